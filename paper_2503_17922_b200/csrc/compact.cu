@@ -5,32 +5,49 @@
 // lower addresses.
 //
 // A parallel copy can still destroy a source row before it has been read: output window w lies on
-// source window w, which an earlier output slot may need.  The kernel therefore gives one thread block
-// a whole (unit, tensor) and lets it walk the output rows in ascending batches: all source rows of a
-// batch are read into registers, the block synchronises, then the batch is written.  Inside a batch
-// every read precedes every write; a later batch reads only rows at or behind its own output rows,
-// which lie behind everything written so far.  Blocks never touch each other's units.
+// source window w, which an earlier output slot may need.  The kernel therefore gives a whole (unit,
+// tensor) to one thread-block cluster and lets it walk the output rows in ascending batches: all source
+// rows of a batch are read into registers, the cluster synchronises, then the batch is written.  Inside
+// a batch every read precedes every write; a later batch reads only rows at or behind its own output
+// rows, which lie behind everything written so far, so one barrier per batch is enough.  Clusters never
+// touch each other's units.
+//
+// Bound by HBM (two passes over the retained rows) once enough SMs have loads in flight: 2 x 64 KB per
+// SM in registers.  One block per (unit, tensor) left 132 of 148 SMs idle when a layer of 8 heads is
+// compacted alone and needed four batches in a row (33 us for 16 MB moved); a cluster of eight takes the
+// same layer in one batch.
 #include "wkv_internal.cuh"
 
 namespace wkv {
 namespace {
 
-constexpr int kThreads = 1024;
-constexpr int kVecs = 8;              // 16-byte vectors per thread and batch: 128 KB per block in flight
+constexpr int kThreads = 512;
+constexpr int kVecs = 8;              // 16-byte vectors per thread and batch: 64 KB per block in flight, two blocks per SM
+constexpr int kMaxCluster = 8;        // portable cluster size
+constexpr int kMinVecs = 2;           // no more blocks per cluster than leave every thread this many vectors
+constexpr int kResident = 264;        // blocks that fit at once in clusters of eight (33 clusters)
 
 struct CompactParams {
     KShape s;
     InplaceTable tab;
     const int *window_idx;
+    int cluster;          // blocks per (unit, tensor)
     int vec_per_row;
     int elem_bytes;
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
+// every access of the cluster's threads before the barrier precedes every access after it
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kThreads, 2)
 compact_inplace_kernel(const __grid_constant__ CompactParams prm)
 {
     const KShape &s = prm.s;
-    const int unit = blockIdx.x, tensor = blockIdx.y;
+    const int cs = prm.cluster, unit = blockIdx.x / cs, rank = blockIdx.x - unit * cs, tensor = blockIdx.y;
     const int b = unit / s.hkv, h = unit % s.hkv;
     const SeqInfo si = seq_info(s, b);
     const int n = si.n;
@@ -46,18 +63,18 @@ compact_inplace_kernel(const __grid_constant__ CompactParams prm)
     const long long row_vecs = s.st * prm.elem_bytes / 16;
     int4 *base = reinterpret_cast<int4 *>(static_cast<char *>(prm.tab.ptr[tensor]) +
                                           (si.off * s.st + b * s.sb + h * s.sh) * (long long)prm.elem_bytes);
-    const int rows_per_batch = max(1, (kThreads * kVecs) / vpr);
+    const int rows_per_batch = max(1, (cs * kThreads * kVecs) / vpr);
     for (int r0 = 0; r0 < kept; r0 += rows_per_batch) {
         const int rows = min(rows_per_batch, kept - r0);
         const int n_vec = rows * vpr;
         int4 val[kVecs];
-        long long doff[kVecs];
+        int dst_row[kVecs];     // -1: nothing to move
 #pragma unroll
         for (int u = 0; u < kVecs; ++u) {
-            const int v = (int)threadIdx.x + u * kThreads;
-            doff[u] = -1;
+            const int v = (int)threadIdx.x + (u * cs + rank) * kThreads;
+            dst_row[u] = -1;
             if (v < n_vec) {
-                const int r = r0 + v / vpr, c = v % vpr;
+                const int r = r0 + v / vpr, c = v - (r - r0) * vpr;
                 int src_row;
                 if (r < review_rows) {
                     const int wi = idx[r / s.omega];
@@ -69,15 +86,17 @@ compact_inplace_kernel(const __grid_constant__ CompactParams prm)
                 }
                 if (src_row >= 0 && src_row < n && src_row != r) {
                     val[u] = base[(long long)src_row * row_vecs + c];
-                    doff[u] = (long long)r * row_vecs + c;
+                    dst_row[u] = r;
                 }
             }
         }
-        __syncthreads();      // every source row of the batch has been read
+        cluster_barrier();      // every source row of the batch has been read
 #pragma unroll
         for (int u = 0; u < kVecs; ++u)
-            if (doff[u] >= 0) base[doff[u]] = val[u];
-        __syncthreads();      // keeps the block in step: the next batch is read after this one is written
+            if (dst_row[u] >= 0) {
+                const int v = (int)threadIdx.x + (u * cs + rank) * kThreads;
+                base[(long long)dst_row[u] * row_vecs + (v - (dst_row[u] - r0) * vpr)] = val[u];
+            }
     }
 }
 
@@ -92,10 +111,28 @@ cudaError_t launch_compact_inplace(const KShape &ks, int elem_bytes, int n_tenso
     prm.window_idx = window_idx;
     prm.vec_per_row = ks.d * elem_bytes / 16;
     prm.elem_bytes = elem_bytes;
-    dim3 grid(ks.batch * ks.hkv, n_tensors);
-    compact_inplace_kernel<<<grid, kThreads, 0, stream>>>(prm);
+    // Blocks per (unit, tensor): as many as are resident at once (with one block of 1,024 threads per SM
+    // only 15 clusters of eight fit, so the sixteenth of a layer of 8 heads ran alone), a power of two up to the portable cluster size, unless the rows are too few to occupy them.
+    const int pairs = ks.batch * ks.hkv * n_tensors;
+    const long long vecs = ((long long)ks.k_max * ks.omega + ks.alpha) * prm.vec_per_row;
+    int cs = 1;
+    while (cs < kMaxCluster && pairs * cs * 2 <= kResident && (long long)cs * kThreads * kMinVecs < vecs) cs *= 2;
+    prm.cluster = cs;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ks.batch * ks.hkv * cs, n_tensors);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, compact_inplace_kernel, prm);
+    if (err != cudaSuccess) return err;
     count_launches(1);
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 }  // namespace wkv

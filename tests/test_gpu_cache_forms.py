@@ -165,3 +165,14 @@ def test_paged_cache_argument_checks():
         binding.wkv_gather_kv_paged(prob, t, None, z, [torch.zeros(8, dtype=torch.bfloat16, device="cuda")], None,
                                     z.view(2, 32)[:, :2].contiguous(), 24, 10, 24 * 128 * 2, 24 * 128, 128)
     assert e.value.status == 2
+
+
+@pytest.mark.parametrize("pattern", ["shift", "tail"])
+@pytest.mark.parametrize("case", [
+    dict(batch=1, max_seqlen=9000, budget_frac=0.9),                       # eight blocks per unit, four batches
+    dict(batch=1, n_q_heads=4, n_kv_heads=1, max_seqlen=257, budget_frac=0.5),   # fewer rows than eight blocks' threads
+    dict(batch=9, max_seqlen=2500, n_layers=4, gamma=4, budget_frac=0.6),  # 144 (unit, tensor) pairs: one block each
+], ids=["clusters-of-8", "few-rows", "no-cluster"])
+def test_compaction_in_place_over_cluster_sizes(case, pattern):
+    """A unit spread over a cluster of blocks: several batches in a row, fewer rows than threads, and one block."""
+    test_compaction_in_place(case, pattern)
