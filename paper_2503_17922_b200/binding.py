@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from typing import List, Optional, Sequence
 
 import numpy as np
@@ -153,27 +154,51 @@ def _ptr(t) -> Optional[int]:
     """Device (or host) address of a torch tensor / numpy array / int / None."""
     if t is None:
         return None
-    if isinstance(t, int):
-        return t
-    if isinstance(t, np.ndarray):
-        return t.ctypes.data
-    return t.data_ptr()
+    try:
+        return t.data_ptr()
+    except AttributeError:
+        pass
+    return t.ctypes.data if isinstance(t, np.ndarray) else t      # or an address already
+
+
+_current_raw_stream = None
+
+
+def _find_current_raw_stream():
+    """The callable behind `torch.cuda.current_stream()` that gives the handle without building a Stream
+    object (0.2 us instead of 2 us of a call); the public way where torch does not have it."""
+    import torch
+    torch.cuda.current_stream()       # initialises CUDA
+    get_device, get_stream = getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if get_device is None or get_stream is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: get_stream(get_device())
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        global _current_raw_stream
+        if _current_raw_stream is None:
+            _current_raw_stream = _find_current_raw_stream()
+        return _current_raw_stream()
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
-def _ptr_array(tensors: Optional[Sequence]) -> Optional[ctypes.Array]:
+_PACK_POINTERS = [struct.Struct(f"{n}P").pack for n in range(WKV_MAX_GROUP_LAYERS + 1)]
+
+
+def _ptr_array(tensors: Optional[Sequence]):
+    """A C array of the tensors' addresses: packed bytes, which cost a third of a ctypes array filled entry by
+    entry (a group call hands over four of them)."""
     if tensors is None:
         return None
-    arr = (ctypes.c_void_p * len(tensors))()
-    for i, t in enumerate(tensors):
-        arr[i] = _ptr(t)
-    return arr
+    try:
+        return _PACK_POINTERS[len(tensors)](*[t.data_ptr() for t in tensors])
+    except (AttributeError, IndexError):      # addresses, numpy arrays or None among them, or too many
+        arr = (ctypes.c_void_p * len(tensors))()
+        for i, t in enumerate(tensors):
+            arr[i] = _ptr(t)
+        return arr
 
 
 class Problem:
