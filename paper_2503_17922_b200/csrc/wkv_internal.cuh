@@ -115,26 +115,40 @@ struct TcPlan {
     int units_per_wave;   // units swept together
     int chunks_per_unit;  // work items per unit
 };
-__host__ __device__ inline TcPlan tc_plan(int units, int max_seqlen, int head_dim)
+// What a wave costs beside its key tiles, in tiles per block: filling the pipeline, the hand-over of the
+// statistics and the pooling take about 8 us, a tile 0.65 us per sweep.
+constexpr int kTcWaveOverhead = 6;
+inline TcPlan tc_plan(int units, int max_seqlen, int head_dim)
 {
-    TcPlan p;
+    // Every number of units per wave whose keys fit the L2 budget and whose blocks are resident together is
+    // tried, and the one with the least (waves x (tiles per block + overhead)) taken.  The largest that fits
+    // is not the best when it leaves a last wave nearly empty: 16 units of 192 tiles as 12 + 4 made 16 tiles
+    // per block and wave, 8 + 8 makes 11.
+    TcPlan best;
+    best.units_per_wave = 1;
+    best.chunks_per_unit = 1;
     const long long unit_bytes = (long long)max_seqlen * head_dim * 2;
-    long long upw = kTcWaveBytes / (unit_bytes > 0 ? unit_bytes : 1);
     const int max_tiles = (max_seqlen + kTcTileKeys - 1) / kTcTileKeys;
-    // A unit needs at least ceil(max_tiles / kTcMaxChunkTiles) blocks: no more units in a wave than
-    // the SMs can take at that rate, or some blocks get two items of a wave and the others wait for
-    // them.
+    // a unit needs at least this many blocks (the token scores of a chunk live in shared memory)
     const int min_chunks = (max_tiles + kTcMaxChunkTiles - 1) / kTcMaxChunkTiles;
-    if (upw > kTcTargetBlocks / min_chunks) upw = kTcTargetBlocks / min_chunks;
-    if (upw < 1) upw = 1;
-    if (upw > units) upw = units;
-    p.units_per_wave = (int)upw;
-    int a = kTcTargetBlocks / p.units_per_wave;
-    const int b = (max_tiles + kTcMaxChunkTiles - 1) / kTcMaxChunkTiles;
-    if (a < 1) a = 1;
-    if (a > max_tiles) a = max_tiles;
-    p.chunks_per_unit = a > b ? a : b;
-    return p;
+    long long most = kTcWaveBytes / (unit_bytes > 0 ? unit_bytes : 1);
+    if (most > kTcTargetBlocks / min_chunks) most = kTcTargetBlocks / min_chunks;
+    if (most > units) most = units;
+    if (most < 1) most = 1;
+    long long best_cost = -1;
+    for (int upw = (int)most; upw >= 1; --upw) {
+        int chunks = kTcTargetBlocks / upw;
+        if (chunks < min_chunks) chunks = min_chunks;
+        if (chunks > max_tiles) chunks = max_tiles;
+        const long long waves = (units + upw - 1) / upw, tiles = (max_tiles + chunks - 1) / chunks;
+        const long long cost = waves * (tiles + kTcWaveOverhead);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best.units_per_wave = upw;
+            best.chunks_per_unit = chunks;
+        }
+    }
+    return best;
 }
 // The pipelined group kernel takes the units in waves too, but keeps TWO waves in flight (the
 // statistics sweep runs one wave ahead of the scoring sweep), so two waves' keys share the L2 budget;
