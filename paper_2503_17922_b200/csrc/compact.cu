@@ -47,6 +47,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 compact_inplace_kernel(const __grid_constant__ CompactParams prm)
 {
     const KShape &s = prm.s;
+    pdl_trigger();
+    pdl_wait();
     const int cs = prm.cluster, unit = blockIdx.x / cs, rank = blockIdx.x - unit * cs, tensor = blockIdx.y;
     const int b = unit / s.hkv, h = unit % s.hkv;
     const SeqInfo si = seq_info(s, b);
@@ -118,18 +120,8 @@ cudaError_t launch_compact_inplace(const KShape &ks, int elem_bytes, int n_tenso
     int cs = 1;
     while (cs < kMaxCluster && pairs * cs * 2 <= kResident && (long long)cs * kThreads * kMinVecs < vecs) cs *= 2;
     prm.cluster = cs;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ks.batch * ks.hkv * cs, n_tensors);
-    cfg.blockDim = dim3(kThreads);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, compact_inplace_kernel, prm);
+    const cudaError_t err = launch_pdl(compact_inplace_kernel, dim3(ks.batch * ks.hkv * cs, n_tensors), kThreads, 0, stream,
+                                       cs, prm);
     if (err != cudaSuccess) return err;
     count_launches(1);
     return cudaSuccess;

@@ -54,6 +54,8 @@ __global__ void __launch_bounds__(kThreads, 4)
 gather_kv_kernel(const __grid_constant__ GatherParams prm)
 {
     const KShape &s = prm.s;
+    pdl_trigger();
+    pdl_wait();
     const int unit = blockIdx.y, tensor = blockIdx.z;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = unit / s.hkv, h = unit % s.hkv;
@@ -203,10 +205,10 @@ cudaError_t launch_gather(const KShape &ks, int elem_bytes, int n_tensors, const
     prm.slots_per_block = (int)per_block;
     const int max_slots = ks.k_max + prm.obs_slots;
     dim3 grid((max_slots + prm.slots_per_block - 1) / prm.slots_per_block, ks.batch * ks.hkv, n_tensors);
-    if (paged) gather_kv_kernel<true><<<grid, kThreads, 0, stream>>>(prm);
-    else gather_kv_kernel<false><<<grid, kThreads, 0, stream>>>(prm);
+    const cudaError_t err = launch_pdl(paged ? gather_kv_kernel<true> : gather_kv_kernel<false>, grid, kThreads, 0, stream, 1, prm);
+    if (err != cudaSuccess) return err;
     count_launches(1);
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 }  // namespace wkv

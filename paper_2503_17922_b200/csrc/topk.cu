@@ -11,6 +11,8 @@ select_topk_kernel(KShape s, const float *__restrict__ window_scores, int *__res
                    int *__restrict__ kept_len)
 {
     __shared__ TopkSmem sm;
+    pdl_trigger();
+    pdl_wait();
     const int unit = blockIdx.x;
     const int b = unit / s.hkv;
     const SeqInfo si = seq_info(s, b);
@@ -26,9 +28,11 @@ cudaError_t launch_topk(const KShape &ks, const float *window_scores, int *windo
                         cudaStream_t stream)
 {
     const int units = ks.batch * ks.hkv;
-    select_topk_kernel<<<units, kThreads, 0, stream>>>(ks, window_scores, window_idx, kept_len);
+    const cudaError_t err =
+        launch_pdl(select_topk_kernel, dim3(units), kThreads, 0, stream, 1, ks, window_scores, window_idx, kept_len);
+    if (err != cudaSuccess) return err;
     count_launches(1);
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 }  // namespace wkv
