@@ -5,6 +5,16 @@
 //   score : logits again, p = exp2(x - lse2), sum over the rows (Eq. 2), then the
 //           Top-p window pooling of Eq. 3-4
 // Summation orders are fixed, so results are bit-identical from run to run.
+//
+// These problems are small (a few thousand keys), so what bounds them is the length of the chain from
+// launch to result and how many SMs take part: a block takes as little as one tile of 64 keys, the eight
+// blocks of a 512-key statistics chunk form a cluster and combine their rows through distributed shared
+// memory, and the score kernel is launched as a programmatic dependent that computes its logits while the
+// statistics kernel is still running.  The row tile follows R (16, 32 or 64 rows), so few rows cost no
+// padding.
+// 2 heads x 1,024 keys, 16 rows, d = 64: one block per 512 keys took 31 + 25 us for the two kernels (whole
+// group 84 us); see simt_tiles_per_block for the sizes where a block takes more tiles.
+#include "score_math.cuh"
 #include "wkv_internal.cuh"
 
 #include <mutex>
@@ -15,9 +25,9 @@ namespace wkv {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kRT = 64;       // rows per logit tile
 constexpr int kKT = 64;       // keys per logit tile
 constexpr int kKPad = kKT + 4;
+constexpr int kChunkTiles = kStatChunk / kKT;
 
 __device__ inline float to_float(float x) { return x; }
 __device__ inline float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
@@ -43,14 +53,15 @@ __device__ inline Vec<T> load_vec(const T *p)
     return r;
 }
 
-// Q of the unit, transposed into shared memory: qs[c * r_pad + r]; rows >= R are zero.
+// Q of the unit, transposed into shared memory: qs[c * r_pad + r]; rows >= R are zero.  Lanes take
+// consecutive rows, so that the transposed stores hit different banks.
 template <typename T>
 __device__ void load_q_transposed(const KShape &s, const T *q_unit, float *qs, int r_pad)
 {
     constexpr int VN = Vec<T>::N;
     const int vec_per_row = s.d / VN;
     for (int idx = threadIdx.x; idx < r_pad * vec_per_row; idx += kThreads) {
-        int r = idx / vec_per_row, cv = idx % vec_per_row;
+        const int cv = idx / r_pad, r = idx - cv * r_pad;
         Vec<T> v;
         if (r < s.R) {
             int g = r / s.alpha, i = r % s.alpha;
@@ -70,8 +81,9 @@ __device__ void load_k_transposed(const KShape &s, const T *k_unit, float *ks, i
 {
     constexpr int VN = Vec<T>::N;
     const int vec_per_row = s.d / VN;
+#pragma unroll 4
     for (int idx = threadIdx.x; idx < kKT * vec_per_row; idx += kThreads) {
-        int jj = idx / vec_per_row, cv = idx % vec_per_row;
+        const int jj = idx % kKT, cv = idx / kKT;
         Vec<T> v;
         if (j0 + jj < n_valid) {
             v = load_vec(k_unit + (long long)(j0 + jj) * s.st + cv * VN);
@@ -84,174 +96,267 @@ __device__ void load_k_transposed(const KShape &s, const T *k_unit, float *ks, i
     }
 }
 
-// 4x4 register tile of raw dot products for rows r0+ty*4.., keys tx*4..
-__device__ inline void logits_4x4(const float *qs, const float *ks, int d, int r_pad, int r0, int ty,
-                                  int tx, float acc[4][4])
+// How the threads share a tile of RB rows x kKT keys: 4 rows x KPT keys each.
+template <int RB>
+struct TileMap {
+    static constexpr int KPT = RB / 16;            // 4, 2, 1
+    static constexpr int TX = kKT / KPT;           // threads along the keys: 16, 32, 64
+    static_assert(RB == 16 || RB == 32 || RB == 64, "row tile");
+    static_assert(kThreads / TX * 4 == RB, "threads do not cover the tile");
+};
+
+// raw dot products of rows r0 + ty*4 .. +3 with keys tx*KPT .. +KPT-1
+template <int RB>
+__device__ inline void logits_tile(const float *qs, const float *ks, int d, int r_pad, int r0, int ty, int tx,
+                                   float (&acc)[4][TileMap<RB>::KPT])
 {
+    constexpr int KPT = TileMap<RB>::KPT;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+        for (int b = 0; b < KPT; ++b) acc[a][b] = 0.f;
     const float *qp = qs + r0 + ty * 4;
-    const float *kp = ks + tx * 4;
-#pragma unroll 4
+    const float *kp = ks + tx * KPT;
+#pragma unroll 8
     for (int c = 0; c < d; ++c) {
-        float4 qv = *reinterpret_cast<const float4 *>(qp + c * r_pad);
-        float4 kv = *reinterpret_cast<const float4 *>(kp + c * kKPad);
-        float qa[4] = {qv.x, qv.y, qv.z, qv.w};
-        float ka[4] = {kv.x, kv.y, kv.z, kv.w};
+        const float4 qv = *reinterpret_cast<const float4 *>(qp + c * r_pad);
+        const float qa[4] = {qv.x, qv.y, qv.z, qv.w};
+        float ka[KPT];
+        if constexpr (KPT == 4) {
+            const float4 kv = *reinterpret_cast<const float4 *>(kp + c * kKPad);
+            ka[0] = kv.x, ka[1] = kv.y, ka[2] = kv.z, ka[3] = kv.w;
+        } else if constexpr (KPT == 2) {
+            const float2 kv = *reinterpret_cast<const float2 *>(kp + c * kKPad);
+            ka[0] = kv.x, ka[1] = kv.y;
+        } else {
+            ka[0] = kp[c * kKPad];
+        }
 #pragma unroll
         for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(qa[a], ka[b], acc[a][b]);
+            for (int b = 0; b < KPT; ++b) acc[a][b] = fmaf(qa[a], ka[b], acc[a][b]);
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-score_stats_simt(KShape s, const T *__restrict__ q, const T *__restrict__ k, float2 *__restrict__ stats,
-                 int n_chunks, int r_pad)
+// (max, sum) pairs of exponentials, to base 2: the pair of the union
+__device__ inline void merge_stats(float &m, float &l, float m2, float l2)
 {
-    extern __shared__ __align__(16) float smem[];
-    float *qs = smem;                    // [d][r_pad]
-    float *ks = smem + s.d * r_pad;      // [d][kKPad]
+    const float mn = fmaxf(m, m2);
+    const float safe = mn == -INFINITY ? 0.f : mn;
+    l = l * exp2f(m - safe) + l2 * exp2f(m2 - safe);
+    m = mn;
+}
 
-    const int unit = blockIdx.y, chunk = blockIdx.x;
+__device__ __forceinline__ float2 ld_cluster(const float2 *p, int rank)
+{
+    uint32_t addr;
+    float2 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+
+// Grid: x = statistics chunk x blocks per chunk (the blocks of a chunk are one cluster), y = unit.
+template <typename T, int RB>
+__global__ void __launch_bounds__(kThreads)
+score_stats_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const T *__restrict__ k,
+                 float2 *__restrict__ stats, int n_chunks, int r_pad, int r_tile, int tiles_per_block)
+{
+    constexpr int KPT = TileMap<RB>::KPT, TX = TileMap<RB>::TX;
+    extern __shared__ __align__(16) float smem[];
+    float *qs = smem;                                                   // [d][r_tile]
+    float *ks = qs + s.d * r_tile;                                      // [d][kKPad]
+    float2 *rows = reinterpret_cast<float2 *>(ks + s.d * kKPad);        // [r_pad] this block's (max, sum) ...
+    float2 *half = rows + (tiles_per_block < kChunkTiles ? r_pad : 0);                                        // ... and, 16-row tiles: the second warps'
+
+    pdl_wait();
+    pdl_trigger();      // the score kernel may read Q and K from here on: what wrote them has completed
+    const int unit = blockIdx.y, cs = kChunkTiles / tiles_per_block;
+    const int chunk = blockIdx.x / cs, rank = blockIdx.x - chunk * cs;
     const int b = unit / s.hkv, h = unit % s.hkv;
     const SeqInfo si = seq_info(s, b);
     const int n = si.n, n_r = n - s.alpha;
+    const int j_begin = chunk * kStatChunk + rank * tiles_per_block * kKT;
+    const int j_end = min(n, j_begin + tiles_per_block * kKT);
+    const bool idle = n_r <= 0 || j_begin >= n;
     float2 *out = stats + ((size_t)unit * n_chunks + chunk) * r_pad;
-    const int j_begin = chunk * kStatChunk;
-    if (n_r <= 0 || j_begin >= n) {
-        for (int r = threadIdx.x; r < r_pad; r += kThreads) out[r] = make_float2(-INFINITY, 0.f);
-        return;
-    }
-    const int j_end = min(n, j_begin + kStatChunk);
-    const T *q_unit = q + b * s.qsb + (long long)h * s.G * s.qsh;
-    const T *k_unit = k + (si.off * s.st + b * s.sb + h * s.sh);
-    load_q_transposed(s, q_unit, qs, r_pad);
-
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    for (int r0 = 0; r0 < r_pad; r0 += kRT) {
-        float m[4], l[4];
-        int pos[4];   // last key each row may attend to
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            m[a] = -INFINITY;
-            l[a] = 0.f;
-            int r = r0 + ty * 4 + a;
-            pos[a] = r < s.R ? n_r + (r % s.alpha) : -1;
-        }
+    if (cs == 1) rows = out;      // nothing to combine: the rows are kept where they go
+    for (int r = threadIdx.x; r < r_pad; r += kThreads) rows[r] = make_float2(-INFINITY, 0.f);
+    if (!idle) {
+        load_q_transposed(s, q + b * s.qsb + (long long)h * s.G * s.qsh, qs, r_tile);
+        const T *k_unit = k + (si.off * s.st + b * s.sb + h * s.sh);
+        const int ty = threadIdx.x / TX, tx = threadIdx.x % TX;
         for (int j0 = j_begin; j0 < j_end; j0 += kKT) {
             __syncthreads();
             load_k_transposed(s, k_unit, ks, j0, n);
             __syncthreads();
-            float acc[4][4];
-            logits_4x4(qs, ks, s.d, r_pad, r0, ty, tx, acc);
+            for (int r0 = 0; r0 < r_tile; r0 += RB) {
+                float acc[4][KPT];
+                logits_tile<RB>(qs, ks, s.d, r_tile, r0, ty, tx, acc);
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                float x[4], tmax = -INFINITY;
+                for (int a = 0; a < 4; ++a) {
+                    const int r = r0 + ty * 4 + a;
+                    const int last = r < s.R ? n_r + (r % s.alpha) : -1;     // last key the row may attend to
+                    float x[KPT], m = -INFINITY;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    int j = j0 + tx * 4 + c;
-                    x[c] = j <= pos[a] ? acc[a][c] * s.scale_log2 : -INFINITY;
-                    tmax = fmaxf(tmax, x[c]);
+                    for (int c = 0; c < KPT; ++c) {
+                        x[c] = j0 + tx * KPT + c <= last ? acc[a][c] * s.scale_log2 : -INFINITY;
+                        m = fmaxf(m, x[c]);
+                    }
+#pragma unroll
+                    for (int o = 1; o < (TX < 32 ? TX : 32); o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                    const float safe = m == -INFINITY ? 0.f : m;
+                    float l = 0.f;
+#pragma unroll
+                    for (int c = 0; c < KPT; ++c) l += exp2f(x[c] - safe);
+#pragma unroll
+                    for (int o = 1; o < (TX < 32 ? TX : 32); o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+                    // one thread per row adds the tile to the block's running pair
+                    if (TX <= 32) {
+                        if (tx == 0) {
+                            float2 p = rows[r];
+                            merge_stats(p.x, p.y, m, l);
+                            rows[r] = p;
+                        }
+                    } else if (tx % 32 == 0) {
+                        float2 *mine = tx == 0 ? rows : half;
+                        float2 p = j0 == j_begin ? make_float2(-INFINITY, 0.f) : mine[r];
+                        merge_stats(p.x, p.y, m, l);
+                        mine[r] = p;
+                    }
                 }
-#pragma unroll
-                for (int o = 1; o < 16; o <<= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
-                // no early exit: both half-warps must reach the shuffles below
-                float m_new = fmaxf(m[a], tmax);
-                float m_safe = m_new == -INFINITY ? 0.f : m_new;
-                float sum = 0.f;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) sum += exp2f(x[c] - m_safe);
-#pragma unroll
-                for (int o = 1; o < 16; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                l[a] = l[a] * exp2f(m[a] - m_safe) + sum;
-                m[a] = m_new;
             }
         }
-        if (tx == 0) {
-#pragma unroll
-            for (int a = 0; a < 4; ++a) out[r0 + ty * 4 + a] = make_float2(m[a], l[a]);
+        if (TX > 32) {
+            __syncthreads();
+            for (int r = threadIdx.x; r < r_tile; r += kThreads) {
+                float2 p = rows[r];
+                merge_stats(p.x, p.y, half[r].x, half[r].y);
+                rows[r] = p;
+            }
         }
+    }
+    if (cs == 1) return;
+    // the chunk's rows: the blocks of the cluster share them out, each combines its rows over all blocks in order
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    for (int r = rank * kThreads + threadIdx.x; r < r_pad; r += cs * kThreads) {
+        float m = -INFINITY, l = 0.f;
+        for (int c = 0; c < cs; ++c) {
+            const float2 p = ld_cluster(rows + r, c);
+            merge_stats(m, l, p.x, p.y);
+        }
+        out[r] = make_float2(m, l);
+    }
+    // no block leaves while another may still read its rows
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Eq. 4 for one window: the sorting network where there is one for its length, else the serial form
+__device__ inline float pool_window(const float *w, int omega, int size, int p)
+{
+    switch (omega) {
+    case 4: return pool_window_sorted<4>(w, size, p);
+    case 8: return pool_window_sorted<8>(w, size, p);
+    case 16: return pool_window_sorted<16>(w, size, p);
+    case 32: return pool_window_sorted<32>(w, size, p);
+    default: return pool_top_p(w, size, p);
     }
 }
 
-template <typename T>
+template <typename T, int RB>
 __global__ void __launch_bounds__(kThreads)
-score_pool_simt(KShape s, const T *__restrict__ q, const T *__restrict__ k,
-                const float2 *__restrict__ stats, const float *__restrict__ lse_obs,
-                float *__restrict__ window_scores, float *__restrict__ token_scores, int n_chunks, int r_pad,
-                int chunk_keys)
+score_pool_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const T *__restrict__ k, const float2 *stats,
+                const float *lse_obs, float *__restrict__ window_scores, float *__restrict__ token_scores, int n_chunks,
+                int r_pad, int r_tile, int chunk_keys)
 {
+    constexpr int KPT = TileMap<RB>::KPT, TX = TileMap<RB>::TX, TY = kThreads / TX;
     extern __shared__ __align__(16) float smem[];
-    float *qs = smem;                          // [d][r_pad]
-    float *ks = qs + s.d * r_pad;              // [d][kKPad]
+    float *qs = smem;                          // [d][r_tile]
+    float *ks = qs + s.d * r_tile;             // [d][kKPad]
     float *lse2 = ks + s.d * kKPad;            // [r_pad]
-    float *part = lse2 + r_pad;                // [16][kKT]
-    float *t_chunk = part + 16 * kKT;          // [chunk_keys rounded up to kKT]
+    float *part = lse2 + r_pad;                // [TY][kKT]
+    float *t_chunk = part + TY * kKT;          // [chunk_keys rounded up to kKT]
 
+    pdl_trigger();
+    // with given normalisers there is no statistics kernel in front that has waited for Q and K
+    if (lse_obs) pdl_wait();
     const int unit = blockIdx.y;
     const int b = unit / s.hkv, h = unit % s.hkv;
     const SeqInfo si = seq_info(s, b);
     const int n = si.n, n_r = n - s.alpha;
     const int j_begin = blockIdx.x * chunk_keys;
-    if (n_r <= 0 || j_begin >= n_r) return;
-    const int j_end = min(n_r, j_begin + chunk_keys);
-    const T *q_unit = q + b * s.qsb + (long long)h * s.G * s.qsh;
-    const T *k_unit = k + (si.off * s.st + b * s.sb + h * s.sh);
-    load_q_transposed(s, q_unit, qs, r_pad);
-
-    // combine the partial statistics of every chunk: lse2 = log2 of the row normaliser
-    // (or, when the caller supplies the natural log of the normalisers, that value in base 2)
-    for (int r = threadIdx.x; r < r_pad; r += kThreads) {
-        if (lse_obs) {
-            const int g = r / s.alpha, i = r - g * s.alpha;
-            lse2[r] = r < s.R ? lse_obs[((size_t)b * s.hq + (size_t)h * s.G + g) * s.alpha + i] * 1.4426950408889634f
-                              : INFINITY;
-            continue;
-        }
-        const float2 *st = stats + (size_t)unit * n_chunks * r_pad + r;
-        float M = -INFINITY;
-        for (int c = 0; c < n_chunks; ++c) M = fmaxf(M, st[(size_t)c * r_pad].x);
-        float L = 0.f;
-        for (int c = 0; c < n_chunks; ++c) {
-            float2 v = st[(size_t)c * r_pad];
-            if (v.y > 0.f) L += v.y * exp2f(v.x - M);
-        }
-        lse2[r] = (r < s.R && L > 0.f) ? M + log2f(L) : INFINITY;
+    if (n_r <= 0 || j_begin >= n_r) {
+        if (!lse_obs) pdl_wait();
+        return;
     }
+    const int j_end = min(n_r, j_begin + chunk_keys);
+    const T *k_unit = k + (si.off * s.st + b * s.sb + h * s.sh);
+    load_q_transposed(s, q + b * s.qsb + (long long)h * s.G * s.qsh, qs, r_tile);
 
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+    const int ty = threadIdx.x / TX, tx = threadIdx.x % TX;
     for (int j0 = j_begin; j0 < j_end; j0 += kKT) {
         __syncthreads();
         load_k_transposed(s, k_unit, ks, j0, n_r);
         __syncthreads();
-        float t_acc = 0.f;   // threads 0..kKT-1: token score of key j0 + tid
-        for (int r0 = 0; r0 < r_pad; r0 += kRT) {
-            float acc[4][4];
-            logits_4x4(qs, ks, s.d, r_pad, r0, ty, tx, acc);
-            float col[4] = {0.f, 0.f, 0.f, 0.f};
+        float col[KPT];
+#pragma unroll
+        for (int c = 0; c < KPT; ++c) col[c] = 0.f;
+        for (int r0 = 0; r0 < r_tile; r0 += RB) {
+            float acc[4][KPT];
+            logits_tile<RB>(qs, ks, s.d, r_tile, r0, ty, tx, acc);
+            if (j0 == j_begin && r0 == 0) {
+                // Only now are the statistics needed.  lse2 = log2 of the row normaliser: the threads of a row
+                // (kThreads / r_pad of them, neighbours) merge every that-many-th chunk, then one another; or the
+                // caller's value (natural log) in base 2
+                if (!lse_obs) pdl_wait();
+                const int tpr = r_pad <= 64 ? 4 : (r_pad <= 128 ? 2 : 1);
+                const int used = (n + kStatChunk - 1) / kStatChunk;
+                for (int rr = threadIdx.x; rr < r_pad * tpr; rr += kThreads) {
+                    const int r = rr / tpr, part_of = rr - r * tpr;
+                    float v = INFINITY;
+                    if (lse_obs) {
+                        const int g = r / s.alpha, i = r - g * s.alpha;
+                        if (r < s.R) v = lse_obs[((size_t)b * s.hq + (size_t)h * s.G + g) * s.alpha + i] * 1.4426950408889634f;
+                    } else {
+                        const float2 *st = stats + (size_t)unit * n_chunks * r_pad + r;
+                        float M = -INFINITY, L = 0.f;
+                        for (int c0 = part_of; c0 < used; c0 += 4 * tpr) {
+                            float2 p[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                p[u] = c0 + u * tpr < used ? __ldcg(st + (size_t)(c0 + u * tpr) * r_pad) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) merge_stats(M, L, p[u].x, p[u].y);
+                        }
+                        for (int o = 1; o < tpr; o <<= 1) {
+                            const float m2 = __shfl_xor_sync(0xffffffffu, M, o), l2 = __shfl_xor_sync(0xffffffffu, L, o);
+                            merge_stats(M, L, m2, l2);
+                        }
+                        if (r < s.R && L > 0.f) v = M + log2f(L);
+                    }
+                    if (part_of == 0) lse2[r] = v;
+                }
+                __syncthreads();
+            }
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                float ls = lse2[r0 + ty * 4 + a];
+                const float ls = lse2[r0 + ty * 4 + a];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) col[c] += exp2f(fmaf(acc[a][c], s.scale_log2, -ls));
+                for (int c = 0; c < KPT; ++c) col[c] += exp2f(fmaf(acc[a][c], s.scale_log2, -ls));
             }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) part[ty * kKT + tx * 4 + c] = col[c];
-            __syncthreads();
-            if (threadIdx.x < kKT) {
-#pragma unroll
-                for (int y = 0; y < 16; ++y) t_acc += part[y * kKT + threadIdx.x];
-            }
-            __syncthreads();
         }
+#pragma unroll
+        for (int c = 0; c < KPT; ++c) part[ty * kKT + tx * KPT + c] = col[c];
+        __syncthreads();
         if (threadIdx.x < kKT) {
-            int j = j0 + threadIdx.x;
-            t_chunk[j - j_begin] = t_acc;
-            if (token_scores && j < n_r) token_scores[(size_t)unit * s.nr_max + j] = t_acc;
+            float t = 0.f;
+#pragma unroll
+            for (int y = 0; y < TY; ++y) t += part[y * kKT + threadIdx.x];
+            const int j = j0 + threadIdx.x;
+            t_chunk[j - j_begin] = t;
+            if (token_scores && j < n_r) token_scores[(size_t)unit * s.nr_max + j] = t;
         }
     }
     __syncthreads();
@@ -259,9 +364,9 @@ score_pool_simt(KShape s, const T *__restrict__ q, const T *__restrict__ k,
     const int w_begin = j_begin / s.omega;
     const int n_win = (j_end - j_begin + s.omega - 1) / s.omega;
     for (int lw = threadIdx.x; lw < n_win; lw += kThreads) {
-        int lo = lw * s.omega;
-        int size = min(s.omega, (j_end - j_begin) - lo);
-        window_scores[(size_t)unit * s.kw_max + w_begin + lw] = pool_top_p(t_chunk + lo, size, s.p);
+        const int lo = lw * s.omega;
+        window_scores[(size_t)unit * s.kw_max + w_begin + lw] =
+            pool_window(t_chunk + lo, s.omega, min(s.omega, (j_end - j_begin) - lo), s.p);
     }
 }
 
@@ -272,7 +377,7 @@ score_pool_simt(KShape s, const T *__restrict__ q, const T *__restrict__ k,
 static cudaError_t allow_dynamic_smem(const void *fn, int dev, int slot, size_t bytes)
 {
     static std::mutex mu;
-    static size_t allowed[kMaxDevices][4] = {};
+    static size_t allowed[kMaxDevices][12] = {};
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (bytes <= allowed[dev][slot]) return cudaSuccess;
@@ -281,59 +386,97 @@ static cudaError_t allow_dynamic_smem(const void *fn, int dev, int slot, size_t 
     return err;
 }
 
-static int simt_chunk_keys(const KShape &ks)
+// Tiles of 64 keys per block: one while the grid is small (latency), more when it fills the GPU many times over
+// anyway, since every block transposes the whole of Q first.  With up to eight blocks per SM resident, 1,184
+// blocks are one wave.
+static int simt_tiles_per_block(const KShape &ks)
 {
-    int per = 512 / ks.omega;
+    const long long tiles = (long long)ks.batch * ks.hkv * ((ks.max_seqlen + kKT - 1) / kKT);
+    if (ks.R > 1024) return kChunkTiles;     // the rows of a cluster's blocks would not fit shared memory beside Q
+    int t = 1;
+    while (t < kChunkTiles && tiles / (2 * t) >= 1184) t *= 2;
+    return t;
+}
+
+// keys per block of the score kernel: whole windows
+static int simt_chunk_keys(const KShape &ks, int tiles_per_block)
+{
+    int per = tiles_per_block * kKT / ks.omega;
     if (per < 1) per = 1;
     return per * ks.omega;
+}
+
+static int simt_row_tile(const KShape &ks) { return ks.R <= 16 ? 16 : (ks.R <= 32 ? 32 : 64); }
+
+static void simt_smem(const KShape &ks, int r_pad, size_t &stats_bytes, size_t &pool_bytes)
+{
+    const int rb = simt_row_tile(ks), r_tile = rb < 64 ? rb : r_pad;
+    const int tpb = simt_tiles_per_block(ks), chunk_keys = simt_chunk_keys(ks, tpb);
+    const size_t tiles = (size_t)ks.d * r_tile + (size_t)ks.d * kKPad;
+    stats_bytes = sizeof(float) * (tiles + (tpb < kChunkTiles ? 2 * (size_t)r_pad : 0) + (rb == 16 ? 2 * (size_t)r_pad : 0));
+    pool_bytes = sizeof(float) * (tiles + (size_t)r_pad + (size_t)(rb / 4) * kKT + (size_t)((chunk_keys + kKT - 1) / kKT) * kKT);
+}
+
+template <typename T, int RB>
+static cudaError_t launch_simt_tile(const KShape &ks, int slot, const void *q, const void *k, float *window_scores,
+                                    float *token_scores, float2 *stats, const Workspace &ws, cudaStream_t stream,
+                                    const float *lse_obs)
+{
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    const int units = ks.batch * ks.hkv, r_pad = ws.r_pad, r_tile = RB < 64 ? RB : r_pad;
+    const int tpb = simt_tiles_per_block(ks), chunk_keys = simt_chunk_keys(ks, tpb);
+    size_t smem1, smem2;
+    simt_smem(ks, r_pad, smem1, smem2);
+    if (!lse_obs) {
+        auto fn = score_stats_simt<T, RB>;
+        err = allow_dynamic_smem(reinterpret_cast<const void *>(fn), dev, slot, smem1);
+        if (err != cudaSuccess) return err;
+        const int cs = kChunkTiles / tpb, chunks = (ks.max_seqlen + kStatChunk - 1) / kStatChunk;
+        err = launch_pdl(fn, dim3(chunks * cs, units), kThreads, smem1, stream, cs, ks, (const T *)q, (const T *)k, stats,
+                         ws.n_stat_chunks, r_pad, r_tile, tpb);
+        if (err != cudaSuccess) return err;
+    }
+    auto fn = score_pool_simt<T, RB>;
+    err = allow_dynamic_smem(reinterpret_cast<const void *>(fn), dev, slot + 1, smem2);
+    if (err != cudaSuccess) return err;
+    const int n_r_max = ks.max_seqlen - ks.alpha;
+    err = launch_pdl(fn, dim3((n_r_max + chunk_keys - 1) / chunk_keys, units), kThreads, smem2, stream, 1, ks, (const T *)q,
+                     (const T *)k, (const float2 *)stats, lse_obs, window_scores, token_scores, ws.n_stat_chunks, r_pad, r_tile,
+                     chunk_keys);
+    if (err == cudaSuccess) count_launches(lse_obs ? 1 : 2);
+    return err;
+}
+
+template <typename T>
+static cudaError_t launch_simt_type(const KShape &ks, int slot, const void *q, const void *k, float *window_scores,
+                                    float *token_scores, float2 *stats, const Workspace &ws, cudaStream_t stream,
+                                    const float *lse_obs)
+{
+    switch (simt_row_tile(ks)) {
+    case 16: return launch_simt_tile<T, 16>(ks, slot, q, k, window_scores, token_scores, stats, ws, stream, lse_obs);
+    case 32: return launch_simt_tile<T, 32>(ks, slot + 2, q, k, window_scores, token_scores, stats, ws, stream, lse_obs);
+    default: return launch_simt_tile<T, 64>(ks, slot + 4, q, k, window_scores, token_scores, stats, ws, stream, lse_obs);
+    }
 }
 
 cudaError_t launch_score_simt(const KShape &ks, int dtype, const void *q, const void *k,
                               float *window_scores, float *token_scores,
                               void *workspace, const Workspace &ws, cudaStream_t stream, const float *lse_obs)
 {
-    const int units = ks.batch * ks.hkv;
-    const int r_pad = ws.r_pad;
     float2 *stats = reinterpret_cast<float2 *>(static_cast<char *>(workspace) + ws.stats_off);
-    const int chunk_keys = simt_chunk_keys(ks);
-    const int n_r_max = ks.max_seqlen - ks.alpha;
-    if (n_r_max <= 0) return cudaSuccess;
-    const int n_score_chunks = (n_r_max + chunk_keys - 1) / chunk_keys;
-    const size_t smem1 = sizeof(float) * ((size_t)ks.d * r_pad + (size_t)ks.d * kKPad);
-    const size_t smem2 = smem1 + sizeof(float) * ((size_t)r_pad + 16 * kKT +
-                                                  (size_t)((chunk_keys + kKT - 1) / kKT) * kKT);
-    dim3 g1(ws.n_stat_chunks, units), g2(n_score_chunks, units);
-    int dev = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err != cudaSuccess) return err;
-#define WKV_LAUNCH_SIMT(T, SLOT)                                                                    \
-    do {                                                                                            \
-        err = allow_dynamic_smem(reinterpret_cast<const void *>(score_stats_simt<T>), dev, SLOT, smem1);     \
-        if (err != cudaSuccess) return err;                                                         \
-        err = allow_dynamic_smem(reinterpret_cast<const void *>(score_pool_simt<T>), dev, SLOT + 1, smem2);  \
-        if (err != cudaSuccess) return err;                                                         \
-        if (!lse_obs)                                                                               \
-            score_stats_simt<T><<<g1, kThreads, smem1, stream>>>(ks, (const T *)q, (const T *)k, stats, \
-                                                                 ws.n_stat_chunks, r_pad);          \
-        score_pool_simt<T><<<g2, kThreads, smem2, stream>>>(ks, (const T *)q, (const T *)k, stats,  \
-                                                            lse_obs, window_scores, token_scores,   \
-                                                            ws.n_stat_chunks, r_pad, chunk_keys);   \
-    } while (0)
-    if (dtype == WKV_F32)
-        WKV_LAUNCH_SIMT(float, 0);
-    else
-        WKV_LAUNCH_SIMT(__nv_bfloat16, 2);
-#undef WKV_LAUNCH_SIMT
-    count_launches(lse_obs ? 1 : 2);
-    return cudaGetLastError();
+    if (ks.max_seqlen <= ks.alpha) return cudaSuccess;
+    return dtype == WKV_F32 ? launch_simt_type<float>(ks, 0, q, k, window_scores, token_scores, stats, ws, stream, lse_obs)
+                            : launch_simt_type<__nv_bfloat16>(ks, 6, q, k, window_scores, token_scores, stats, ws, stream, lse_obs);
 }
 
 // shared-memory need of the CUDA-core kernels, for the host-side support check
 size_t score_simt_smem_bytes(const KShape &ks, int r_pad)
 {
-    const int chunk_keys = simt_chunk_keys(ks);
-    return sizeof(float) * ((size_t)ks.d * r_pad + (size_t)ks.d * kKPad + (size_t)r_pad + 16 * kKT +
-                            (size_t)((chunk_keys + kKT - 1) / kKT) * kKT);
+    size_t a, b;
+    simt_smem(ks, r_pad, a, b);
+    return a > b ? a : b;
 }
 
 }  // namespace wkv
