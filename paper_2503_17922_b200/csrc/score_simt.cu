@@ -53,25 +53,30 @@ __device__ inline Vec<T> load_vec(const T *p)
     return r;
 }
 
-// Q of the unit, transposed into shared memory: qs[c * r_pad + r]; rows >= R are zero.  Lanes take
-// consecutive rows, so that the transposed stores hit different banks.
-template <typename T>
-__device__ void load_q_transposed(const KShape &s, const T *q_unit, float *qs, int r_pad)
+// Q of the unit, transposed into shared memory: qs[c * r_tile + r]; rows >= R are zero.  Lanes take
+// consecutive rows, so that the transposed stores hit different banks; a thread keeps its row for all of the
+// row's vectors, so the index arithmetic is done once per row.  last[r]: the last key row r may attend to.
+template <typename T, int RB>
+__device__ void load_q_transposed(const KShape &s, const T *q_unit, float *qs, int *last, int n_r, int r_tile)
 {
     constexpr int VN = Vec<T>::N;
     const int vec_per_row = s.d / VN;
-    for (int idx = threadIdx.x; idx < r_pad * vec_per_row; idx += kThreads) {
-        const int cv = idx / r_pad, r = idx - cv * r_pad;
-        Vec<T> v;
-        if (r < s.R) {
-            int g = r / s.alpha, i = r % s.alpha;
-            v = load_vec(q_unit + g * s.qsh + i * s.qst + cv * VN);
-        } else {
+    for (int r = threadIdx.x % RB; r < r_tile; r += RB) {
+        const int g = r / s.alpha, i = r - g * s.alpha;
+        const T *row = q_unit + g * s.qsh + i * s.qst;
+        if (last && threadIdx.x < RB) last[r] = r < s.R ? n_r + i : -1;
+#pragma unroll 4
+        for (int cv = threadIdx.x / RB; cv < vec_per_row; cv += kThreads / RB) {
+            Vec<T> v;
+            if (r < s.R) {
+                v = load_vec(row + cv * VN);
+            } else {
 #pragma unroll
-            for (int e = 0; e < VN; ++e) v.v[e] = T(0.f);
+                for (int e = 0; e < VN; ++e) v.v[e] = T(0.f);
+            }
+#pragma unroll
+            for (int e = 0; e < VN; ++e) qs[(cv * VN + e) * r_tile + r] = to_float(v.v[e]);
         }
-#pragma unroll
-        for (int e = 0; e < VN; ++e) qs[(cv * VN + e) * r_pad + r] = to_float(v.v[e]);
     }
 }
 
@@ -81,12 +86,13 @@ __device__ void load_k_transposed(const KShape &s, const T *k_unit, float *ks, i
 {
     constexpr int VN = Vec<T>::N;
     const int vec_per_row = s.d / VN;
+    const int jj = threadIdx.x % kKT;
+    const T *row = k_unit + (long long)(j0 + jj) * s.st;
 #pragma unroll 4
-    for (int idx = threadIdx.x; idx < kKT * vec_per_row; idx += kThreads) {
-        const int jj = idx % kKT, cv = idx / kKT;
+    for (int cv = threadIdx.x / kKT; cv < vec_per_row; cv += kThreads / kKT) {
         Vec<T> v;
         if (j0 + jj < n_valid) {
-            v = load_vec(k_unit + (long long)(j0 + jj) * s.st + cv * VN);
+            v = load_vec(row + cv * VN);
         } else {
 #pragma unroll
             for (int e = 0; e < VN; ++e) v.v[e] = T(0.f);
@@ -167,7 +173,8 @@ score_stats_simt(const __grid_constant__ KShape s, const T *__restrict__ q, cons
     float *qs = smem;                                                   // [d][r_tile]
     float *ks = qs + s.d * r_tile;                                      // [d][kKPad]
     float2 *rows = reinterpret_cast<float2 *>(ks + s.d * kKPad);        // [r_pad] this block's (max, sum) ...
-    float2 *half = rows + (tiles_per_block < kChunkTiles ? r_pad : 0);                                        // ... and, 16-row tiles: the second warps'
+    float2 *half = rows + (tiles_per_block < kChunkTiles ? r_pad : 0);  // ... and, 16-row tiles: the second warps'
+    int *last = reinterpret_cast<int *>(half + (RB == 16 ? r_pad : 0)); // [r_tile] last key of each row
 
     pdl_wait();
     pdl_trigger();      // the score kernel may read Q and K from here on: what wrote them has completed
@@ -183,7 +190,7 @@ score_stats_simt(const __grid_constant__ KShape s, const T *__restrict__ q, cons
     if (cs == 1) rows = out;      // nothing to combine: the rows are kept where they go
     for (int r = threadIdx.x; r < r_pad; r += kThreads) rows[r] = make_float2(-INFINITY, 0.f);
     if (!idle) {
-        load_q_transposed(s, q + b * s.qsb + (long long)h * s.G * s.qsh, qs, r_tile);
+        load_q_transposed<T, RB>(s, q + b * s.qsb + (long long)h * s.G * s.qsh, qs, last, n_r, r_tile);
         const T *k_unit = k + (si.off * s.st + b * s.sb + h * s.sh);
         const int ty = threadIdx.x / TX, tx = threadIdx.x % TX;
         for (int j0 = j_begin; j0 < j_end; j0 += kKT) {
@@ -196,11 +203,11 @@ score_stats_simt(const __grid_constant__ KShape s, const T *__restrict__ q, cons
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
                     const int r = r0 + ty * 4 + a;
-                    const int last = r < s.R ? n_r + (r % s.alpha) : -1;     // last key the row may attend to
+                    const int jl = last[r] - j0 - tx * KPT;      // of this thread's keys, those up to jl count
                     float x[KPT], m = -INFINITY;
 #pragma unroll
                     for (int c = 0; c < KPT; ++c) {
-                        x[c] = j0 + tx * KPT + c <= last ? acc[a][c] * s.scale_log2 : -INFINITY;
+                        x[c] = c <= jl ? acc[a][c] * s.scale_log2 : -INFINITY;
                         m = fmaxf(m, x[c]);
                     }
 #pragma unroll
@@ -293,7 +300,7 @@ score_pool_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const
     }
     const int j_end = min(n_r, j_begin + chunk_keys);
     const T *k_unit = k + (si.off * s.st + b * s.sb + h * s.sh);
-    load_q_transposed(s, q + b * s.qsb + (long long)h * s.G * s.qsh, qs, r_tile);
+    load_q_transposed<T, RB>(s, q + b * s.qsb + (long long)h * s.G * s.qsh, qs, nullptr, n_r, r_tile);
 
     const int ty = threadIdx.x / TX, tx = threadIdx.x % TX;
     for (int j0 = j_begin; j0 < j_end; j0 += kKT) {
@@ -413,7 +420,7 @@ static void simt_smem(const KShape &ks, int r_pad, size_t &stats_bytes, size_t &
     const int rb = simt_row_tile(ks), r_tile = rb < 64 ? rb : r_pad;
     const int tpb = simt_tiles_per_block(ks), chunk_keys = simt_chunk_keys(ks, tpb);
     const size_t tiles = (size_t)ks.d * r_tile + (size_t)ks.d * kKPad;
-    stats_bytes = sizeof(float) * (tiles + (tpb < kChunkTiles ? 2 * (size_t)r_pad : 0) + (rb == 16 ? 2 * (size_t)r_pad : 0));
+    stats_bytes = sizeof(float) * (tiles + (tpb < kChunkTiles ? 2 * (size_t)r_pad : 0) + (rb == 16 ? 2 * (size_t)r_pad : 0) + (size_t)r_tile);
     pool_bytes = sizeof(float) * (tiles + (size_t)r_pad + (size_t)(rb / 4) * kKT + (size_t)((chunk_keys + kKT - 1) / kKT) * kKT);
 }
 
