@@ -515,7 +515,10 @@ def main() -> None:
         dt = time.perf_counter() - t0
         dt = replicas.max_over_ranks(dt, "cuda")
         nb = lambda t: t.numel() * t.element_size()
-        h2d = nb(hsets[0]["q"]) + sum(nb(x) for x in hsets[0]["k"] + hsets[0]["v"])
+        # in: the queries and the leader's keys whole, of every other tensor the retained rows (the gather reads them
+        # from the pinned host memory)
+        row_bytes = w.head_dim * hsets[0]["q"].element_size()
+        h2d = nb(hsets[0]["q"]) + nb(hsets[0]["k"][0]) + (2 * w.gamma - 1) * int(h_kept.sum()) * row_bytes
         d2h = sum(nb(x) for x in h_k_out + h_v_out) + nb(h_idx) + nb(h_kept)
         e2e = {"value": tokens * world * e2e_steps / dt, "unit": UNIT, "h2d_bytes_per_step": h2d,
                "d2h_bytes_per_step": d2h, "steps": e2e_steps}

@@ -363,14 +363,16 @@ int wkv_group_plan_launch(wkv_group_plan *plan, void *cuda_stream);
 void wkv_group_plan_destroy(wkv_group_plan *plan);
 
 /*
- * The same group with every tensor in HOST memory (pinned memory recommended): the
- * inputs are copied to caller-provided DEVICE staging buffers, the group is
- * compressed there, and indices, kept lengths and the compact caches are copied
- * back; the function returns after everything it enqueued has completed.  The copies
- * dominate, so the call runs as a pipeline over the layers: the leader's keys first
- * (scored and selected as soon as they have landed), then layer by layer copy in, gather,
- * and copy back on a second stream of the call's own, so that both copy directions are
- * busy at once.  (This creates and destroys one stream and one event per call.)
+ * The same group with every tensor in HOST memory (pinned memory recommended): the group is
+ * compressed on the device and indices, kept lengths and the compact caches are copied back; the
+ * function returns after everything it enqueued has completed.  What crosses the bus dominates, so
+ * only what is needed crosses: the leader's keys whole (they are copied to their DEVICE staging buffer
+ * first and scored as soon as they have landed), and of every other tensor the retained rows, which the
+ * gather reads straight from the host memory where that is pinned and mapped.  A tensor in memory that
+ * is not, or of which more than half the rows are retained, is copied to its staging buffer whole.  The
+ * staging buffers are scratch: what they hold after the call is unspecified.  Each layer's compact cache
+ * travels back on a second stream while the next layer is coming in.  (That stream and its event are made
+ * at a thread's first call on a device and given back when the thread ends.)
  *   *_host arguments    HOST pointers / HOST arrays of HOST pointers
  *   *_dev arguments     DEVICE staging of the same sizes (HOST arrays of DEVICE pointers)
  *   bytes_per_layer     size of one K (or V) tensor; out_bytes_per_layer of one compact cache

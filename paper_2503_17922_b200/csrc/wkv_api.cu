@@ -2,7 +2,10 @@
 // carve-up and kernel sequencing.  No device memory is allocated here.
 #include "wkv_internal.cuh"
 
+#include <cuda.h>
+
 #include <atomic>
+#include <mutex>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -721,6 +724,69 @@ int wkv_compress_group_lse(const wkv_shape *s, int32_t n_layers, const void *q_o
                                 workspace_bytes, cuda_stream);
 }
 
+// The stream and the event of the copies back: one pair per thread and device, made at a thread's first call on a
+// device (making and destroying a stream costs 100-180 us, a fifth of a small call) and given back when the
+// thread ends.
+struct CopyBack {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t event = nullptr;
+};
+struct CopyBackSet {
+    CopyBack of_device[kMaxDevices];
+    ~CopyBackSet()
+    {
+        for (CopyBack &cb : of_device) {
+            if (cb.event) (void)cudaEventDestroy(cb.event);
+            if (cb.stream) (void)cudaStreamDestroy(cb.stream);
+        }
+    }
+};
+static CopyBack *copy_back()
+{
+    static thread_local CopyBackSet set;
+    int dev = 0;
+    if (check_cuda(cudaGetDevice(&dev), "current device") != WKV_OK) return nullptr;
+    if (dev >= kMaxDevices) {
+        set_error_detail("device ordinal beyond %d", kMaxDevices - 1);
+        return nullptr;
+    }
+    CopyBack &cb = set.of_device[dev];
+    if (!cb.stream && check_cuda(cudaStreamCreateWithFlags(&cb.stream, cudaStreamNonBlocking), "stream for the copies back") != WKV_OK) {
+        cb.stream = nullptr;
+        return nullptr;
+    }
+    if (!cb.event && check_cuda(cudaEventCreateWithFlags(&cb.event, cudaEventDisableTiming), "event") != WKV_OK) {
+        cb.event = nullptr;
+        return nullptr;
+    }
+    return &cb;
+}
+
+// Whether the GPU can read `bytes` bytes of host memory at `p` in place: all of it inside one pinned (or
+// registered) allocation that is mapped at the same address.
+static bool mapped_host_range(const void *p, size_t bytes)
+{
+    static CUresult (*get)(void *, CUpointer_attribute, CUdeviceptr) = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            get = reinterpret_cast<decltype(get)>(fn);
+        (void)cudaGetLastError();
+    });
+    if (!get) return false;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    unsigned type = 0;
+    CUdeviceptr dev = 0, start = 0;
+    size_t size = 0;
+    return get(&type, CU_POINTER_ATTRIBUTE_MEMORY_TYPE, at) == CUDA_SUCCESS && type == CU_MEMORYTYPE_HOST &&
+           get(&dev, CU_POINTER_ATTRIBUTE_DEVICE_POINTER, at) == CUDA_SUCCESS && dev == at &&
+           get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) == CUDA_SUCCESS && start <= at &&
+           get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) == CUDA_SUCCESS && size >= bytes && at - start <= size - bytes;
+}
+
 int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_obs_host, size_t q_bytes,
                             const void *const *k_layers_host, const void *const *v_layers_host,
                             size_t bytes_per_layer, void *const *k_out_layers_host,
@@ -771,15 +837,25 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_
         }
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    // The copies in dominate this call, so it is laid out as a pipeline over the layers: the leader's
-    // keys go first and are scored as soon as they have landed; every layer is gathered behind its own
-    // copy in, and its compact cache travels back on a second stream while the next layer is still
-    // coming in (the two copy directions run at the same time).
-    cudaStream_t back = nullptr;
-    cudaEvent_t ready = nullptr;
-    st = check_cuda(cudaStreamCreateWithFlags(&back, cudaStreamNonBlocking), "stream for the copies back");
-    if (st != WKV_OK) return st;
-    st = check_cuda(cudaEventCreateWithFlags(&ready, cudaEventDisableTiming), "event");
+    // What crosses the bus dominates this call.  Only the leader's keys are needed whole (every key is scored); of
+    // every other tensor the retained rows are, so where the GPU can read the caller's host memory the gather takes
+    // them straight from there and the rest never moves.  The crossing of 16 KB of a head's consecutive windows is as
+    // fast as a copy (4 layers x 8,192 keys, 12 %: 31 MB instead of 134 MB).  With most rows retained, or memory
+    // that is not pinned, a tensor is copied to its staging buffer first.
+    // The call is a pipeline over the layers: the leader's keys are scored as soon as they have landed, every layer
+    // is gathered in turn, and its compact cache travels back on a second stream while the next layer is coming in
+    // (the two directions run at the same time).
+    double kept_rows = 0;
+    for (int b = 0; b < s->batch; ++b) {
+        const int n = s->cu_seqlens_host ? s->cu_seqlens_host[b + 1] - s->cu_seqlens_host[b] : s->max_seqlen;
+        kept_rows += (double)num_selected(n, s->l_obs, s->window, s->budgets_host ? s->budgets_host[b] : s->budget) * s->window +
+                     s->l_obs;
+    }
+    const bool few_rows = kept_rows <= 0.5 * ks.total_rows;
+    CopyBack *cb = copy_back();
+    if (!cb) return WKV_ERR_CUDA;
+    const cudaStream_t back = cb->stream;
+    const cudaEvent_t ready = cb->event;
     const size_t units = (size_t)ks.batch * ks.hkv;
     auto h2d = [&](void *dst, const void *src, size_t bytes, const char *what) {
         if (st == WKV_OK) st = check_cuda(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, stream), what);
@@ -800,19 +876,29 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_
     d2h_after(window_idx_host, window_idx_dev, units * ks.k_max * sizeof(int32_t), "copy of window_idx");
     d2h_after(kept_len_host, kept_len_dev, units * sizeof(int32_t), "copy of kept_len");
     for (int l = 0; l < n_layers && st == WKV_OK; ++l) {
-        if (l > 0) h2d(k_layers_dev[l], k_layers_host[l], bytes_per_layer, "copy of K");
-        h2d(v_layers_dev[l], v_layers_host[l], bytes_per_layer, "copy of V");
-        if (st == WKV_OK)
-            st = wkv_gather_kv(s, 1, k_layers_dev + l, v_layers_dev + l, window_idx_dev, k_out_layers_dev + l,
-                               v_out_layers_dev + l, nullptr, keep_capacity, cuda_stream);
-        hand_over();
-        d2h_after(k_out_layers_host[l], k_out_layers_dev[l], out_bytes_per_layer, "copy of compact K");
-        d2h_after(v_out_layers_host[l], v_out_layers_dev[l], out_bytes_per_layer, "copy of compact V");
+        // each of the layer's tensors from where it can be read: staging, or the host memory itself
+        const void *src[2] = {k_layers_dev[l], v_layers_dev[l]};
+        const void *const from[2] = {k_layers_host[l], v_layers_host[l]};
+        void *const staging[2] = {k_layers_dev[l], v_layers_dev[l]};
+        for (int t = l == 0 ? 1 : 0; t < 2; ++t) {
+            if (few_rows && aligned16(from[t]) && mapped_host_range(from[t], bytes_per_layer)) src[t] = from[t];
+            else h2d(staging[t], from[t], bytes_per_layer, t ? "copy of V" : "copy of K");
+        }
+        // The last layer in two steps, so that less is left to travel back when the gather is over
+        const bool last = l == n_layers - 1;
+        for (int t = 0; t < (last ? 2 : 1); ++t) {
+            void *const out[2] = {k_out_layers_dev[l], v_out_layers_dev[l]};
+            void *const out_host[2] = {k_out_layers_host[l], v_out_layers_host[l]};
+            if (st == WKV_OK)
+                st = wkv_gather_kv(s, 1, &src[t], last ? nullptr : &src[1], window_idx_dev, &out[t], last ? nullptr : &out[1], nullptr,
+                                   keep_capacity, cuda_stream);
+            hand_over();
+            d2h_after(out_host[t], out[t], out_bytes_per_layer, t ? "copy of compact V" : "copy of compact K");
+            if (!last) d2h_after(out_host[1], out[1], out_bytes_per_layer, "copy of compact V");
+        }
     }
     // both streams are drained before the call returns, whatever happened above
     const cudaError_t e1 = cudaStreamSynchronize(stream), e2 = cudaStreamSynchronize(back);
-    if (ready) cudaEventDestroy(ready);
-    cudaStreamDestroy(back);
     if (st != WKV_OK) return st;
     if (e1 != cudaSuccess) return check_cuda(e1, "stream synchronisation");
     return check_cuda(e2, "stream synchronisation (copies back)");

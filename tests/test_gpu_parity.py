@@ -557,6 +557,23 @@ def test_host_buffer_entry_point(which):
             np.testing.assert_array_equal(got["v_out"][layer], ref["v_out"][layer])
 
 
+@pytest.mark.parametrize("pinned", [True, False], ids=["pinned", "pageable"])
+@pytest.mark.parametrize("budget_frac", [0.05, 0.49, 0.9])
+@pytest.mark.parametrize("n_layers", [1, 3])
+def test_host_buffer_entry_point_reads_only_what_it_needs(monkeypatch, pinned, budget_frac, n_layers):
+    """Pinned memory with few retained rows is read in place, anything else is copied whole: the compact caches
+    are the oracle's gather either way."""
+    w = small(budget_frac=budget_frac, n_layers=n_layers, gamma=n_layers)
+    grp = wl.make_group(w, 0)
+    if not pinned:
+        monkeypatch.setattr(torch.Tensor, "pin_memory", lambda t: t)
+    got = _run_host_entry(w, grp)
+    ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
+    got["window_scores"] = ref["window_scores"]
+    pu.check_selection(w, grp, got, ref)
+    pu.check_gather(w, grp, got)
+
+
 @pytest.mark.parametrize("impl", ["simt", "tc", "pipe"])
 def test_stale_device_copy_of_cu_seqlens_stays_in_bounds(impl):
     """cu_seqlens and budgets exist as a host and a device copy, and sizes are derived from the host
