@@ -100,13 +100,25 @@ __device__ __forceinline__ void score_accumulate(const float (&v)[N], const floa
 // Eq. 4 for one window of compile-time length (a power of two) by one thread: a bitonic sorting
 // network in registers (every compare-exchange of a stage is independent of the others, so the
 // thread is not latency-bound), then the p largest are summed in descending order.  Positions
-// beyond `size` (ragged last window) hold -inf and sort to the end.
+// beyond `size` (ragged last window) hold -inf and sort to the end.  `w` is 16-byte aligned shared memory that holds
+// omega values.
 template <int omega>
 __device__ __forceinline__ float pool_window_sorted(const float *w, int size, int p)
 {
+    // Neighbouring lanes take neighbouring windows, so a lane starts with another 16-byte piece of its window than the
+    // lanes it would share banks with; the network does not care in which register an element starts.
+    constexpr int kPieces = omega / 4;
+    const int turn = ((threadIdx.x & 31) * kPieces) >> 3;
     float v[omega];
 #pragma unroll
-    for (int x = 0; x < omega; ++x) v[x] = x < size ? w[x] : -INFINITY;
+    for (int i = 0; i < kPieces; ++i) {
+        const int c = (i + turn) % kPieces;
+        const float4 x = *reinterpret_cast<const float4 *>(w + 4 * c);
+        v[4 * i] = 4 * c < size ? x.x : -INFINITY;
+        v[4 * i + 1] = 4 * c + 1 < size ? x.y : -INFINITY;
+        v[4 * i + 2] = 4 * c + 2 < size ? x.z : -INFINITY;
+        v[4 * i + 3] = 4 * c + 3 < size ? x.w : -INFINITY;
+    }
 #pragma unroll
     for (int k = 2; k <= omega; k <<= 1)
 #pragma unroll

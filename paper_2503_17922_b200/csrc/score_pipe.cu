@@ -396,7 +396,7 @@ group_pipeline_tc(const __grid_constant__ CUtensorMap kmap, const __grid_constan
     __shared__ int abort_s;
     __shared__ float2 part[kBufs][128];                  // a compute group's (max, sum) of the rows on its lanes
     __shared__ __align__(16) float neg_lse2[128];        // -log2 of the row normaliser; -inf for padding rows
-    __shared__ float t_chunk[kChunkCap];                 // token scores of the item being scored
+    __shared__ __align__(16) float t_chunk[kChunkCap];                 // token scores of the item being scored
     __shared__ TopkSmem topk_sm;
 
     const KShape &s = a.s;

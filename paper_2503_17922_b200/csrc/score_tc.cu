@@ -16,7 +16,8 @@
 // Units are taken in waves whose keys fit L2 together.  A work item is (unit, chunk of <= 17 key
 // tiles); the persistent blocks (at most one per SM) take the items of a wave round-robin.
 //
-// Warp roles: warp 0 issues the TMA tile loads (4-stage ring), warp 1 issues the MMAs into four
+// Warp roles: warp 0 issues the TMA tile loads (4-stage ring), warp 1 issues the MMAs (each as a whole
+// converged warp, one elected lane acting) into four
 // accumulator buffers of 128 columns in tensor memory, and four compute groups of four warps (one
 // warp per 32-lane quarter of tensor memory) take the accumulators round-robin, each with its own
 // buffer, 32 columns at a time.  With more than 128 observation rows (up to 256) every key tile
@@ -162,7 +163,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     __shared__ int abort_s;
     __shared__ float2 part[NG][1][128];                    // sweep 1: a group's (max, sum) of the rows on its lanes
     __shared__ __align__(16) float neg_lse2_all[256];    // -log2 of the row normaliser; -inf for padding rows
-    __shared__ float t_chunk[MB][kChunkCap];              // sweep 2: per half, the key's sum over that half's rows
+    __shared__ __align__(16) float t_chunk[MB][kChunkCap];              // sweep 2: per half, the key's sum over that half's rows
     __shared__ TopkSmem topk_sm;
 
     const KShape &s = a.s;
@@ -175,6 +176,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     uint8_t *k_stage0 = q_img + a.kblocks * q_region;
     const int stage_bytes = a.kblocks * kRegion;
     const int ksteps = s.d / 16;
+    const uint32_t leader = elect_one();     // lane that acts for its warp where a whole warp issues
 
     if (threadIdx.x == 0) {
         init_barriers(bar);
@@ -271,25 +273,25 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
             const int st = g % kStages;
             if (im.reuse && t < kStages) {
                 // the stage holds this tile already: complete the phase without a load
-                mbar_arrive(&bar.full[st]);
+                if (leader) mbar_arrive(&bar.full[st]);
                 ++p_issued;
                 continue;
             }
             if (g >= kStages && !mbar_wait(&bar.empty[st], ((g / kStages) - 1) & 1, &abort_s)) return;
-            mbar_arrive_expect_tx(&bar.full[st], (uint32_t)stage_bytes);
+            mbar_arrive_expect_tx_if(leader, &bar.full[st], (uint32_t)stage_bytes);
             const int tok = tok0 + tile_at(im, t) * kTile;
             const int c1 = a.slot_tok == 1 ? tok : (a.slot_h == 1 ? im.h : bcoord);
             const int c2 = a.slot_tok == 2 ? tok : (a.slot_h == 2 ? im.h : bcoord);
             const int c3 = a.slot_tok == 3 ? tok : (a.slot_h == 3 ? im.h : bcoord);
             for (int kb = 0; kb < a.kblocks; ++kb)
-                tma_load_4d(k_stage0 + st * stage_bytes + kb * kRegion, &tmap, &bar.full[st], kb * 64, c1, c2, c3);
+                tma_load_4d_if(leader, k_stage0 + st * stage_bytes + kb * kRegion, &tmap, &bar.full[st], kb * 64, c1, c2, c3);
             ++p_issued;
         }
     };
 
     // MMA issue for one item.  sweep 1: D[rows, keys] = Q K^T; sweep 2: D[keys, rows] = K Q^T; per key
     // tile one accumulator per 128-row block of Q.
-    // One thread issues everything, so its instruction count per tile is on the critical path: the
+    // One warp issues everything, so its instruction count per tile is on the critical path: the
     // matrix descriptors of Q and of stage 0 are built once, and every k-step only adds a
     // compile-time constant to the address field (the fields above it never change).
     const uint64_t q_desc0 = umma_desc_sw128(smem_u32(q_img));
@@ -301,11 +303,12 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
         for (int ks = 0; ks < KSTEPS; ++ks) {
             const uint32_t qo = (uint32_t)((ks >> 2) * q_region + (ks & 3) * 32) >> 4;
             const uint32_t ko = (uint32_t)((ks >> 2) * kRegion + (ks & 3) * 32) >> 4;
-            if (sweep2) umma_bf16(d_tmem, k_desc + ko, q_desc + qo, idesc, ks > 0);
-            else umma_bf16(d_tmem, q_desc + qo, k_desc + ko, idesc, ks > 0);
+            if (sweep2) umma_bf16_if(leader, d_tmem, k_desc + ko, q_desc + qo, idesc, ks > 0);
+            else umma_bf16_if(leader, d_tmem, q_desc + qo, k_desc + ko, idesc, ks > 0);
         }
     };
-    auto issue_mma = [&](const Item &im, bool sweep2) {
+    auto issue_mma = [&](const Item &im, auto sweep2_tag) {
+        constexpr bool sweep2 = decltype(sweep2_tag)::value;
         const uint32_t stage_step = (uint32_t)stage_bytes >> 4;
         for (int t = 0; t < im.n_tiles; ++t) {
             const uint32_t g = it + t;
@@ -325,9 +328,9 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                 const uint32_t d_tmem = tmem_base + buf * buf_cols;
                 if (ksteps == 8) issue_tile(std::integral_constant<int, 8>{}, d_tmem, k_desc, q_desc, idesc, sweep2);
                 else issue_tile(std::integral_constant<int, 4>{}, d_tmem, k_desc, q_desc, idesc, sweep2);
-                umma_commit(&bar.tfull[buf]);
+                umma_commit_if(leader, &bar.tfull[buf]);
             }
-            umma_commit(&bar.empty[st]);
+            umma_commit_if(leader, &bar.empty[st]);
         }
     };
 
@@ -420,13 +423,13 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                 // the first tiles leave before the loads of the Q image (they land while those are
                 // being issued); the rest of the ring's burst follows once the Q loads are on their way
                 const int early = min(kEarlyTiles, im.n_tiles);
-                if (lane == 0) produce(im, 0, early);
+                produce(im, 0, early);
                 asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
-                if (lane == 0) produce(im, early, im.n_tiles);
+                produce(im, early, im.n_tiles);
             } else {
                 load_q_image(im, true);
                 if (warp == 1) {
-                    if (lane == 0) issue_mma(im, false);
+                    issue_mma(im, std::false_type{});
                 } else {
                     compute_stats(im);
                 }
@@ -492,16 +495,16 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                 // ahead of the small loads of this item: the tiles the ring still holds (no traffic), or,
                 // when this is the only sweep, the first tiles from HBM as in sweep 1
                 const int ahead = im.reuse ? kStages : (a.lse_obs ? min(kEarlyTiles, im.n_tiles) : 0);
-                if (lane == 0) produce(im, 0, ahead);
+                produce(im, 0, ahead);
                 asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
-                if (lane == 0) produce(im, ahead, im.n_tiles);
+                produce(im, ahead, im.n_tiles);
             } else {
                 load_q_image(im, false);
                 if (warp == 1) {
                     // the MMAs do not need the normalisers: the first accumulators fill while the
                     // compute warps merge the statistics
                     go_producer();
-                    if (lane == 0) issue_mma(im, true);
+                    issue_mma(im, std::true_type{});
                 } else {
                 // Eq. 1's normaliser of every row: merge the partial statistics of the unit's chunks.
                 // kMergers threads share a row (each takes every kMergers-th chunk), then one of them
