@@ -33,6 +33,7 @@ struct CompactParams {
     const int *window_idx;
     int cluster;          // blocks per (unit, tensor)
     int vec_per_row;
+    int vec_shift, omega_shift;   // log2 of vec_per_row and of omega where they are powers of two, else -1
     int elem_bytes;
 };
 
@@ -51,53 +52,62 @@ compact_inplace_kernel(const __grid_constant__ CompactParams prm)
     pdl_wait();
     const int cs = prm.cluster, unit = blockIdx.x / cs, rank = blockIdx.x - unit * cs, tensor = blockIdx.y;
     const int b = unit / s.hkv, h = unit % s.hkv;
+    const int *idx = prm.window_idx + (size_t)unit * s.k_max;
+    const int vpr = prm.vec_per_row;
+    const int rows_per_batch = max(1, (cs * kThreads * kVecs) / vpr);
+    // row and window slot of the thread's vectors in the batch at row r0
+    auto over = [](int x, int by, int shift) { return shift >= 0 ? x >> shift : x / by; };
+    auto row_of = [&](int r0, int u) { return r0 + over((int)threadIdx.x + (u * cs + rank) * kThreads, vpr, prm.vec_shift); };
+    // A vector's window index waits in the registers that its 16 bytes go to.  The first batch's windows and the unit's
+    // last one are looked up before it is known how many are selected, which takes a trip to memory of its own.
+    int4 val[kVecs];
+    auto load_windows = [&](int r0) {
+#pragma unroll
+        for (int u = 0; u < kVecs; ++u) {
+            const int slot = over(row_of(r0, u), s.omega, prm.omega_shift);
+            val[u].x = slot < s.k_max ? idx[slot] : -1;
+        }
+    };
+    load_windows(0);
+    const int wi_last = idx[s.k_max - 1];
     const SeqInfo si = seq_info(s, b);
     const int n = si.n;
     const int n_r = n > s.alpha ? n - s.alpha : 0;
     const int kw = num_windows(n, s.alpha, s.omega);
     const int k = num_selected_capped(n, s.alpha, s.omega, si.budget, s.k_max);
-    const int *idx = prm.window_idx + (size_t)unit * s.k_max;
     int review_rows = k * s.omega;
-    if (k > 0 && idx[k - 1] == kw - 1) review_rows -= kw * s.omega - n_r;
+    if (k > 0 && (k == s.k_max ? wi_last : idx[k - 1]) == kw - 1) review_rows -= kw * s.omega - n_r;
     const int kept = review_rows + (n - n_r);
 
-    const int vpr = prm.vec_per_row;
     const long long row_vecs = s.st * prm.elem_bytes / 16;
     int4 *base = reinterpret_cast<int4 *>(static_cast<char *>(prm.tab.ptr[tensor]) +
                                           (si.off * s.st + b * s.sb + h * s.sh) * (long long)prm.elem_bytes);
-    const int rows_per_batch = max(1, (cs * kThreads * kVecs) / vpr);
     for (int r0 = 0; r0 < kept; r0 += rows_per_batch) {
-        const int rows = min(rows_per_batch, kept - r0);
-        const int n_vec = rows * vpr;
-        int4 val[kVecs];
-        int dst_row[kVecs];     // -1: nothing to move
+        const int n_vec = min(rows_per_batch, kept - r0) * vpr;
+        if (r0 > 0) load_windows(r0);
+        unsigned moves = 0u;      // bit u: vector u of the thread has somewhere to go
 #pragma unroll
         for (int u = 0; u < kVecs; ++u) {
             const int v = (int)threadIdx.x + (u * cs + rank) * kThreads;
-            dst_row[u] = -1;
             if (v < n_vec) {
-                const int r = r0 + v / vpr, c = v - (r - r0) * vpr;
+                const int r = row_of(r0, u), slot = over(r, s.omega, prm.omega_shift), wi = val[u].x;
                 int src_row;
-                if (r < review_rows) {
-                    const int wi = idx[r / s.omega];
-                    // an entry that is no window of this sequence, or that lies before its own slot (a
-                    // list that is not an ascending selection), is skipped: the row stays as it is
-                    src_row = (wi < r / s.omega || wi >= kw) ? -1 : wi * s.omega + r % s.omega;
-                } else {
-                    src_row = n_r + (r - review_rows);
-                }
+                // an entry that is no window of this sequence, or that lies before its own slot (a
+                // list that is not an ascending selection), is skipped: the row stays as it is
+                if (r < review_rows) src_row = wi < slot || wi >= kw ? -1 : (wi - slot) * s.omega + r;
+                else src_row = n_r + (r - review_rows);
                 if (src_row >= 0 && src_row < n && src_row != r) {
-                    val[u] = base[(long long)src_row * row_vecs + c];
-                    dst_row[u] = r;
+                    val[u] = base[(long long)src_row * row_vecs + (v - (r - r0) * vpr)];
+                    moves |= 1u << u;
                 }
             }
         }
         cluster_barrier();      // every source row of the batch has been read
 #pragma unroll
         for (int u = 0; u < kVecs; ++u)
-            if (dst_row[u] >= 0) {
-                const int v = (int)threadIdx.x + (u * cs + rank) * kThreads;
-                base[(long long)dst_row[u] * row_vecs + (v - (dst_row[u] - r0) * vpr)] = val[u];
+            if (moves >> u & 1u) {
+                const int v = (int)threadIdx.x + (u * cs + rank) * kThreads, r = row_of(r0, u);
+                base[(long long)r * row_vecs + (v - (r - r0) * vpr)] = val[u];
             }
     }
 }
@@ -113,6 +123,11 @@ cudaError_t launch_compact_inplace(const KShape &ks, int elem_bytes, int n_tenso
     prm.window_idx = window_idx;
     prm.vec_per_row = ks.d * elem_bytes / 16;
     prm.elem_bytes = elem_bytes;
+    prm.vec_shift = prm.omega_shift = -1;
+    for (int sh = 0; sh < 16; ++sh) {
+        if ((1 << sh) == prm.vec_per_row) prm.vec_shift = sh;
+        if ((1 << sh) == ks.omega) prm.omega_shift = sh;
+    }
     // Blocks per (unit, tensor): as many as are resident at once (with one block of 1,024 threads per SM
     // only 15 clusters of eight fit, so the sixteenth of a layer of 8 heads ran alone), a power of two up to the portable cluster size, unless the rows are too few to occupy them.
     const int pairs = ks.batch * ks.hkv * n_tensors;

@@ -59,17 +59,23 @@ gather_kv_kernel(const __grid_constant__ GatherParams prm)
     const int unit = blockIdx.y, tensor = blockIdx.z;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = unit / s.hkv, h = unit % s.hkv;
+    // The warp's first two windows and the unit's last one are looked up before it is known how many are selected
+    // (that takes a trip to memory of its own): the chain from launch to the first row is one trip shorter.
+    const int *idx = prm.window_idx + (size_t)unit * s.k_max;
+    const int first_slot = blockIdx.x * prm.slots_per_block + warp;
+    int wi_next = first_slot < s.k_max ? idx[first_slot] : -1;
+    int wi_after = first_slot + kWarps < s.k_max ? idx[first_slot + kWarps] : -1;
+    const int wi_last = idx[s.k_max - 1];
     const SeqInfo si = seq_info(s, b);
     const int n = si.n;
     const int n_r = n > s.alpha ? n - s.alpha : 0;
     const int kw = num_windows(n, s.alpha, s.omega);
     const int k = num_selected_capped(n, s.alpha, s.omega, si.budget, s.k_max);
-    const int *idx = prm.window_idx + (size_t)unit * s.k_max;
 
     // rows of the unit: the selected windows (only the last window of the sequence can be short,
     // and it can only be the last selected one), then the observation rows
     int review_rows = k * s.omega;
-    if (k > 0 && idx[k - 1] == kw - 1) review_rows -= kw * s.omega - n_r;
+    if (k > 0 && (k == s.k_max ? wi_last : idx[k - 1]) == kw - 1) review_rows -= kw * s.omega - n_r;
     const int obs_rows = n - n_r;
 
     const int vpr = prm.vec_per_row;
@@ -94,12 +100,14 @@ gather_kv_kernel(const __grid_constant__ GatherParams prm)
     if (paged) dst = reinterpret_cast<int4 *>(prm.tab.dst[tensor]) + (long long)h * prm.head_vecs;
 
     const int slot_end = min(k + prm.obs_slots, (int)(blockIdx.x + 1) * prm.slots_per_block);
-    for (int slot = blockIdx.x * prm.slots_per_block + warp; slot < slot_end; slot += kWarps) {
+    for (int slot = first_slot; slot < slot_end; slot += kWarps) {
+        const int wi = wi_next;
+        wi_next = wi_after;
+        if (slot + 2 * kWarps < min(k, slot_end)) wi_after = idx[slot + 2 * kWarps];
         int src_row0, dst_row0, n_rows;
         if (slot < k) {
             // an entry that is no window of this sequence (a list that no selection has written, or
             // that the caller filled wrongly) is skipped: the kernel never leaves the tensors
-            const int wi = idx[slot];
             if (wi < 0 || wi >= kw) continue;
             src_row0 = wi * s.omega;
             n_rows = min(s.omega, n_r - src_row0);

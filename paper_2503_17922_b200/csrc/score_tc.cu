@@ -187,6 +187,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_s;
+    pdl_wait();                 // nothing above touches memory of anybody else
     if (warp == 0 && lane == 0) tma_prefetch_desc(&tmap);
 
     // Row layout of the Q image: image row r holds observation row (r mod Rp); with Rp < 128 the rows
@@ -638,8 +639,27 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
             // chunk is usually a short one, so its block is done early and the selection does not sit
             // on the path of a block that the next wave is waiting for.  The other blocks only count
             // themselves, without waiting for an answer.
+            // With given normalisers nothing else makes a block wait for another, and the selection does not
+            // either: the block that counts itself last selects, so the launch need not be cooperative.
             int *ticket = a.sync + kSyncTickets + kSyncWordsPerUnit * im.unit;
-            if (im.chunk != used2 - 1) {
+            bool selects = im.chunk == used2 - 1;
+            if (a.lse_obs) {
+                selects = false;
+                if (a.window_idx) {
+                    __syncthreads();
+                    if (threadIdx.x == 0) {
+                        __threadfence();             // publishes the window scores the whole block wrote
+                        const int before = atomicAdd(ticket, 1);
+                        if (before == used2 - 1) atomicExch(ticket, 0);
+                        if (before < 0 || before >= used2) atomicOr(a.status, kStatusWaitExpired);   // workspace not cleared
+                        __threadfence();
+                        topk_sm.remaining = before;
+                    }
+                    __syncthreads();
+                    selects = topk_sm.remaining == used2 - 1;
+                    __syncthreads();                 // the word is the selection's own from here on
+                }
+            } else if (!selects) {
                 if (a.window_idx) {
                     __syncthreads();
                     // release, cumulative: publishes the window scores the whole block wrote
@@ -654,12 +674,12 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                     atomicExch(ticket + 1, 0);
                 }
                 __syncthreads();
-                if (a.window_idx && !abort_s) {
-                    select_topk_block<kThreads>(topk_sm, a.window_scores + (size_t)im.unit * s.kw_max, kw,
-                                                num_selected_capped(im.n, s.alpha, s.omega, budget, s.k_max), s.k_max,
-                                                a.window_idx + (size_t)im.unit * s.k_max, a.kept_len + im.unit,
-                                                im.n, s.alpha, s.omega);
-                }
+            }
+            if (selects && a.window_idx && !abort_s) {
+                select_topk_block<kThreads>(topk_sm, a.window_scores + (size_t)im.unit * s.kw_max, kw,
+                                            num_selected_capped(im.n, s.alpha, s.omega, budget, s.k_max), s.k_max,
+                                            a.window_idx + (size_t)im.unit * s.k_max, a.kept_len + im.unit,
+                                            im.n, s.alpha, s.omega);
             }
             __syncthreads();   // t_chunk, neg_lse2 and the selection scratch are reused by the next item
         }
@@ -877,7 +897,10 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
     const __nv_bfloat16 *qp = static_cast<const __nv_bfloat16 *>(q);
     if (err == cudaSuccess) {
         void *params[3] = {&tmap, &a, &qp};
-        err = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), params, smem, stream);
+        // with given normalisers no block waits for another: a plain launch, which may start while the kernel in front
+        // drains (a cooperative one may not: 2 us)
+        if (lse_obs) err = launch_pdl(mb == 1 ? score_windows_tc<1> : score_windows_tc<2>, dim3(grid), threads, smem, stream, 1, tmap, a, qp);
+        else err = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), params, smem, stream);
     }
     if (err != cudaSuccess) {
         set_error_detail("tensor-core score kernel (grid %d x %d threads, %zu bytes of shared memory): %s", grid,
