@@ -176,3 +176,21 @@ def test_paged_cache_argument_checks():
 def test_compaction_in_place_over_cluster_sizes(case, pattern):
     """A unit spread over a cluster of blocks: several batches in a row, fewer rows than threads, and one block."""
     test_compaction_in_place(case, pattern)
+
+
+@pytest.mark.parametrize("pattern", ["selected", "shift", "tail", "front"])
+@pytest.mark.parametrize("case", [
+    # 40 (sequence, head) pairs x 4 tensors: one block each, so that few rows are already several batches
+    dict(max_seqlen=16 + 8 * 400 + 3, budget_frac=0.45),                   # short last window, nearly half retained: long chains
+    dict(max_seqlen=16 + 8 * 420 + 1, budget_frac=0.3),                    # last window of one token
+    dict(l_obs=61, window=16, max_seqlen=3000, budget_frac=0.3),           # observation rows over four windows, not aligned
+    dict(l_obs=64, window=8, max_seqlen=2500, budget_frac=0.3),            # ... over eight
+    dict(window=7, max_seqlen=3200, budget_frac=0.2, l_obs=5),
+    dict(window=200, max_seqlen=5000, budget_frac=0.3, n_planted=2),       # windows of several pieces
+    dict(layout="bnhd", max_seqlen=3001, budget_frac=0.4, dtype="f32", head_dim=64, l_obs=8),
+    dict(ragged=True, max_seqlen=4000, budget_frac=0.3),
+], ids=lambda c: "-".join(f"{k}{v}" for k, v in c.items()))
+def test_compaction_in_place_by_chains(case, pattern):
+    """More rows than one batch and at most half of the windows retained: every chain of slots that read one another's
+    windows, and the stretch that the observation rows overwrite, in all the ways they can meet."""
+    test_compaction_in_place(dict(batch=20, n_q_heads=4, n_kv_heads=2) | case, pattern)
