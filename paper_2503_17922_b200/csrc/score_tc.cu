@@ -13,7 +13,7 @@
 //            exp2(x_ij - lse2_i) over the rows (Eq. 2); the block then pools its windows (Eq. 3-4).
 //            The block re-reads the keys it streamed in sweep 1, now from L2.
 //   select   the block of a unit's last chunk waits for the unit's other blocks and runs the selection.
-// Units are taken in waves whose keys fit L2 together.  A work item is (unit, chunk of <= 17 key
+// Units are taken in waves of as many as the blocks can share (tc_plan).  A work item is (unit, chunk of <= 37 key
 // tiles); the persistent blocks (at most one per SM) take the items of a wave round-robin.
 //
 // Warp roles: warp 0 issues the TMA tile loads (4-stage ring), warp 1 issues the MMAs (each as a whole
@@ -43,14 +43,17 @@ namespace {
 
 using namespace tc;
 
-constexpr int kStages = 4;
+constexpr int kMaxStages = 4;
+// Ring depth: two 128-row blocks of Q and their two buffers of token scores leave room for three stages (a key tile
+// lasts twice as long there; the fourth stage made no difference)
+__host__ __device__ constexpr int stages_for(int mb) { return mb == 2 ? 3 : kMaxStages; }
 constexpr int kEarlyTiles = 2;                           // key tiles requested ahead of the Q image at the start of an item
 constexpr int kMaxGroups = 4;
 __host__ __device__ constexpr int groups_for(int) { return 4; }
 __host__ __device__ constexpr int block_threads(int mb) { return 64 + groups_for(mb) * 128; }
 constexpr int kTile = kTcTileKeys;                       // keys per tile
 constexpr int kRegion = kTile * 128;                     // bytes of one 64-column block of a key tile
-constexpr int kChunkCap = kTcMaxChunkTiles * kTile + kTcMaxWindow;   // token scores a block may hold
+constexpr int kChunkCap = kTcChunkCap;                   // token scores a block may hold
 
 struct TcArgs {
     KShape s;
@@ -75,15 +78,15 @@ __device__ __forceinline__ uint8_t *align_1024(uint8_t *p)
 }
 
 struct Barriers {
-    uint64_t full[kStages];        // TMA -> MMA: the stage holds a key tile
-    uint64_t empty[kStages];       // MMA -> TMA: the MMAs that read the stage have completed
+    uint64_t full[kMaxStages];        // TMA -> MMA: the stage holds a key tile
+    uint64_t empty[kMaxStages];       // MMA -> TMA: the MMAs that read the stage have completed
     uint64_t tfull[kMaxGroups];    // MMA -> compute group: the accumulator buffer is complete
     uint64_t tempty[kMaxGroups];   // compute group -> MMA: the accumulator buffer has been read
 };
 
 __device__ __forceinline__ void init_barriers(Barriers &bar)
 {
-    for (int i = 0; i < kStages; ++i) {
+    for (int i = 0; i < kMaxStages; ++i) {
         mbar_init(&bar.full[i], 1);
         mbar_init(&bar.empty[i], 1);
     }
@@ -128,12 +131,13 @@ struct Item {
 };
 // Tile taken at step u of an item.  Sweep 1 and a sweep 2 that has to load everything go through the
 // tiles in ascending order.  A block that scores the item it has just taken statistics of still holds
-// that item's last kStages tiles in the ring, in ring order: it scores those first, without
+// that item's last STAGES tiles in the ring, in ring order: it scores those first, without
 // loading them again, and then walks down through the rest.
+template <int STAGES>
 __device__ __forceinline__ int tile_at(const Item &im, int u)
 {
     if (!im.reuse) return u;
-    return u < kStages ? im.n_tiles - kStages + u : im.n_tiles - 1 - u;
+    return u < STAGES ? im.n_tiles - STAGES + u : im.n_tiles - 1 - u;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -145,7 +149,7 @@ __global__ void __launch_bounds__(block_threads(MB), 1)
 score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ TcArgs a,
                  const __nv_bfloat16 *__restrict__ q)
 {
-    constexpr int NG = groups_for(MB);
+    constexpr int NG = groups_for(MB), kStages = stages_for(MB);
     constexpr int kThreads = block_threads(MB);
     constexpr int q_rows = MB * 128;
     constexpr int q_region = q_rows * 128;                // bytes of one 64-column block of the Q image
@@ -280,7 +284,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
             }
             if (g >= kStages && !mbar_wait(&bar.empty[st], ((g / kStages) - 1) & 1, &abort_s)) return;
             mbar_arrive_expect_tx_if(leader, &bar.full[st], (uint32_t)stage_bytes);
-            const int tok = tok0 + tile_at(im, t) * kTile;
+            const int tok = tok0 + tile_at<kStages>(im, t) * kTile;
             const int c1 = a.slot_tok == 1 ? tok : (a.slot_h == 1 ? im.h : bcoord);
             const int c2 = a.slot_tok == 2 ? tok : (a.slot_h == 2 ? im.h : bcoord);
             const int c3 = a.slot_tok == 3 ? tok : (a.slot_h == 3 ? im.h : bcoord);
@@ -396,7 +400,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                 score_accumulate<16>(vt, neg_lse2 + n32 * 32, c, a0, a1, a2, a3);
             }
             const float tj = (a0 + a1) + (a2 + a3);
-            const int j = im.j_begin + tile_at(im, t) * kTile + L;
+            const int j = im.j_begin + tile_at<kStages>(im, t) * kTile + L;
             if (j < im.j_end) {
                 t_chunk[rh][j - im.j_begin] = tj;
                 if (MB == 1 && a.token_scores) a.token_scores[(size_t)im.unit * s.nr_max + j] = tj;
@@ -814,7 +818,7 @@ DeviceInfo *device_info()
 
 size_t tc_smem_bytes(int kblocks, int mb)
 {
-    return 1024 + (size_t)kblocks * mb * 128 * 128 + (size_t)kStages * kblocks * kRegion;
+    return 1024 + (size_t)kblocks * mb * 128 * 128 + (size_t)stages_for(mb) * kblocks * kRegion;
 }
 
 }  // namespace
@@ -853,7 +857,7 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
     a.n_stat_chunks = ws.n_stat_chunks;
     a.r_pad = ws.r_pad;
     const int units = ks.batch * ks.hkv;
-    const TcPlan plan = tc_plan(units, ks.max_seqlen, ks.d);
+    const TcPlan plan = tc_plan(units, ks.max_seqlen, ks.omega);
     a.chunks_per_unit = plan.chunks_per_unit;
     a.units_per_wave = plan.units_per_wave;
     a.kblocks = ks.d / 64;

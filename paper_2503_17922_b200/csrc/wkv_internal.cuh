@@ -107,9 +107,13 @@ constexpr int kTcMaxChunkTiles = 16;
 constexpr int kTcTargetBlocks = 148;
 constexpr int kTcMaxWindow = 1024;
 
-// The tensor-core kernel works through the units in waves whose keys fit the L2 cache together, so
-// that the second sweep over a wave's keys is served from L2.  kTcWaveBytes is the budget.
+// The pipelined kernel works through the units in waves whose keys fit the L2 cache together.
 constexpr long long kTcWaveBytes = 80ll << 20;
+
+// Key tiles a block of the tensor-core kernel may take per item: what its buffer of token scores holds when the
+// chunk is rounded up to whole windows (37 tiles for windows of up to 128 tokens, 30 for 1,024).
+constexpr int kTcChunkCap = 4864;
+__host__ __device__ inline int tc_max_chunk_tiles(int omega) { return (kTcChunkCap - omega) / kTcTileKeys; }
 
 struct TcPlan {
     int units_per_wave;   // units swept together
@@ -118,25 +122,25 @@ struct TcPlan {
 // What a wave costs beside its key tiles, in tiles per block: filling the pipeline, the hand-over of the
 // statistics and the pooling take about 8 us, a tile 0.65 us per sweep.
 constexpr int kTcWaveOverhead = 6;
-inline TcPlan tc_plan(int units, int max_seqlen, int head_dim)
+inline TcPlan tc_plan(int units, int max_seqlen, int omega)
 {
-    // Every number of units per wave whose keys fit the L2 budget and whose blocks are resident together is
-    // tried, and the one with the least (waves x (tiles per block + overhead)) taken.  The largest that fits
-    // is not the best when it leaves a last wave nearly empty: 16 units of 192 tiles as 12 + 4 made 16 tiles
-    // per block and wave, 8 + 8 makes 11.
+    // Every number of units per wave whose blocks are resident together is tried, and the one with the least (waves x
+    // (tiles per block + overhead)) taken.  The largest is not the best when it leaves a last wave nearly empty: 16
+    // units of 192 tiles as 12 + 4 made 16 tiles per block and wave, 8 + 8 makes 11.  Whether a wave's keys fit L2
+    // between the two sweeps does not count: a wave costs more than reading keys from HBM again beside the
+    // exponentials (8 sequences of 32-64 K keys, R = 256, scoring: 80 MB waves 690 us, 104 MB 630 us, 170 MB 560 us).
     TcPlan best;
     best.units_per_wave = 1;
     best.chunks_per_unit = 1;
-    const long long unit_bytes = (long long)max_seqlen * head_dim * 2;
     const int max_tiles = (max_seqlen + kTcTileKeys - 1) / kTcTileKeys;
     // a unit needs at least this many blocks (the token scores of a chunk live in shared memory)
-    const int min_chunks = (max_tiles + kTcMaxChunkTiles - 1) / kTcMaxChunkTiles;
-    long long most = kTcWaveBytes / (unit_bytes > 0 ? unit_bytes : 1);
-    if (most > kTcTargetBlocks / min_chunks) most = kTcTargetBlocks / min_chunks;
+    const int chunk_tiles = tc_max_chunk_tiles(omega);
+    const int min_chunks = (max_tiles + chunk_tiles - 1) / chunk_tiles;
+    int most = kTcTargetBlocks / min_chunks;
     if (most > units) most = units;
     if (most < 1) most = 1;
     long long best_cost = -1;
-    for (int upw = (int)most; upw >= 1; --upw) {
+    for (int upw = most; upw >= 1; --upw) {
         int chunks = kTcTargetBlocks / upw;
         if (chunks < min_chunks) chunks = min_chunks;
         if (chunks > max_tiles) chunks = max_tiles;
