@@ -11,7 +11,7 @@
 //            observation window).  K comes from HBM.
 //   sweep 2  D[keys, rows] = K Q^T with the keys on the lanes: one thread owns one key and sums
 //            exp2(x_ij - lse2_i) over the rows (Eq. 2); the block then pools its windows (Eq. 3-4).
-//            The block re-reads the keys it streamed in sweep 1, now from L2.
+//            The block re-reads the keys it streamed in sweep 1, as far as they fit from L2.
 //   select   the block of a unit's last chunk waits for the unit's other blocks and runs the selection.
 // Units are taken in waves of as many as the blocks can share (tc_plan).  A work item is (unit, chunk of <= 37 key
 // tiles); the persistent blocks (at most one per SM) take the items of a wave round-robin.

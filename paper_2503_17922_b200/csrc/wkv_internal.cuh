@@ -128,7 +128,8 @@ inline TcPlan tc_plan(int units, int max_seqlen, int omega)
     // (tiles per block + overhead)) taken.  The largest is not the best when it leaves a last wave nearly empty: 16
     // units of 192 tiles as 12 + 4 made 16 tiles per block and wave, 8 + 8 makes 11.  Whether a wave's keys fit L2
     // between the two sweeps does not count: a wave costs more than reading keys from HBM again beside the
-    // exponentials (8 sequences of 32-64 K keys, R = 256, scoring: 80 MB waves 690 us, 104 MB 630 us, 170 MB 560 us).
+    // exponentials (8 sequences of 32-64 K keys, R = 256, one layer: 669 us with waves of at most 104 MB, 599 us with up
+    // to 170 MB).
     TcPlan best;
     best.units_per_wave = 1;
     best.chunks_per_unit = 1;
