@@ -3,7 +3,8 @@
 //   stats : per row of the unit, partial (max, sum exp2) over a chunk of keys
 //           (Eq. 1's normaliser, causal mask applied)
 //   score : logits again, p = exp2(x - lse2), sum over the rows (Eq. 2), then the
-//           Top-p window pooling of Eq. 3-4
+//           Top-p window pooling of Eq. 3-4 and, when asked, the selection by the
+//           block that finishes a unit last
 // Summation orders are fixed, so results are bit-identical from run to run.
 //
 // These problems are small (a few thousand keys), so what bounds them is the length of the chain from
@@ -15,6 +16,7 @@
 // 2 heads x 1,024 keys, 16 rows, d = 64: one block per 512 keys took 31 + 25 us for the two kernels (whole
 // group 84 us); see simt_tiles_per_block for the sizes where a block takes more tiles.
 #include "score_math.cuh"
+#include "topk_block.cuh"
 #include "wkv_internal.cuh"
 
 #include <mutex>
@@ -260,6 +262,11 @@ score_stats_simt(const __grid_constant__ KShape s, const T *__restrict__ q, cons
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// the selection that the score kernel's last block of a unit runs (window_idx null: none)
+struct SimtSelect {
+    int *window_idx, *kept_len, *status, *sync;
+};
+
 // Eq. 4 for one window: the sorting network where there is one for its length, else the serial form
 __device__ inline float pool_window(const float *w, int omega, int size, int p)
 {
@@ -277,8 +284,8 @@ template <typename T, int RB>
 // of the kernel its place beside the statistics kernel's blocks: 44.6 us instead of 42.1 us for 4 heads x 6,000 keys)
 __global__ void __launch_bounds__(kThreads, 5)
 score_pool_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const T *__restrict__ k, const float2 *stats,
-                const float *lse_obs, float *__restrict__ window_scores, float *__restrict__ token_scores, int n_chunks,
-                int r_pad, int r_tile, int chunk_keys)
+                const float *lse_obs, float *window_scores, float *__restrict__ token_scores, int n_chunks,
+                int r_pad, int r_tile, int chunk_keys, const __grid_constant__ SimtSelect sel)
 {
     constexpr int KPT = TileMap<RB>::KPT, TX = TileMap<RB>::TX, TY = kThreads / TX;
     extern __shared__ __align__(16) float smem[];
@@ -287,6 +294,7 @@ score_pool_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const
     float *lse2 = ks + s.d * kKPad;            // [r_pad]
     float *part = lse2 + r_pad;                // [TY][kKT]
     float *t_chunk = part + TY * kKT;          // [chunk_keys rounded up to kKT]
+    TopkSmem &topk_sm = *reinterpret_cast<TopkSmem *>(smem);   // the selection comes when all of these are done with
 
     pdl_trigger();
     // with given normalisers there is no statistics kernel in front that has waited for Q and K
@@ -298,6 +306,10 @@ score_pool_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const
     const int j_begin = blockIdx.x * chunk_keys;
     if (n_r <= 0 || j_begin >= n_r) {
         if (!lse_obs) pdl_wait();
+        // a unit without review context still gets its (empty) selection
+        if (sel.window_idx && n_r <= 0 && blockIdx.x == 0)
+            select_topk_block<kThreads>(topk_sm, window_scores, 0, 0, s.k_max, sel.window_idx + (size_t)unit * s.k_max,
+                                        sel.kept_len + unit, n, s.alpha, s.omega);
         return;
     }
     const int j_end = min(n_r, j_begin + chunk_keys);
@@ -377,6 +389,26 @@ score_pool_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const
         window_scores[(size_t)unit * s.kw_max + w_begin + lw] =
             pool_window(t_chunk + lo, s.omega, min(s.omega, (j_end - j_begin) - lo), s.p);
     }
+    if (!sel.window_idx) return;
+    // The block that counts itself last on the unit's ticket word selects for the unit and clears the word.
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const int used = (n_r + chunk_keys - 1) / chunk_keys;
+        int *ticket = sel.sync + kSyncTickets + kSyncWordsPerUnit * unit;
+        __threadfence();                 // publishes the window scores the whole block wrote
+        const int before = atomicAdd(ticket, 1);
+        if (before == used - 1) atomicExch(ticket, 0);
+        if (before < 0 || before >= used) atomicOr(sel.status, kStatusWaitExpired);   // the workspace was not cleared
+        __threadfence();
+        topk_sm.remaining = before == used - 1;
+    }
+    __syncthreads();
+    const bool selects = topk_sm.remaining != 0;
+    __syncthreads();                     // the word is the selection's own from here on
+    if (selects)
+        select_topk_block<kThreads>(topk_sm, window_scores + (size_t)unit * s.kw_max, num_windows(n, s.alpha, s.omega),
+                                    num_selected_capped(n, s.alpha, s.omega, si.budget, s.k_max), s.k_max,
+                                    sel.window_idx + (size_t)unit * s.k_max, sel.kept_len + unit, n, s.alpha, s.omega);
 }
 
 }  // namespace
@@ -424,12 +456,13 @@ static void simt_smem(const KShape &ks, int r_pad, size_t &stats_bytes, size_t &
     const size_t tiles = (size_t)ks.d * r_tile + (size_t)ks.d * kKPad;
     stats_bytes = sizeof(float) * (tiles + (tpb < kChunkTiles ? 2 * (size_t)r_pad : 0) + (rb == 16 ? 2 * (size_t)r_pad : 0) + (size_t)r_tile);
     pool_bytes = sizeof(float) * (tiles + (size_t)r_pad + (size_t)(rb / 4) * kKT + (size_t)((chunk_keys + kKT - 1) / kKT) * kKT);
+    if (pool_bytes < sizeof(TopkSmem)) pool_bytes = sizeof(TopkSmem);
 }
 
 template <typename T, int RB>
 static cudaError_t launch_simt_tile(const KShape &ks, int slot, const void *q, const void *k, float *window_scores,
                                     float *token_scores, float2 *stats, const Workspace &ws, cudaStream_t stream,
-                                    const float *lse_obs)
+                                    const float *lse_obs, const SimtSelect &sel)
 {
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -453,7 +486,7 @@ static cudaError_t launch_simt_tile(const KShape &ks, int slot, const void *q, c
     const int n_r_max = ks.max_seqlen - ks.alpha;
     err = launch_pdl(fn, dim3((n_r_max + chunk_keys - 1) / chunk_keys, units), kThreads, smem2, stream, 1, ks, (const T *)q,
                      (const T *)k, (const float2 *)stats, lse_obs, window_scores, token_scores, ws.n_stat_chunks, r_pad, r_tile,
-                     chunk_keys);
+                     chunk_keys, sel);
     if (err == cudaSuccess) count_launches(lse_obs ? 1 : 2);
     return err;
 }
@@ -461,23 +494,38 @@ static cudaError_t launch_simt_tile(const KShape &ks, int slot, const void *q, c
 template <typename T>
 static cudaError_t launch_simt_type(const KShape &ks, int slot, const void *q, const void *k, float *window_scores,
                                     float *token_scores, float2 *stats, const Workspace &ws, cudaStream_t stream,
-                                    const float *lse_obs)
+                                    const float *lse_obs, const SimtSelect &sel)
 {
     switch (simt_row_tile(ks)) {
-    case 16: return launch_simt_tile<T, 16>(ks, slot, q, k, window_scores, token_scores, stats, ws, stream, lse_obs);
-    case 32: return launch_simt_tile<T, 32>(ks, slot + 2, q, k, window_scores, token_scores, stats, ws, stream, lse_obs);
-    default: return launch_simt_tile<T, 64>(ks, slot + 4, q, k, window_scores, token_scores, stats, ws, stream, lse_obs);
+    case 16: return launch_simt_tile<T, 16>(ks, slot, q, k, window_scores, token_scores, stats, ws, stream, lse_obs, sel);
+    case 32: return launch_simt_tile<T, 32>(ks, slot + 2, q, k, window_scores, token_scores, stats, ws, stream, lse_obs, sel);
+    default: return launch_simt_tile<T, 64>(ks, slot + 4, q, k, window_scores, token_scores, stats, ws, stream, lse_obs, sel);
     }
 }
 
 cudaError_t launch_score_simt(const KShape &ks, int dtype, const void *q, const void *k,
                               float *window_scores, float *token_scores,
-                              void *workspace, const Workspace &ws, cudaStream_t stream, const float *lse_obs)
+                              void *workspace, const Workspace &ws, cudaStream_t stream, const float *lse_obs,
+                              int *window_idx, int *kept_len)
 {
     float2 *stats = reinterpret_cast<float2 *>(static_cast<char *>(workspace) + ws.stats_off);
-    if (ks.max_seqlen <= ks.alpha) return cudaSuccess;
-    return dtype == WKV_F32 ? launch_simt_type<float>(ks, 0, q, k, window_scores, token_scores, stats, ws, stream, lse_obs)
-                            : launch_simt_type<__nv_bfloat16>(ks, 6, q, k, window_scores, token_scores, stats, ws, stream, lse_obs);
+    if (ks.max_seqlen <= ks.alpha) return window_idx ? launch_topk(ks, window_scores, window_idx, kept_len, stream) : cudaSuccess;
+    // The selection inside the score kernel where a block keeps the unit's window scores in registers (eight per
+    // thread): one launch less.  Longer lists go to the kernel with four times the threads.
+    const bool inside = window_idx && ks.kw_max <= 8 * kThreads;
+    SimtSelect sel = {};
+    if (inside) {
+        sel.window_idx = window_idx;
+        sel.kept_len = kept_len;
+        sel.status = reinterpret_cast<int *>(static_cast<char *>(workspace) + ws.status_off);
+        sel.sync = reinterpret_cast<int *>(static_cast<char *>(workspace) + ws.sync_off);
+    }
+    const cudaError_t err =
+        dtype == WKV_F32
+            ? launch_simt_type<float>(ks, 0, q, k, window_scores, token_scores, stats, ws, stream, lse_obs, sel)
+            : launch_simt_type<__nv_bfloat16>(ks, 6, q, k, window_scores, token_scores, stats, ws, stream, lse_obs, sel);
+    if (err != cudaSuccess || !window_idx || inside) return err;
+    return launch_topk(ks, window_scores, window_idx, kept_len, stream);
 }
 
 // shared-memory need of the CUDA-core kernels, for the host-side support check

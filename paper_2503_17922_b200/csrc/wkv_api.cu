@@ -255,12 +255,9 @@ int do_score(const wkv_shape *s, const KShape &ks, const Workspace &ws, const vo
         if (st != WKV_ERR_UNSUPPORTED || forced) return st;
         if (score_simt_smem_bytes(ks, ws.r_pad) > 227u * 1024u) return st;
     }
-    st = check_cuda(launch_score_simt(ks, s->dtype, q, k, window_scores, token_scores, workspace, ws, stream,
-                                      lse_obs),
-                    "score kernels");
-    if (st == WKV_OK && window_idx)
-        st = check_cuda(launch_topk(ks, window_scores, window_idx, kept_len, stream), "selection kernel");
-    return st;
+    return check_cuda(launch_score_simt(ks, s->dtype, q, k, window_scores, token_scores, workspace, ws, stream, lse_obs,
+                                        window_idx, kept_len),
+                      "score kernels");
 }
 
 static int fill_table(int n_layers, const void *const *k_layers, const void *const *v_layers,

@@ -232,7 +232,8 @@ Workspace plan_workspace(const KShape &ks);
 cudaError_t launch_score_simt(const KShape &ks, int dtype, const void *q, const void *k,
                               float *window_scores, float *token_scores,
                               void *workspace, const Workspace &ws, cudaStream_t stream,
-                              const float *lse_obs = nullptr);
+                              const float *lse_obs = nullptr, int *window_idx = nullptr,
+                              int *kept_len = nullptr);
 bool score_tc_supported(const KShape &ks, int dtype);
 // window_idx / kept_len non-null: the selection is fused into the same launch.
 // lse_obs non-null: float [B, H_q, alpha], natural log of Eq. 1's normaliser of every observation

@@ -574,6 +574,29 @@ def test_host_buffer_entry_point_reads_only_what_it_needs(monkeypatch, pinned, b
     pu.check_gather(w, grp, got)
 
 
+@pytest.mark.parametrize("n_windows", [1, 15, 17, 2048, 2049])
+def test_selection_inside_and_behind_the_cuda_core_score_kernel(n_windows):
+    """Up to 2,048 windows per unit are selected by the score kernel's last block of the unit, more by the kernel of its
+    own; twice on one workspace, whose ticket words clear themselves."""
+    w = small(dtype="f32", head_dim=64, n_q_heads=4, l_obs=8, window=4, n_planted=0, budget_frac=0.25, batch=1,
+              max_seqlen=8 + 4 * n_windows - (1 if n_windows > 1 else 0))
+    grp = wl.make_group(w, 0)
+    ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
+    prob = binding.Problem.from_workload(w)
+    assert prob.kw_max == n_windows
+    q, k = binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0])
+    work, out = prob.alloc_workspace(), prob.alloc_outputs(0)
+    for _ in range(2):
+        out["window_idx"].fill_(-7)
+        out["kept_len"].fill_(-7)
+        binding.wkv_select_leader_windows(prob, q, k, out["window_scores"], out["window_idx"], out["kept_len"], work)
+        torch.cuda.synchronize()
+        assert binding.device_status(work) == 0
+        got = {"prob": prob, "window_scores": out["window_scores"].cpu().numpy(),
+               "window_idx": out["window_idx"].cpu().numpy(), "kept_len": out["kept_len"].cpu().numpy()}
+        pu.check_selection(w, grp, got, ref)
+
+
 @pytest.mark.parametrize("impl", ["simt", "tc", "pipe"])
 def test_stale_device_copy_of_cu_seqlens_stays_in_bounds(impl):
     """cu_seqlens and budgets exist as a host and a device copy, and sizes are derived from the host
