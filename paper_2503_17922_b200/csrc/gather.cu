@@ -8,10 +8,15 @@
 // once per vector.  The observation rows are handled as extra windows behind the selected ones.
 #include "wkv_internal.cuh"
 
+#include <algorithm>
+
 namespace wkv {
 namespace {
 
 constexpr int kThreads = 256;
+// Rows that the GPU reads over the bus: so many blocks of 32 KB in flight fill it, and leave the copies that go back at
+// the same time their share (4 layers x 8,192 keys from pinned memory: 854 us, with all blocks at once 889 us).
+constexpr int kBusBlocks = 16;
 constexpr int kBatch = 8;             // independent 16-byte loads in flight per lane
 
 struct GatherParams {
@@ -47,8 +52,8 @@ __device__ __forceinline__ void st_stream(int4 *p, const int4 &v)
 }
 
 // PAGED is a separate instantiation: its per-row page arithmetic would otherwise cost the plain copy
-// registers it needs for its loads in flight.
-template <bool PAGED>
+// registers it needs for its loads in flight; so is STRIDED, in which the grid may be smaller than the work.
+template <bool PAGED, bool STRIDED>
 __global__ void __launch_bounds__(kThreads, 4)
 gather_kv_kernel(const __grid_constant__ GatherParams prm)
 {
@@ -61,8 +66,9 @@ gather_kv_kernel(const __grid_constant__ GatherParams prm)
     // The window and the unit's last one are looked up before it is known how many are selected (that takes a trip to
     // memory of its own): the chain from launch to the first row is one trip shorter.
     const int *idx = prm.window_idx + (size_t)unit * s.k_max;
-    const int slot = (blockIdx.x * kThreads + threadIdx.x) >> prm.lanes_shift, lane = threadIdx.x & (lanes - 1);
-    const int wi = slot < s.k_max ? idx[slot] : -1;
+    int slot = (blockIdx.x * kThreads + threadIdx.x) >> prm.lanes_shift;
+    const int lane = threadIdx.x & (lanes - 1);
+    int wi = slot < s.k_max ? idx[slot] : -1;
     const int wi_last = idx[s.k_max - 1];
     const SeqInfo si = seq_info(s, b);
     const int n = si.n;
@@ -97,75 +103,82 @@ gather_kv_kernel(const __grid_constant__ GatherParams prm)
     const int *pages = paged ? prm.block_table + (size_t)b * prm.max_pages : nullptr;
     if (paged) dst = reinterpret_cast<int4 *>(prm.tab.dst[tensor]) + (long long)h * prm.head_vecs;
 
-    if (slot >= k + prm.obs_slots) return;
-    int src_row0, dst_row0, n_rows;
-    if (slot < k) {
-        // an entry that is no window of this sequence (a list that no selection has written, or
-        // that the caller filled wrongly) is skipped: the kernel never leaves the tensors
-        if (wi < 0 || wi >= kw) return;
-        src_row0 = wi * s.omega;
-        n_rows = min(s.omega, n_r - src_row0);
-        dst_row0 = slot * s.omega;
-    } else {
-        const int o = (slot - k) * s.omega;
-        src_row0 = n_r + o;
-        n_rows = min(s.omega, obs_rows - o);
-        dst_row0 = review_rows + o;
-    }
-    if (n_rows <= 0) return;
-    // dense output: a unit owns keep_capacity rows (cannot trigger while the device copies of
-    // cu_seqlens / budgets equal the host copies the capacity was checked against)
-    if (!prm.cu_out && !paged && dst_row0 + n_rows > prm.keep_capacity) return;
-    if (paged) {
-        // every row finds its page; a row whose page entry is missing or negative is skipped
+    auto move = [&](int slot, int wi) {
+        int src_row0, dst_row0, n_rows;
+        if (slot < k) {
+            // an entry that is no window of this sequence (a list that no selection has written, or
+            // that the caller filled wrongly) is skipped: the kernel never leaves the tensors
+            if (wi < 0 || wi >= kw) return;
+            src_row0 = wi * s.omega;
+            n_rows = min(s.omega, n_r - src_row0);
+            dst_row0 = slot * s.omega;
+        } else {
+            const int o = (slot - k) * s.omega;
+            src_row0 = n_r + o;
+            n_rows = min(s.omega, obs_rows - o);
+            dst_row0 = review_rows + o;
+        }
+        if (n_rows <= 0) return;
+        // dense output: a unit owns keep_capacity rows (cannot trigger while the device copies of
+        // cu_seqlens / budgets equal the host copies the capacity was checked against)
+        if (!prm.cu_out && !paged && dst_row0 + n_rows > prm.keep_capacity) return;
+        if (paged) {
+            // every row finds its page; a row whose page entry is missing or negative is skipped
+            const int n_vec = n_rows * vpr;
+            for (int v0 = lane; v0 < n_vec; v0 += lanes * kBatch) {
+                int4 val[kBatch];
+                long long doff[kBatch];
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    const int v = v0 + u * lanes;
+                    doff[u] = -1;
+                    if (v < n_vec) {
+                        const int r = prm.vec_shift >= 0 ? v >> prm.vec_shift : v / vpr;
+                        const int c = v - r * vpr;
+                        const int row = dst_row0 + r, page = row / prm.page_size;
+                        const int phys = page < prm.max_pages ? pages[page] : -1;
+                        if (phys >= 0 && phys < prm.num_pages)
+                            doff[u] = (long long)phys * prm.page_vecs + (long long)(row - page * prm.page_size) * prm.row_vecs + c;
+                        val[u] = ld_stream(src + (long long)(src_row0 + r) * src_row_vecs + c);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u)
+                    if (doff[u] >= 0) st_stream(dst + doff[u], val[u]);
+            }
+            return;
+        }
+        const int4 *sp = src + src_row0 * src_row_vecs;
+        int4 *dp = dst + dst_row0 * dst_row_vecs;
         const int n_vec = n_rows * vpr;
         for (int v0 = lane; v0 < n_vec; v0 += lanes * kBatch) {
             int4 val[kBatch];
-            long long doff[kBatch];
+            int soff[kBatch], doff[kBatch];   // offsets inside one window: small
 #pragma unroll
             for (int u = 0; u < kBatch; ++u) {
                 const int v = v0 + u * lanes;
-                doff[u] = -1;
                 if (v < n_vec) {
-                    const int r = prm.vec_shift >= 0 ? v >> prm.vec_shift : v / vpr;
-                    const int c = v - r * vpr;
-                    const int row = dst_row0 + r, page = row / prm.page_size;
-                    const int phys = page < prm.max_pages ? pages[page] : -1;
-                    if (phys >= 0 && phys < prm.num_pages)
-                        doff[u] = (long long)phys * prm.page_vecs + (long long)(row - page * prm.page_size) * prm.row_vecs + c;
-                    val[u] = ld_stream(src + (long long)(src_row0 + r) * src_row_vecs + c);
+                    soff[u] = v;
+                    doff[u] = v;
+                    if (!src_dense || !dst_dense) {
+                        const int r = prm.vec_shift >= 0 ? v >> prm.vec_shift : v / vpr;
+                        const int c = v - r * vpr;
+                        if (!src_dense) soff[u] = r * (int)src_row_vecs + c;
+                        if (!dst_dense) doff[u] = r * (int)dst_row_vecs + c;
+                    }
+                    val[u] = ld_stream(sp + soff[u]);
                 }
             }
 #pragma unroll
             for (int u = 0; u < kBatch; ++u)
-                if (doff[u] >= 0) st_stream(dst + doff[u], val[u]);
+                if (v0 + u * lanes < n_vec) st_stream(dp + doff[u], val[u]);
         }
-        return;
-    }
-    const int4 *sp = src + src_row0 * src_row_vecs;
-    int4 *dp = dst + dst_row0 * dst_row_vecs;
-    const int n_vec = n_rows * vpr;
-    for (int v0 = lane; v0 < n_vec; v0 += lanes * kBatch) {
-        int4 val[kBatch];
-        int soff[kBatch], doff[kBatch];   // offsets inside one window: small
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-            const int v = v0 + u * lanes;
-            if (v < n_vec) {
-                soff[u] = v;
-                doff[u] = v;
-                if (!src_dense || !dst_dense) {
-                    const int r = prm.vec_shift >= 0 ? v >> prm.vec_shift : v / vpr;
-                    const int c = v - r * vpr;
-                    if (!src_dense) soff[u] = r * (int)src_row_vecs + c;
-                    if (!dst_dense) doff[u] = r * (int)dst_row_vecs + c;
-                }
-                val[u] = ld_stream(sp + soff[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u)
-            if (v0 + u * lanes < n_vec) st_stream(dp + doff[u], val[u]);
+    };
+    if (STRIDED) {
+        const int stride = gridDim.x * (kThreads >> prm.lanes_shift);
+        for (; slot < k + prm.obs_slots; slot += stride, wi = slot < k ? idx[slot] : -1) move(slot, wi);
+    } else if (slot < k + prm.obs_slots) {
+        move(slot, wi);
     }
 }
 
@@ -173,7 +186,7 @@ gather_kv_kernel(const __grid_constant__ GatherParams prm)
 
 cudaError_t launch_gather(const KShape &ks, int elem_bytes, int n_tensors, const LayerTable &tab,
                           const int *window_idx, const int *cu_out, int keep_capacity,
-                          cudaStream_t stream, const PagedOut *paged)
+                          cudaStream_t stream, const PagedOut *paged, bool over_bus)
 {
     GatherParams prm;
     prm.block_table = nullptr;
@@ -207,8 +220,10 @@ cudaError_t launch_gather(const KShape &ks, int elem_bytes, int n_tensors, const
     while (prm.lanes_shift > 3 && window_vecs <= (kBatch << (prm.lanes_shift - 1))) --prm.lanes_shift;
     const int slots_per_block = kThreads >> prm.lanes_shift;
     const int max_slots = ks.k_max + prm.obs_slots;
-    dim3 grid((max_slots + slots_per_block - 1) / slots_per_block, ks.batch * ks.hkv, n_tensors);
-    const cudaError_t err = launch_pdl(paged ? gather_kv_kernel<true> : gather_kv_kernel<false>, grid, kThreads, 0, stream, 1, prm);
+    int blocks = (max_slots + slots_per_block - 1) / slots_per_block;
+    if (over_bus) blocks = std::max(1, std::min(blocks, kBusBlocks / (ks.batch * ks.hkv * n_tensors)));
+    dim3 grid(blocks, ks.batch * ks.hkv, n_tensors);
+    const cudaError_t err = launch_pdl(paged ? gather_kv_kernel<true, false> : (over_bus ? gather_kv_kernel<false, true> : gather_kv_kernel<false, false>), grid, kThreads, 0, stream, 1, prm);
     if (err != cudaSuccess) return err;
     count_launches(1);
     return cudaSuccess;

@@ -531,10 +531,10 @@ int wkv_select_topk_windows(const wkv_shape *s, const float *window_scores, int3
                       "selection kernel");
 }
 
-int wkv_gather_kv(const wkv_shape *s, int32_t n_layers, const void *const *k_layers,
+static int gather_kv_entry(const wkv_shape *s, int32_t n_layers, const void *const *k_layers,
                   const void *const *v_layers, const int32_t *window_idx, void *const *k_out_layers,
                   void *const *v_out_layers, const int32_t *cu_seqlens_out, int32_t keep_capacity,
-                  void *cuda_stream)
+                  void *cuda_stream, bool over_bus)
 {
     KShape ks;
     int st = resolve(s, ks);
@@ -552,8 +552,17 @@ int wkv_gather_kv(const wkv_shape *s, int32_t n_layers, const void *const *k_lay
         return WKV_ERR_SHAPE;
     }
     return check_cuda(launch_gather(ks, elem_bytes(s->dtype), n_tensors, tab, window_idx, cu_seqlens_out,
-                                    keep_capacity, static_cast<cudaStream_t>(cuda_stream)),
+                                    keep_capacity, static_cast<cudaStream_t>(cuda_stream), nullptr, over_bus),
                       "gather kernel");
+}
+
+int wkv_gather_kv(const wkv_shape *s, int32_t n_layers, const void *const *k_layers,
+                  const void *const *v_layers, const int32_t *window_idx, void *const *k_out_layers,
+                  void *const *v_out_layers, const int32_t *cu_seqlens_out, int32_t keep_capacity,
+                  void *cuda_stream)
+{
+    return gather_kv_entry(s, n_layers, k_layers, v_layers, window_idx, k_out_layers, v_out_layers, cu_seqlens_out,
+                           keep_capacity, cuda_stream, false);
 }
 
 int wkv_gather_kv_paged(const wkv_shape *s, int32_t n_layers, const void *const *k_layers,
@@ -887,8 +896,8 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_
             void *const out[2] = {k_out_layers_dev[l], v_out_layers_dev[l]};
             void *const out_host[2] = {k_out_layers_host[l], v_out_layers_host[l]};
             if (st == WKV_OK)
-                st = wkv_gather_kv(s, 1, &src[t], last ? nullptr : &src[1], window_idx_dev, &out[t], last ? nullptr : &out[1], nullptr,
-                                   keep_capacity, cuda_stream);
+                st = gather_kv_entry(s, 1, &src[t], last ? nullptr : &src[1], window_idx_dev, &out[t], last ? nullptr : &out[1],
+                                     nullptr, keep_capacity, cuda_stream, src[t] != staging[t] || src[1] != staging[1]);
             hand_over();
             d2h_after(out_host[t], out[t], out_bytes_per_layer, t ? "copy of compact V" : "copy of compact K");
             if (!last) d2h_after(out_host[1], out[1], out_bytes_per_layer, "copy of compact V");

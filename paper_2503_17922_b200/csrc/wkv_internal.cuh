@@ -268,9 +268,10 @@ struct PagedOut {
     int max_pages, page_size, num_pages;
     long long page_stride, head_stride, row_stride;
 };
+// over_bus: the rows are read from host memory (not for paged output)
 cudaError_t launch_gather(const KShape &ks, int elem_bytes, int n_tensors, const LayerTable &tab,
                           const int *window_idx, const int *cu_out, int keep_capacity,
-                          cudaStream_t stream, const PagedOut *paged = nullptr);
+                          cudaStream_t stream, const PagedOut *paged = nullptr, bool over_bus = false);
 // compaction of every layer's K/V inside its own buffer (compact.cu)
 struct InplaceTable {
     void *ptr[2 * WKV_MAX_GROUP_LAYERS];
