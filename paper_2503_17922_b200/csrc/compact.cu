@@ -256,6 +256,7 @@ cudaError_t launch_compact_inplace(const KShape &ks, int elem_bytes, int n_tenso
     const long long vecs = ((long long)ks.k_max * ks.omega + ks.alpha) * prm.vec_per_row;
     int cs = 1;
     while (cs < kMaxCluster && pairs * cs * 2 <= kResident && (long long)cs * kThreads * kMinVecs < vecs) cs *= 2;
+    while (cs * kThreads * kVecs < prm.vec_per_row) cs *= 2;      // a batch is at least one row (of at most 128 KB)
     prm.cluster = cs;
     // By chains where a cluster would need more than one batch (every batch is a trip to memory and back behind a
     // barrier: 18.6 us against 14.8 us a layer at 8 heads x 32,768 keys, 12 %; with one batch the cluster is faster,

@@ -194,3 +194,11 @@ def test_compaction_in_place_by_chains(case, pattern):
     """More rows than one batch and at most half of the windows retained: every chain of slots that read one another's
     windows, and the stretch that the observation rows overwrite, in all the ways they can meet."""
     test_compaction_in_place(dict(batch=20, n_q_heads=4, n_kv_heads=2) | case, pattern)
+
+
+@pytest.mark.parametrize("pattern", ["shift", "tail"])
+def test_compaction_in_place_of_rows_wider_than_a_block_moves_at_once(pattern):
+    """Rows of 80 KB (the entry point takes up to 128 KB) in 136 (unit, tensor) pairs, which get one block each as far as
+    occupancy goes: a block moves 64 KB at once."""
+    test_compaction_in_place(dict(batch=34, n_layers=1, gamma=1, n_q_heads=2, n_kv_heads=2, head_dim=40960, max_seqlen=20,
+                                  l_obs=2, window=3, top_p=2, budget_frac=0.8, n_planted=0), pattern)
