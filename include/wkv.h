@@ -272,7 +272,7 @@ int wkv_gather_kv_paged(const wkv_shape *s, int32_t n_layers,
  * in the tensor's own layout: afterwards row r < kept_len of unit (b, h) holds what wkv_gather_kv would
  * have written to row r of the compact cache; rows from kept_len on hold leftovers.  Rows only move
  * toward lower addresses; the kernel orders the reads of a stretch of rows before the writes that land
- * on them (one thread block walks a unit's rows in ascending batches), so the result is exact.
+ * on them, so the result is exact.
  *   k_layers, v_layers   HOST arrays [n_layers] of DEVICE pointers, read AND written (v_layers may be NULL)
  *   window_idx           DEVICE int32 [B, H_kv, wkv_k_max()], an ascending selection as written by
  *                        wkv_select_topk_windows; entries that are no window of the sequence or lie

@@ -38,6 +38,13 @@ def _indices(w, grp, prob, pattern):
                 lo = 1 if k < kw else 0
             elif pattern == "tail":
                 lo = kw - k
+            elif pattern == "run":      # half of them a run from window 2 on, the rest spread over what follows
+                half = min(k // 2, kw - 2) if kw > 2 else 0
+                rest = np.random.Generator(np.random.Philox(key=h)).permutation(np.arange(2 + half, kw))[: k - half]
+                if half + len(rest) == k:
+                    idx[b, h, :k] = np.concatenate([np.arange(2, 2 + half), np.sort(rest)])
+                    continue
+                lo = 0
             else:
                 lo = 0
             idx[b, h, :k] = np.arange(lo, lo + k)
@@ -55,9 +62,11 @@ def _indices(w, grp, prob, pattern):
 ], ids=lambda c: "-".join(f"{k}{v}" for k, v in c.items()) or "base")
 def test_compaction_in_place(case, pattern):
     case = dict(case)
-    layout = case.pop("layout", "bhnd")
+    layout, budgets = case.pop("layout", "bhnd"), case.pop("budgets", None)
     w = _case(**case)
     grp = wl.make_group(w, 0)
+    if budgets is not None:
+        grp["budgets"] = np.array(budgets, dtype=np.int32)
     prob = binding.Problem(dtype=w.dtype, batch=w.batch, n_q_heads=w.n_q_heads, n_kv_heads=w.n_kv_heads,
                            head_dim=w.head_dim, l_obs=w.l_obs, window=w.window, task=w.task, top_p=w.top_p,
                            max_seqlen=w.max_seqlen, budgets=grp["budgets"], cu_seqlens=grp["cu_seqlens"],
@@ -202,3 +211,46 @@ def test_compaction_in_place_of_rows_wider_than_a_block_moves_at_once(pattern):
     occupancy goes: a block moves 64 KB at once."""
     test_compaction_in_place(dict(batch=34, n_layers=1, gamma=1, n_q_heads=2, n_kv_heads=2, head_dim=40960, max_seqlen=20,
                                   l_obs=2, window=3, top_p=2, budget_frac=0.8, n_planted=0), pattern)
+
+
+@pytest.mark.parametrize("pattern", ["shift", "run", "tail"])
+@pytest.mark.parametrize("case", [
+    dict(batch=1, n_layers=1, gamma=1, window=16, l_obs=32, max_seqlen=20805, budget_frac=0.5),   # clusters of sixteen
+    dict(batch=8, n_layers=4, gamma=4, max_seqlen=6001, budget_frac=0.2),       # two blocks per pair, several free stretches
+    dict(batch=3, ragged=True, max_seqlen=4000, budgets=[3600, 300, 17]),       # a sequence that keeps nine tenths beside others
+    dict(batch=20, head_dim=96, max_seqlen=3001, budget_frac=0.3),              # rows whose vectors do not divide a batch
+    dict(batch=1, n_q_heads=4, n_kv_heads=1, head_dim=64, window=1, l_obs=3, top_p=1, max_seqlen=30000,
+         budgets=[13000]),                                                      # a list longer than shared memory takes
+], ids=["clusters-of-16", "two-blocks", "nine-tenths", "ragged-vectors", "long-list"])
+def test_compaction_in_place_by_free_stretches(case, pattern):
+    """Runs of retained windows with a spread rest behind them: batches that need a barrier, stretches that need none, and
+    every change from one to the other."""
+    test_compaction_in_place(dict(n_q_heads=4, n_kv_heads=2, n_planted=0) | case, pattern)
+
+
+def test_compaction_time_depends_on_the_number_of_rows_only():
+    """8 heads x 65,536 keys, 12 % retained: windows that all move by one place must not take longer than spread ones.
+    What is measured differs by a fifth; the bound of three allows for a disturbed run."""
+    H, n, omega, alpha, d = 8, 65536, 16, 32, 128
+    prob = binding.Problem(dtype="bf16", batch=1, n_q_heads=32, n_kv_heads=H, head_dim=d, l_obs=alpha, window=omega, task=0,
+                           top_p=8, max_seqlen=n, budgets=[n * 12 // 100])
+    kw, k = prob.kw_max, prob.k_max
+    rng = np.random.Generator(np.random.Philox(key=5))
+    lists = {"spread": np.stack([np.sort(rng.permutation(kw)[:k]) for _ in range(H)]),
+             "by one": np.tile(np.arange(1, k + 1), (H, 1)),
+             "run": np.tile(np.concatenate([np.arange(3, 3 + k // 2), kw - np.arange(k - k // 2, 0, -1)]), (H, 1))}
+    t = [torch.zeros((1, H, n, d), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    us = {}
+    for name, rows in lists.items():
+        idx = torch.from_numpy(rows[None].astype(np.int32)).cuda()
+        samples = []
+        for _ in range(9):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(4):
+                binding.wkv_compact_kv_inplace(prob, t[:1], t[1:], idx)
+            b.record()
+            torch.cuda.synchronize()
+            samples.append(a.elapsed_time(b))
+        us[name] = sorted(samples)[len(samples) // 2]
+    assert us["by one"] < 3 * us["spread"] and us["run"] < 3 * us["spread"], us
