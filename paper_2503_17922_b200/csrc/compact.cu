@@ -80,6 +80,7 @@ compact_inplace_kernel(const __grid_constant__ CompactParams prm)
     __syncthreads();
     int review_rows = k * s.omega;
     if (k > 0 && idx[k - 1] == kw - 1) review_rows -= kw * s.omega - n_r;
+    if (review_rows > n_r) review_rows = n_r;      // a list of all windows whose last entry is not the last window
     const int kept = review_rows + (n - n_r);
     if (kept <= 0) return;
 

@@ -80,6 +80,7 @@ gather_kv_kernel(const __grid_constant__ GatherParams prm)
     // and it can only be the last selected one), then the observation rows
     int review_rows = k * s.omega;
     if (k > 0 && (k == s.k_max ? wi_last : idx[k - 1]) == kw - 1) review_rows -= kw * s.omega - n_r;
+    if (review_rows > n_r) review_rows = n_r;      // a list of all windows whose last entry is not the last window
     const int obs_rows = n - n_r;
 
     const int vpr = prm.vec_per_row;

@@ -254,3 +254,22 @@ def test_compaction_time_depends_on_the_number_of_rows_only():
             samples.append(a.elapsed_time(b))
         us[name] = sorted(samples)[len(samples) // 2]
     assert us["by one"] < 3 * us["spread"] and us["run"] < 3 * us["spread"], us
+
+
+def test_a_list_that_misses_the_last_window_stays_inside_the_tensors():
+    """Everything is to be kept, but the list holds no window (nothing has been selected into it yet): the observation rows
+    keep their place, in the packed cache and inside the buffer, and nothing is written behind the sequence."""
+    H, n, alpha, omega, d, guard = 2, 61, 7, 8, 64, 16                     # 54 review rows: seven windows, the last of six
+    prob = binding.Problem(dtype="bf16", batch=1, n_q_heads=4, n_kv_heads=H, head_dim=d, l_obs=alpha, window=omega, task=0,
+                           top_p=4, max_seqlen=n, budgets=[1000], cu_seqlens=[0, n])
+    assert prob.k_max == prob.kw_max == 7
+    idx = torch.full((1, H, 7), -1, dtype=torch.int32, device="cuda")
+    k = torch.randn((n + guard, H, d), device="cuda").to(torch.bfloat16)
+    before = k.clone()
+    out = torch.full((n + guard, H, d), -3.0, dtype=torch.bfloat16, device="cuda")
+    binding.wkv_gather_kv(prob, [k], None, idx, [out], None, cu_seqlens_out=torch.tensor([0, n], dtype=torch.int32, device="cuda"))
+    binding.wkv_compact_kv_inplace(prob, [k], None, idx)
+    torch.cuda.synchronize()
+    assert torch.equal(k, before)
+    assert torch.equal(out[n - alpha:n], before[n - alpha:n])
+    assert bool((out[:n - alpha] == -3.0).all()) and bool((out[n:] == -3.0).all())
