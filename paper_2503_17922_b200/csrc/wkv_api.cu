@@ -842,6 +842,14 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_
             return WKV_ERR_SHAPE;
         }
     }
+    // staging and compact caches as the gather would have them, whether or not a tensor passes through its staging
+    // buffer (misaligned or missing pointers, a cache that is its own staging buffer)
+    {
+        LayerTable tab;
+        int n_tensors = 0;
+        st = fill_table(n_layers, k_layers_dev, v_layers_dev, k_out_layers_dev, v_out_layers_dev, tab, n_tensors);
+        if (st != WKV_OK) return st;
+    }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     // What crosses the bus dominates this call.  Only the leader's keys are needed whole (every key is scored); of
     // every other tensor the retained rows are, so where the GPU can read the caller's host memory the gather takes

@@ -158,6 +158,27 @@ def test_host_entry_refuses_byte_counts_that_disagree_with_the_shape(L):
     assert L.wkv_launch_count() == 0
 
 
+def test_host_entry_refuses_staging_that_the_gather_would_refuse(L):
+    """Missing, misaligned and shared staging buffers are refused whatever way the rows take (no GPU needed)."""
+    s = _shape()
+    cap = L.wkv_keep_max(ctypes.byref(s))
+    need = L.wkv_workspace_bytes(ctypes.byref(s))
+    table = lambda *xs: (ctypes.c_void_p * 2)(*xs)
+    good = dict(k_dev=table(0x1000, 0x2000), v_dev=table(0x3000, 0x4000), k_out=table(0x5000, 0x6000), v_out=table(0x7000, 0x8000))
+    host = table(0x1000, 0x1000)
+
+    def call(**kw):
+        t = good | kw
+        return L.wkv_compress_group_host(ctypes.byref(s), 2, 0x1000, 4 * 8 * 64 * 2, host, host, 2 * 1024 * 64 * 2, host, host,
+                                         2 * cap * 64 * 2, 0x1000, 0x1000, 0x1000, t["k_dev"], t["v_dev"], t["k_out"],
+                                         t["v_out"], 0x1000, 0x1000, cap, 0x1000, need, None)
+    for name in good:
+        assert call(**{name: table(0x9000, None)}) == 1, name                       # WKV_ERR_NULL
+        assert call(**{name: table(0x9000, 0x9008)}) == 6, name                     # WKV_ERR_ALIGN
+    assert call(k_out=table(0x5000, 0x2000)) == 2 and call(v_out=table(0x3000, 0x8000)) == 2     # WKV_ERR_SHAPE
+    assert L.wkv_launch_count() == 0
+
+
 def test_gather_refuses_a_cache_that_is_its_own_input(L):
     s = _shape()
     a = (ctypes.c_void_p * 2)(0x1000, 0x2000)
