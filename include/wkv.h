@@ -17,8 +17,9 @@
  * General conventions
  *   - Every pointer marked DEVICE is device memory owned by the caller; HOST
  *     pointers are ordinary host memory read before the function returns.
- *     The library allocates and frees nothing and keeps no state between
- *     calls other than a launch counter.
+ *     The library allocates and frees no memory and keeps no state between
+ *     calls other than a launch counter and, for the host-buffer entry points, a
+ *     stream and an event per thread and device.
  *   - All device work is enqueued on `cuda_stream` (a cudaStream_t passed as
  *     void*; NULL = the legacy default stream) and the functions return
  *     without synchronising.
@@ -363,16 +364,14 @@ int wkv_group_plan_launch(wkv_group_plan *plan, void *cuda_stream);
 void wkv_group_plan_destroy(wkv_group_plan *plan);
 
 /*
- * The same group with every tensor in HOST memory (pinned memory recommended): the group is
- * compressed on the device and indices, kept lengths and the compact caches are copied back; the
- * function returns after everything it enqueued has completed.  What crosses the bus dominates, so
- * only what is needed crosses: the leader's keys whole (they are copied to their DEVICE staging buffer
- * first and scored as soon as they have landed), and of every other tensor the retained rows, which the
- * gather reads straight from the host memory where that is pinned and mapped.  A tensor in memory that
- * is not, or of which more than half the rows are retained, is copied to its staging buffer whole.  The
- * staging buffers are scratch: what they hold after the call is unspecified.  Each layer's compact cache
- * travels back on a second stream while the next layer is coming in.  (That stream and its event are made
- * at a thread's first call on a device and given back when the thread ends.)
+ * The same group with every tensor in HOST memory (pinned memory recommended): the
+ * inputs are copied to caller-provided DEVICE staging buffers, the group is
+ * compressed there, and indices, kept lengths and the compact caches are copied
+ * back; the function returns after everything it enqueued has completed, and the staging buffers
+ * hold the inputs then.  The copies dominate, so the call runs as a pipeline over the layers: the
+ * leader's keys first (scored and selected as soon as they have landed), then layer by layer copy in,
+ * gather, and copy back on a second stream, so that both copy directions are busy at once.  (That stream
+ * and its event are made at a thread's first call on a device and given back when the thread ends.)
  *   *_host arguments    HOST pointers / HOST arrays of HOST pointers
  *   *_dev arguments     DEVICE staging of the same sizes (HOST arrays of DEVICE pointers)
  *   bytes_per_layer     size of one K (or V) tensor; out_bytes_per_layer of one compact cache
@@ -389,6 +388,24 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers,
                             void *const *k_out_layers_dev, void *const *v_out_layers_dev,
                             int32_t *window_idx_dev, int32_t *kept_len_dev, int32_t keep_capacity,
                             void *workspace, size_t workspace_bytes, void *cuda_stream);
+/*
+ * The same for callers that want the results only: the staging buffers of K and V are scratch, and what
+ * they hold after the call is unspecified.  Then only what is needed has to cross the bus: the leader's keys
+ * whole (they are all scored), and of every other tensor the retained rows, which the gather reads straight
+ * from the host memory where that is pinned and mapped.  A tensor in memory that is not, or of which more than half
+ * the rows are retained, is copied to its staging buffer whole.  Arguments as above.
+ */
+int wkv_compress_group_host_rows(const wkv_shape *s, int32_t n_layers,
+                                 const void *q_obs_host, size_t q_bytes,
+                                 const void *const *k_layers_host, const void *const *v_layers_host,
+                                 size_t bytes_per_layer,
+                                 void *const *k_out_layers_host, void *const *v_out_layers_host,
+                                 size_t out_bytes_per_layer,
+                                 int32_t *window_idx_host, int32_t *kept_len_host,
+                                 void *q_obs_dev, void *const *k_layers_dev, void *const *v_layers_dev,
+                                 void *const *k_out_layers_dev, void *const *v_out_layers_dev,
+                                 int32_t *window_idx_dev, int32_t *kept_len_dev, int32_t keep_capacity,
+                                 void *workspace, size_t workspace_bytes, void *cuda_stream);
 
 /*
  * Measurement aid (no counterpart in the paper): launches a kernel that does nothing but evaluate

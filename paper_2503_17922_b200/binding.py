@@ -25,7 +25,7 @@ WKV_MAX_GROUP_LAYERS = 32
 EXPORTED_SYMBOLS = [
     "wkv_num_windows", "wkv_num_selected", "wkv_keep_len", "wkv_workspace_sync_words", "wkv_kw_max", "wkv_k_max", "wkv_keep_max", "wkv_group_budgets", "wkv_jaccard_windows",
     "wkv_workspace_bytes", "wkv_score_windows", "wkv_score_windows_static", "wkv_select_topk_windows", "wkv_gather_kv", "wkv_gather_kv_paged", "wkv_compact_kv_inplace",
-    "wkv_compress_group", "wkv_compress_group_host", "wkv_score_windows_lse", "wkv_compress_group_lse",
+    "wkv_compress_group", "wkv_compress_group_host", "wkv_compress_group_host_rows", "wkv_score_windows_lse", "wkv_compress_group_lse",
     "wkv_select_leader_windows", "wkv_probe_ex2_rate", "wkv_probe_colsum_rate", "wkv_group_plan_create", "wkv_group_plan_launch", "wkv_group_plan_destroy", "wkv_status_string", "wkv_last_error_detail",
     "wkv_launch_count",
 ]
@@ -126,9 +126,10 @@ def lib() -> ctypes.CDLL:
     L.wkv_group_plan_launch.argtypes = [vp, vp]
     L.wkv_group_plan_destroy.restype = None
     L.wkv_group_plan_destroy.argtypes = [vp]
-    L.wkv_compress_group_host.restype = ctypes.c_int
-    L.wkv_compress_group_host.argtypes = [sp, i32, vp, sz, vp, vp, sz, vp, vp, sz, vp, vp,
-                                          vp, vp, vp, vp, vp, vp, vp, i32, vp, sz, vp]
+    for host_entry in (L.wkv_compress_group_host, L.wkv_compress_group_host_rows):
+        host_entry.restype = ctypes.c_int
+        host_entry.argtypes = [sp, i32, vp, sz, vp, vp, sz, vp, vp, sz, vp, vp,
+                               vp, vp, vp, vp, vp, vp, vp, i32, vp, sz, vp]
     L.wkv_probe_ex2_rate.restype = ctypes.c_int
     L.wkv_probe_ex2_rate.argtypes = [vp, i32, i32, i32, ctypes.POINTER(ctypes.c_int64), vp]
     L.wkv_probe_colsum_rate.restype = ctypes.c_int
@@ -487,10 +488,13 @@ def prepare_gather_kv(prob: Problem, k_layers, v_layers, window_idx, k_out_layer
 def wkv_compress_group_host(prob: Problem, q_obs_host, k_layers_host, v_layers_host, k_out_host, v_out_host,
                             window_idx_host, kept_len_host, q_obs_dev, k_layers_dev, v_layers_dev,
                             k_out_dev, v_out_dev, window_idx_dev, kept_len_dev, keep_capacity, workspace,
-                            stream=None) -> None:
-    """Host-buffer entry: copies in, compresses, copies out, synchronises (host tensors: torch CPU, pinned)."""
+                            stream=None, keep_staged: bool = False) -> None:
+    """Host-buffer entry: copies in, compresses, copies out, synchronises (host tensors: torch CPU, pinned).
+    The staging tensors `k_layers_dev`, `v_layers_dev` are scratch (wkv_compress_group_host_rows); with `keep_staged` they
+    hold the whole inputs afterwards (the C entry of this name), which takes every tensor over the bus whole."""
     nbytes = lambda t: t.numel() * t.element_size()
-    _check(lib().wkv_compress_group_host(
+    call = lib().wkv_compress_group_host if keep_staged else lib().wkv_compress_group_host_rows
+    _check(call(
         ctypes.byref(prob.shape), len(k_layers_host), _ptr(q_obs_host), nbytes(q_obs_host),
         _ptr_array(k_layers_host), _ptr_array(v_layers_host), nbytes(k_layers_host[0]),
         _ptr_array(k_out_host), _ptr_array(v_out_host), nbytes(k_out_host[0]),

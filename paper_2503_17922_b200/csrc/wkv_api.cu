@@ -793,7 +793,8 @@ static bool mapped_host_range(const void *p, size_t bytes)
            get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) == CUDA_SUCCESS && size >= bytes && at - start <= size - bytes;
 }
 
-int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_obs_host, size_t q_bytes,
+// `in_place`: rows may be read where the caller's host memory is, past the staging buffers
+static int compress_group_host_entry(const wkv_shape *s, int32_t n_layers, const void *q_obs_host, size_t q_bytes,
                             const void *const *k_layers_host, const void *const *v_layers_host,
                             size_t bytes_per_layer, void *const *k_out_layers_host,
                             void *const *v_out_layers_host, size_t out_bytes_per_layer,
@@ -801,7 +802,8 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_
                             void *const *k_layers_dev, void *const *v_layers_dev,
                             void *const *k_out_layers_dev, void *const *v_out_layers_dev,
                             int32_t *window_idx_dev, int32_t *kept_len_dev, int32_t keep_capacity,
-                            void *workspace, size_t workspace_bytes, void *cuda_stream)
+                            void *workspace, size_t workspace_bytes, void *cuda_stream,
+                            bool in_place)
 {
     KShape ks;
     int st = resolve(s, ks);
@@ -852,7 +854,8 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     // What crosses the bus dominates this call.  Only the leader's keys are needed whole (every key is scored); of
-    // every other tensor the retained rows are, so where the GPU can read the caller's host memory the gather takes
+    // every other tensor the retained rows are, so where the caller does not ask for the staging buffers to be
+    // filled and the GPU can read the host memory the gather takes
     // them straight from there and the rest never moves.  The crossing of 16 KB of a head's consecutive windows is as
     // fast as a copy (4 layers x 8,192 keys, 12 %: 31 MB instead of 134 MB).  With most rows retained, or memory
     // that is not pinned, a tensor is copied to its staging buffer first.
@@ -865,7 +868,7 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_
         kept_rows += (double)num_selected(n, s->l_obs, s->window, s->budgets_host ? s->budgets_host[b] : s->budget) * s->window +
                      s->l_obs;
     }
-    const bool few_rows = kept_rows <= 0.5 * ks.total_rows;
+    const bool few_rows = in_place && kept_rows <= 0.5 * ks.total_rows;
     CopyBack *cb = copy_back();
     if (!cb) return WKV_ERR_CUDA;
     const cudaStream_t back = cb->stream;
@@ -916,6 +919,40 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_
     if (st != WKV_OK) return st;
     if (e1 != cudaSuccess) return check_cuda(e1, "stream synchronisation");
     return check_cuda(e2, "stream synchronisation (copies back)");
+}
+
+int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers, const void *q_obs_host, size_t q_bytes,
+                            const void *const *k_layers_host, const void *const *v_layers_host,
+                            size_t bytes_per_layer, void *const *k_out_layers_host,
+                            void *const *v_out_layers_host, size_t out_bytes_per_layer,
+                            int32_t *window_idx_host, int32_t *kept_len_host, void *q_obs_dev,
+                            void *const *k_layers_dev, void *const *v_layers_dev,
+                            void *const *k_out_layers_dev, void *const *v_out_layers_dev,
+                            int32_t *window_idx_dev, int32_t *kept_len_dev, int32_t keep_capacity,
+                            void *workspace, size_t workspace_bytes, void *cuda_stream)
+{
+    return compress_group_host_entry(s, n_layers, q_obs_host, q_bytes, k_layers_host, v_layers_host, bytes_per_layer,
+                                     k_out_layers_host, v_out_layers_host, out_bytes_per_layer, window_idx_host,
+                                     kept_len_host, q_obs_dev, k_layers_dev, v_layers_dev, k_out_layers_dev,
+                                     v_out_layers_dev, window_idx_dev, kept_len_dev, keep_capacity, workspace,
+                                     workspace_bytes, cuda_stream, false);
+}
+
+int wkv_compress_group_host_rows(const wkv_shape *s, int32_t n_layers, const void *q_obs_host, size_t q_bytes,
+                                 const void *const *k_layers_host, const void *const *v_layers_host,
+                                 size_t bytes_per_layer, void *const *k_out_layers_host,
+                                 void *const *v_out_layers_host, size_t out_bytes_per_layer,
+                                 int32_t *window_idx_host, int32_t *kept_len_host, void *q_obs_dev,
+                                 void *const *k_layers_dev, void *const *v_layers_dev,
+                                 void *const *k_out_layers_dev, void *const *v_out_layers_dev,
+                                 int32_t *window_idx_dev, int32_t *kept_len_dev, int32_t keep_capacity,
+                                 void *workspace, size_t workspace_bytes, void *cuda_stream)
+{
+    return compress_group_host_entry(s, n_layers, q_obs_host, q_bytes, k_layers_host, v_layers_host, bytes_per_layer,
+                                     k_out_layers_host, v_out_layers_host, out_bytes_per_layer, window_idx_host,
+                                     kept_len_host, q_obs_dev, k_layers_dev, v_layers_dev, k_out_layers_dev,
+                                     v_out_layers_dev, window_idx_dev, kept_len_dev, keep_capacity, workspace,
+                                     workspace_bytes, cuda_stream, true);
 }
 
 const char *wkv_status_string(int status)

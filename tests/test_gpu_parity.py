@@ -510,7 +510,7 @@ def test_ragged_batch_with_a_tiny_sequence():
         np.testing.assert_array_equal(binding.to_host_bits(out["v_out"][layer]), ref["v_out"][layer])
 
 
-def _run_host_entry(w, grp):
+def _run_host_entry(w, grp, **kw):
     """wkv_compress_group_host on pinned host tensors; returns host outputs in the oracle's conventions."""
     prob = binding.Problem.from_workload(w)
     pin = lambda a: binding.to_device(a, "cpu").pin_memory()
@@ -527,13 +527,13 @@ def _run_host_entry(w, grp):
     before = binding.wkv_launch_count()
     binding.wkv_compress_group_host(prob, hq, hk, hv, h_k_out, h_v_out, h_idx, h_kept, stage_q, stage_k, stage_v,
                                     out["k_out"], out["v_out"], out["window_idx"], out["kept_len"],
-                                    out["keep_capacity"], work)
+                                    out["keep_capacity"], work, **kw)
     # the call returns after synchronising its stream: the host buffers are complete here
     assert binding.wkv_launch_count() - before >= 2
     assert binding.device_status(work) == 0
     return {"prob": prob, "window_idx": h_idx.numpy().copy(), "kept_len": h_kept.numpy().copy(),
             "k_out": [binding.to_host_bits(t) for t in h_k_out], "v_out": [binding.to_host_bits(t) for t in h_v_out],
-            "window_scores": None}
+            "window_scores": None, "staged": [binding.to_host_bits(t) for t in stage_k + stage_v]}
 
 
 @pytest.mark.parametrize("which", ["small", "small-f32", "config2"])
@@ -571,6 +571,20 @@ def test_host_buffer_entry_point_reads_only_what_it_needs(monkeypatch, pinned, b
     ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
     got["window_scores"] = ref["window_scores"]
     pu.check_selection(w, grp, got, ref)
+    pu.check_gather(w, grp, got)
+
+
+@pytest.mark.parametrize("budget_frac", [0.05, 0.9])
+def test_host_buffer_entry_point_keeps_the_staged_inputs(budget_frac):
+    """Asked to, the call leaves the whole inputs in the staging buffers, few rows retained or many;
+    the results are the same."""
+    w = small(budget_frac=budget_frac, n_layers=3, gamma=3)
+    grp = wl.make_group(w, 0)
+    got, rows = _run_host_entry(w, grp, keep_staged=True), _run_host_entry(w, grp)
+    for staged, given in zip(got["staged"], grp["k_layers"] + grp["v_layers"]):
+        np.testing.assert_array_equal(staged, given)
+    for name in ("window_idx", "kept_len", "k_out", "v_out"):
+        np.testing.assert_array_equal(np.asarray(got[name]), np.asarray(rows[name]))
     pu.check_gather(w, grp, got)
 
 
