@@ -574,6 +574,18 @@ def test_host_buffer_entry_point_reads_only_what_it_needs(monkeypatch, pinned, b
     pu.check_gather(w, grp, got)
 
 
+@pytest.mark.parametrize("batch,kv_heads", [(1, 8), (9, 1), (3, 4)], ids=["16-pairs", "18-pairs", "24-pairs"])
+def test_host_buffer_entry_point_with_as_many_pairs_as_blocks_and_more(batch, kv_heads):
+    """Rows read in place are moved by sixteen blocks: one for each (unit, tensor) of a layer, or one for several of them."""
+    w = small(batch=batch, n_kv_heads=kv_heads, n_q_heads=2 * kv_heads, budget_frac=0.2, n_layers=2, gamma=2)
+    grp = wl.make_group(w, 0)
+    got = _run_host_entry(w, grp)
+    ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
+    got["window_scores"] = ref["window_scores"]
+    pu.check_selection(w, grp, got, ref)
+    pu.check_gather(w, grp, got)
+
+
 @pytest.mark.parametrize("budget_frac", [0.05, 0.9])
 def test_host_buffer_entry_point_keeps_the_staged_inputs(budget_frac):
     """Asked to, the call leaves the whole inputs in the staging buffers, few rows retained or many;
