@@ -901,17 +901,21 @@ static int compress_group_host_entry(const wkv_shape *s, int32_t n_layers, const
             if (few_rows && aligned16(from[t]) && mapped_host_range(from[t], bytes_per_layer)) src[t] = from[t];
             else h2d(staging[t], from[t], bytes_per_layer, t ? "copy of V" : "copy of K");
         }
-        // The last layer in two steps, so that less is left to travel back when the gather is over
-        const bool last = l == n_layers - 1;
-        for (int t = 0; t < (last ? 2 : 1); ++t) {
+        // The last layer in two steps, so that less is left to travel back when the gather is over.  A launch reads over
+        // the bus when one of its tensors does.  (The leader's keys have landed already; in a launch of their own ahead of
+        // the values' they start to travel back earlier, but beside the values that come in: 4 layers x 8,192 keys 860 us
+        // instead of 853 us.)
+        const bool over_bus[2] = {src[0] != staging[0], src[1] != staging[1]};
+        const bool apart = l == n_layers - 1;
+        for (int t = 0; t < (apart ? 2 : 1); ++t) {
             void *const out[2] = {k_out_layers_dev[l], v_out_layers_dev[l]};
             void *const out_host[2] = {k_out_layers_host[l], v_out_layers_host[l]};
             if (st == WKV_OK)
-                st = gather_kv_entry(s, 1, &src[t], last ? nullptr : &src[1], window_idx_dev, &out[t], last ? nullptr : &out[1],
-                                     nullptr, keep_capacity, cuda_stream, src[t] != staging[t] || src[1] != staging[1]);
+                st = gather_kv_entry(s, 1, &src[t], apart ? nullptr : &src[1], window_idx_dev, &out[t], apart ? nullptr : &out[1],
+                                     nullptr, keep_capacity, cuda_stream, over_bus[t] || (!apart && over_bus[1]));
             hand_over();
             d2h_after(out_host[t], out[t], out_bytes_per_layer, t ? "copy of compact V" : "copy of compact K");
-            if (!last) d2h_after(out_host[1], out[1], out_bytes_per_layer, "copy of compact V");
+            if (!apart) d2h_after(out_host[1], out[1], out_bytes_per_layer, "copy of compact V");
         }
     }
     // both streams are drained before the call returns, whatever happened above
