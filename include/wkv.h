@@ -392,8 +392,8 @@ int wkv_compress_group_host(const wkv_shape *s, int32_t n_layers,
  * The same for callers that want the results only: the staging buffers of K and V are scratch, and what
  * they hold after the call is unspecified.  Then only what is needed has to cross the bus: the leader's keys
  * whole (they are all scored), and of every other tensor the retained rows, which the gather reads straight
- * from the host memory where that is pinned and mapped.  A tensor in memory that is not, or of which more than half
- * the rows are retained, is copied to its staging buffer whole.  Arguments as above.
+ * from the host memory where that is pinned and mapped.  A tensor in memory that is not, or of which more than three
+ * quarters of the rows are retained, is copied to its staging buffer whole.  Arguments as above.
  */
 int wkv_compress_group_host_rows(const wkv_shape *s, int32_t n_layers,
                                  const void *q_obs_host, size_t q_bytes,

@@ -856,9 +856,9 @@ static int compress_group_host_entry(const wkv_shape *s, int32_t n_layers, const
     // What crosses the bus dominates this call.  Only the leader's keys are needed whole (every key is scored); of
     // every other tensor the retained rows are, so where the caller does not ask for the staging buffers to be
     // filled and the GPU can read the host memory the gather takes
-    // them straight from there and the rest never moves.  The crossing of 16 KB of a head's consecutive windows is as
-    // fast as a copy (4 layers x 8,192 keys, 12 %: 31 MB instead of 134 MB).  With most rows retained, or memory
-    // that is not pinned, a tensor is copied to its staging buffer first.
+    // them straight from there and the rest never moves (4 layers x 8,192 keys, 12 %: 31 MB instead of 134 MB; at 48-50
+    // GB/s, where a copy runs at 54).  With more than three quarters of the rows retained, or memory that is not pinned,
+    // a tensor is copied to its staging buffer first.
     // The call is a pipeline over the layers: the leader's keys are scored as soon as they have landed, every layer
     // is gathered in turn, and its compact cache travels back on a second stream while the next layer is coming in
     // (the two directions run at the same time).
@@ -868,7 +868,10 @@ static int compress_group_host_entry(const wkv_shape *s, int32_t n_layers, const
         kept_rows += (double)num_selected(n, s->l_obs, s->window, s->budgets_host ? s->budgets_host[b] : s->budget) * s->window +
                      s->l_obs;
     }
-    const bool few_rows = in_place && kept_rows <= 0.5 * ks.total_rows;
+    // Copying whole tensors runs into the copies back (both directions at once move less than either alone), so rows read
+    // one by one win well beyond their lower rate.  4 layers x 8,192 keys, in place / whole, us: 60 % retained 2,600 /
+    // 3,180, 70 % 2,960 / 3,260, 80 % 3,320 / 3,320, 90 % 3,680 / 3,300; 2 sequences, 3,000 keys and 2 heads alike.
+    const bool few_rows = in_place && kept_rows <= 0.75 * ks.total_rows;
     CopyBack *cb = copy_back();
     if (!cb) return WKV_ERR_CUDA;
     const cudaStream_t back = cb->stream;

@@ -586,6 +586,21 @@ def test_host_buffer_entry_point_with_as_many_pairs_as_blocks_and_more(batch, kv
     pu.check_gather(w, grp, got)
 
 
+@pytest.mark.parametrize("budget_frac", [0.72, 0.78])
+def test_host_buffer_entry_point_on_both_sides_of_three_quarters(budget_frac):
+    """Rows are read in place up to three quarters of a tensor, and tensors copied whole beyond."""
+    w = small(budget_frac=budget_frac, n_layers=2, gamma=2)
+    grp = wl.make_group(w, 0)
+    got = _run_host_entry(w, grp)
+    ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
+    got["window_scores"] = ref["window_scores"]
+    pu.check_selection(w, grp, got, ref)
+    pu.check_gather(w, grp, got)
+    if budget_frac > 0.75:
+        for staged, given in zip(got["staged"], grp["k_layers"] + grp["v_layers"]):
+            np.testing.assert_array_equal(staged, given)
+
+
 @pytest.mark.parametrize("budget_frac", [0.05, 0.9])
 def test_host_buffer_entry_point_keeps_the_staged_inputs(budget_frac):
     """Asked to, the call leaves the whole inputs in the staging buffers, few rows retained or many;
