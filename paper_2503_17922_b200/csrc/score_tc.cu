@@ -857,7 +857,7 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
     a.n_stat_chunks = ws.n_stat_chunks;
     a.r_pad = ws.r_pad;
     const int units = ks.batch * ks.hkv;
-    const TcPlan plan = tc_plan(units, ks.max_seqlen, ks.omega);
+    const TcPlan plan = tc_plan(units, ks.max_seqlen, ks.omega, ks.R);
     a.chunks_per_unit = plan.chunks_per_unit;
     a.units_per_wave = plan.units_per_wave;
     a.kblocks = ks.d / 64;

@@ -36,7 +36,7 @@ Workspace plan_workspace(const KShape &ks)
     const size_t units = (size_t)ks.batch * ks.hkv;
     w.r_pad = (ks.R + 63) / 64 * 64;
     w.n_stat_chunks = (ks.max_seqlen + kStatChunk - 1) / kStatChunk;
-    const int tc_chunks = tc_plan((int)units, ks.max_seqlen, ks.omega).chunks_per_unit;
+    const int tc_chunks = tc_plan((int)units, ks.max_seqlen, ks.omega, ks.R).chunks_per_unit;
     if (tc_chunks > w.n_stat_chunks) w.n_stat_chunks = tc_chunks;
     const int pipe_chunks = pipe_plan((int)units, ks.max_seqlen, ks.d).chunks_per_unit;
     if (pipe_chunks > w.n_stat_chunks) w.n_stat_chunks = pipe_chunks;

@@ -120,16 +120,20 @@ struct TcPlan {
     int chunks_per_unit;  // work items per unit
 };
 // What a wave costs beside its key tiles, in tiles per block: filling the pipeline, the hand-over of the
-// statistics and the pooling take about 8 us, a tile 0.65 us per sweep.
-constexpr int kTcWaveOverhead = 6;
-inline TcPlan tc_plan(int units, int max_seqlen, int omega)
+// statistics and the pooling take about 8 us, a tile 0.65 us per sweep with up to 128 observation rows and, with two
+// accumulators per tile, about twice that with more.  Measured on shapes where the number decides (select call, us):
+//   R = 128   35 units of 54 tiles, 1 wave of 27 tiles / 2 of 11: 62 / 69      40 of 465, 4 of 34 / 5 of 26: 261 / 273
+//   R = 256   128 units of 165 tiles, 5 waves of 33 / 8 of 19: 530 / 509       40 of 465, 4 of 34 / 5 of 26: 429 / 426
+//             32 of 460, 3 of 36 / 4 of 26: 343 / 345                          112 of 39, 2 of 20 / 4 of 8: 147 / 152
+constexpr int tc_wave_overhead(int rows) { return rows <= 128 ? 6 : 4; }
+inline TcPlan tc_plan(int units, int max_seqlen, int omega, int rows)
 {
     // Every number of units per wave whose blocks are resident together is tried, and the one with the least (waves x
-    // (tiles per block + overhead)) taken.  The largest is not the best when it leaves a last wave nearly empty: 16
-    // units of 192 tiles as 12 + 4 made 16 tiles per block and wave, 8 + 8 makes 11.  Whether a wave's keys fit L2
-    // between the two sweeps does not count: a wave costs more than reading keys from HBM again beside the
-    // exponentials (8 sequences of 32-64 K keys, R = 256, one layer: 669 us with waves of at most 104 MB, 599 us with up
-    // to 170 MB).
+    // (tiles per block + overhead)) taken; tiles are those of the longest sequence.  The largest is not the best when
+    // it leaves a last wave nearly empty: 24 units of 256 tiles as 21 + 3 are two waves of 37 tiles per block, as 12 + 12
+    // two of 22.  Whether a wave's keys fit L2 between the two sweeps does not count: a wave costs more than reading
+    // keys from HBM again beside the exponentials (8 sequences of 32-64 K keys, R = 256, one layer: 669 us with waves of at
+    // most 104 MB, 599 us with up to 170 MB).
     TcPlan best;
     best.units_per_wave = 1;
     best.chunks_per_unit = 1;
@@ -146,7 +150,7 @@ inline TcPlan tc_plan(int units, int max_seqlen, int omega)
         if (chunks < min_chunks) chunks = min_chunks;
         if (chunks > max_tiles) chunks = max_tiles;
         const long long waves = (units + upw - 1) / upw, tiles = (max_tiles + chunks - 1) / chunks;
-        const long long cost = waves * (tiles + kTcWaveOverhead);
+        const long long cost = waves * (tiles + tc_wave_overhead(rows));
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best.units_per_wave = upw;

@@ -557,6 +557,14 @@ def test_host_buffer_entry_point(which):
             np.testing.assert_array_equal(got["v_out"][layer], ref["v_out"][layer])
 
 
+@pytest.mark.parametrize("l_obs", [32, 33, 64])
+def test_units_that_share_waves_by_the_number_of_rows(l_obs):
+    """75 units of 15 key tiles: one wave with R = 128 observation rows; with R = 132 and 256, where a tile costs twice as
+    much beside what a wave costs, two waves of more blocks per unit."""
+    w = small(batch=25, n_kv_heads=3, n_q_heads=12, l_obs=l_obs, max_seqlen=1913, n_layers=1, gamma=1, window=16)
+    pu.full_check(w, score_impl=IMPLS["tc"])
+
+
 @pytest.mark.parametrize("pinned", [True, False], ids=["pinned", "pageable"])
 @pytest.mark.parametrize("budget_frac", [0.05, 0.49, 0.9])
 @pytest.mark.parametrize("n_layers", [1, 3])
