@@ -200,7 +200,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     const int Rp = MB == 2 ? 256 : (s.R <= 32 ? 32 : (s.R <= 64 ? 64 : 128));
     int q_unit_loaded = -1;
     uint32_t it = 0;            // key tiles this block has pushed through the pipeline so far
-    uint32_t p_issued = 0;      // producer thread only: tiles whose loads have been issued
+    uint32_t p_issued = 0;      // producer warp: tiles whose loads have been issued (by its leader)
     int s1_unit = -1, s1_chunk = -1, s1_tiles = 0;   // the sweep-1 item whose last tiles the ring holds ...
     uint32_t s1_it = 0;                              // ... as long as `it` still has this value
 
@@ -691,9 +691,10 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
 
     // ------------------------------------------------------------------ teardown
     __syncthreads();
-    if (warp == 0 && lane == 0) {
+    if (warp == 0 && leader) {
         // nothing of this block may be in flight when it ends: the last MMAs must have released
-        // their stages; after a failed wait, the loads already issued must still land
+        // their stages; after a failed wait, the loads already issued must still land.  (The lane that issued
+        // them knows how many: the lanes of the warp may give up at different tiles.)
         for (uint32_t g = p_issued > kStages ? p_issued - kStages : 0; g < p_issued; ++g) {
             const int st = g % kStages;
             if (!mbar_wait(&bar.empty[st], (g / kStages) & 1, &abort_s)) {
