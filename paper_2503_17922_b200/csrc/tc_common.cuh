@@ -268,13 +268,6 @@ __device__ __forceinline__ void mbar_arrive_expect_tx_if(uint32_t leader, uint64
                  "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(smem_u32(bar)), "r"(bytes), "r"(leader)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_if(uint32_t leader, uint64_t *bar)
-{
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-                 "@q mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(smem_u32(bar)), "r"(leader)
-                 : "memory");
-}
-
 __device__ __forceinline__ float fast_exp2(float x)
 {
     float y;
