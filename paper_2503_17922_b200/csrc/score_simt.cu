@@ -427,15 +427,20 @@ static cudaError_t allow_dynamic_smem(const void *fn, int dev, int slot, size_t 
     return err;
 }
 
-// Tiles of 64 keys per block: one while the grid is small (latency), more when it fills the GPU many times over
-// anyway, since every block transposes the whole of Q first.  With up to eight blocks per SM resident, 1,184
-// blocks are one wave.
+// Tiles of 64 keys per block: one while the blocks fit the GPU once or twice (latency), two and four when they fill it
+// more often, since every block transposes the whole of Q first.  A wave is 740 blocks, five per SM (the score kernel's
+// bound; at d = 128 shared memory leaves three).  Select call, fp32, R = 64, d = 64 / 128, us with 1, 2, 4, 8 tiles:
+//     376 tiles   36  42  52  85   /   54  65  73 140       1,504 tiles   97  93 110 167  /  179 151 146 206
+//   4,096 tiles  222 196 181 218   /  450 372 366 458      16,384 tiles  851 732 669 652  /  1709 1416 1269 1300
+// R = 16, 32 and 128 lie alike.
+constexpr int kBlocksPerWave = 740;
+constexpr int kMaxBlockTiles = 4;
 static int simt_tiles_per_block(const KShape &ks)
 {
     const long long tiles = (long long)ks.batch * ks.hkv * ((ks.max_seqlen + kKT - 1) / kKT);
     if (ks.R > 1024) return kChunkTiles;     // the rows of a cluster's blocks would not fit shared memory beside Q
     int t = 1;
-    while (t < kChunkTiles && tiles / (2 * t) >= 1184) t *= 2;
+    while (t < kMaxBlockTiles && tiles / (2 * t) >= kBlocksPerWave) t *= 2;
     return t;
 }
 

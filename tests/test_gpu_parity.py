@@ -557,6 +557,14 @@ def test_host_buffer_entry_point(which):
             np.testing.assert_array_equal(got["v_out"][layer], ref["v_out"][layer])
 
 
+@pytest.mark.parametrize("tiles_per_unit", [46, 47, 92, 93])
+def test_cuda_core_blocks_of_one_two_and_four_tiles(tiles_per_unit):
+    """32 units: 1,472 tiles of 64 keys are blocks of one tile, 1,504 and 2,944 of two, 2,976 of four; a last tile of 29 keys."""
+    w = small(dtype="f32", batch=8, n_kv_heads=4, n_q_heads=8, head_dim=64, l_obs=8, max_seqlen=64 * tiles_per_unit - 35,
+              n_layers=1, gamma=1)
+    pu.full_check(w, score_impl=IMPLS["simt"])
+
+
 @pytest.mark.parametrize("l_obs", [32, 33, 64])
 def test_units_that_share_waves_by_the_number_of_rows(l_obs):
     """75 units of 15 key tiles: one wave with R = 128 observation rows; with R = 132 and 256, where a tile costs twice as
