@@ -201,7 +201,10 @@ constexpr int kStatusWaitExpired = 1;   // a bounded wait inside a kernel ran ou
 // kernel before it in the stream still runs, once every block of that one has called pdl_trigger() or
 // ended.  It must call pdl_wait() before it touches global memory; the wait ends when the kernel before it
 // has completed and its writes are visible.  Because every kernel launched this way waits, "the kernel
-// before it has completed" includes everything earlier in the stream.  Takes about 2 us off the gap
+// before it has completed" includes everything earlier in the stream.  One exception to waiting first: the CUDA-core
+// score kernel reads Q and K (which no kernel of this library writes) ahead of its wait, because the statistics
+// kernel in front of it triggers only after its own wait, behind which everything that wrote them lies; what the
+// statistics kernel writes is read, and anything is written, after the wait.  Takes about 2 us off the gap
 // between two kernels (a chain of short kernels: 4.1 us each without, 2.0 us with).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
