@@ -1090,6 +1090,7 @@ int launch_group_pipeline(const KShape &ks, const void *q, const void *k, float 
         err = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kThreads), params, smem, stream);
     }
     if (err != cudaSuccess) {
+        (void)cudaGetLastError();
         set_error_detail("pipelined group kernel (grid %d x %d threads, %zu bytes of shared memory): %s", grid, kThreads,
                          smem, cudaGetErrorString(err));
         return WKV_ERR_CUDA;

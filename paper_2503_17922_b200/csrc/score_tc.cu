@@ -908,6 +908,7 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
         else err = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), params, smem, stream);
     }
     if (err != cudaSuccess) {
+        (void)cudaGetLastError();
         set_error_detail("tensor-core score kernel (grid %d x %d threads, %zu bytes of shared memory): %s", grid,
                          threads, smem, cudaGetErrorString(err));
         return WKV_ERR_CUDA;

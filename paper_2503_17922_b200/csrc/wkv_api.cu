@@ -179,6 +179,7 @@ int resolve(const wkv_shape *s, KShape &ks)
 int check_cuda(cudaError_t e, const char *what)
 {
     if (e == cudaSuccess) return WKV_OK;
+    (void)cudaGetLastError();      // reported by this call, not by a later one as well
     set_error_detail("%s: %s", what, cudaGetErrorString(e));
     return WKV_ERR_CUDA;
 }

@@ -273,3 +273,16 @@ def test_a_list_that_misses_the_last_window_stays_inside_the_tensors():
     assert torch.equal(k, before)
     assert torch.equal(out[n - alpha:n], before[n - alpha:n])
     assert bool((out[:n - alpha] == -3.0).all()) and bool((out[n:] == -3.0).all())
+
+
+def test_a_refused_launch_is_reported_once():
+    """More (sequence, head) pairs than a grid takes: the gather reports it, and the next call is none the worse."""
+    prob = binding.Problem(dtype="bf16", batch=65536, n_q_heads=1, n_kv_heads=1, head_dim=8, l_obs=1, window=1, task=0, top_p=1,
+                           max_seqlen=2, budgets=[2] * 65536)
+    k = torch.zeros((65536, 1, 2, 8), dtype=torch.bfloat16, device="cuda")
+    idx = torch.zeros((65536, 1, 1), dtype=torch.int32, device="cuda")
+    with pytest.raises(binding.WkvError) as e:
+        binding.wkv_gather_kv(prob, [k], None, idx, [torch.zeros_like(k)], None, keep_capacity=2)
+    assert e.value.status == 8
+    binding.wkv_probe_ex2_rate(torch.zeros(4, dtype=torch.float32, device="cuda"), 1, 32, 1)
+    torch.cuda.synchronize()
