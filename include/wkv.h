@@ -179,7 +179,9 @@ int wkv_workspace_sync_words(const wkv_shape *s, int32_t unit, size_t *ticket_by
  *                  (bit 0: a bounded wait inside a kernel expired, results invalid); the words
  *                  behind it synchronise the blocks of a launch and reset themselves when the
  *                  launch ends normally.  After a non-zero status zero the workspace again.
- *                  One workspace serves one launch at a time.
+ *                  One workspace serves one launch at a time.  It may serve different shapes in turn if it
+ *                  is large enough for each of them and none has more than 2,048 (sequence, KV head) pairs;
+ *                  else, and before a WKV_SCORE_TCGEN05_PIPELINED call that follows another shape's, zero it in between.
  */
 int wkv_score_windows(const wkv_shape *s, const void *q_obs, const void *k_leader,
                       float *window_scores, float *token_scores,

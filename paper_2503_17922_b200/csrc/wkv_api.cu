@@ -30,7 +30,7 @@ size_t score_simt_smem_bytes(const KShape &ks, int r_pad);
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-Workspace plan_workspace(const KShape &ks)
+Workspace plan_workspace(const KShape &ks, int sync_units)
 {
     Workspace w;
     const size_t units = (size_t)ks.batch * ks.hkv;
@@ -44,7 +44,8 @@ Workspace plan_workspace(const KShape &ks)
     w.status_off = off;
     off = 64;
     w.sync_off = off;
-    off = align_up(off + (kSyncTickets + kSyncWordsPerUnit * (size_t)units) * sizeof(int), 256);
+    const size_t sync_room = units > (size_t)sync_units ? units : (size_t)sync_units;
+    off = align_up(off + (kSyncTickets + kSyncWordsPerUnit * sync_room) * sizeof(int), 256);
     w.pstats_off = off;
     off = align_up(off + (ks.R <= 128 ? units * w.n_stat_chunks * 128 * sizeof(unsigned long long) : 0), 256);
     w.stats_off = off;

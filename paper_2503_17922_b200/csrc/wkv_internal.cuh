@@ -94,6 +94,9 @@ struct Workspace {
 // and gather job counter (the last two only in the kernel that also gathers)
 constexpr int kSyncTickets = 16;
 constexpr int kSyncWordsPerUnit = 4;
+// The area has room for at least this many units whatever the shape (32 KB), so that what lies behind it never lands on
+// the words of another shape: one workspace may serve shapes of up to so many units in turn.
+constexpr int kSyncUnits = 2048;
 
 // per-device host state (kernel attributes, device properties) is kept for this many device ordinals
 constexpr int kMaxDevices = 64;
@@ -233,7 +236,7 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, 
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-Workspace plan_workspace(const KShape &ks);
+Workspace plan_workspace(const KShape &ks, int sync_units = kSyncUnits);
 
 // Launchers (each returns a cudaError_t from the launch).
 cudaError_t launch_score_simt(const KShape &ks, int dtype, const void *q, const void *k,

@@ -557,6 +557,26 @@ def test_host_buffer_entry_point(which):
             np.testing.assert_array_equal(got["v_out"][layer], ref["v_out"][layer])
 
 
+@pytest.mark.parametrize("impl", ["simt", "tc"])
+def test_one_workspace_for_different_shapes_in_turn(impl):
+    """An engine's one workspace: few units with many rows leave their statistics where the words of many units would lie if
+    the words took only the room that each shape needs."""
+    cases = [small(l_obs=40, batch=1, n_layers=1, gamma=1), small(batch=33, max_seqlen=300, n_layers=1, gamma=1),
+             small(l_obs=64, batch=3, n_layers=1, gamma=1), small(batch=60, max_seqlen=200, l_obs=40, n_layers=1, gamma=1)]
+    probs = [binding.Problem.from_workload(w, score_impl=IMPLS[impl]) for w in cases]
+    work = torch.zeros(max(p.workspace_bytes for p in probs), dtype=torch.uint8, device="cuda")
+    for w, prob in zip(cases * 2, probs * 2):
+        grp = wl.make_group(w, 0)
+        ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
+        out = prob.alloc_outputs(0)
+        binding.wkv_select_leader_windows(prob, binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0]),
+                                          out["window_scores"], out["window_idx"], out["kept_len"], work)
+        assert binding.device_status(work) == 0
+        pu.check_selection(w, grp, {"prob": prob, "window_scores": out["window_scores"].cpu().numpy(),
+                                    "window_idx": out["window_idx"].cpu().numpy(),
+                                    "kept_len": out["kept_len"].cpu().numpy()}, ref)
+
+
 @pytest.mark.parametrize("tiles_per_unit", [46, 47, 92, 93])
 def test_cuda_core_blocks_of_one_two_and_four_tiles(tiles_per_unit):
     """32 units: 1,472 tiles of 64 keys are blocks of one tile, 1,504 and 2,944 of two, 2,976 of four; a last tile of 29 keys."""
