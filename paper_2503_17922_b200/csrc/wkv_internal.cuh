@@ -103,8 +103,9 @@ constexpr int kMaxDevices = 64;
 
 constexpr int kStatChunk = 512;   // keys per partial-statistics chunk of the CUDA-core kernels
 
-// Tensor-core kernels: key tiles of 128, at most 16 (+1 for window alignment) tiles per block, and a
-// grid aimed at one wave of the 148 SMs of a B200 when the problem is small enough for that.
+// Tensor-core kernels: key tiles of 128 (at most 16, +1 for window alignment, per item of the pipelined kernel;
+// tc_max_chunk_tiles below for the other), and a grid aimed at one wave of the 148 SMs of a B200 when the
+// problem is small enough for that.
 constexpr int kTcTileKeys = 128;
 constexpr int kTcMaxChunkTiles = 16;
 constexpr int kTcTargetBlocks = 148;
