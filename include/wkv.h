@@ -156,8 +156,8 @@ int wkv_jaccard_windows(const int32_t *idx_a, const int32_t *idx_b, int32_t unit
 size_t wkv_workspace_bytes(const wkv_shape *s);
 
 /* Byte offsets, inside the workspace of this shape, of the two words through which the blocks of a
- * launch synchronise on `unit` (a ticket count and a count of arrived statistics chunks; both are
- * zero between launches).  Diagnostic helper (no counterpart in the paper): lets a test or a
+ * launch synchronise on `unit` (a ticket count and, in the pipelined kernel, a count of arrived
+ * statistics chunks; both are zero between launches).  Diagnostic helper (no counterpart in the paper): lets a test or a
  * debugger inspect or disturb the hand-over without knowing the workspace layout.  Either output
  * may be NULL.  The status word is always at byte 0. */
 int wkv_workspace_sync_words(const wkv_shape *s, int32_t unit, size_t *ticket_byte_offset,
@@ -191,7 +191,7 @@ int wkv_score_windows(const wkv_shape *s, const void *q_obs, const void *k_leade
  * The same stage for callers that cannot allocate device memory (no counterpart in the paper: an
  * engineering variant).  A serving engine that gave all of HBM to its own cache pool at start-up,
  * or code running where cudaMalloc is forbidden, has no way to provide the workspace above; here
- * the scratch is a fixed area of WKV_STATIC_SCRATCH_BYTES inside the library image, which every
+ * the scratch is a fixed area of twice WKV_STATIC_SCRATCH_BYTES inside the library image, which every
  * GPU that loads the library holds until the process exits.  The function allocates and frees
  * nothing.
  *   - Shapes whose wkv_workspace_bytes() exceeds WKV_STATIC_SCRATCH_BYTES are refused with
@@ -199,11 +199,10 @@ int wkv_score_windows(const wkv_shape *s, const void *q_obs, const void *k_leade
  *   - The first call on each device looks up the area's device address (with that device current);
  *     make that first call outside any stream capture.
  *   - All calls on a device share the one area: two calls whose kernels may overlap on the GPU
- *     (different streams, no dependency) race on it.  Every call first clears the status and
- *     synchronisation words at the head of the area, so an overlapping call does more than
- *     corrupt scores: it wipes the arrival counts of the kernel already running, whose blocks
- *     then sit in their bounded waits for one to two seconds and end with status bit 0 set (in
- *     either call); the scores of both calls are invalid.  Calls on one stream are safe.
+ *     (different streams, no dependency) race on it and on the words at its head, which every
+ *     call clears first: the scores of both calls are invalid, and blocks may sit in their bounded
+ *     waits for one to two seconds and end with status bit 0 set (in either call).  Calls on one
+ *     stream are safe.
  *   - The looked-up address belongs to the device's primary context; after cudaDeviceReset() in
  *     this process the entry point must not be used again.
  *   - device_status  DEVICE out or NULL: receives 0, or the error bits a kernel set

@@ -41,6 +41,78 @@ __device__ __forceinline__ bool poll_until_at_least(const int *word, int target,
     }
     return true;
 }
+
+// A published word: value and tag travel together in one 16-byte access (a .b128 access is performed as a whole), so a
+// reader that finds the tag has the value, without a fence on either side.
+struct __align__(16) StatEntry {
+    unsigned long long value, tag;
+};
+__device__ __forceinline__ void publish_entry(StatEntry *p, unsigned long long value, unsigned long long tag)
+{
+    asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p), "l"(value), "l"(tag)
+                 : "memory");
+}
+__device__ __forceinline__ StatEntry read_entry(const StatEntry *p)
+{
+    StatEntry e;
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}" : "=l"(e.value), "=l"(e.tag)
+                 : "l"(p)
+                 : "memory");
+    return e;
+}
+// Up to N words that are or will be published: word u is at p + u * step, those in the mask `wanted` count.  All that
+// are still missing are looked at together, so that each look is one trip.  Bounded like every wait.
+template <int N>
+__device__ __forceinline__ void wait_entries(const StatEntry *p, size_t step, unsigned wanted, unsigned long long tag,
+                                             StatEntry (&e)[N], volatile int *abort_flag)
+{
+    unsigned long long t0 = 0;
+    for (uint32_t spin = 1;; ++spin) {
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+            if (wanted >> u & 1u) e[u] = read_entry(p + u * step);
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+            if ((wanted >> u & 1u) && e[u].tag == tag) wanted &= ~(1u << u);
+        if (!wanted || *abort_flag) return;
+        if ((spin & 255u) == 0u) {
+            const unsigned long long now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > 2 * kWaitLimitNs) {
+                *abort_flag = 1;
+                return;
+            }
+        }
+    }
+}
+
+// Launches on a workspace, counted so that each has a tag of its own.  Every block reads the count before it counts
+// itself, and the launch's last block to do so raises it: the blocks of one launch agree on it, the next one's
+// find it changed.
+struct LaunchCount {
+    unsigned blocks, unused[3];
+    unsigned long long launches;
+};
+// The tag's upper bits make its upper word a NaN with a payload that no arithmetic produces, so that neither numbers
+// nor counters that another shape has left at the place of a tag equal one.
+constexpr unsigned long long kTagBits = 0xffb5000000000000ull;
+__device__ __forceinline__ unsigned long long launches_so_far(const LaunchCount *c)
+{
+    unsigned long long n;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(n) : "l"(&c->launches) : "memory");
+    return n;
+}
+__device__ __forceinline__ unsigned long long launch_tag(unsigned long long launches, unsigned salt)
+{
+    return kTagBits | (unsigned long long)(salt & 0xffu) << 40 | ((launches + 1) & 0xffffffffffull);
+}
+__device__ __forceinline__ unsigned long long launch_of(unsigned long long tag) { return tag & 0xffffffffffull; }
+// one thread per block, `launch` being one more than what it has read
+__device__ __forceinline__ void count_launch(LaunchCount *c, unsigned long long launch)
+{
+    if (atomicInc(&c->blocks, gridDim.x - 1) == gridDim.x - 1) c->launches = launch;
+}
+
 __device__ __forceinline__ bool warp_wait_arrivals(const int *word, int target, volatile int *abort_flag, int lane)
 {
     int ok = 1;
@@ -103,12 +175,12 @@ __device__ __forceinline__ void score_accumulate(const float (&v)[N], const floa
 // beyond `size` (ragged last window) hold -inf and sort to the end.  `w` is 16-byte aligned shared memory that holds
 // omega values.
 template <int omega>
-__device__ __forceinline__ float pool_window_sorted(const float *w, int size, int p)
+__device__ __forceinline__ float pool_window_sorted(const float *w, int size, int p, int lane)
 {
     // Neighbouring lanes take neighbouring windows, so a lane starts with another 16-byte piece of its window than the
     // lanes it would share banks with; the network does not care in which register an element starts.
     constexpr int kPieces = omega / 4;
-    const int turn = ((threadIdx.x & 31) * kPieces) >> 3;
+    const int turn = (lane * kPieces) >> 3;
     float v[omega];
 #pragma unroll
     for (int i = 0; i < kPieces; ++i) {

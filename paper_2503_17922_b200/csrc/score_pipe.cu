@@ -643,8 +643,8 @@ group_pipeline_tc(const __grid_constant__ CUtensorMap kmap, const __grid_constan
             if (e.n_tiles == 0) {
                 // a unit without review context still gets its (empty) selection, from its first item
                 if (a.window_idx && e.n_r <= 0 && e.chunk == 0) {
-                    select_topk_block<kComputeThreads, kBarCompute, 64>(
-                        topk_sm, a.window_scores + (size_t)e.unit * s.kw_max, 0, 0, s.k_max,
+                    select_topk_block<kComputeThreads, kBarCompute>(
+                        tl, topk_sm, WrittenScores{a.window_scores + (size_t)e.unit * s.kw_max, -1}, 0, 0, s.k_max,
                         a.window_idx + (size_t)e.unit * s.k_max, a.kept_len + e.unit, e.n, s.alpha, s.omega);
                     compute_sync();
                     if (gathers && tl == 0) {
@@ -776,10 +776,10 @@ group_pipeline_tc(const __grid_constant__ CUtensorMap kmap, const __grid_constan
                     for (int i = tl; i < n_win; i += kComputeThreads) {
                         const int lo = i * s.omega, size = min(s.omega, n_tok - lo);
                         float r;
-                        if (s.omega == 16) r = pool_window_sorted<16>(t_chunk + lo, size, s.p);
-                        else if (s.omega == 8) r = pool_window_sorted<8>(t_chunk + lo, size, s.p);
-                        else if (s.omega == 32) r = pool_window_sorted<32>(t_chunk + lo, size, s.p);
-                        else r = pool_window_sorted<4>(t_chunk + lo, size, s.p);
+                        if (s.omega == 16) r = pool_window_sorted<16>(t_chunk + lo, size, s.p, lane);
+                        else if (s.omega == 8) r = pool_window_sorted<8>(t_chunk + lo, size, s.p, lane);
+                        else if (s.omega == 32) r = pool_window_sorted<32>(t_chunk + lo, size, s.p, lane);
+                        else r = pool_window_sorted<4>(t_chunk + lo, size, s.p, lane);
                         ws_out[i] = r;
                     }
                 } else if (s.omega == 64 || s.omega == 128) {
@@ -828,8 +828,8 @@ group_pipeline_tc(const __grid_constant__ CUtensorMap kmap, const __grid_constan
                     for (int i = tl; i < used1 * 128; i += kComputeThreads) st[i] = 0ull;
                 }
                 if (a.window_idx) {
-                    select_topk_block<kComputeThreads, kBarCompute, 64>(
-                        topk_sm, a.window_scores + (size_t)e.unit * s.kw_max, kw,
+                    select_topk_block<kComputeThreads, kBarCompute>(
+                        tl, topk_sm, WrittenScores{a.window_scores + (size_t)e.unit * s.kw_max, topk_hint(s.R, e.n)}, kw,
                         num_selected_capped(e.n, s.alpha, s.omega, budget, s.k_max), s.k_max,
                         a.window_idx + (size_t)e.unit * s.k_max, a.kept_len + e.unit, e.n, s.alpha, s.omega);
                     if (gathers) {

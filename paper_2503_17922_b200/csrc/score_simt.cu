@@ -271,10 +271,10 @@ struct SimtSelect {
 __device__ inline float pool_window(const float *w, int omega, int size, int p)
 {
     switch (omega) {
-    case 4: return pool_window_sorted<4>(w, size, p);
-    case 8: return pool_window_sorted<8>(w, size, p);
-    case 16: return pool_window_sorted<16>(w, size, p);
-    case 32: return pool_window_sorted<32>(w, size, p);
+    case 4: return pool_window_sorted<4>(w, size, p, threadIdx.x & 31);
+    case 8: return pool_window_sorted<8>(w, size, p, threadIdx.x & 31);
+    case 16: return pool_window_sorted<16>(w, size, p, threadIdx.x & 31);
+    case 32: return pool_window_sorted<32>(w, size, p, threadIdx.x & 31);
     default: return pool_top_p(w, size, p);
     }
 }
@@ -308,7 +308,7 @@ score_pool_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const
         if (!lse_obs) pdl_wait();
         // a unit without review context still gets its (empty) selection
         if (sel.window_idx && n_r <= 0 && blockIdx.x == 0)
-            select_topk_block<kThreads>(topk_sm, window_scores, 0, 0, s.k_max, sel.window_idx + (size_t)unit * s.k_max,
+            select_topk_block<kThreads>((int)threadIdx.x, topk_sm, WrittenScores{window_scores, -1}, 0, 0, s.k_max, sel.window_idx + (size_t)unit * s.k_max,
                                         sel.kept_len + unit, n, s.alpha, s.omega);
         return;
     }
@@ -406,7 +406,7 @@ score_pool_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const
     const bool selects = topk_sm.remaining != 0;
     __syncthreads();                     // the word is the selection's own from here on
     if (selects)
-        select_topk_block<kThreads>(topk_sm, window_scores + (size_t)unit * s.kw_max, num_windows(n, s.alpha, s.omega),
+        select_topk_block<kThreads>((int)threadIdx.x, topk_sm, WrittenScores{window_scores + (size_t)unit * s.kw_max, topk_hint(s.R, n)}, num_windows(n, s.alpha, s.omega),
                                     num_selected_capped(n, s.alpha, s.omega, si.budget, s.k_max), s.k_max,
                                     sel.window_idx + (size_t)unit * s.k_max, sel.kept_len + unit, n, s.alpha, s.omega);
 }

@@ -5,10 +5,11 @@
 // that must not synchronise the device, or under a memory budget audited at load time.  Such a
 // caller cannot size and allocate the workspace wkv_score_windows() asks for.  This entry point
 // needs none: its partial row statistics live in a fixed array that is part of the library image.
-// Every GPU that loads the library therefore holds WKV_STATIC_SCRATCH_BYTES of device memory
+// Every GPU that loads the library therefore holds twice WKV_STATIC_SCRATCH_BYTES of device memory
 // until the process exits, whether or not the entry point is ever called.
 #include "wkv_internal.cuh"
 
+#include <atomic>
 #include <mutex>
 
 namespace wkv {
@@ -16,7 +17,8 @@ namespace {
 
 // The one scratch area, shared by every call on a device.  In host code this name is only a
 // handle for cudaGetSymbolAddress(); the device address is looked up once per device below.
-static __device__ __align__(256) unsigned char g_static_scratch[WKV_STATIC_SCRATCH_BYTES];
+// (Shapes are admitted by what they would need with statistics of eight bytes each; the tensor-core kernel's take sixteen.)
+static __device__ __align__(256) unsigned char g_static_scratch[2 * WKV_STATIC_SCRATCH_BYTES];
 
 std::mutex g_setup_mutex;
 void *g_scratch_addr[kMaxDevices] = {};
@@ -62,23 +64,29 @@ extern "C" int wkv_score_windows_static(const wkv_shape *s, const void *q_obs, c
         set_error_detail("q_obs / k_leader / window_scores is NULL");
         return WKV_ERR_NULL;
     }
-    const Workspace ws = plan_workspace(ks, 0);      // cleared on every call: no room for other shapes' words
+    Workspace ws = plan_workspace(ks, 0);            // cleared on every call: no room for other shapes' words
     // window_scores is the caller's here, so the part of the workspace that would hold them is not needed
-    if (ws.scores_off > (size_t)WKV_STATIC_SCRATCH_BYTES) {
+    if (ws.counted_off > (size_t)WKV_STATIC_SCRATCH_BYTES) {
         set_error_detail("this shape needs %zu bytes of scratch, the built-in area holds %zu: "
                          "use wkv_score_windows with a caller-provided workspace",
-                         ws.scores_off, (size_t)WKV_STATIC_SCRATCH_BYTES);
+                         ws.counted_off, (size_t)WKV_STATIC_SCRATCH_BYTES);
         return WKV_ERR_LIMIT;
     }
     void *scratch = nullptr;
     st = static_scratch(&scratch);
     if (st != WKV_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    // the status word and the grid-synchronisation words behind it are the only part of the area
-    // that must start from zero; the kernels write every statistic they later read
-    st = check_cuda(cudaMemsetAsync(static_cast<char *>(scratch) + ws.status_off, 0, ws.stats_off - ws.status_off,
-                                    stream),
-                    "clearing the status and synchronisation words");
+    // Scoring alone starts from the status word and the count of blocks; the number of the launch behind them goes on
+    // counting, so that nothing an earlier call left behind passes for this one's.  (Two calls that overlap upset the
+    // count of blocks and may leave the number as it was: the salt tells the next calls from them.)
+    static std::atomic<unsigned> calls{0};
+    ws.salt = 1u + calls.fetch_add(1u, std::memory_order_relaxed) % 255u;
+    st = check_cuda(cudaMemsetAsync(static_cast<char *>(scratch) + ws.status_off, 0, ws.count_off + 16 - ws.status_off, stream),
+                    "clearing the status word");
+    // the pipelined kernel's words and statistics must start from zero
+    if (st == WKV_OK && s->score_impl == WKV_SCORE_TCGEN05_PIPELINED)
+        st = check_cuda(cudaMemsetAsync(static_cast<char *>(scratch) + ws.sync_off, 0, ws.stats_off - ws.sync_off, stream),
+                        "clearing the synchronisation words");
     if (st != WKV_OK) return st;
     st = do_score(s, ks, ws, q_obs, k_leader, window_scores, token_scores, nullptr, nullptr, scratch, stream);
     if (st != WKV_OK) return st;

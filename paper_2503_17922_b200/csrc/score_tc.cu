@@ -4,7 +4,7 @@
 // The token score of Eq. 2, t_j = sum_i exp(s_ij) / Z_i, needs every row's softmax normaliser
 // Z_i (a reduction over all keys) before any column sum can be finished, so the keys are swept
 // twice; a block starts normalising a unit's keys once all chunks of that unit have delivered their
-// sweep-1 statistics (a per-unit arrival count, no grid-wide barrier):
+// sweep-1 statistics (published words that say themselves whether they are there, no grid-wide barrier):
 //   sweep 1  D[rows, keys] = Q K^T per 128-key tile with the observation rows on the tensor-memory
 //            lanes: one thread owns one row and keeps its running (max, sum exp2) without any
 //            cross-thread traffic (Eq. 1's normaliser, causal mask on the tiles that touch the
@@ -53,11 +53,13 @@ __host__ __device__ constexpr int groups_for(int) { return 4; }
 __host__ __device__ constexpr int block_threads(int mb) { return 64 + groups_for(mb) * 128; }
 constexpr int kTile = kTcTileKeys;                       // keys per tile
 constexpr int kRegion = kTile * 128;                     // bytes of one 64-column block of a key tile
+constexpr uint32_t kTmemCols = 512;                      // all of tensor memory: four accumulator buffers
 constexpr int kChunkCap = kTcChunkCap;                   // token scores a block may hold
 
 struct TcArgs {
     KShape s;
-    float2 *stats;          // [units][n_stat_chunks][r_pad]
+    StatEntry *stats;       // [units][n_stat_chunks][r_pad]: published statistics of sweep 1
+    StatEntry *scores;      // [units][kw_max]: published window scores, for the block that selects
     float *window_scores;
     float *token_scores;
     const float *lse_obs;   // [B, H_q, alpha] natural log of Eq. 1's normalisers from the caller, or null
@@ -65,10 +67,13 @@ struct TcArgs {
     int *kept_len;
     int *status;
     int *sync;
+    LaunchCount *count;
+    unsigned salt;          // part of the launch's tag
     int n_stat_chunks, r_pad;
     int chunks_per_unit, units_per_wave;
     int kblocks;            // head_dim / 64
     int slot_tok, slot_h, slot_b;   // which tensor-map coordinate (1..3) carries token / head / batch
+    unsigned alpha_inverse; // ceil(2^16 / alpha): r * alpha_inverse >> 16 is r / alpha for r, alpha <= 256
     int r16;                // observation rows rounded up to a multiple of 16
 };
 
@@ -113,14 +118,55 @@ __device__ __forceinline__ void warp_release(uint64_t *bar, int lane)
     if (lane == 0) mbar_arrive(bar);
 }
 
-// Hand-over between the sweeps, per unit (all blocks are resident: cooperative launch).  A block that
-// has written the sweep-1 statistics of one chunk adds one to the unit's arrival word; a block about
-// to normalise keys of the unit waits until all of the unit's chunks have arrived.  No block waits
-// before it has finished all its sweep-1 work, so every wait ends.  In sweep 2 every block counts
-// itself on the unit's ticket word when it is done; the block of the unit's last chunk waits for
-// that count (every waiter of the unit is past its wait by then), clears both words for the next
-// launch and selects.  Bounded: a warp that waits longer than two seconds gives up and sets the
-// block's abort flag.
+// Hand-over between blocks (all are resident: cooperative launch): every partial statistic and, where the launch
+// selects, every window score is published as one 16-byte word of value and tag, written and read as a whole, so that
+// it says itself whether it is there: no fence, no counter, and the data arrives with the answer.  The tag holds the
+// number of this launch on the workspace (LaunchCount), which what an earlier launch has left behind, of whatever
+// shape, cannot equal.  8 heads x 4,096 keys: 2.3 us from the end of sweep 1 to the normalisers and 3.3 us from the pooled
+// windows to the selection; with counters raised by a release and polled it was 3.7 and 4.6 us.
+// No block waits before it has finished all its sweep-1 work, so every wait ends.  Bounded: a thread that
+// looks for longer than two seconds gives up and sets the block's abort flag.
+
+// The selection reads the published window scores, waiting for those that are still to come: LOOK words at a time.
+template <int LOOK>
+struct PublishedScores {
+    const StatEntry *entries;
+    unsigned long long tag;
+    volatile int *abort_flag;
+    int hint;
+    template <int N>
+    __device__ __forceinline__ void keys(unsigned (&key)[N], int lo, int hi) const
+    {
+        constexpr int kLook = N < LOOK ? N : LOOK;
+#pragma unroll
+        for (int e0 = 0; e0 < N; e0 += kLook) {
+            StatEntry v[kLook];
+            const int left = hi - lo - e0;
+            wait_entries<kLook>(entries + lo + e0, 1, left >= kLook ? (1u << kLook) - 1u : left > 0 ? (1u << left) - 1u : 0u, tag, v,
+                                abort_flag);
+#pragma unroll
+            for (int e = 0; e < kLook; ++e) key[e0 + e] = e < left ? topk_order_key(__uint_as_float((unsigned)v[e].value)) : 0u;
+        }
+    }
+    __device__ __forceinline__ void wait(int lo, int hi) const
+    {
+        unsigned unused[LOOK];
+        for (int w = lo; w < hi; w += LOOK) keys(unused, w, min(hi, w + LOOK));
+    }
+    __device__ __forceinline__ unsigned key(int w) const
+    {
+        return topk_order_key(__ldcg(reinterpret_cast<const float *>(&entries[w].value)));
+    }
+};
+
+// The value, but nothing that is computed from it before this point: what only the ends of an item need would otherwise
+// be computed ahead of the tile loops and take their registers.
+__device__ __forceinline__ int late(int x)
+{
+    asm volatile("" : "+r"(x));
+    return x;
+}
+
 // geometry of one work item
 struct Item {
     int unit, chunk, b, h;
@@ -134,20 +180,182 @@ struct Item {
 // that item's last STAGES tiles in the ring, in ring order: it scores those first, without
 // loading them again, and then walks down through the rest.
 template <int STAGES>
-__device__ __forceinline__ int tile_at(const Item &im, int u)
+__device__ __forceinline__ int tile_at(bool reuse, int n_tiles, int u)
 {
-    if (!im.reuse) return u;
-    return u < STAGES ? im.n_tiles - STAGES + u : im.n_tiles - 1 - u;
+    if (!reuse) return u;
+    return u < STAGES ? n_tiles - STAGES + u : n_tiles - 1 - u;
+}
+
+// The compute groups' part of the two sweeps.  Accumulators are numbered v = tile * MB + row half across the block's tile
+// stream, `it` tiles lie before the item's, and group `grp` of NG takes those with v mod NG = grp.  Shared memory is passed
+// by its 32-bit addresses, so that it is known as such in the calls below too.
+struct GroupBarriers {
+    uint32_t tfull, tempty, abort_flag;
+};
+template <typename T>
+__device__ __forceinline__ T *shared_at(uint32_t addr)
+{
+    return static_cast<T *>(__cvta_shared_to_generic(addr));
+}
+struct StatsSweep {
+    int nslot, col0;        // 32-column slots of an accumulator this thread reduces, and the first one's column
+    int limit;              // last key the thread's row may attend to
+    int j_begin, j_plain;   // first key of the item; tiles that end before j_plain need no masking
+};
+template <int MB>
+__device__ __forceinline__ float2 stats_sweep(GroupBarriers gb, StatsSweep w, uint32_t taddr, uint32_t it, int n_tiles, int grp, float c)
+{
+    constexpr int NG = groups_for(MB);
+    uint64_t *const tfull = shared_at<uint64_t>(gb.tfull), *const tempty = shared_at<uint64_t>(gb.tempty);
+    volatile int *const abort_flag = shared_at<volatile int>(gb.abort_flag);
+    const int lane = threadIdx.x & 31;
+    float m = -INFINITY, l = 0.f;
+    for (uint32_t v = it * MB; v < (it + n_tiles) * MB; ++v) {
+        if ((int)(v % NG) != grp) continue;
+        const int tile0 = w.j_begin + (int)(v / MB - it) * kTile;
+        if (!warp_wait(tfull, (v / NG) & 1, abort_flag, lane)) break;
+        tc_fence_after_sync();
+        const bool fast = tile0 + kTile - 1 < w.j_plain;     // no masking
+        for (int sl = 0; sl < w.nslot; ++sl) {
+            float x[32];
+            tmem_ld32(taddr + sl * 32, x);
+            if (sl + 1 == w.nslot) warp_release(tempty, lane);   // the buffer may be overwritten now
+            stats_update(x, fast, tile0 + w.col0 + sl * 32, w.limit, c, m, l);
+        }
+    }
+    return make_float2(m, l);
+}
+struct ScoreSweep {
+    int rows;               // of the group's half: 32-row slices; a 16-row tail follows if their number has bit 4 set
+    uint32_t neg_lse2, t_out;
+    int n_keys;
+    bool reuse;
+    float *token_out;       // or null
+};
+template <int MB>
+__device__ __forceinline__ void score_sweep(GroupBarriers gb, ScoreSweep w, uint32_t taddr, uint32_t it, int n_tiles, int grp, int L, float c)
+{
+    constexpr int NG = groups_for(MB);
+    uint64_t *const tfull = shared_at<uint64_t>(gb.tfull), *const tempty = shared_at<uint64_t>(gb.tempty);
+    volatile int *const abort_flag = shared_at<volatile int>(gb.abort_flag);
+    const float *const neg_lse2 = shared_at<const float>(w.neg_lse2);
+    float *const t_out = shared_at<float>(w.t_out);
+    const int lane = threadIdx.x & 31;
+    const int n32 = w.rows >> 5;
+    const bool tail = (w.rows & 16) != 0;
+    for (uint32_t v = it * MB; v < (it + n_tiles) * MB; ++v) {
+        if ((int)(v % NG) != grp) continue;
+        if (!warp_wait(tfull, (v / NG) & 1, abort_flag, lane)) break;
+        tc_fence_after_sync();
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+        for (int sl = 0; sl < n32; ++sl) {
+            float x[32];
+            tmem_ld32(taddr + sl * 32, x);
+            if (sl + 1 == n32 && !tail) warp_release(tempty, lane);   // the buffer may be overwritten now
+            score_accumulate<32>(x, neg_lse2 + sl * 32, c, a0, a1, a2, a3);
+        }
+        if (tail) {
+            float x[16];
+            tmem_ld16(taddr + n32 * 32, x);
+            warp_release(tempty, lane);
+            score_accumulate<16>(x, neg_lse2 + n32 * 32, c, a0, a1, a2, a3);
+        }
+        const float tj = (a0 + a1) + (a2 + a3);
+        const int j = tile_at<stages_for(MB)>(w.reuse, n_tiles, (int)(v / MB - it)) * kTile + L;
+        if (j < w.n_keys) {
+            t_out[j] = tj;
+            if (w.token_out) w.token_out[j] = tj;
+        }
+    }
+}
+// Eq. 1's normaliser of every row from the published statistics of a unit's `used` chunks (row r's of chunk c at
+// st[c * r_pad + r]) -> -log2 of it in neg_lse2.  `tl`: number of the compute thread; MERGERS neighbouring ones share a row.
+// LOOK of a thread's words are looked at together.
+template <int MERGERS, int LOOK>
+__device__ __forceinline__ void merge_stats(const StatEntry *st, int used, int rows, int r_pad, unsigned long long tag, int tl,
+                                            float *neg_lse2, volatile int *abort_flag)
+{
+    const int r = tl / MERGERS, mp = tl % MERGERS;
+    float M = -INFINITY, sum = 0.f;
+    if (r < rows) {
+        for (int c0 = mp; c0 < used; c0 += LOOK * MERGERS) {
+            unsigned wanted = 0u;
+#pragma unroll
+            for (int u = 0; u < LOOK; ++u) wanted |= (c0 + u * MERGERS < used ? 1u : 0u) << u;
+            StatEntry e[LOOK];
+            wait_entries<LOOK>(st + r + (size_t)c0 * r_pad, (size_t)MERGERS * r_pad, wanted, tag, e, abort_flag);
+            float2 p[LOOK];
+            float Mn = M;
+#pragma unroll
+            for (int u = 0; u < LOOK; ++u) {
+                p[u] = make_float2(wanted >> u & 1u ? __uint_as_float((unsigned)e[u].value) : -INFINITY,
+                                   wanted >> u & 1u ? __uint_as_float((unsigned)(e[u].value >> 32)) : 0.f);
+                Mn = fmaxf(Mn, p[u].x);
+            }
+            if (Mn > -INFINITY) {
+                sum *= fast_exp2(M - Mn);
+#pragma unroll
+                for (int u = 0; u < LOOK; ++u)
+                    if (p[u].y > 0.f) sum += p[u].y * fast_exp2(p[u].x - Mn);
+                M = Mn;
+            }
+        }
+    }
+    __syncwarp();
+    float Ma = M;
+#pragma unroll
+    for (int o = 1; o < MERGERS; o <<= 1) Ma = fmaxf(Ma, __shfl_xor_sync(0xffffffffu, Ma, o));
+    sum = sum > 0.f ? sum * fast_exp2(M - Ma) : 0.f;
+#pragma unroll
+    for (int o = 1; o < MERGERS; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (mp == 0) neg_lse2[r] = sum > 0.f ? -(Ma + log2f(sum)) : -INFINITY;
 }
 
 // ---------------------------------------------------------------------------------------------
 // the kernel
 // ---------------------------------------------------------------------------------------------
-template <int MB>   // 128-row blocks of observation rows: 1 (R <= 128) or 2 (R <= 256)
-// 18 warps put five on one SM sub-partition (16K registers): 96 registers per thread at most
-__global__ void __launch_bounds__(block_threads(MB), 1)
-score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ TcArgs a,
-                 const __nv_bfloat16 *__restrict__ q)
+// A block's state in shared memory, beside the images of Q and of the key tiles
+// what a block takes from wave to wave
+struct Carry {
+    uint32_t it;          // key tiles it has pushed through the pipeline so far
+    uint32_t issued;      // tiles whose loads have been issued
+    int q_unit_loaded;    // unit whose Q image is in shared memory, -1: none
+};
+template <int MB>
+struct Shared {
+    int counted;                               // the block is among the launch's counted blocks
+    __align__(8) Barriers bar;
+    uint32_t tmem_base;
+    int abort;
+    unsigned long long tag;                    // what this launch marks its published words with
+    float2 part[groups_for(MB)][128 + 8];      // sweep 1: a group's (max, sum) of the rows on its lanes
+    __align__(16) float neg_lse2[256];         // -log2 of the row normaliser; -inf for padding rows
+    __align__(16) float t_chunk[MB][kChunkCap];   // sweep 2: per half, the key's sum over that half's rows
+    TopkSmem topk;
+};
+template <int MB>
+__device__ __forceinline__ Shared<MB> &shared_state()
+{
+    __shared__ Shared<MB> state;
+    return state;
+}
+extern __shared__ uint8_t smem_raw[];
+
+// The selection as a call, where a block goes through several waves: its registers would otherwise be laid over what
+// lives from wave to wave.
+template <int MB>
+__device__ __noinline__ void select_call(PublishedScores<1> src, int kw, int k, int k_max, int *out, int *kept_len, int n, int alpha, int omega)
+{
+    select_topk_block<block_threads(MB)>((int)threadIdx.x, shared_state<MB>().topk, src, kw, k, k_max, out, kept_len, n, alpha, omega);
+}
+
+// One wave of a block.  The sweeps have no registers to spare, and inside a loop over waves or items everything that
+// lives on counts: 8 heads x 65,536 keys, 128 rows, one wave, take 58.1 us as ONE and 61.0 us as the form with a
+// loop (65.2 us where that looks at five published words at a time and has the selection inlined, as ONE does).  MB: 128-row blocks of observation rows, 1 (R <= 128) or 2 (R <= 256).  SINGLE: no block has more
+// than one item of a wave.  ONE: and there is one wave, so that nothing is kept from item to item.
+template <int MB, bool ONE, bool SINGLE>
+__device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs &a, const __nv_bfloat16 *__restrict__ q, int u0,
+                                          Carry &carry)
 {
     constexpr int NG = groups_for(MB), kStages = stages_for(MB);
     constexpr int kThreads = block_threads(MB);
@@ -157,22 +365,17 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     // two row blocks); accumulators are numbered v = tile * MB + rh across the block's whole tile
     // stream, and buffers and compute groups take them round-robin (v mod NG).  With two row blocks a
     // group therefore always works on the same half (NG is even).
-    constexpr uint32_t buf_cols = 128;                    // accumulator buffer stride in tensor memory
-    constexpr uint32_t tmem_cols = 512;
-    static_assert(NG * buf_cols <= tmem_cols, "accumulator buffers exceed tensor memory");
+    constexpr uint32_t buf_cols = kTmemCols / NG;         // accumulator buffer stride in tensor memory
+    static_assert(buf_cols >= kTile, "accumulator buffers exceed tensor memory");
 
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) Barriers bar;
-    __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s;
-    __shared__ float2 part[NG][1][128];                    // sweep 1: a group's (max, sum) of the rows on its lanes
-    __shared__ __align__(16) float neg_lse2_all[256];    // -log2 of the row normaliser; -inf for padding rows
-    __shared__ __align__(16) float t_chunk[MB][kChunkCap];              // sweep 2: per half, the key's sum over that half's rows
-    __shared__ TopkSmem topk_sm;
-
+    Shared<MB> &sh = shared_state<MB>();
+    Barriers &bar = sh.bar;
     const KShape &s = a.s;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int units = s.batch * s.hkv;
+    // (Computed anew in every wave where there are several: kept across the steps at the end of an item it would cost the
+    // sweeps their registers.)
+    const int tid = ONE ? (int)threadIdx.x : late((int)threadIdx.x);
+    const int warp = tid >> 5, lane = tid & 31;
+    const int units = ONE ? a.units_per_wave : s.batch * s.hkv;
     const int cpu = a.chunks_per_unit;
     const float c = s.scale_log2;
 
@@ -182,33 +385,22 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     const int ksteps = s.d / 16;
     const uint32_t leader = elect_one();     // lane that acts for its warp where a whole warp issues
 
-    if (threadIdx.x == 0) {
-        init_barriers(bar);
-        abort_s = 0;
-    }
-    if (warp == 1) tmem_alloc(&tmem_base_s, tmem_cols);
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    const uint32_t tmem_base = tmem_base_s;
-    pdl_wait();                 // nothing above touches memory of anybody else
-    if (warp == 0 && lane == 0) tma_prefetch_desc(&tmap);
+    const uint32_t tmem_base = sh.tmem_base;
+    uint32_t &it = carry.it, &p_issued = carry.issued;
+    int &q_unit_loaded = carry.q_unit_loaded;
 
     // Row layout of the Q image: image row r holds observation row (r mod Rp); with Rp < 128 the rows
     // repeat so that all 128 lanes work in sweep 1, each copy taking its own slice of a tile's columns.
     // Rows [0, r16) of the image are the B operand of sweep 2.
     const int Rp = MB == 2 ? 256 : (s.R <= 32 ? 32 : (s.R <= 64 ? 64 : 128));
-    int q_unit_loaded = -1;
-    uint32_t it = 0;            // key tiles this block has pushed through the pipeline so far
-    uint32_t p_issued = 0;      // producer warp: tiles whose loads have been issued (by its leader)
-    int s1_unit = -1, s1_chunk = -1, s1_tiles = 0;   // the sweep-1 item whose last tiles the ring holds ...
-    uint32_t s1_it = 0;                              // ... as long as `it` still has this value
 
+    // the query head, within the unit's G, that observation row r < 256 belongs to: r / alpha
+    auto head_of = [&](int r) { return (int)((unsigned)r * a.alpha_inverse >> 16); };
     auto make_item = [&](int unit, int chunk, int review_only, Item &im) {
         im.unit = unit;
         im.chunk = chunk;
         im.b = unit / s.hkv;
-        im.h = unit % s.hkv;
+        im.h = unit - im.b * s.hkv;
         if (s.cu) {
             const int lo = min(max(s.cu[im.b], 0), s.total_rows);
             im.n = min(min(max(s.cu[im.b + 1] - s.cu[im.b], 0), s.n_cap), s.total_rows - lo);
@@ -233,25 +425,29 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     constexpr int kLoaders = kThreads - 32;
     auto go_producer = [&]() { asm volatile("bar.arrive 2, %0;" ::"n"(kThreads) : "memory"); };
     auto load_q_image = [&](const Item &im, bool signal) {
-        if (q_unit_loaded != im.unit) {
+        if (ONE ? q_unit_loaded < 0 : q_unit_loaded != im.unit) {
+            unsigned long long launches = 0;
+            const bool first = q_unit_loaded < 0;      // the number is raised while the launch runs: it is read once
+            if (first && threadIdx.x == 32) launches = launches_so_far(a.count);
             const __nv_bfloat16 *q_unit = q + im.b * s.qsb + (long long)im.h * s.G * s.qsh;
+            const int loader = late((int)threadIdx.x) - 32;
             const int vshift = s.d == 128 ? 4 : 3;            // log2(16-byte vectors per row)
             const int total = q_rows << vshift;
-            for (int base = threadIdx.x - 32; base < total; base += kLoaders * 4) {
+            for (int base = loader; base < total; base += kLoaders * 4) {
                 int4 v[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int idx = base + u * kLoaders;
                     v[u] = make_int4(0, 0, 0, 0);
                     if (idx < total) {
-                        const int rq = (idx >> vshift) % Rp, cc = idx & ((1 << vshift) - 1);
+                        const int rq = (idx >> vshift) & (Rp - 1), cc = idx & ((1 << vshift) - 1);
                         if (rq < s.R) {
-                            const int g = rq / s.alpha, i = rq - g * s.alpha;
+                            const int g = head_of(rq), i = rq - g * s.alpha;
                             v[u] = __ldg(reinterpret_cast<const int4 *>(q_unit + g * s.qsh + i * s.qst + cc * 8));
                         }
                     }
                 }
-                if (signal && base == (int)threadIdx.x - 32) go_producer();
+                if (signal && base == loader) go_producer();
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int idx = base + u * kLoaders;
@@ -261,12 +457,13 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                     }
                 }
             }
-            if (signal && (int)threadIdx.x - 32 >= total) go_producer();   // a thread without a share of the image
+            if (signal && loader >= total) go_producer();   // a thread without a share of the image
             fence_proxy_async_smem();
+            if (first && threadIdx.x == 32) sh.tag = launch_tag(launches, a.salt);
+            asm volatile("bar.sync 1, %0;" ::"n"(kLoaders) : "memory");
         } else if (signal) {
             go_producer();
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(kLoaders) : "memory");
     };
 
     // producer: the item's key tiles into the stage ring (the block-wide tile counter `it` keeps the phases)
@@ -276,20 +473,20 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
         for (int t = t_begin; t < t_end; ++t) {
             const uint32_t g = it + t;
             const int st = g % kStages;
+            if (g >= kStages && !mbar_wait(&bar.empty[st], ((g / kStages) - 1) & 1, &sh.abort)) return;
             if (im.reuse && t < kStages) {
                 // the stage holds this tile already: complete the phase without a load
                 if (leader) mbar_arrive(&bar.full[st]);
                 ++p_issued;
                 continue;
             }
-            if (g >= kStages && !mbar_wait(&bar.empty[st], ((g / kStages) - 1) & 1, &abort_s)) return;
             mbar_arrive_expect_tx_if(leader, &bar.full[st], (uint32_t)stage_bytes);
-            const int tok = tok0 + tile_at<kStages>(im, t) * kTile;
+            const int tok = tok0 + tile_at<kStages>(im.reuse, im.n_tiles, t) * kTile;
             const int c1 = a.slot_tok == 1 ? tok : (a.slot_h == 1 ? im.h : bcoord);
             const int c2 = a.slot_tok == 2 ? tok : (a.slot_h == 2 ? im.h : bcoord);
             const int c3 = a.slot_tok == 3 ? tok : (a.slot_h == 3 ? im.h : bcoord);
             for (int kb = 0; kb < a.kblocks; ++kb)
-                tma_load_4d_if(leader, k_stage0 + st * stage_bytes + kb * kRegion, &tmap, &bar.full[st], kb * 64, c1, c2, c3);
+                tma_load_4d_if(leader, k_stage0 + st * stage_bytes + kb * kRegion, tmap, &bar.full[st], kb * 64, c1, c2, c3);
             ++p_issued;
         }
     };
@@ -318,13 +515,13 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
         for (int t = 0; t < im.n_tiles; ++t) {
             const uint32_t g = it + t;
             const int st = g % kStages;
-            if (!mbar_wait(&bar.full[st], (g / kStages) & 1, &abort_s)) return;
+            if (!mbar_wait(&bar.full[st], (g / kStages) & 1, &sh.abort)) return;
             const uint64_t k_desc = k_desc0 + (uint64_t)(st * stage_step);
 #pragma unroll
             for (int rh = 0; rh < MB; ++rh) {
                 const uint32_t v = g * MB + rh;
                 const int buf = v % NG;
-                if (v >= NG && !mbar_wait(&bar.tempty[buf], ((v / NG) - 1) & 1, &abort_s)) return;
+                if (v >= NG && !mbar_wait(&bar.tempty[buf], ((v / NG) - 1) & 1, &sh.abort)) return;
                 tc_fence_after_sync();
                 // sweep 2: the rows of this half are the N dimension (a multiple of 16)
                 const int n_rows = rh == 0 ? min(a.r16, 128) : a.r16 - 128;
@@ -343,371 +540,308 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     const int L = quarter * 32 + lane;
     const uint32_t taddr_grp = tmem_base + ((uint32_t)(quarter * 32) << 16) + grp * buf_cols;
 
-    // sweep-1 compute: the row's partial (max, sum exp2) over the item's keys -> part[grp][.][L]
+    const GroupBarriers gb = {smem_u32(&bar.tfull[grp]), smem_u32(&bar.tempty[grp]), smem_u32(&sh.abort)};
+    // sweep-1 compute: the row's partial (max, sum exp2) over the item's keys -> part[grp][L]
     auto compute_stats = [&](const Item &im) {
-        const int ncols = MB == 2 ? kTile : Rp;             // columns of a tile this thread reduces
-        const int col0 = MB == 2 ? 0 : (L / Rp) * Rp;       // warp-uniform: Rp is a multiple of 32
-        const int nslot = ncols >> 5;                       // 32-column slots of an accumulator this thread reduces
-        float m0 = -INFINITY, l0 = 0.f;
-        int limit0;                                         // last key the thread's row may attend to
-        {
-            const int row = MB == 2 ? (grp & 1) * 128 + L : L % Rp;
-            limit0 = row < s.R ? min(im.n_r + row % s.alpha, im.j_end - 1) : -1;
-        }
-        const uint32_t taddr = taddr_grp + col0;
-        for (uint32_t v = it * MB; v < (it + im.n_tiles) * MB; ++v) {
-            if ((int)(v % NG) != grp) continue;
-            const int t = (int)(v / MB - it);
-            if (!warp_wait(&bar.tfull[grp], (v / NG) & 1, &abort_s, lane)) break;
-            tc_fence_after_sync();
-            const int tile0 = im.j_begin + t * kTile;
-            const int j0 = tile0 + col0;
-            const bool fast = (tile0 + kTile - 1 <= im.n_r) && (tile0 + kTile - 1 < im.j_end);   // no masking
-            for (int sl = 0; sl < nslot; ++sl) {
-                float x[32];
-                tmem_ld32(taddr + sl * 32, x);
-                if (sl + 1 == nslot) warp_release(&bar.tempty[grp], lane);   // the buffer may be overwritten now
-                stats_update(x, fast, j0 + sl * 32, limit0, c, m0, l0);
-            }
-        }
-        part[grp][0][L] = make_float2(m0, l0);
+        StatsSweep w;
+        w.nslot = MB == 2 ? kTile / 32 : Rp >> 5;
+        w.col0 = MB == 2 ? 0 : L & ~(Rp - 1);               // warp-uniform: Rp is a multiple of 32
+        const int row = MB == 2 ? (grp & 1) * 128 + L : L & (Rp - 1);
+        w.limit = row < s.R ? min(im.n_r + row - head_of(row) * s.alpha, im.j_end - 1) : -1;
+        w.j_begin = im.j_begin;
+        w.j_plain = min(im.n_r + 1, im.j_end);
+        const uint32_t taddr = taddr_grp + w.col0;
+        sh.part[grp][L] = stats_sweep<MB>(gb, w, taddr, it, im.n_tiles, grp, c);
+    };
+
+    // kMergers neighbouring threads share an observation row when partial statistics are merged, within the block and
+    // between the chunks; both in a fixed order
+    constexpr int kComputeThreads = kThreads - 64;
+    constexpr int kMergers = kComputeThreads / q_rows;
+    auto compute_barrier = [&]() { asm volatile("bar.sync 3, %0;" ::"n"(kComputeThreads) : "memory"); };
+
+    // combines the compute groups and the column slices of each row and publishes the item's statistics
+    auto publish_stats = [&](const Item &im) {
+        const int tl = late((int)threadIdx.x) - 64, r = tl / kMergers, mp = tl % kMergers;
+        // with two row blocks a row lives in the groups of its half (group index odd or even)
+        const float2 *mine = MB == 2 ? &sh.part[(r >> 7) + 2 * mp][r & 127] : &sh.part[mp][r];
+        float2 p[4];
+#pragma unroll
+        for (int cp = 0; cp < 4; ++cp) p[cp] = (MB == 2 ? cp == 0 : (r < Rp && cp * Rp < 128)) ? mine[cp * Rp] : make_float2(-INFINITY, 0.f);
+        float M = fmaxf(fmaxf(p[0].x, p[1].x), fmaxf(p[2].x, p[3].x));
+#pragma unroll
+        for (int o = 1; o < kMergers; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+        float sum = 0.f;
+#pragma unroll
+        for (int cp = 0; cp < 4; ++cp)
+            if (p[cp].y > 0.f) sum += p[cp].y * fast_exp2((p[cp].x - M) * c);
+#pragma unroll
+        for (int o = 1; o < kMergers; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (mp == 0 && r < s.R && !*static_cast<volatile int *>(&sh.abort))
+            publish_entry(a.stats + ((size_t)im.unit * a.n_stat_chunks + im.chunk) * a.r_pad + r,
+                          (unsigned long long)__float_as_uint(M * c) | (unsigned long long)__float_as_uint(sum) << 32, sh.tag);
     };
 
     // sweep-2 compute: token score of key L of every tile of the item -> t_chunk (and token_scores)
     auto compute_scores = [&](const Item &im) {
-        // rows of the group's half: 32-row slices; a 16-row tail follows if their number has bit 4 set
         const int rh = MB == 2 ? (grp & 1) : 0;
-        const int rows_h = rh == 0 ? min(a.r16, 128) : a.r16 - 128;
-        const int n32 = rows_h >> 5;
-        const bool tail = (rows_h & 16) != 0;
-        const float *neg_lse2 = neg_lse2_all + rh * 128;
-        for (uint32_t av = it * MB; av < (it + im.n_tiles) * MB; ++av) {
-            if ((int)(av % NG) != grp) continue;
-            const int t = (int)(av / MB - it);
-            if (!warp_wait(&bar.tfull[grp], (av / NG) & 1, &abort_s, lane)) break;
-            tc_fence_after_sync();
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-            for (int sl = 0; sl < n32; ++sl) {
-                float v[32];
-                tmem_ld32(taddr_grp + sl * 32, v);
-                if (sl + 1 == n32 && !tail) warp_release(&bar.tempty[grp], lane);   // the buffer may be overwritten now
-                score_accumulate<32>(v, neg_lse2 + sl * 32, c, a0, a1, a2, a3);
-            }
-            if (tail) {
-                float vt[16];
-                tmem_ld16(taddr_grp + n32 * 32, vt);
-                warp_release(&bar.tempty[grp], lane);
-                score_accumulate<16>(vt, neg_lse2 + n32 * 32, c, a0, a1, a2, a3);
-            }
-            const float tj = (a0 + a1) + (a2 + a3);
-            const int j = im.j_begin + tile_at<kStages>(im, t) * kTile + L;
-            if (j < im.j_end) {
-                t_chunk[rh][j - im.j_begin] = tj;
-                if (MB == 1 && a.token_scores) a.token_scores[(size_t)im.unit * s.nr_max + j] = tj;
-            }
-        }
+        ScoreSweep w;
+        w.rows = rh == 0 ? min(a.r16, 128) : a.r16 - 128;
+        w.neg_lse2 = smem_u32(sh.neg_lse2 + rh * 128);
+        w.t_out = smem_u32(sh.t_chunk[rh]);
+        w.n_keys = im.j_end - im.j_begin;
+        w.reuse = im.reuse;
+        w.token_out = MB == 1 && a.token_scores ? a.token_scores + (size_t)im.unit * s.nr_max + im.j_begin : nullptr;
+        score_sweep<MB>(gb, w, taddr_grp, it, im.n_tiles, grp, L, c);
     };
 
-    const int n_waves = (units + a.units_per_wave - 1) / a.units_per_wave;
-    for (int wave = 0; wave < n_waves && !abort_s; ++wave) {
-        const int u0 = wave * a.units_per_wave;
-        const int nu = min(a.units_per_wave, units - u0);
-        const int n_items = nu * cpu;
+    auto block_barrier = [&]() {
+        tc_fence_before_sync();
+        __syncthreads();
+        tc_fence_after_sync();
+    };
+    const int n_items = ONE ? (int)gridDim.x : min(a.units_per_wave, units - u0) * cpu;
+    int item;
 
-        // ------------------------------------------------------------------ sweep 1
-        // (not needed when the caller supplies the normalisers: sweep 2 then reads the keys from HBM)
-        for (int item = blockIdx.x; item < n_items && !a.lse_obs; item += gridDim.x) {
-            Item im;
-            make_item(u0 + item / cpu, item % cpu, 0, im);
-            float2 *out = a.stats + ((size_t)im.unit * a.n_stat_chunks + im.chunk) * a.r_pad;
-            if (im.n_r <= 0 || im.n_tiles == 0) {
-                for (int r = threadIdx.x; r < a.r_pad; r += kThreads) out[r] = make_float2(-INFINITY, 0.f);
-                continue;
-            }
-            if (warp == 0) {
-                // the first tiles leave before the loads of the Q image (they land while those are
-                // being issued); the rest of the ring's burst follows once the Q loads are on their way
-                const int early = min(kEarlyTiles, im.n_tiles);
-                produce(im, 0, early);
-                asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
-                produce(im, early, im.n_tiles);
+    // ------------------------------------------------------------------ sweep 1
+    // (not needed when the caller supplies the normalisers: sweep 2 then reads the keys from HBM)
+    item = blockIdx.x;
+    if (!a.lse_obs && (ONE || item < n_items)) do {
+        Item im;
+        const int nth = item / cpu;
+        make_item(u0 + nth, item - nth * cpu, 0, im);
+        if (im.n_r <= 0 || im.n_tiles == 0) continue;
+        if (!ONE && q_unit_loaded != im.unit && q_unit_loaded >= 0) block_barrier();   // the image is still being read
+        if (warp == 0) {
+            // the first tiles leave before the loads of the Q image (they land while those are
+            // being issued); the rest of the ring's burst follows once the Q loads are on their way
+            const int early = min(kEarlyTiles, im.n_tiles);
+            produce(im, 0, early);
+            asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+            produce(im, early, im.n_tiles);
+        } else {
+            load_q_image(im, true);
+            if (warp == 1) {
+                issue_mma(im, std::false_type{});
             } else {
-                load_q_image(im, true);
-                if (warp == 1) {
-                    issue_mma(im, std::false_type{});
-                } else {
-                    compute_stats(im);
-                }
+                compute_stats(im);
+                compute_barrier();
+                publish_stats(im);
             }
-            q_unit_loaded = im.unit;
-            it += im.n_tiles;
-            s1_unit = im.unit;
-            s1_chunk = im.chunk;
-            s1_tiles = im.n_tiles;
-            s1_it = it;
-            tc_fence_before_sync();
-            __syncthreads();
-            tc_fence_after_sync();
-            if (abort_s) break;
-            // combine the compute groups and the column slices of each row, in a fixed order
-            const int copies = MB == 2 ? 1 : 128 / Rp;
-            for (int r = threadIdx.x; r < a.r_pad; r += kThreads) {
-                float2 res = make_float2(-INFINITY, 0.f);
-                if (r < s.R) {
-                    const int mb = MB == 2 ? r >> 7 : 0, base = MB == 2 ? (r & 127) : r;
-                    // with two row blocks a row lives in the groups of its half (group index odd or even)
-                    float M = -INFINITY;
-                    for (int g = 0; g < NG; ++g)
-                        for (int cp = 0; cp < copies; ++cp)
-                            if (MB == 1 || (g & 1) == mb) M = fmaxf(M, part[g][0][base + cp * Rp].x);
-                    float sum = 0.f;
-                    for (int g = 0; g < NG; ++g)
-                        for (int cp = 0; cp < copies; ++cp) {
-                            const float2 p = part[g][0][base + cp * Rp];
-                            if ((MB == 1 || (g & 1) == mb) && p.y > 0.f) sum += p.y * fast_exp2((p.x - M) * c);
-                        }
-                    res = make_float2(M * c, sum);
-                }
-                out[r] = res;
-            }
-            __syncthreads();   // `part` is rewritten by the next item
-            // release: cumulative over what the block wrote before the barrier above
-            if (threadIdx.x == 0) red_release_gpu_add(a.sync + kSyncTickets + kSyncWordsPerUnit * im.unit + 1, 1);
         }
-        if (abort_s) break;
+        // No barrier of the whole block here: the TMA and MMA warps run on into the second sweep, whose first
+        // accumulators fill as the last ones of this one are read.
+        q_unit_loaded = im.unit;
+        it += im.n_tiles;
+        if (!SINGLE && item + (int)gridDim.x < n_items) block_barrier();   // `part` is rewritten by the next item
+    } while (!SINGLE && (item += gridDim.x) < n_items);
 
-        // ------------------------------------------------------------------ sweep 2 (+ selection)
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-            Item im;
-            make_item(u0 + item / cpu, item % cpu, 1, im);
-            const int kw = num_windows(im.n, s.alpha, s.omega);
-            // read now, needed only by the block that selects: the load is long done by then
-            const int budget = a.window_idx ? (s.budgets ? __ldg(s.budgets + im.b) : s.budget) : 0;
-            if (im.n_r <= 0 || im.n_tiles == 0) {
-                // a unit without review context still gets its (empty) selection, from its first item
-                if (a.window_idx && im.n_r <= 0 && im.chunk == 0) {
-                    select_topk_block<kThreads>(topk_sm, a.window_scores + (size_t)im.unit * s.kw_max, 0, 0, s.k_max,
-                                                a.window_idx + (size_t)im.unit * s.k_max, a.kept_len + im.unit,
-                                                im.n, s.alpha, s.omega);
-                    __syncthreads();
-                }
-                continue;
+    // ------------------------------------------------------------------ sweep 2 (+ selection)
+    item = blockIdx.x;
+    if (ONE || item < n_items) do {
+        Item im;
+        const int nth = item / cpu;
+        make_item(u0 + nth, item - nth * cpu, 1, im);
+        // read now, needed only by the block that selects: the load is long done by then
+        const int budget = a.window_idx ? (s.budgets ? __ldg(s.budgets + im.b) : s.budget) : 0;
+        if (im.n_r <= 0 || im.n_tiles == 0) {
+            // a unit without review context still gets its (empty) selection, from its first item
+            if (a.window_idx && im.n_r <= 0 && im.chunk == 0) {
+                for (int x = threadIdx.x; x < s.k_max; x += kThreads) a.window_idx[(size_t)im.unit * s.k_max + x] = -1;
+                if (threadIdx.x == 0) a.kept_len[im.unit] = min(im.n, s.alpha);
             }
-            const int len1 = tc_chunk_len(im.n, cpu, 1);
-            im.reuse = im.unit == s1_unit && im.chunk == s1_chunk && it == s1_it && im.n_tiles == s1_tiles &&
-                       im.n_tiles >= kStages && im.chunk * len1 == im.j_begin;
-            if (warp == 0) {
-                // ahead of the small loads of this item: the tiles the ring still holds (no traffic), or,
-                // when this is the only sweep, the first tiles from HBM as in sweep 1
-                const int ahead = im.reuse ? kStages : (a.lse_obs ? min(kEarlyTiles, im.n_tiles) : 0);
-                produce(im, 0, ahead);
-                asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
-                produce(im, ahead, im.n_tiles);
-            } else {
-                load_q_image(im, false);
-                if (warp == 1) {
-                    // the MMAs do not need the normalisers: the first accumulators fill while the
-                    // compute warps merge the statistics
-                    go_producer();
-                    issue_mma(im, std::true_type{});
-                } else {
-                // Eq. 1's normaliser of every row: merge the partial statistics of the unit's chunks.
-                // kMergers threads share a row (each takes every kMergers-th chunk), then one of them
-                // merges their results; both steps in a fixed order.
-                constexpr int kComputeThreads = kThreads - 64;
-                constexpr int kMergers = kComputeThreads / q_rows;
-                float2 *merged = &part[0][0][0];
-                const int tl = threadIdx.x - 64;
-                if (a.lse_obs) {
-                    // the caller's normalisers, to base 2; row r = (query head g of the group, position i)
-                    if (tl < 256) {
-                        float v = -INFINITY;
-                        if (tl < s.R) {
-                            const int g = tl / s.alpha, i = tl - g * s.alpha;
-                            v = -1.4426950408889634f *
-                                __ldg(a.lse_obs + ((size_t)im.b * s.hq + (size_t)im.h * s.G + g) * s.alpha + i);
-                        }
-                        neg_lse2_all[tl] = v;
-                    }
-                    go_producer();
-                    asm volatile("bar.sync 3, %0;" ::"n"(kComputeThreads) : "memory");
-                    compute_scores(im);
-                } else {
-                const int used1 = (im.n + len1 - 1) / len1;   // chunks of the unit that hold keys in sweep 1
-                const bool arrived =
-                    warp_wait_arrivals(a.sync + kSyncTickets + kSyncWordsPerUnit * im.unit + 1, used1, &abort_s, lane);
-                if (tl < kMergers * q_rows && arrived) {
-                    const int r = tl % q_rows, mp = tl / q_rows;
-                    float M = -INFINITY, sum = 0.f;
-                    const int used = r < s.R ? used1 : 0;
-                    const float2 *st = a.stats + (size_t)im.unit * a.n_stat_chunks * a.r_pad + r;
-                    for (int c0 = mp; c0 < used || c0 == mp; c0 += 8 * kMergers) {
-                        float2 p[8];
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const int cidx = c0 + u * kMergers;
-                            p[u] = cidx < used ? __ldcg(st + (size_t)cidx * a.r_pad) : make_float2(-INFINITY, 0.f);
-                        }
-                        if (c0 == mp) go_producer();   // this thread's first loads are on their way
-                        float Mn = M;
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) Mn = fmaxf(Mn, p[u].x);
-                        if (Mn > -INFINITY) {
-                            sum *= fast_exp2(M - Mn);
-#pragma unroll
-                            for (int u = 0; u < 8; ++u)
-                                if (p[u].y > 0.f) sum += p[u].y * fast_exp2(p[u].x - Mn);
-                            M = Mn;
-                        }
-                    }
-                    merged[mp * q_rows + r] = make_float2(M, sum);
-                } else {
-                    go_producer();
+            __syncthreads();   // as at the end of every item: what made the block give up has been seen by all
+            continue;
+        }
+        if (!SINGLE && q_unit_loaded != im.unit && q_unit_loaded >= 0) block_barrier();   // the image is still being read
+        const int len1 = tc_chunk_len(im.n, cpu, 1);
+        // the ring holds the last tiles of the block's one item of the wave, if they are this sweep's tiles too
+        const int keys1 = min(im.n - im.chunk * len1, len1);
+        im.reuse = !a.lse_obs && (SINGLE || (item == (int)blockIdx.x && item + (int)gridDim.x >= n_items)) &&
+                   im.n_tiles >= kStages && im.chunk * len1 == im.j_begin && (keys1 + kTile - 1) / kTile == im.n_tiles;
+        if (warp == 0) {
+            // ahead of the small loads of this item: the tiles the ring still holds (no traffic), or
+            // the first tiles as in sweep 1
+            const int ahead = im.reuse ? kStages : min(kEarlyTiles, im.n_tiles);
+            produce(im, 0, ahead);
+            asm volatile("bar.sync 2, %0;" ::"n"(kThreads) : "memory");
+            produce(im, ahead, im.n_tiles);
+        } else {
+            load_q_image(im, false);
+            if (warp == 1) {
+                // the MMAs do not need the normalisers: the first accumulators fill while the
+                // compute warps merge the statistics
+                go_producer();
+                issue_mma(im, std::true_type{});
+                // the block counts itself, once, now that it has read the number of launches
+                if (lane == 0 && (ONE || !sh.counted)) {
+                    count_launch(a.count, launch_of(sh.tag));
+                    sh.counted = 1;
                 }
-                asm volatile("bar.sync 3, %0;" ::"n"(kComputeThreads) : "memory");
+            } else {
+            const int tl = late((int)threadIdx.x) - 64;
+            if (a.lse_obs) {
+                // the caller's normalisers, to base 2; row r = (query head g of the group, position i)
                 if (tl < 256) {
                     float v = -INFINITY;
                     if (tl < s.R) {
-                        float M = -INFINITY, sum = 0.f;
-#pragma unroll
-                        for (int mp = 0; mp < kMergers; ++mp) {
-                            const float2 p = merged[mp * q_rows + tl];
-                            if (p.y > 0.f) {
-                                const float Mn = fmaxf(M, p.x);
-                                sum = sum * fast_exp2(M - Mn) + p.y * fast_exp2(p.x - Mn);
-                                M = Mn;
-                            }
-                        }
-                        if (sum > 0.f) v = -(M + log2f(sum));
+                        const int g = head_of(tl), i = tl - g * s.alpha;
+                        v = -1.4426950408889634f *
+                            __ldg(a.lse_obs + ((size_t)im.b * s.hq + (size_t)im.h * s.G + g) * s.alpha + i);
                     }
-                    neg_lse2_all[tl] = v;
+                    sh.neg_lse2[tl] = v;
                 }
-                asm volatile("bar.sync 3, %0;" ::"n"(kComputeThreads) : "memory");
-                compute_scores(im);
-                }
-                }
-            }
-            q_unit_loaded = im.unit;
-            it += im.n_tiles;
-            tc_fence_before_sync();
-            __syncthreads();
-            tc_fence_after_sync();
-            if (abort_s) break;
-            float *t_item = &t_chunk[0][0];
-            if (MB == 2) {
-                // Eq. 2 sums over all rows: add the two halves' sums of every key
-                for (int x = threadIdx.x; x < im.j_end - im.j_begin; x += kThreads) {
-                    const float tj = t_chunk[0][x] + t_chunk[MB - 1][x];
-                    t_item[x] = tj;
-                    if (a.token_scores) a.token_scores[(size_t)im.unit * s.nr_max + im.j_begin + x] = tj;
-                }
-                __syncthreads();
-            }
-            // Eq. 3-4: the item's windows (its first key is a multiple of omega)
-            {
-                const int n_tok = im.j_end - im.j_begin;
-                float *ws_out = a.window_scores + (size_t)im.unit * s.kw_max + im.j_begin / s.omega;
-                const int n_win = (n_tok + s.omega - 1) / s.omega;
-                if (s.omega == 16 || s.omega == 8 || s.omega == 32 || s.omega == 4) {
-                    // consecutive windows go to different warps so that all four schedulers take part
-                    for (int i = threadIdx.x; i < n_win; i += kThreads) {
-                        const int lw = i;
-                        const int lo = lw * s.omega, size = min(s.omega, n_tok - lo);
-                        float r;
-                        if (s.omega == 16) r = pool_window_sorted<16>(t_item + lo, size, s.p);
-                        else if (s.omega == 8) r = pool_window_sorted<8>(t_item + lo, size, s.p);
-                        else if (s.omega == 32) r = pool_window_sorted<32>(t_item + lo, size, s.p);
-                        else r = pool_window_sorted<4>(t_item + lo, size, s.p);
-                        ws_out[lw] = r;
-                    }
-                }
-                else if (s.omega == 64 || s.omega == 128) {
-                    // one warp per window
-                    for (int lw = warp; lw < n_win; lw += kThreads / 32) {
-                        const int lo = lw * s.omega, size = min(s.omega, n_tok - lo);
-                        const float r = s.omega == 64 ? pool_window_warp<64>(t_item + lo, size, s.p, lane)
-                                                      : pool_window_warp<128>(t_item + lo, size, s.p, lane);
-                        if (lane == 0) ws_out[lw] = r;
-                    }
-                }
-                else {
-                    for (int lw = threadIdx.x; lw < n_win; lw += kThreads) {
-                        const int lo = lw * s.omega;
-                        ws_out[lw] = pool_top_p(t_item + lo, min(s.omega, n_tok - lo), s.p);
-                    }
-                }
-            }
-            const int len2 = tc_chunk_len(im.n_r, cpu, s.omega);
-            const int used2 = (im.n_r + len2 - 1) / len2;   // chunks of the unit that hold keys in sweep 2
-            // The block of the unit's last chunk selects for the unit (and clears the unit's words): that
-            // chunk is usually a short one, so its block is done early and the selection does not sit
-            // on the path of a block that the next wave is waiting for.  The other blocks only count
-            // themselves, without waiting for an answer.
-            // With given normalisers nothing else makes a block wait for another, and the selection does not
-            // either: the block that counts itself last selects, so the launch need not be cooperative.
-            int *ticket = a.sync + kSyncTickets + kSyncWordsPerUnit * im.unit;
-            bool selects = im.chunk == used2 - 1;
-            if (a.lse_obs) {
-                selects = false;
-                if (a.window_idx) {
-                    __syncthreads();
-                    if (threadIdx.x == 0) {
-                        __threadfence();             // publishes the window scores the whole block wrote
-                        const int before = atomicAdd(ticket, 1);
-                        if (before == used2 - 1) atomicExch(ticket, 0);
-                        if (before < 0 || before >= used2) atomicOr(a.status, kStatusWaitExpired);   // workspace not cleared
-                        __threadfence();
-                        topk_sm.remaining = before;
-                    }
-                    __syncthreads();
-                    selects = topk_sm.remaining == used2 - 1;
-                    __syncthreads();                 // the word is the selection's own from here on
-                }
-            } else if (!selects) {
-                if (a.window_idx) {
-                    __syncthreads();
-                    // release, cumulative: publishes the window scores the whole block wrote
-                    if (threadIdx.x == 0) red_release_gpu_add(ticket, 1);
-                } else if (threadIdx.x == 0) {
-                    atomicAdd(ticket, 1);
-                }
+                go_producer();
             } else {
-                __syncthreads();
-                if (threadIdx.x == 0 && poll_until_at_least(ticket, used2 - 1, &abort_s)) {
-                    atomicExch(ticket, 0);       // every other block of the unit is past its waits
-                    atomicExch(ticket + 1, 0);
-                }
-                __syncthreads();
+                go_producer();
+                const StatEntry *st = a.stats + (size_t)im.unit * a.n_stat_chunks * a.r_pad;
+                const int used1 = (im.n + len1 - 1) / len1;    // chunks of the unit that hold keys in sweep 1
+                merge_stats<kMergers, ONE ? 5 : 2>(st, used1, s.R, a.r_pad, sh.tag, tl, sh.neg_lse2, &sh.abort);
             }
-            if (selects && a.window_idx && !abort_s) {
-                select_topk_block<kThreads>(topk_sm, a.window_scores + (size_t)im.unit * s.kw_max, kw,
-                                            num_selected_capped(im.n, s.alpha, s.omega, budget, s.k_max), s.k_max,
-                                            a.window_idx + (size_t)im.unit * s.k_max, a.kept_len + im.unit,
-                                            im.n, s.alpha, s.omega);
+            compute_barrier();
+            compute_scores(im);
             }
-            __syncthreads();   // t_chunk, neg_lse2 and the selection scratch are reused by the next item
         }
+        q_unit_loaded = im.unit;
+        it += im.n_tiles;
+        block_barrier();
+        if (sh.abort) break;
+        float *t_item = &sh.t_chunk[0][0];
+        if (MB == 2) {
+            // Eq. 2 sums over all rows: add the two halves' sums of every key
+            for (int x = threadIdx.x; x < im.j_end - im.j_begin; x += kThreads) {
+                const float tj = sh.t_chunk[0][x] + sh.t_chunk[MB - 1][x];
+                t_item[x] = tj;
+                if (a.token_scores) a.token_scores[(size_t)im.unit * s.nr_max + im.j_begin + x] = tj;
+            }
+            __syncthreads();
+        }
+        const int tid = late((int)threadIdx.x);
+        // the unit's ticket counts the blocks that are past all waiting for one another
+        int *ticket = a.sync + kSyncTickets + kSyncWordsPerUnit * im.unit;
+        const bool last_chunk = im.j_end == im.n_r;     // of those that hold keys in sweep 2
+        if (a.window_idx && !a.lse_obs && !last_chunk && threadIdx.x == 0) atomicAdd(ticket, 1);
+        // Eq. 3-4: the item's windows (its first key is a multiple of omega)
+        {
+            const int n_tok = im.j_end - im.j_begin;
+            const int omega = late(s.omega);
+            const size_t w0 = (size_t)im.unit * s.kw_max + im.j_begin / omega;
+            float *ws_out = a.window_scores + w0;
+            auto put = [&](int lw, float r) {
+                ws_out[lw] = r;
+                if (a.window_idx) publish_entry(a.scores + w0 + lw, __float_as_uint(r), sh.tag);
+            };
+            const int n_win = (n_tok + omega - 1) / omega;
+            if (s.omega == 16 || s.omega == 8 || s.omega == 32 || s.omega == 4) {
+                // consecutive windows go to different warps so that all four schedulers take part
+                for (int lw = tid; lw < n_win; lw += kThreads) {
+                    const int lo = lw * s.omega, size = min(s.omega, n_tok - lo);
+                    float r;
+                    if (s.omega == 16) r = pool_window_sorted<16>(t_item + lo, size, s.p, tid & 31);
+                    else if (s.omega == 8) r = pool_window_sorted<8>(t_item + lo, size, s.p, tid & 31);
+                    else if (s.omega == 32) r = pool_window_sorted<32>(t_item + lo, size, s.p, tid & 31);
+                    else r = pool_window_sorted<4>(t_item + lo, size, s.p, tid & 31);
+                    put(lw, r);
+                }
+            }
+            else if (s.omega == 64 || s.omega == 128) {
+                // one warp per window
+                for (int lw = tid >> 5; lw < n_win; lw += kThreads / 32) {
+                    const int lo = lw * s.omega, size = min(s.omega, n_tok - lo);
+                    const float r = s.omega == 64 ? pool_window_warp<64>(t_item + lo, size, s.p, tid & 31)
+                                                  : pool_window_warp<128>(t_item + lo, size, s.p, tid & 31);
+                    if ((tid & 31) == 0) put(lw, r);
+                }
+            }
+            else {
+                for (int lw = tid; lw < n_win; lw += kThreads) {
+                    const int lo = lw * s.omega;
+                    put(lw, pool_top_p(t_item + lo, min(s.omega, n_tok - lo), s.p));
+                }
+            }
+        }
+        // The block of the unit's last chunk selects for the unit, from the published scores: that
+        // chunk is usually a short one, so its block is done early and the selection does not sit
+        // on the path of a block that the next wave is waiting for.
+        // With given normalisers nothing else makes a block wait for another, and the selection does not
+        // either: the block that counts itself last selects, so the launch need not be cooperative.
+        bool selects = last_chunk;
+        if (a.lse_obs && a.window_idx) {
+            if (threadIdx.x == 0) {
+                const int before = atomicAdd(ticket, 1);
+                const int len2 = tc_chunk_len(im.n_r, cpu, late(s.omega)), used2 = (im.n_r + len2 - 1) / len2;
+                if (before == used2 - 1) atomicExch(ticket, 0);
+                if (before < 0 || before >= used2) atomicOr(a.status, kStatusWaitExpired);   // workspace not cleared
+                sh.topk.remaining = before == used2 - 1;
+            }
+            __syncthreads();
+            selects = sh.topk.remaining != 0;
+        }
+        if (a.window_idx && selects) {
+            __syncthreads();                 // a wait that expires from here on is seen by all at the same place
+            const PublishedScores<ONE ? 4 : 1> src = {a.scores + (size_t)im.unit * s.kw_max, sh.tag, &sh.abort, topk_hint(s.R, im.n)};
+            const int kw = num_windows(im.n, s.alpha, late(s.omega));
+            const int k = num_selected_capped(im.n, s.alpha, late(s.omega), budget, s.k_max);
+            int *const out = a.window_idx + (size_t)im.unit * s.k_max;
+            if constexpr (ONE) select_topk_block<kThreads>((int)threadIdx.x, sh.topk, src, kw, k, s.k_max, out, a.kept_len + im.unit, im.n, s.alpha, s.omega);
+            else select_call<MB>(src, kw, k, s.k_max, out, a.kept_len + im.unit, im.n, s.alpha, s.omega);
+            // the others counted themselves before they published what has just been read: no wait in practice
+            if (!a.lse_obs && threadIdx.x == 0 && poll_until_at_least(ticket, im.chunk, &sh.abort)) atomicExch(ticket, 0);
+        }
+        if (!ONE) __syncthreads();   // t_chunk, neg_lse2 and the selection scratch are reused by the next item
+    } while (!SINGLE && (item += gridDim.x) < n_items);
+}
+
+template <int MB, bool ONE, bool SINGLE>
+// 18 warps put five on one SM sub-partition (16K registers): 96 registers per thread at most
+__global__ void __launch_bounds__(block_threads(MB), 1)
+score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ TcArgs a,
+                 const __nv_bfloat16 *__restrict__ q)
+{
+    constexpr int kStages = stages_for(MB);
+    Shared<MB> &sh = shared_state<MB>();
+    Barriers &bar = sh.bar;
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        init_barriers(bar);
+        sh.abort = 0;
+        sh.counted = 0;
+    }
+    if (warp == 1) tmem_alloc(&sh.tmem_base, kTmemCols);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    pdl_wait();                 // nothing above touches memory of anybody else
+    if (threadIdx.x == 0) tma_prefetch_desc(&tmap);
+
+    Carry carry = {0, 0, -1};
+    if (ONE) {
+        take_wave<MB, true, true>(&tmap, a, q, 0, carry);
+    } else {
+        for (int u0 = 0; u0 < a.s.batch * a.s.hkv && !*static_cast<volatile int *>(&sh.abort); u0 += a.units_per_wave)
+            take_wave<MB, false, SINGLE>(&tmap, a, q, u0, carry);
     }
 
     // ------------------------------------------------------------------ teardown
     __syncthreads();
-    if (warp == 0 && leader) {
+    if (threadIdx.x == 32 && !sh.counted) count_launch(a.count, launches_so_far(a.count) + 1);    // a block without an item
+    if (warp == 0 && elect_one()) {
         // nothing of this block may be in flight when it ends: the last MMAs must have released
         // their stages; after a failed wait, the loads already issued must still land.  (The lane that issued
         // them knows how many: the lanes of the warp may give up at different tiles.)
-        for (uint32_t g = p_issued > kStages ? p_issued - kStages : 0; g < p_issued; ++g) {
+        for (uint32_t g = carry.issued > kStages ? carry.issued - kStages : 0; g < carry.issued; ++g) {
             const int st = g % kStages;
-            if (!mbar_wait(&bar.empty[st], (g / kStages) & 1, &abort_s)) {
+            if (!mbar_wait(&bar.empty[st], (g / kStages) & 1, &sh.abort)) {
                 volatile int never = 0;
                 mbar_wait(&bar.full[st], (g / kStages) & 1, &never);
             }
         }
-        if (abort_s) atomicOr(a.status, kStatusWaitExpired);
+        if (sh.abort) atomicOr(a.status, kStatusWaitExpired);
     }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    if (warp == 1) tmem_dealloc(tmem_base, tmem_cols);
+    if (warp == 1) tmem_dealloc(sh.tmem_base, kTmemCols);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -792,7 +926,7 @@ struct DeviceInfo {
     int cc_major = -1;
     int sm_count = 0;
     int cooperative = 0;
-    int blocks_per_sm[2] = {-1, -1};   // resident blocks of each instantiation at its largest footprint
+    int blocks_per_sm[2][3] = {{-1, -1, -1}, {-1, -1, -1}};   // resident blocks of each instantiation at its largest footprint
 };
 std::mutex g_device_mutex;
 DeviceInfo g_device_info[kMaxDevices];
@@ -847,7 +981,10 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
 
     TcArgs a;
     a.s = ks;
-    a.stats = reinterpret_cast<float2 *>(static_cast<char *>(workspace) + ws.stats_off);
+    a.stats = reinterpret_cast<StatEntry *>(static_cast<char *>(workspace) + ws.stats_off);
+    a.scores = reinterpret_cast<StatEntry *>(static_cast<char *>(workspace) + ws.entries_off);
+    a.count = reinterpret_cast<LaunchCount *>(static_cast<char *>(workspace) + ws.count_off);
+    a.salt = ws.salt;
     a.window_scores = window_scores;
     a.lse_obs = lse_obs;
     a.token_scores = token_scores;
@@ -855,26 +992,34 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
     a.kept_len = kept_len;
     a.status = reinterpret_cast<int *>(static_cast<char *>(workspace) + ws.status_off);
     a.sync = reinterpret_cast<int *>(static_cast<char *>(workspace) + ws.sync_off);
-    a.n_stat_chunks = ws.n_stat_chunks;
     a.r_pad = ws.r_pad;
     const int units = ks.batch * ks.hkv;
     const TcPlan plan = tc_plan(units, ks.max_seqlen, ks.omega, ks.R);
+    a.n_stat_chunks = plan.chunks_per_unit;
     a.chunks_per_unit = plan.chunks_per_unit;
     a.units_per_wave = plan.units_per_wave;
     a.kblocks = ks.d / 64;
     a.slot_tok = slot[0];
     a.slot_h = slot[1];
     a.slot_b = slot[2];
+    a.alpha_inverse = (65536u + ks.alpha - 1) / ks.alpha;
     a.r16 = (ks.R + 15) / 16 * 16;
 
     const int mb = ks.R > 128 ? 2 : 1;
     const int threads = block_threads(mb);
     const size_t smem = tc_smem_bytes(a.kblocks, mb);
-    const void *fn = mb == 1 ? reinterpret_cast<const void *>(score_windows_tc<1>)
-                             : reinterpret_cast<const void *>(score_windows_tc<2>);
+    // persistent blocks, one per SM at most; every block of a cooperative launch is resident, which
+    // the hand-over of the statistics between the sweeps relies on
+    int grid = plan.units_per_wave * plan.chunks_per_unit;
+    if (grid > di.sm_count) grid = di.sm_count;
+    const int form = grid < plan.units_per_wave * plan.chunks_per_unit ? 0 : (plan.units_per_wave < units ? 1 : 2);
+    const auto kernel = mb == 1 ? (form == 2 ? score_windows_tc<1, true, true> : form == 1 ? score_windows_tc<1, false, true> : score_windows_tc<1, false, false>)
+                                : (form == 2 ? score_windows_tc<2, true, true> : form == 1 ? score_windows_tc<2, false, true> : score_windows_tc<2, false, false>);
+    const void *fn = reinterpret_cast<const void *>(kernel);
+    int &blocks_per_sm = di.blocks_per_sm[mb - 1][form];
     cudaError_t err = cudaSuccess;
     std::unique_lock<std::mutex> setup_lock(g_device_mutex);
-    if (di.blocks_per_sm[mb - 1] < 0) {
+    if (blocks_per_sm < 0) {
         // once per device and instantiation: allow its largest shared-memory request (head_dim 128) and ask how
         // many of its blocks an SM holds at that size
         const size_t smem_max = tc_smem_bytes(2, mb);
@@ -891,20 +1036,16 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
                                  "of shared memory)", threads, fa.numRegs, smem_max, fa.sharedSizeBytes);
                 return WKV_ERR_CUDA;
             }
-            di.blocks_per_sm[mb - 1] = occ;
+            blocks_per_sm = occ;
         }
     }
     setup_lock.unlock();
-    // persistent blocks, one per SM at most; every block of a cooperative launch is resident, which
-    // the hand-over of the statistics between the sweeps relies on
-    int grid = plan.units_per_wave * plan.chunks_per_unit;
-    if (grid > di.sm_count) grid = di.sm_count;
     const __nv_bfloat16 *qp = static_cast<const __nv_bfloat16 *>(q);
     if (err == cudaSuccess) {
         void *params[3] = {&tmap, &a, &qp};
         // with given normalisers no block waits for another: a plain launch, which may start while the kernel in front
         // drains (a cooperative one may not: 2 us)
-        if (lse_obs) err = launch_pdl(mb == 1 ? score_windows_tc<1> : score_windows_tc<2>, dim3(grid), threads, smem, stream, 1, tmap, a, qp);
+        if (lse_obs) err = launch_pdl(kernel, dim3(grid), threads, smem, stream, 1, tmap, a, qp);
         else err = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), params, smem, stream);
     }
     if (err != cudaSuccess) {

@@ -42,6 +42,7 @@ Workspace plan_workspace(const KShape &ks, int sync_units)
     if (pipe_chunks > w.n_stat_chunks) w.n_stat_chunks = pipe_chunks;
     size_t off = 0;
     w.status_off = off;
+    w.count_off = 16;
     off = 64;
     w.sync_off = off;
     const size_t sync_room = units > (size_t)sync_units ? units : (size_t)sync_units;
@@ -49,11 +50,16 @@ Workspace plan_workspace(const KShape &ks, int sync_units)
     w.pstats_off = off;
     off = align_up(off + (ks.R <= 128 ? units * w.n_stat_chunks * 128 * sizeof(unsigned long long) : 0), 256);
     w.stats_off = off;
-    off = align_up(off + units * w.n_stat_chunks * w.r_pad * sizeof(float2), 256);
+    const size_t stats = (size_t)w.n_stat_chunks * sizeof(float2), words = (size_t)tc_chunks * 16;
+    off = align_up(off + units * w.r_pad * (stats > words ? stats : words), 256);
     w.lse_off = off;
     off = align_up(off + units * w.r_pad * sizeof(float), 256);
     w.scores_off = off;
+    w.counted_off = align_up(align_up(w.stats_off + units * w.r_pad * stats, 256) + units * w.r_pad * sizeof(float), 256);
+    w.salt = 0;
     off = align_up(off + units * (size_t)ks.kw_max * sizeof(float), 256);
+    w.entries_off = off;
+    off = align_up(off + units * (size_t)ks.kw_max * 16, 256);
     w.total = off;
     return w;
 }

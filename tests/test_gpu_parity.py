@@ -861,3 +861,56 @@ def test_config5_packed_output():
     dense = pu.run_gpu_group(w, grp)
     np.testing.assert_array_equal(idx_h, dense["window_idx"])
     np.testing.assert_array_equal(kept.cpu().numpy(), dense["kept_len"])
+
+
+def _expected_selection(scores, k):
+    """Of given fp32 window scores: the k highest, ties to the lower index, in ascending order."""
+    return np.sort(np.lexsort((np.arange(len(scores)), -scores))[:k])
+
+
+@pytest.mark.parametrize("n_windows", [1, 64, 65, 576, 577, 2304, 2305, 4608, 4609])
+@pytest.mark.parametrize("keys", ["normal", "one-takes-all", "equal"])
+def test_fused_selection_is_exact_on_its_own_scores(n_windows, keys):
+    """The selection inside the score kernel against a sort of the scores that the same call returns, on both sides of its
+    limits (candidates ranked directly, windows per thread) and where scores leave the range its first pass looks at:
+    one key takes all of the attention and the other windows' scores underflow to zero or nearly so, or all are equal."""
+    w = small(head_dim=64, n_q_heads=4, n_kv_heads=2, batch=1, l_obs=8, window=4, n_planted=0, n_layers=1, gamma=1,
+              budget_frac=0.3, max_seqlen=8 + 4 * n_windows - (1 if n_windows > 1 else 0))
+    grp = wl.make_group(w, 0)
+    q, k = binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0])
+    if keys == "equal":
+        k.copy_(k[:, :, :1].expand_as(k))
+    elif keys == "one-takes-all":
+        for h in range(2):
+            k[0, h, min(5, k.shape[2] - 1)] = 40 * torch.nn.functional.normalize(q[0, 2 * h:2 * h + 2].float().sum((0, 1)), dim=0)
+    prob = binding.Problem.from_workload(w, score_impl=IMPLS["tc"])
+    assert prob.kw_max == n_windows
+    work, out = prob.alloc_workspace(), prob.alloc_outputs(0)
+    for _ in range(2):
+        out["window_idx"].fill_(-7)
+        binding.wkv_select_leader_windows(prob, q, k, out["window_scores"], out["window_idx"], out["kept_len"], work)
+    assert binding.device_status(work) == 0
+    scores, idx = out["window_scores"].cpu().numpy(), out["window_idx"].cpu().numpy()
+    for h in range(2):
+        chosen = idx[0, h][idx[0, h] >= 0]
+        np.testing.assert_array_equal(chosen, _expected_selection(scores[0, h, :n_windows], len(chosen)))
+        last = 4 if n_windows == 1 else 3
+        rows = 4 * len(chosen) - (4 - last if n_windows - 1 in chosen else 0) + 8
+        assert int(out["kept_len"][0, h]) == rows
+
+
+def test_a_sequence_with_more_chunks_than_blocks():
+    """Beyond 148 x 37 key tiles a block takes several items of one wave; its ring and its image of Q pass from one to the next."""
+    w = small(head_dim=64, n_q_heads=1, n_kv_heads=1, batch=1, l_obs=8, window=64, n_planted=0, n_layers=1, gamma=1,
+              budget_frac=0.01, max_seqlen=148 * 37 * 128 + 5000)
+    grp = wl.make_group(w, 0)
+    ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
+    prob = binding.Problem.from_workload(w, score_impl=IMPLS["tc"])
+    work, out = prob.alloc_workspace(), prob.alloc_outputs(0)
+    for _ in range(2):
+        binding.wkv_select_leader_windows(prob, binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0]),
+                                          out["window_scores"], out["window_idx"], out["kept_len"], work)
+        assert binding.device_status(work) == 0
+        pu.check_selection(w, grp, {"prob": prob, "window_scores": out["window_scores"].cpu().numpy(),
+                                    "window_idx": out["window_idx"].cpu().numpy(),
+                                    "kept_len": out["kept_len"].cpu().numpy()}, ref)
