@@ -265,6 +265,7 @@ score_stats_simt(const __grid_constant__ KShape s, const T *__restrict__ q, cons
 // the selection that the score kernel's last block of a unit runs (window_idx null: none)
 struct SimtSelect {
     int *window_idx, *kept_len, *status, *sync;
+    bool release_early;     // the gather behind it waits before it looks at the indices
 };
 
 // Eq. 4 for one window: the sorting network where there is one for its length, else the serial form
@@ -296,7 +297,7 @@ score_pool_simt(const __grid_constant__ KShape s, const T *__restrict__ q, const
     float *t_chunk = part + TY * kKT;          // [chunk_keys rounded up to kKT]
     TopkSmem &topk_sm = *reinterpret_cast<TopkSmem *>(smem);   // the selection comes when all of these are done with
 
-    pdl_trigger();
+    if (sel.release_early) pdl_trigger();
     // with given normalisers there is no statistics kernel in front that has waited for Q and K
     if (lse_obs) pdl_wait();
     const int unit = blockIdx.y;
@@ -511,7 +512,7 @@ static cudaError_t launch_simt_type(const KShape &ks, int slot, const void *q, c
 cudaError_t launch_score_simt(const KShape &ks, int dtype, const void *q, const void *k,
                               float *window_scores, float *token_scores,
                               void *workspace, const Workspace &ws, cudaStream_t stream, const float *lse_obs,
-                              int *window_idx, int *kept_len)
+                              int *window_idx, int *kept_len, bool group)
 {
     float2 *stats = reinterpret_cast<float2 *>(static_cast<char *>(workspace) + ws.stats_off);
     if (ks.max_seqlen <= ks.alpha) return window_idx ? launch_topk(ks, window_scores, window_idx, kept_len, stream) : cudaSuccess;
@@ -519,6 +520,7 @@ cudaError_t launch_score_simt(const KShape &ks, int dtype, const void *q, const 
     // thread): one launch less.  Longer lists go to the kernel with four times the threads.
     const bool inside = window_idx && ks.kw_max <= 8 * kThreads;
     SimtSelect sel = {};
+    sel.release_early = group;
     if (inside) {
         sel.window_idx = window_idx;
         sel.kept_len = kept_len;

@@ -11,7 +11,7 @@ select_topk_kernel(KShape s, const float *__restrict__ window_scores, int *__res
                    int *__restrict__ kept_len)
 {
     __shared__ TopkSmem sm;
-    pdl_trigger();
+    // (no early release: a gather behind it fetches rows by the indices it finds, ahead of its wait)
     pdl_wait();
     const int unit = blockIdx.x;
     const int b = unit / s.hkv;

@@ -264,7 +264,7 @@ int do_score(const wkv_shape *s, const KShape &ks, const Workspace &ws, const vo
         if (score_simt_smem_bytes(ks, ws.r_pad) > 227u * 1024u) return st;
     }
     return check_cuda(launch_score_simt(ks, s->dtype, q, k, window_scores, token_scores, workspace, ws, stream, lse_obs,
-                                        window_idx, kept_len),
+                                        window_idx, kept_len, gather != nullptr),
                       "score kernels");
 }
 
@@ -560,7 +560,7 @@ static int gather_kv_entry(const wkv_shape *s, int32_t n_layers, const void *con
         return WKV_ERR_SHAPE;
     }
     return check_cuda(launch_gather(ks, elem_bytes(s->dtype), n_tensors, tab, window_idx, cu_seqlens_out,
-                                    keep_capacity, static_cast<cudaStream_t>(cuda_stream), nullptr, over_bus),
+                                    keep_capacity, static_cast<cudaStream_t>(cuda_stream), nullptr, over_bus, true),
                       "gather kernel");
 }
 

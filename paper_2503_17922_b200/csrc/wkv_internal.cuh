@@ -217,6 +217,24 @@ constexpr int kStatusWaitExpired = 1;   // a bounded wait inside a kernel ran ou
 // between two kernels (a chain of short kernels: 4.1 us each without, 2.0 us with).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A window's rows into L2, ahead of pdl_wait(): `lanes` lanes take its lines in turn.  Nothing is read that the kernel
+// goes on with (L2 is where the GPU's memory is coherent: a line fetched early and written later is the written one), and
+// an index that is not yet the final one is no more than a wasted fetch inside the tensor.
+__device__ __forceinline__ void fetch_window(const KShape &s, const char *tensor, int elem_bytes, int unit, int window, int lane,
+                                             int lanes)
+{
+    const int b = unit / s.hkv, h = unit - b * s.hkv;
+    const SeqInfo si = seq_info(s, b);
+    const int n_r = si.n - s.alpha, row0 = window * s.omega;
+    if (window < 0 || window >= num_windows(si.n, s.alpha, s.omega)) return;
+    const long long row_bytes = s.st * elem_bytes;
+    const int row_lines = (s.d * elem_bytes + 127) >> 7, rows = min(s.omega, n_r - row0);
+    const char *at = tensor + (si.off * s.st + b * s.sb + h * s.sh) * (long long)elem_bytes + row0 * row_bytes;
+    for (int x = lane; x < rows * row_lines; x += lanes) {
+        const int r = x / row_lines;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(at + r * row_bytes + (long long)(x - r * row_lines) * 128));
+    }
+}
 // `cluster`: blocks per cluster along x (1: none)
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
@@ -249,7 +267,7 @@ cudaError_t launch_score_simt(const KShape &ks, int dtype, const void *q, const 
                               float *window_scores, float *token_scores,
                               void *workspace, const Workspace &ws, cudaStream_t stream,
                               const float *lse_obs = nullptr, int *window_idx = nullptr,
-                              int *kept_len = nullptr);
+                              int *kept_len = nullptr, bool group = false);
 bool score_tc_supported(const KShape &ks, int dtype);
 // window_idx / kept_len non-null: the selection is fused into the same launch.
 // lse_obs non-null: float [B, H_q, alpha], natural log of Eq. 1's normaliser of every observation
@@ -284,10 +302,13 @@ struct PagedOut {
     int max_pages, page_size, num_pages;
     long long page_stride, head_stride, row_stride;
 };
-// over_bus: the rows are read from host memory (not for paged output)
+// over_bus: the rows are read from host memory (not for paged output).  early: the windows' rows are fetched into L2
+// before the kernel in front has ended; for calls of their own, whose indices are final by then (a kernel that writes
+// them releases nobody before it ends).  Not in the group call, whose gather may be released earlier.
 cudaError_t launch_gather(const KShape &ks, int elem_bytes, int n_tensors, const LayerTable &tab,
                           const int *window_idx, const int *cu_out, int keep_capacity,
-                          cudaStream_t stream, const PagedOut *paged = nullptr, bool over_bus = false);
+                          cudaStream_t stream, const PagedOut *paged = nullptr, bool over_bus = false,
+                          bool early = false);
 // compaction of every layer's K/V inside its own buffer (compact.cu)
 struct InplaceTable {
     void *ptr[2 * WKV_MAX_GROUP_LAYERS];

@@ -286,3 +286,45 @@ def test_a_refused_launch_is_reported_once():
     assert e.value.status == 8
     binding.wkv_probe_ex2_rate(torch.zeros(4, dtype=torch.float32, device="cuda"), 1, 32, 1)
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("inplace", [False, True])
+@pytest.mark.parametrize("layout", ["bhnd", "bnhd"])
+def test_rows_that_the_kernel_in_front_writes(layout, inplace):
+    """A gather or compaction fetches rows into L2 before the kernel in front has ended; what it then reads is what that
+    kernel wrote.  Here a gather writes the keys that the next call takes rows from, at odd sizes and with a short last
+    window, several times back to back."""
+    B, H, n, d, alpha, omega, k = 2, 3, 4999, 128, 8, 16, 60
+    rows = k * omega + alpha
+    rng = np.random.default_rng(5)
+
+    def problem(length, layout):
+        return binding.Problem(dtype="bf16", batch=B, n_q_heads=H, n_kv_heads=H, head_dim=d, l_obs=alpha, window=omega, task=0,
+                               top_p=omega, max_seqlen=length, budgets=[rows] * B, kv_layout=layout)
+
+    first, second = problem(n, layout), problem(rows, "bhnd")
+    assert first.k_max == k and second.k_max == k
+    kw = -(-(n - alpha) // omega)
+    idx = np.stack([np.stack([np.sort(rng.permutation(kw)[:k]) for _ in range(H)]) for _ in range(B)]).astype(np.int32)
+    idx[0, 0, -1] = kw - 1                                 # the short last window
+    again = np.tile(np.arange(k, dtype=np.int32), (B, H, 1))
+    again[:, :, 7:] = -1                                   # of the compact rows: the first seven windows and the last rows
+    shape = (B, H, n, d) if layout == "bhnd" else (B, n, H, d)
+    idx_d, again_d = torch.from_numpy(idx).cuda(), torch.from_numpy(again).cuda()
+    for seed in range(4):
+        src = torch.randn(shape, dtype=torch.bfloat16, device="cuda", generator=torch.Generator("cuda").manual_seed(seed))
+        mid = torch.zeros((B, H, rows, d), dtype=torch.bfloat16, device="cuda")
+        out = torch.zeros_like(mid)
+        binding.wkv_gather_kv(first, [src], [src], idx_d, [mid], [torch.empty_like(mid)], keep_capacity=rows)
+        if inplace:
+            binding.wkv_compact_kv_inplace(second, [mid], None, again_d)
+        else:
+            binding.wkv_gather_kv(second, [mid], [mid], again_d, [out], [torch.empty_like(out)], keep_capacity=rows)
+        got = (mid if inplace else out).float().cpu()
+        full = (src if layout == "bhnd" else src.transpose(1, 2)).float().cpu()
+        for b in range(B):
+            for h in range(H):
+                taken = torch.cat([full[b, h, w * omega:min((w + 1) * omega, n - alpha)] for w in idx[b, h, :7]])
+                assert torch.equal(got[b, h, :7 * omega], taken)
+
+
