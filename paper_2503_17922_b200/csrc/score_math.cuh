@@ -4,6 +4,7 @@
 #pragma once
 
 #include "tc_common.cuh"
+#include "topk_block.cuh"
 #include "wkv_internal.cuh"
 
 namespace wkv {
@@ -107,18 +108,43 @@ __device__ __forceinline__ unsigned long long launch_tag(unsigned long long laun
     return kTagBits | (unsigned long long)(salt & 0xffu) << 40 | ((launches + 1) & 0xffffffffffull);
 }
 __device__ __forceinline__ unsigned long long launch_of(unsigned long long tag) { return tag & 0xffffffffffull; }
-// one thread per block, `launch` being one more than what it has read
-__device__ __forceinline__ void count_launch(LaunchCount *c, unsigned long long launch)
+// one thread of each of the launch's `blocks` blocks, `launch` being one more than what it has read
+__device__ __forceinline__ void count_launch(LaunchCount *c, unsigned long long launch, unsigned blocks)
 {
-    if (atomicInc(&c->blocks, gridDim.x - 1) == gridDim.x - 1) c->launches = launch;
+    if (atomicInc(&c->blocks, blocks - 1) == blocks - 1) c->launches = launch;
 }
 
-__device__ __forceinline__ bool warp_wait_arrivals(const int *word, int target, volatile int *abort_flag, int lane)
-{
-    int ok = 1;
-    if (lane == 0) ok = poll_until_at_least(word, target, abort_flag) ? 1 : 0;
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
-}
+// The selection reads the published window scores, waiting for those that are still to come: LOOK words at a time.
+template <int LOOK>
+struct PublishedScores {
+    const StatEntry *entries;
+    unsigned long long tag;
+    volatile int *abort_flag;
+    int hint;
+    template <int N>
+    __device__ __forceinline__ void keys(unsigned (&key)[N], int lo, int hi) const
+    {
+        constexpr int kLook = N < LOOK ? N : LOOK;
+#pragma unroll
+        for (int e0 = 0; e0 < N; e0 += kLook) {
+            StatEntry v[kLook];
+            const int left = hi - lo - e0;
+            wait_entries<kLook>(entries + lo + e0, 1, left >= kLook ? (1u << kLook) - 1u : left > 0 ? (1u << left) - 1u : 0u, tag, v,
+                                abort_flag);
+#pragma unroll
+            for (int e = 0; e < kLook; ++e) key[e0 + e] = e < left ? topk_order_key(__uint_as_float((unsigned)v[e].value)) : 0u;
+        }
+    }
+    __device__ __forceinline__ void wait(int lo, int hi) const
+    {
+        unsigned unused[LOOK];
+        for (int w = lo; w < hi; w += LOOK) keys(unused, w, min(hi, w + LOOK));
+    }
+    __device__ __forceinline__ unsigned key(int w) const
+    {
+        return topk_order_key(__ldcg(reinterpret_cast<const float *>(&entries[w].value)));
+    }
+};
 
 // acc + 2^x for x <= 0 on the FMA pipe: 2^x = 2^t * 2^f with t the nearest integer, and 2^f by a polynomial of degree six
 // (a Remez fit of the relative error on [-1/2, 1/2]: 1.9e-9, below the rounding of the evaluation and of ex2.approx).

@@ -1,5 +1,5 @@
 // CUDA-core (FFMA) score kernels: Eq. 1-4 for fp32 inputs and for shapes the
-// tensor-core kernels do not cover.  Two kernels per call:
+// tensor-core kernels do not cover.  One kernel per call where its blocks are resident together (score_fused_simt), else two:
 //   stats : per row of the unit, partial (max, sum exp2) over a chunk of keys
 //           (Eq. 1's normaliser, causal mask applied)
 //   score : logits again, p = exp2(x - lse2), sum over the rows (Eq. 2), then the
@@ -262,12 +262,6 @@ score_stats_simt(const __grid_constant__ KShape s, const T *__restrict__ q, cons
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// the selection that the score kernel's last block of a unit runs (window_idx null: none)
-struct SimtSelect {
-    int *window_idx, *kept_len, *status, *sync;
-    bool release_early;     // the gather behind it waits before it looks at the indices
-};
-
 // Eq. 4 for one window: the sorting network where there is one for its length, else the serial form
 __device__ inline float pool_window(const float *w, int omega, int size, int p)
 {
@@ -279,6 +273,204 @@ __device__ inline float pool_window(const float *w, int omega, int size, int p)
     default: return pool_top_p(w, size, p);
     }
 }
+
+// ---------------------------------------------------------------------------------------------
+// one launch for statistics, scores and selection
+// ---------------------------------------------------------------------------------------------
+struct FusedArgs {
+    KShape s;
+    StatEntry *stats;       // [units][n_chunks][r_pad]: published statistics of 512 keys
+    StatEntry *entries;     // [units][kw_max]: published window scores, for the block that selects
+    float *window_scores, *token_scores;
+    int *window_idx, *kept_len;     // null: no selection
+    int *status;
+    LaunchCount *count;
+    unsigned salt;
+    int n_chunks, r_pad, r_tile;
+};
+
+// Where all blocks are resident at once (cooperative launch) the logits of a block's one tile stay in its registers
+// while the unit's statistics are put together: the tiles of Q and K are transposed and multiplied once instead of twice,
+// and two kernel boundaries go.  The blocks of 512 keys are a cluster and combine their rows through distributed shared
+// memory; chunks and window scores are handed over as self-validating words; the block of the unit's last review
+// keys selects.  Windows must not straddle tiles.  Bounded, like the other kernels that wait: status bit 0.
+// Grid: x = tiles rounded up to whole clusters, y = unit.
+template <typename T, int RB, int PASSES>
+__global__ void __launch_bounds__(kThreads, 4)
+score_fused_simt(const __grid_constant__ FusedArgs a, const T *__restrict__ q, const T *__restrict__ k)
+{
+    constexpr int KPT = TileMap<RB>::KPT, TX = TileMap<RB>::TX, TY = kThreads / TX;
+    constexpr int kSharers = TX < 32 ? TX : 32;              // neighbouring lanes that share a row
+    extern __shared__ __align__(16) float smem[];
+    const KShape &s = a.s;
+    float *qs = smem;                                        // [d][r_tile]
+    float *ks = qs + s.d * a.r_tile;                         // [d][kKPad]
+    float2 *rows = reinterpret_cast<float2 *>(ks + s.d * kKPad);   // [2][r_pad] this block's (max, sum) per row
+    float *lse2 = reinterpret_cast<float *>(rows + 2 * a.r_pad);   // [r_pad]
+    float *part = lse2 + a.r_pad;                            // [TY][kKT]
+    float *t_tile = part + TY * kKT;                         // [kKT]
+    int *last = reinterpret_cast<int *>(t_tile + kKT);       // [r_tile]
+    TopkSmem &topk_sm = *reinterpret_cast<TopkSmem *>(smem); // the selection comes when all of these are done with
+    __shared__ int abort_s;
+    __shared__ unsigned long long tag_s;
+
+    const int unit = blockIdx.y, chunk = blockIdx.x / kChunkTiles, rank = blockIdx.x - chunk * kChunkTiles;
+    const int b = unit / s.hkv, h = unit - b * s.hkv;
+    const SeqInfo si = seq_info(s, b);
+    const int n = si.n, n_r = n - s.alpha, j0 = blockIdx.x * kKT;
+    const int ty = threadIdx.x / TX, tx = threadIdx.x % TX;
+    unsigned long long launches = 0;
+    if (threadIdx.x == 0) launches = launches_so_far(a.count);
+    const bool idle = n_r <= 0 || j0 >= n;
+    float acc[PASSES][4][KPT];
+    if (!idle) {
+        load_q_transposed<T, RB>(s, q + b * s.qsb + (long long)h * s.G * s.qsh, qs, last, n_r, a.r_tile);
+        load_k_transposed(s, k + (si.off * s.st + b * s.sb + h * s.sh), ks, j0, n);
+    }
+    if (threadIdx.x == 0) {
+        abort_s = 0;
+        tag_s = launch_tag(launches, a.salt);
+    }
+    for (int r = threadIdx.x; r < 2 * a.r_pad; r += kThreads) rows[r] = make_float2(-INFINITY, 0.f);
+    __syncthreads();
+    if (threadIdx.x == 32) count_launch(a.count, launch_of(tag_s), gridDim.x * gridDim.y);
+    if (!idle) {
+#pragma unroll
+        for (int p = 0; p < PASSES; ++p) {
+            logits_tile<RB>(qs, ks, s.d, a.r_tile, p * RB, ty, tx, acc[p]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = p * RB + ty * 4 + i, jl = last[r] - j0 - tx * KPT;      // of this thread's keys, those up to jl count
+                float m = -INFINITY;
+#pragma unroll
+                for (int c = 0; c < KPT; ++c) {
+                    acc[p][i][c] *= s.scale_log2;
+                    if (c <= jl) m = fmaxf(m, acc[p][i][c]);
+                }
+#pragma unroll
+                for (int o = 1; o < kSharers; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                const float safe = m == -INFINITY ? 0.f : m;
+                float l = 0.f;
+#pragma unroll
+                for (int c = 0; c < KPT; ++c)
+                    if (c <= jl) l += exp2f(acc[p][i][c] - safe);
+#pragma unroll
+                for (int o = 1; o < kSharers; o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+                if (tx % kSharers == 0) rows[(tx / kSharers) * a.r_pad + r] = make_float2(m, l);
+            }
+        }
+    }
+    // the chunk's rows: each block of the cluster combines a share of them over all blocks, a lane per block
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const int share = a.r_pad / kChunkTiles;
+    if ((int)threadIdx.x < share * kChunkTiles) {            // whole warps: r_pad is a multiple of 64
+        const int r = rank * share + threadIdx.x / kChunkTiles, from = threadIdx.x % kChunkTiles;
+        float2 v = ld_cluster(rows + r, from);
+        if (TX > 32) {
+            const float2 second = ld_cluster(rows + a.r_pad + r, from);
+            merge_stats(v.x, v.y, second.x, second.y);
+        }
+#pragma unroll
+        for (int o = 1; o < kChunkTiles; o <<= 1)
+            merge_stats(v.x, v.y, __shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
+        if (from == 0 && r < s.R && chunk * kStatChunk < n)
+            publish_entry(a.stats + ((size_t)unit * a.n_chunks + chunk) * a.r_pad + r,
+                          (unsigned long long)__float_as_uint(v.x) | (unsigned long long)__float_as_uint(v.y) << 32, tag_s);
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // this block has read its peers' rows
+
+    const int j_end = min(n_r, j0 + kKT);
+    if (j0 < n_r) {
+        // log2 of every row's normaliser from the unit's chunks: neighbouring threads share a row
+        const int used = (n + kStatChunk - 1) / kStatChunk;
+        const int tpr = a.r_pad <= 64 ? 4 : 2;
+        {
+            const int r = threadIdx.x / tpr, of = threadIdx.x - r * tpr;
+            float M = -INFINITY, L = 0.f;
+            if (r < s.R) {
+                const StatEntry *st = a.stats + (size_t)unit * a.n_chunks * a.r_pad + r;
+                for (int c0 = of; c0 < used; c0 += 4 * tpr) {
+                    unsigned wanted = 0u;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) wanted |= (c0 + u * tpr < used ? 1u : 0u) << u;
+                    StatEntry e[4];
+                    wait_entries<4>(st + (size_t)c0 * a.r_pad, (size_t)tpr * a.r_pad, wanted, tag_s, e, &abort_s);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (wanted >> u & 1u)
+                            merge_stats(M, L, __uint_as_float((unsigned)e[u].value), __uint_as_float((unsigned)(e[u].value >> 32)));
+                }
+            }
+            __syncwarp();
+            for (int o = 1; o < tpr; o <<= 1) {
+                const float m2 = __shfl_xor_sync(0xffffffffu, M, o), l2 = __shfl_xor_sync(0xffffffffu, L, o);
+                merge_stats(M, L, m2, l2);
+            }
+            if (of == 0 && r < a.r_pad) lse2[r] = r < s.R && L > 0.f ? M + log2f(L) : INFINITY;
+        }
+        __syncthreads();
+        float col[KPT];
+#pragma unroll
+        for (int c = 0; c < KPT; ++c) col[c] = 0.f;
+#pragma unroll
+        for (int p = 0; p < PASSES; ++p)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float ls = lse2[p * RB + ty * 4 + i];
+#pragma unroll
+                for (int c = 0; c < KPT; ++c) col[c] += exp2f(acc[p][i][c] - ls);
+            }
+#pragma unroll
+        for (int c = 0; c < KPT; ++c) part[ty * kKT + tx * KPT + c] = col[c];
+        __syncthreads();
+        if (threadIdx.x < kKT) {
+            float t = 0.f;
+#pragma unroll
+            for (int y = 0; y < TY; ++y) t += part[y * kKT + threadIdx.x];
+            t_tile[threadIdx.x] = t;
+            if (a.token_scores && j0 + (int)threadIdx.x < n_r) a.token_scores[(size_t)unit * s.nr_max + j0 + threadIdx.x] = t;
+        }
+        __syncthreads();
+        // Eq. 3-4: the tile's windows
+        const int n_win = (j_end - j0 + s.omega - 1) / s.omega;
+        if ((int)threadIdx.x < n_win) {
+            const int lo = threadIdx.x * s.omega;
+            const float r = pool_window(t_tile + lo, s.omega, min(s.omega, j_end - j0 - lo), s.p);
+            const size_t w = (size_t)unit * s.kw_max + j0 / s.omega + threadIdx.x;
+            a.window_scores[w] = r;
+            if (a.window_idx) publish_entry(a.entries + w, __float_as_uint(r), tag_s);
+        }
+    }
+    // no block leaves, or overwrites its rows, while another may still read them
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (a.window_idx) {
+        if (n_r <= 0) {
+            // a unit without review context still gets its (empty) selection
+            if (blockIdx.x == 0) {
+                for (int x = threadIdx.x; x < s.k_max; x += kThreads) a.window_idx[(size_t)unit * s.k_max + x] = -1;
+                if (threadIdx.x == 0) a.kept_len[unit] = min(n, s.alpha);
+            }
+        } else if (j0 < n_r && j_end == n_r) {
+            __syncthreads();
+            select_topk_block<kThreads>((int)threadIdx.x, topk_sm,
+                                        PublishedScores<4>{a.entries + (size_t)unit * s.kw_max, tag_s, &abort_s, topk_hint(s.R, n)},
+                                        num_windows(n, s.alpha, s.omega), num_selected_capped(n, s.alpha, s.omega, si.budget, s.k_max),
+                                        s.k_max, a.window_idx + (size_t)unit * s.k_max, a.kept_len + unit, n, s.alpha, s.omega);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && abort_s) atomicOr(a.status, kStatusWaitExpired);
+}
+
+// the selection that the score kernel's last block of a unit runs (window_idx null: none)
+struct SimtSelect {
+    int *window_idx, *kept_len, *status, *sync;
+    bool release_early;     // the gather behind it waits before it looks at the indices
+};
 
 template <typename T, int RB>
 // (five blocks per SM: the sorting network of long windows would take it beyond 48 registers, which costs the beginning
@@ -497,6 +689,99 @@ static cudaError_t launch_simt_tile(const KShape &ks, int slot, const void *q, c
     return err;
 }
 
+// Launches the fused kernel where its clusters are all resident at once, else leaves `taken` false: more blocks than that
+// would wait for blocks that cannot start.  Wherever they fit it is the faster way; select call, fp32, us, two launches /
+// one: 2 heads x 600 keys, 16 rows, d = 64 12.4 / 10.6; 8 heads x 4,000, 16 rows 24.1 / 17.0; 4 heads x 6,000, 64 rows
+// 30.9 / 20.6 (d = 128: 48.2 / 30.8); 2 heads x 6,000, 128 rows 33.6 / 24.3 (d = 128: 49.8 / 34.9).
+template <typename T, int RB, int PASSES>
+static cudaError_t launch_fused_tile(const KShape &ks, const void *q, const void *k, float *window_scores, float *token_scores,
+                                     void *workspace, const Workspace &ws, cudaStream_t stream, int *window_idx, int *kept_len,
+                                     bool &taken)
+{
+    FusedArgs a;
+    char *base = static_cast<char *>(workspace);
+    a.s = ks;
+    a.stats = reinterpret_cast<StatEntry *>(base + ws.stats_off);
+    a.entries = reinterpret_cast<StatEntry *>(base + ws.entries_off);
+    a.window_scores = window_scores;
+    a.token_scores = token_scores;
+    a.window_idx = window_idx;
+    a.kept_len = kept_len;
+    a.status = reinterpret_cast<int *>(base + ws.status_off);
+    a.count = reinterpret_cast<LaunchCount *>(base + ws.count_off);
+    a.salt = ws.salt;
+    a.n_chunks = (ks.max_seqlen + kStatChunk - 1) / kStatChunk;
+    a.r_pad = ws.r_pad;
+    a.r_tile = RB * PASSES;
+    size_t smem = sizeof(float) * ((size_t)ks.d * (a.r_tile + kKPad) + 5 * (size_t)a.r_pad + (RB / 4 + 1) * kKT + a.r_tile);
+    if (smem < sizeof(TopkSmem)) smem = sizeof(TopkSmem);
+
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    const auto fn = score_fused_simt<T, RB, PASSES>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a.n_chunks * kChunkTiles, ks.batch * ks.hkv);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kChunkTiles;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    {
+        // clusters that are resident at once: a property of device, kernel and shared-memory size, asked for once each
+        static std::mutex mu;
+        static size_t allowed[kMaxDevices] = {};
+        static size_t asked[kMaxDevices][4] = {};
+        static int resident[kMaxDevices][4] = {};
+        if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+        std::lock_guard<std::mutex> lock(mu);
+        if (smem > 48u * 1024u && smem > allowed[dev]) {
+            err = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (err != cudaSuccess) return err;
+            allowed[dev] = smem;
+        }
+        int slot = 0;
+        while (slot < 4 && asked[dev][slot] != smem && asked[dev][slot] != 0) ++slot;
+        int fits = slot < 4 ? resident[dev][slot] : 0;
+        if (slot == 4 || asked[dev][slot] == 0) {
+            err = cudaOccupancyMaxActiveClusters(&fits, fn, &cfg);
+            if (err != cudaSuccess) {
+                (void)cudaGetLastError();      // a device without such clusters: the two kernels
+                fits = 0;
+            }
+            if (slot < 4) {
+                asked[dev][slot] = smem;
+                resident[dev][slot] = fits;
+            }
+        }
+        if (a.n_chunks * ks.batch * ks.hkv > fits) return cudaSuccess;
+    }
+    cfg.numAttrs = 2;
+    err = cudaLaunchKernelEx(&cfg, fn, a, (const T *)q, (const T *)k);
+    if (err != cudaSuccess) return err;
+    taken = true;
+    count_launches(1);
+    return cudaSuccess;
+}
+
+template <typename T>
+static cudaError_t launch_fused_type(const KShape &ks, const void *q, const void *k, float *window_scores, float *token_scores,
+                                     void *workspace, const Workspace &ws, cudaStream_t stream, int *window_idx, int *kept_len,
+                                     bool &taken)
+{
+    if (ks.R <= 16) return launch_fused_tile<T, 16, 1>(ks, q, k, window_scores, token_scores, workspace, ws, stream, window_idx, kept_len, taken);
+    if (ks.R <= 32) return launch_fused_tile<T, 32, 1>(ks, q, k, window_scores, token_scores, workspace, ws, stream, window_idx, kept_len, taken);
+    if (ks.R <= 64) return launch_fused_tile<T, 64, 1>(ks, q, k, window_scores, token_scores, workspace, ws, stream, window_idx, kept_len, taken);
+    return launch_fused_tile<T, 64, 2>(ks, q, k, window_scores, token_scores, workspace, ws, stream, window_idx, kept_len, taken);
+}
+
 template <typename T>
 static cudaError_t launch_simt_type(const KShape &ks, int slot, const void *q, const void *k, float *window_scores,
                                     float *token_scores, float2 *stats, const Workspace &ws, cudaStream_t stream,
@@ -516,6 +801,14 @@ cudaError_t launch_score_simt(const KShape &ks, int dtype, const void *q, const 
 {
     float2 *stats = reinterpret_cast<float2 *>(static_cast<char *>(workspace) + ws.stats_off);
     if (ks.max_seqlen <= ks.alpha) return window_idx ? launch_topk(ks, window_scores, window_idx, kept_len, stream) : cudaSuccess;
+    if (!lse_obs && simt_fused_shape(ks)) {
+        bool taken = false;
+        const cudaError_t err = dtype == WKV_F32 ? launch_fused_type<float>(ks, q, k, window_scores, token_scores, workspace, ws,
+                                                                            stream, window_idx, kept_len, taken)
+                                                 : launch_fused_type<__nv_bfloat16>(ks, q, k, window_scores, token_scores, workspace,
+                                                                                    ws, stream, window_idx, kept_len, taken);
+        if (err != cudaSuccess || taken) return err;
+    }
     // The selection inside the score kernel where a block keeps the unit's window scores in registers (eight per
     // thread): one launch less.  Longer lists go to the kernel with four times the threads.
     const bool inside = window_idx && ks.kw_max <= 8 * kThreads;

@@ -127,38 +127,6 @@ __device__ __forceinline__ void warp_release(uint64_t *bar, int lane)
 // No block waits before it has finished all its sweep-1 work, so every wait ends.  Bounded: a thread that
 // looks for longer than two seconds gives up and sets the block's abort flag.
 
-// The selection reads the published window scores, waiting for those that are still to come: LOOK words at a time.
-template <int LOOK>
-struct PublishedScores {
-    const StatEntry *entries;
-    unsigned long long tag;
-    volatile int *abort_flag;
-    int hint;
-    template <int N>
-    __device__ __forceinline__ void keys(unsigned (&key)[N], int lo, int hi) const
-    {
-        constexpr int kLook = N < LOOK ? N : LOOK;
-#pragma unroll
-        for (int e0 = 0; e0 < N; e0 += kLook) {
-            StatEntry v[kLook];
-            const int left = hi - lo - e0;
-            wait_entries<kLook>(entries + lo + e0, 1, left >= kLook ? (1u << kLook) - 1u : left > 0 ? (1u << left) - 1u : 0u, tag, v,
-                                abort_flag);
-#pragma unroll
-            for (int e = 0; e < kLook; ++e) key[e0 + e] = e < left ? topk_order_key(__uint_as_float((unsigned)v[e].value)) : 0u;
-        }
-    }
-    __device__ __forceinline__ void wait(int lo, int hi) const
-    {
-        unsigned unused[LOOK];
-        for (int w = lo; w < hi; w += LOOK) keys(unused, w, min(hi, w + LOOK));
-    }
-    __device__ __forceinline__ unsigned key(int w) const
-    {
-        return topk_order_key(__ldcg(reinterpret_cast<const float *>(&entries[w].value)));
-    }
-};
-
 // The value, but nothing that is computed from it before this point: what only the ends of an item need would otherwise
 // be computed ahead of the tile loops and take their registers.
 __device__ __forceinline__ int late(int x)
@@ -675,7 +643,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                 issue_mma(im, std::true_type{});
                 // the block counts itself, once, now that it has read the number of launches
                 if (lane == 0 && (ONE || !sh.counted)) {
-                    count_launch(a.count, launch_of(sh.tag));
+                    count_launch(a.count, launch_of(sh.tag), gridDim.x);
                     sh.counted = 1;
                 }
             } else {
@@ -824,7 +792,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
 
     // ------------------------------------------------------------------ teardown
     __syncthreads();
-    if (threadIdx.x == 32 && !sh.counted) count_launch(a.count, launches_so_far(a.count) + 1);    // a block without an item
+    if (threadIdx.x == 32 && !sh.counted) count_launch(a.count, launches_so_far(a.count) + 1, gridDim.x);    // a block without an item
     if (warp == 0 && elect_one()) {
         // nothing of this block may be in flight when it ends: the last MMAs must have released
         // their stages; after a failed wait, the loads already issued must still land.  (The lane that issued

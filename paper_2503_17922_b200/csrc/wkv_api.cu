@@ -50,7 +50,7 @@ Workspace plan_workspace(const KShape &ks, int sync_units)
     w.pstats_off = off;
     off = align_up(off + (ks.R <= 128 ? units * w.n_stat_chunks * 128 * sizeof(unsigned long long) : 0), 256);
     w.stats_off = off;
-    const size_t stats = (size_t)w.n_stat_chunks * sizeof(float2), words = (size_t)tc_chunks * 16;
+    const size_t stats = (size_t)w.n_stat_chunks * sizeof(float2), words = (size_t)(simt_fused_shape(ks) && w.n_stat_chunks > tc_chunks ? w.n_stat_chunks : tc_chunks) * 16;
     off = align_up(off + units * w.r_pad * (stats > words ? stats : words), 256);
     w.lse_off = off;
     off = align_up(off + units * w.r_pad * sizeof(float), 256);

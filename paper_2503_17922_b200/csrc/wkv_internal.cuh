@@ -124,6 +124,14 @@ constexpr long long kTcWaveBytes = 80ll << 20;
 constexpr int kTcChunkCap = 4864;
 __host__ __device__ inline int tc_max_chunk_tiles(int omega) { return (kTcChunkCap - omega) / kTcTileKeys; }
 
+// Shapes that the CUDA-core path may score and select in one launch, if its blocks, one per 64 keys, are resident together:
+// up to 128 observation rows and windows that do not straddle 64 keys.
+inline bool simt_fused_shape(const KShape &ks)
+{
+    const long long chunks = (ks.max_seqlen + kStatChunk - 1) / kStatChunk;
+    return ks.R <= 128 && 64 % ks.omega == 0 && chunks * ks.batch * ks.hkv <= 128;
+}
+
 struct TcPlan {
     int units_per_wave;   // units swept together
     int chunks_per_unit;  // work items per unit

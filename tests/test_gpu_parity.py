@@ -914,3 +914,28 @@ def test_a_sequence_with_more_chunks_than_blocks():
         pu.check_selection(w, grp, {"prob": prob, "window_scores": out["window_scores"].cpu().numpy(),
                                     "window_idx": out["window_idx"].cpu().numpy(),
                                     "kept_len": out["kept_len"].cpu().numpy()}, ref)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("rows,window,n,batch", [
+    (16, 8, 64, 1), (16, 4, 65, 2), (17, 16, 512, 1), (32, 64, 513, 2), (33, 32, 577, 1), (64, 2, 1024 + 8, 1), (64, 1, 200, 1),
+    (65, 16, 1100, 3), (128, 8, 1031, 2), (129, 8, 700, 1), (16, 48, 700, 1), (16, 8, 9, 1), (16, 8, 72, 1),
+    (16, 16, 3000, 20), (16, 16, 3000, 40)])
+def test_cuda_core_path_in_one_launch_and_in_two(dtype, rows, window, n, batch):
+    """Statistics, scores and selection in one launch where its blocks of 64 keys are resident together: both sides of its
+    limits (128 rows, windows that do not straddle tiles, clusters that fit), every row tile, first and last tiles with only
+    observation keys or one review key.  Twice on one workspace, with other inputs: nothing of the first call passes for the second's."""
+    alpha = rows if rows % 8 else 8
+    w = small(dtype=dtype, head_dim=64, n_kv_heads=2, n_q_heads=2 * rows // alpha, l_obs=alpha, window=window, batch=batch,
+              max_seqlen=max(n, alpha + 1), n_layers=1, gamma=1, n_planted=0, budget_frac=0.4, top_p=max(1, window // 2))
+    prob = binding.Problem.from_workload(w, score_impl=IMPLS["simt"])
+    work, out = prob.alloc_workspace(), prob.alloc_outputs(0)
+    for config in (10, 11):
+        grp = wl.make_group(wl.scaled(w, config_id=config), 0)
+        ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
+        binding.wkv_select_leader_windows(prob, binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0]),
+                                          out["window_scores"], out["window_idx"], out["kept_len"], work)
+        assert binding.device_status(work) == 0
+        pu.check_selection(w, grp, {"prob": prob, "window_scores": out["window_scores"].cpu().numpy(),
+                                    "window_idx": out["window_idx"].cpu().numpy(),
+                                    "kept_len": out["kept_len"].cpu().numpy()}, ref)
