@@ -163,15 +163,18 @@ __device__ __forceinline__ void add_exp2_fma(float &acc, float x)
     p = fmaf(p, f, 1.f);
     acc = fmaf(p, __int_as_float((__float_as_int(shifted) << 23) + 0x3f800000), acc);
 }
-// One exponential in eight of both sweeps goes that way: the special-function pipe is what bounds them where keys come
-// fast enough, and the FMA pipe is half idle.  Select call, us, none / one in eight / 3 in 16 / one in four: 8 packed sequences of
-// 32-64 K keys, 256 rows, 552 / 533 / 528 / 538; 8 heads x 32,768 keys, 128 rows, 35.8 / 35.0 / 35.0 / 36.1; 16 heads x 24,576
-// keys 47.4 / 46.3 / 46.7 / 47.1.  Scores against 64 bits: 3.4-6.5e-7 rms with and without.
+// FMA_SHARE: one exponential in eight of both sweeps goes that way.  The special-function pipe is what bounds them where
+// keys come fast enough, and the FMA pipe is half idle.  Select call, us, none / one in eight / 3 in 16 / one in four: 8
+// heads x 32,768 keys, 128 rows, 35.8 / 35.0 / 35.0 / 36.1; 16 heads x 24,576 keys 47.4 / 46.3 / 46.7 / 47.1; 8 heads x 65,536
+// keys, 256 rows, 99.2 / 93.3.  Launches of several waves run long enough to meet the power limit, where the added work
+// costs what it saves: a whole group of 8 sequences of 32-64 K keys with 256 rows 1,033 / 1,050, so they go without.
+// Scores against 64 bits: 3.4-6.5e-7 rms with and without.
 
 // ---------------------------------------------------------------------------------------------
 // per-element work of the two sweeps
 // ---------------------------------------------------------------------------------------------
 // sweep 1: online-softmax update of one row with 32 more logits (raw dot products; c = log2(e)/sqrt(d))
+template <bool FMA_SHARE = false>
 __device__ __forceinline__ void stats_update(float (&v)[32], bool fast, int jb, int limit, float c, float &m,
                                              float &l)
 {
@@ -195,7 +198,7 @@ __device__ __forceinline__ void stats_update(float (&v)[32], bool fast, int jb, 
             a0 += fast_exp2(fmaf(v[x], c, -mc));
             a1 += fast_exp2(fmaf(v[x + 1], c, -mc));
             a2 += fast_exp2(fmaf(v[x + 2], c, -mc));
-            if (x % 8 == 0) add_exp2_fma(a3, fmaf(v[x + 3], c, -mc));
+            if (FMA_SHARE && x % 8 == 0) add_exp2_fma(a3, fmaf(v[x + 3], c, -mc));
             else a3 += fast_exp2(fmaf(v[x + 3], c, -mc));
         }
         const float add = (a0 + a1) + (a2 + a3);
@@ -204,7 +207,7 @@ __device__ __forceinline__ void stats_update(float (&v)[32], bool fast, int jb, 
     }
 }
 // sweep 2: adds exp2(x*c - lse2) of 32 (or 16) rows to the four partial sums of a key
-template <int N>
+template <int N, bool FMA_SHARE = false>
 __device__ __forceinline__ void score_accumulate(const float (&v)[N], const float *nl_base, float c, float &a0,
                                                  float &a1, float &a2, float &a3)
 {
@@ -214,7 +217,7 @@ __device__ __forceinline__ void score_accumulate(const float (&v)[N], const floa
         a0 += fast_exp2(fmaf(v[x], c, nl.x));
         a1 += fast_exp2(fmaf(v[x + 1], c, nl.y));
         a2 += fast_exp2(fmaf(v[x + 2], c, nl.z));
-        if (x % 8 == 0) add_exp2_fma(a3, fmaf(v[x + 3], c, nl.w));
+        if (FMA_SHARE && x % 8 == 0) add_exp2_fma(a3, fmaf(v[x + 3], c, nl.w));
         else a3 += fast_exp2(fmaf(v[x + 3], c, nl.w));
     }
 }

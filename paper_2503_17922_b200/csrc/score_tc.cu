@@ -170,7 +170,7 @@ struct StatsSweep {
     int limit;              // last key the thread's row may attend to
     int j_begin, j_plain;   // first key of the item; tiles that end before j_plain need no masking
 };
-template <int MB>
+template <int MB, bool FMA_SHARE>
 __device__ __forceinline__ float2 stats_sweep(GroupBarriers gb, StatsSweep w, uint32_t taddr, uint32_t it, int n_tiles, int grp, float c)
 {
     constexpr int NG = groups_for(MB);
@@ -188,7 +188,7 @@ __device__ __forceinline__ float2 stats_sweep(GroupBarriers gb, StatsSweep w, ui
             float x[32];
             tmem_ld32(taddr + sl * 32, x);
             if (sl + 1 == w.nslot) warp_release(tempty, lane);   // the buffer may be overwritten now
-            stats_update(x, fast, tile0 + w.col0 + sl * 32, w.limit, c, m, l);
+            stats_update<FMA_SHARE>(x, fast, tile0 + w.col0 + sl * 32, w.limit, c, m, l);
         }
     }
     return make_float2(m, l);
@@ -200,7 +200,7 @@ struct ScoreSweep {
     bool reuse;
     float *token_out;       // or null
 };
-template <int MB>
+template <int MB, bool FMA_SHARE>
 __device__ __forceinline__ void score_sweep(GroupBarriers gb, ScoreSweep w, uint32_t taddr, uint32_t it, int n_tiles, int grp, int L, float c)
 {
     constexpr int NG = groups_for(MB);
@@ -220,13 +220,13 @@ __device__ __forceinline__ void score_sweep(GroupBarriers gb, ScoreSweep w, uint
             float x[32];
             tmem_ld32(taddr + sl * 32, x);
             if (sl + 1 == n32 && !tail) warp_release(tempty, lane);   // the buffer may be overwritten now
-            score_accumulate<32>(x, neg_lse2 + sl * 32, c, a0, a1, a2, a3);
+            score_accumulate<32, FMA_SHARE>(x, neg_lse2 + sl * 32, c, a0, a1, a2, a3);
         }
         if (tail) {
             float x[16];
             tmem_ld16(taddr + n32 * 32, x);
             warp_release(tempty, lane);
-            score_accumulate<16>(x, neg_lse2 + n32 * 32, c, a0, a1, a2, a3);
+            score_accumulate<16, FMA_SHARE>(x, neg_lse2 + n32 * 32, c, a0, a1, a2, a3);
         }
         const float tj = (a0 + a1) + (a2 + a3);
         const int j = tile_at<stages_for(MB)>(w.reuse, n_tiles, (int)(v / MB - it)) * kTile + L;
@@ -519,7 +519,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         w.j_begin = im.j_begin;
         w.j_plain = min(im.n_r + 1, im.j_end);
         const uint32_t taddr = taddr_grp + w.col0;
-        sh.part[grp][L] = stats_sweep<MB>(gb, w, taddr, it, im.n_tiles, grp, c);
+        sh.part[grp][L] = stats_sweep<MB, ONE>(gb, w, taddr, it, im.n_tiles, grp, c);
     };
 
     // kMergers neighbouring threads share an observation row when partial statistics are merged, within the block and
@@ -560,7 +560,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         w.n_keys = im.j_end - im.j_begin;
         w.reuse = im.reuse;
         w.token_out = MB == 1 && a.token_scores ? a.token_scores + (size_t)im.unit * s.nr_max + im.j_begin : nullptr;
-        score_sweep<MB>(gb, w, taddr_grp, it, im.n_tiles, grp, L, c);
+        score_sweep<MB, ONE>(gb, w, taddr_grp, it, im.n_tiles, grp, L, c);
     };
 
     auto block_barrier = [&]() {
