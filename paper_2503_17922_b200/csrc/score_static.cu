@@ -64,7 +64,7 @@ extern "C" int wkv_score_windows_static(const wkv_shape *s, const void *q_obs, c
         set_error_detail("q_obs / k_leader / window_scores is NULL");
         return WKV_ERR_NULL;
     }
-    Workspace ws = plan_workspace(ks, 0);            // cleared on every call: no room for other shapes' words
+    Workspace ws = plan_workspace(ks, 0);            // scoring alone uses no unit's words but in the form that clears them
     // window_scores is the caller's here, so the part of the workspace that would hold them is not needed
     if (ws.counted_off > (size_t)WKV_STATIC_SCRATCH_BYTES) {
         set_error_detail("this shape needs %zu bytes of scratch, the built-in area holds %zu: "
