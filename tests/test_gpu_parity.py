@@ -868,7 +868,7 @@ def _expected_selection(scores, k):
     return np.sort(np.lexsort((np.arange(len(scores)), -scores))[:k])
 
 
-@pytest.mark.parametrize("n_windows", [1, 64, 65, 576, 577, 2304, 2305, 4608, 4609])
+@pytest.mark.parametrize("n_windows", [1, 64, 65, 576, 577, 2304, 2305, 4608, 4609, 9216, 9217])
 @pytest.mark.parametrize("keys", ["normal", "one-takes-all", "equal"])
 def test_fused_selection_is_exact_on_its_own_scores(n_windows, keys):
     """The selection inside the score kernel against a sort of the scores that the same call returns, on both sides of its
