@@ -735,25 +735,26 @@ static cudaError_t launch_fused_tile(const KShape &ks, const void *q, const void
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     {
-        // clusters that are resident at once: a property of device, kernel and shared-memory size, asked for once each
+        // clusters that are resident at once: a property of device, kernel and shared-memory size, asked for once each.
+        // None where a block is refused that much shared memory: with long rows the two kernels need 1.3 to 2.6 KB less
+        // than this one (head dimension 288 with 65-128 rows: 225.25 and 227.75 KB of the 227 there are).
         static std::mutex mu;
         static size_t allowed[kMaxDevices] = {};
         static size_t asked[kMaxDevices][4] = {};
         static int resident[kMaxDevices][4] = {};
         if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
         std::lock_guard<std::mutex> lock(mu);
-        if (smem > 48u * 1024u && smem > allowed[dev]) {
-            err = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (err != cudaSuccess) return err;
-            allowed[dev] = smem;
-        }
         int slot = 0;
         while (slot < 4 && asked[dev][slot] != smem && asked[dev][slot] != 0) ++slot;
         int fits = slot < 4 ? resident[dev][slot] : 0;
         if (slot == 4 || asked[dev][slot] == 0) {
-            err = cudaOccupancyMaxActiveClusters(&fits, fn, &cfg);
+            if (smem > 48u * 1024u && smem > allowed[dev]) {
+                err = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (err == cudaSuccess) allowed[dev] = smem;
+            }
+            if (err == cudaSuccess) err = cudaOccupancyMaxActiveClusters(&fits, fn, &cfg);
             if (err != cudaSuccess) {
-                (void)cudaGetLastError();      // a device without such clusters: the two kernels
+                (void)cudaGetLastError();      // too much shared memory, or a device without such clusters: the two kernels
                 fits = 0;
             }
             if (slot < 4) {

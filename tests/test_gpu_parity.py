@@ -939,3 +939,30 @@ def test_cuda_core_path_in_one_launch_and_in_two(dtype, rows, window, n, batch):
         pu.check_selection(w, grp, {"prob": prob, "window_scores": out["window_scores"].cpu().numpy(),
                                     "window_idx": out["window_idx"].cpu().numpy(),
                                     "kept_len": out["kept_len"].cpu().numpy()}, ref)
+
+
+def _select_leader(w, grp, prob, lse_obs=None):
+    """Runs score, pooling and selection of the leader; returns the outputs on the host."""
+    work, out = prob.alloc_workspace(), prob.alloc_outputs(0)
+    binding.wkv_select_leader_windows(prob, binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0]),
+                                      out["window_scores"], out["window_idx"], out["kept_len"], work,
+                                      lse_obs=None if lse_obs is None else torch.from_numpy(lse_obs).cuda())
+    assert binding.device_status(work) == 0
+    return {"prob": prob, "window_scores": out["window_scores"].cpu().numpy(),
+            "window_idx": out["window_idx"].cpu().numpy(), "kept_len": out["kept_len"].cpu().numpy()}
+
+
+@pytest.mark.parametrize("dtype,rows,head_dim,launches", [
+    ("f32", 16, 680, 1), ("f32", 16, 684, 2), ("f32", 32, 568, 1), ("f32", 32, 572, 2), ("f32", 128, 284, 1),
+    ("f32", 128, 288, 2), ("bf16", 128, 280, 1), ("bf16", 96, 288, 2)])
+def test_cuda_core_path_with_rows_too_long_for_one_launch(dtype, rows, head_dim, launches):
+    """The kernel that does everything in one launch needs up to 2.6 KB of shared memory more than the two: the longest rows
+    that the two take go to the two."""
+    w = small(dtype=dtype, head_dim=head_dim, n_kv_heads=1, n_q_heads=rows // 8, l_obs=8, batch=1, max_seqlen=600,
+              n_layers=1, gamma=1, n_planted=0)
+    grp = wl.make_group(w, 0)
+    ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
+    before = binding.wkv_launch_count()
+    got = _select_leader(w, grp, binding.Problem.from_workload(w, score_impl=IMPLS["simt"]))
+    assert binding.wkv_launch_count() - before == launches
+    pu.check_selection(w, grp, got, ref)
