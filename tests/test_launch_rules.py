@@ -1,0 +1,78 @@
+"""Which kernels a call on the CUDA-core path launches, and what becomes of a launch that the CUDA runtime refuses.
+
+The library's own launch code is built over a stand-in for the runtime (fake_cuda_runtime.cu) that records the launches
+and refuses what a case says; nothing runs on a GPU."""
+import ctypes
+import itertools
+import os
+import subprocess
+
+import pytest
+
+from paper_2503_17922_b200 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+SMEM = 227 * 1024                   # what a block may have; a kernel's static words come off the dynamic ones
+TOO_LARGE, ILLEGAL = 720, 700       # cudaErrorCooperativeLaunchTooLarge, cudaErrorIllegalAddress
+ONE, TWO = "score_fused_simt", "score_stats_simt score_pool_simt"
+_device = itertools.count()         # what the library has asked of one device it does not ask again
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    nvcc = build._nvcc()
+    try:
+        subprocess.check_output([nvcc, "--version"])
+    except OSError:
+        pytest.skip("no nvcc")
+    so = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    # (PTX alone: the device code is never loaded.  The stand-in's functions, not those of a runtime that the process has.)
+    subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=compute_100a", "-O0", "-Xcicc", "-O0", "-std=c++17",
+                           "-Xcompiler", "-fPIC", "-shared", "-cudart", "none", "-Xlinker", "-Bsymbolic", "-I", os.path.join(build.ROOT, "include"),
+                           "-I", build.CSRC, "-o", so, os.path.join(build.CSRC, "score_simt.cu"),
+                           os.path.join(HERE, "fake_cuda_runtime.cu")])
+    lib = ctypes.CDLL(so)
+
+    def select(rows=16, head_dim=64, n=600, window=8, f32=True, clusters=16, cooperative_error=0, smem=SMEM - 16, device=None):
+        log, pending = ctypes.create_string_buffer(256), ctypes.c_int(0)
+        err = lib.fake_select(ctypes.c_int(next(_device) if device is None else device), ctypes.c_size_t(smem), clusters,
+                              cooperative_error, int(f32), rows, head_dim, n, window, log, ctypes.c_size_t(256),
+                              ctypes.byref(pending))
+        return err, log.value.decode(), pending.value
+    return select
+
+
+@pytest.mark.parametrize("case,kernels", [
+    (dict(), ONE),
+    (dict(clusters=1), TWO),                                   # 600 keys are two clusters
+    (dict(clusters=2), ONE),
+    (dict(window=12), TWO),                                    # windows straddle tiles
+    (dict(rows=129), TWO),
+    (dict(rows=128, head_dim=284), ONE),
+    (dict(rows=128, head_dim=288), TWO),                       # only the two kernels fit shared memory
+    (dict(rows=16, head_dim=684), TWO),
+    (dict(n=16 + 8 * 2048, clusters=0), TWO),
+    (dict(n=16 + 8 * 2049, clusters=0), TWO + " select_topk"),
+])
+def test_one_launch_or_two(fake, case, kernels):
+    assert fake(**case) == (0, kernels, 0)
+
+
+@pytest.mark.parametrize("f32", [True, False])
+@pytest.mark.parametrize("rows", [16, 32, 64, 128])
+def test_a_cooperative_launch_that_is_refused_is_served_by_the_two_kernels(fake, rows, f32):
+    """The query may answer for more SMs than the context has: then the launch is refused, and the two kernels, none of whose
+    blocks waits for another, take the call.  The refusal is not left behind for the next call to report."""
+    assert fake(rows=rows, f32=f32, cooperative_error=TOO_LARGE) == (0, TWO, 0)
+
+
+def test_other_launch_errors_reach_the_caller(fake):
+    err, kernels, _ = fake(cooperative_error=ILLEGAL)
+    assert err == ILLEGAL and kernels == ""
+
+
+def test_a_size_that_does_not_fit_is_remembered(fake):
+    device = next(_device)
+    for _ in range(2):
+        assert fake(rows=128, head_dim=288, device=device) == (0, TWO, 0)
+        assert fake(rows=128, head_dim=64, device=device) == (0, ONE, 0)
