@@ -966,3 +966,22 @@ def test_cuda_core_path_with_rows_too_long_for_one_launch(dtype, rows, head_dim,
     got = _select_leader(w, grp, binding.Problem.from_workload(w, score_impl=IMPLS["simt"]))
     assert binding.wkv_launch_count() - before == launches
     pu.check_selection(w, grp, got, ref)
+
+
+@pytest.mark.parametrize("impl", ["simt", "tc"])
+@pytest.mark.parametrize("rows", [16, 128, 256])
+def test_weights_below_the_smallest_normal_number_add_nothing(rows, impl):
+    """Review keys 320 nats below the observation keys, for every row: their softmax weights are zero in fp32, so are the
+    token scores, whatever computes the exponentials."""
+    w = small(head_dim=64, n_kv_heads=1, n_q_heads=rows // 8, l_obs=8, batch=1, max_seqlen=700, n_layers=1, gamma=1, n_planted=0)
+    sign = torch.where(torch.rand(64, generator=torch.Generator().manual_seed(rows)) < 0.5, -1.0, 1.0)
+    q = (2.0 * sign).expand(1, rows // 8, 8, 64).to(torch.bfloat16).cuda().contiguous()
+    k = (-20.0 * sign).repeat(1, 1, 700, 1)
+    k[:, :, -8:] = 0.0                                        # logits: 64 * 2 * -20 / 8 = -320, and 0
+    prob = binding.Problem.from_workload(w, score_impl=IMPLS[impl])
+    scores = torch.full((1, 1, prob.kw_max), -1.0, dtype=torch.float32, device="cuda")
+    tokens = torch.full((1, 1, prob.nr_max), -1.0, dtype=torch.float32, device="cuda")
+    work = prob.alloc_workspace()
+    binding.wkv_score_windows(prob, q, k.to(torch.bfloat16).cuda(), scores, tokens, work)
+    assert binding.device_status(work) == 0
+    assert float(tokens.abs().max()) == 0.0 and float(scores.abs().max()) == 0.0
