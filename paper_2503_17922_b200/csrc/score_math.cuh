@@ -146,12 +146,15 @@ struct PublishedScores {
     }
 };
 
-// acc + 2^x for x <= 0 on the FMA pipe: 2^x = 2^t * 2^f with t the nearest integer, and 2^f by a polynomial of degree six
+// acc + 2^x on the FMA pipe: 2^x = 2^t * 2^f with t the nearest integer, and 2^f by a polynomial of degree six
 // (a Remez fit of the relative error on [-1/2, 1/2]).  With its coefficients in fp32 it is off by 1.6e-8 at most, evaluated in
-// fp32 by 7.9e-8.  From t = -127 on the power of two is zero, so that below -126.5 nothing is added; a NaN stays one.
+// fp32 by 7.9e-8.  From t = -127 on the power of two is zero, so that below -126.5 nothing is added, and at t = 128 it is infinite, so that beyond
+// 127.5 the result is; a NaN stays one.  AT_MOST_ZERO: x is not above zero (but for its rounding).
+template <bool AT_MOST_ZERO>
 __device__ __forceinline__ void add_exp2_fma(float &acc, float x)
 {
     asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x));      // -127
+    if (!AT_MOST_ZERO) asm("min.NaN.f32 %0, %0, 0f43000000;" : "+f"(x));      // 128
     const float shifted = x + 12582912.f;                  // 1.5 * 2^23: the integer is in the low bits
     const float f = x - (shifted - 12582912.f);
     float p = 1.5345812e-4f;
@@ -198,7 +201,7 @@ __device__ __forceinline__ void stats_update(float (&v)[32], bool fast, int jb, 
             a0 += fast_exp2(fmaf(v[x], c, -mc));
             a1 += fast_exp2(fmaf(v[x + 1], c, -mc));
             a2 += fast_exp2(fmaf(v[x + 2], c, -mc));
-            if (FMA_SHARE && x % 8 == 0) add_exp2_fma(a3, fmaf(v[x + 3], c, -mc));
+            if (FMA_SHARE && x % 8 == 0) add_exp2_fma<true>(a3, fmaf(v[x + 3], c, -mc));
             else a3 += fast_exp2(fmaf(v[x + 3], c, -mc));
         }
         const float add = (a0 + a1) + (a2 + a3);
@@ -217,7 +220,7 @@ __device__ __forceinline__ void score_accumulate(const float (&v)[N], const floa
         a0 += fast_exp2(fmaf(v[x], c, nl.x));
         a1 += fast_exp2(fmaf(v[x + 1], c, nl.y));
         a2 += fast_exp2(fmaf(v[x + 2], c, nl.z));
-        if (FMA_SHARE && x % 8 == 0) add_exp2_fma(a3, fmaf(v[x + 3], c, nl.w));
+        if (FMA_SHARE && x % 8 == 0) add_exp2_fma<false>(a3, fmaf(v[x + 3], c, nl.w));   // (a caller's normaliser may be too low)
         else a3 += fast_exp2(fmaf(v[x + 3], c, nl.w));
     }
 }

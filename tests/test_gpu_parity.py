@@ -985,3 +985,33 @@ def test_weights_below_the_smallest_normal_number_add_nothing(rows, impl):
     binding.wkv_score_windows(prob, q, k.to(torch.bfloat16).cuda(), scores, tokens, work)
     assert binding.device_status(work) == 0
     assert float(tokens.abs().max()) == 0.0 and float(scores.abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("impl", ["simt", "tc"])
+@pytest.mark.parametrize("row", [2, 3])
+@pytest.mark.parametrize("low", [60.0, 86.0, 150.0])
+def test_given_normalisers_that_are_too_low(low, row, impl):
+    """One observation row's normaliser is too low by so many nats: its weights are too high by that factor, and infinite where
+    fp32 does not hold them; the other KV head is as it was.  (Token scores within 1e-4: the exponent is rounded at 2^-17.)"""
+    w = small(head_dim=64, n_kv_heads=2, n_q_heads=8, l_obs=8, batch=1, max_seqlen=700, n_layers=1, gamma=1, n_planted=0)
+    grp = wl.make_group(w, 0)
+    lse = pu.lse_obs_reference(w, grp)
+    lse[0, 4, row] -= low                                     # first query head of KV head 1
+    q, k = (wl.to_f32(x).astype(np.float64) for x in (grp["q_obs"], grp["k_layers"][0]))
+    n_r = w.max_seqlen - w.l_obs
+    expected = np.zeros((2, n_r))
+    for hq in range(8):
+        expected[hq // 4] += np.exp(q[0, hq] @ k[0, hq // 4, :n_r].T / 8.0 - lse[0, hq].astype(np.float64)[:, None]).sum(0)
+    prob = binding.Problem.from_workload(w, score_impl=IMPLS[impl])
+    scores = torch.zeros((1, 2, prob.kw_max), dtype=torch.float32, device="cuda")
+    tokens = torch.zeros((1, 2, prob.nr_max), dtype=torch.float32, device="cuda")
+    work = prob.alloc_workspace()
+    binding.wkv_score_windows_lse(prob, binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0]),
+                                  torch.from_numpy(lse).cuda(), scores, tokens, work)
+    assert binding.device_status(work) == 0
+    got = tokens[0, :, :n_r].cpu().numpy().astype(np.float64)
+    top = float(np.finfo(np.float32).max)
+    held, beyond = expected < top / 4, expected > top * 4
+    assert held[0].all() and (low > 100 or held.all()) and (low < 100 or beyond[1].all())
+    np.testing.assert_allclose(got[held], expected[held], rtol=1e-4)
+    assert np.isposinf(got[beyond]).all()
