@@ -431,6 +431,19 @@ int wkv_probe_ex2_rate(float *scratch_dev, int32_t blocks, int32_t threads, int3
 int wkv_probe_colsum_rate(float *scratch_dev, int32_t blocks, int32_t threads, int32_t iters,
                           int64_t *elements_per_launch, void *cuda_stream);
 
+/*
+ * Test aid (no counterpart in the paper): the selection that the score kernels run on scores which other blocks
+ * publish, by one block, on words that the caller has written.  A published word is 16 bytes: a score (float) in the
+ * low half of the first eight, a tag in the second eight; a word whose tag is not `tag` is missing, and is waited for, two
+ * seconds at most.
+ *   words_dev       DEVICE  in,  n_words words, 16-byte aligned
+ *   window_idx_dev  DEVICE  out, int32 [k]: the k <= n_words highest, ascending; after an expired wait whatever the block has
+ *                   written, which is nothing where the list is longer than the block keeps in registers (4,096 words)
+ *   status_dev      DEVICE  int32, OR-ed with 1 if the wait expired
+ */
+int wkv_probe_published_select(const void *words_dev, int32_t n_words, uint64_t tag, int32_t k, int32_t *window_idx_dev,
+                               int32_t *status_dev, void *cuda_stream);
+
 const char *wkv_status_string(int status);
 const char *wkv_last_error_detail(void);
 /* Number of kernels the library has launched from this process (all threads). */

@@ -1,8 +1,10 @@
-// Measurement aid (no counterpart in the paper): the rate at which this GPU evaluates
+// Measurement and test aids (no counterpart in the paper).  First the rate at which this GPU evaluates
 // ex2.approx.ftz.f32, the instruction both sweeps of the score kernels spend most of their issue
 // slots on.  The benchmark times this kernel with CUDA events and uses the measured rate, instead of
 // an assumed one, as the special-function floor of the score stage.
+#include "score_math.cuh"
 #include "tc_common.cuh"
+#include "topk_block.cuh"
 #include "wkv_internal.cuh"
 
 namespace wkv {
@@ -60,8 +62,46 @@ colsum_rate_kernel(float *out, int iters, float seed)
     if (keep == 123.456f) out[0] = keep;
 }
 
+// The score kernels' selection from published words, by one block on words that the caller has written: with all of them
+// there it must select, with one missing its wait must end by itself.
+constexpr int kSelectThreads = 256;
+__global__ void __launch_bounds__(kSelectThreads)
+published_select_kernel(const StatEntry *words, int n_words, unsigned long long tag, int k, int *window_idx, int *status)
+{
+    __shared__ TopkSmem sm;
+    __shared__ int abort_s, kept;
+    if (threadIdx.x == 0) abort_s = 0;
+    __syncthreads();
+    select_topk_block<kSelectThreads>((int)threadIdx.x, sm, PublishedScores<4>{words, tag, &abort_s, -1}, n_words, k, k, window_idx,
+                                      &kept, n_words + 1, 1, 1);
+    __syncthreads();
+    if (threadIdx.x == 0 && abort_s) atomicOr(status, kStatusWaitExpired);
+}
+
 }  // namespace
 }  // namespace wkv
+
+extern "C" int wkv_probe_published_select(const void *words_dev, int32_t n_words, uint64_t tag, int32_t k, int32_t *window_idx_dev,
+                                          int32_t *status_dev, void *cuda_stream)
+{
+    using namespace wkv;
+    if (!words_dev || !window_idx_dev || !status_dev) {
+        set_error_detail("words_dev / window_idx_dev / status_dev is NULL");
+        return WKV_ERR_NULL;
+    }
+    if (reinterpret_cast<uintptr_t>(words_dev) & 15u) {
+        set_error_detail("words_dev is not 16-byte aligned");
+        return WKV_ERR_ALIGN;
+    }
+    if (n_words < 1 || k < 1 || k > n_words) {
+        set_error_detail("probe shape: %d words, %d selected", n_words, k);
+        return WKV_ERR_SHAPE;
+    }
+    published_select_kernel<<<1, kSelectThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+        static_cast<const StatEntry *>(words_dev), n_words, tag, k, window_idx_dev, status_dev);
+    count_launches(1);
+    return check_cuda(cudaGetLastError(), "selection probe kernel");
+}
 
 extern "C" int wkv_probe_colsum_rate(float *scratch_dev, int32_t blocks, int32_t threads, int32_t iters,
                                      int64_t *elements_per_launch, void *cuda_stream)

@@ -117,6 +117,7 @@ __device__ __forceinline__ void count_launch(LaunchCount *c, unsigned long long 
 // The selection reads the published window scores, waiting for those that are still to come: LOOK words at a time.
 template <int LOOK>
 struct PublishedScores {
+    static constexpr bool kWaits = true;
     const StatEntry *entries;
     unsigned long long tag;
     volatile int *abort_flag;
@@ -140,6 +141,8 @@ struct PublishedScores {
         unsigned unused[LOOK];
         for (int w = lo; w < hi; w += LOOK) keys(unused, w, min(hi, w + LOOK));
     }
+    // behind a barrier of all that wait
+    __device__ __forceinline__ bool gave_up() const { return *abort_flag != 0; }
     __device__ __forceinline__ unsigned key(int w) const
     {
         return topk_order_key(__ldcg(reinterpret_cast<const float *>(&entries[w].value)));

@@ -89,6 +89,7 @@ __device__ __forceinline__ int topk_hint(int rows, int n)
 // window scores in memory, read through L2: those written by other blocks of the same grid are seen once the caller
 // has synchronised with them
 struct WrittenScores {
+    static constexpr bool kWaits = false;
     const float *scores;
     int hint;            // topk_hint(), or negative: nothing is known about the scores' range
     template <int N>
@@ -98,6 +99,7 @@ struct WrittenScores {
         for (int e = 0; e < N; ++e) key[e] = lo + e < hi ? topk_order_key(__ldcg(scores + lo + e)) : 0u;
     }
     __device__ __forceinline__ void wait(int, int) const {}
+    __device__ __forceinline__ bool gave_up() const { return false; }
     __device__ __forceinline__ unsigned key(int w) const { return topk_order_key(__ldcg(scores + w)); }
 };
 
@@ -140,8 +142,8 @@ __device__ __forceinline__ void topk_find_bin(int tid, TopkSmem &sm, int remaini
 }
 
 // All NT threads of the block call this.  `src.keys(key, lo, hi)` gives the order keys of the unit's windows lo .. hi - 1 (at
-// most as many as `key` holds) once they are there; for longer lists `src.wait(lo, hi)` waits for them and `src.key(w)`
-// reads one. `out` receives k ascending indices followed by -1 up to k_max.
+// most as many as `key` holds) once they are there; for longer lists `src.wait(lo, hi)` waits for them, `src.gave_up()` tells
+// whether a wait of the block's has expired (kWaits: one may) and `src.key(w)` reads one. `out` receives k ascending indices followed by -1 up to k_max.
 // Thread t owns the windows [t*E, (t+1)*E), E = ceil(kw / NT).  With E <= REGS (4, 8 or 16) the keys
 // are read once and stay in registers through the radix passes and the compaction (one trip to L2
 // instead of several); REGS = 0: longer lists are re-read.
@@ -162,7 +164,15 @@ __device__ __forceinline__ void select_topk_impl(int tid, TopkSmem &sm, const Sr
     constexpr int kTopkRegs = IN_REGS ? REGS : 1;
     unsigned keys[kTopkRegs];
     if (IN_REGS) src.keys(keys, w_lo, w_hi);
-    else src.wait(w_lo, w_hi);
+    else {
+        src.wait(w_lo, w_hi);
+        // What is still missing after a wait that expired may come while the passes below read the list, and they write by
+        // counts that hold for an unchanged list alone: no selection then.
+        if (Src::kWaits) {
+            topk_sync<NT, BAR>();
+            if (src.gave_up()) return;
+        }
+    }
     auto key_at = [&](int e) -> unsigned { return IN_REGS ? keys[e] : src.key(w_lo + e); };
     // runs f(e, key) over the thread's own keys
     auto for_own = [&](auto f) {

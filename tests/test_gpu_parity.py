@@ -1015,3 +1015,29 @@ def test_given_normalisers_that_are_too_low(low, row, impl):
     assert held[0].all() and (low > 100 or held.all()) and (low < 100 or beyond[1].all())
     np.testing.assert_allclose(got[held], expected[held], rtol=1e-4)
     assert np.isposinf(got[beyond]).all()
+
+
+@pytest.mark.parametrize("n_words,k", [(1, 1), (700, 60), (4096, 500), (4097, 500), (9000, 8999)])
+@pytest.mark.parametrize("missing", [False, True])
+def test_selection_from_published_words_that_do_not_all_come(n_words, k, missing):
+    """The words that blocks hand one another are waited for within bounds: with one that is never published the block gives
+    up after two seconds, its status bit is set, nothing is written outside the output, and the next call is none the
+    worse.  A list that is read several times is not selected from then: its missing words might still come meanwhile."""
+    tag = 0xffb5000000000007
+    scores = np.random.default_rng(n_words).standard_normal(n_words).astype(np.float32)
+    words = np.zeros((n_words, 2), dtype=np.uint64)
+    words[:, 0] = scores.view(np.uint32)
+    words[:, 1] = tag
+    if missing:
+        words[n_words // 2, 1] -= np.uint64(1)                   # the launch before
+    idx = torch.full((k + 128,), -7, dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    binding.wkv_probe_published_select(torch.from_numpy(words.view(np.int64)).cuda(), tag, idx[64:64 + k], status)
+    torch.cuda.synchronize()
+    got = idx.cpu().numpy()
+    assert (got[:64] == -7).all() and (got[64 + k:] == -7).all()
+    assert int(status) == int(missing)
+    if not missing:
+        np.testing.assert_array_equal(got[64:64 + k], _expected_selection(scores, k))
+    elif n_words > 4096:
+        assert (got == -7).all()
