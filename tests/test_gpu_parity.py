@@ -171,9 +171,11 @@ def test_layer_by_layer_use_equals_the_group_call(given_lse, impl):
         np.testing.assert_array_equal(binding.to_host_bits(out["v_out"][l]), ref["v_out"][l])
 
 
-def test_group_plan_replays_the_group_call():
-    """A recorded group must give what the direct call gives, on whatever the buffers hold at launch."""
-    w = small(task=wl.TASK_AGGREGATION, top_p=31, window=32, l_obs=32)
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_group_plan_replays_the_group_call(dtype):
+    """A recorded group must give what the direct call gives, on whatever the buffers hold at launch: the tensor-core
+    kernel, and in fp32 the CUDA-core form of one launch (a cooperative launch of clusters)."""
+    w = small(dtype=dtype, task=wl.TASK_AGGREGATION, top_p=31, window=32, l_obs=32)
     prob = binding.Problem.from_workload(w)
     grps = [wl.make_group(w, 0), wl.make_group(wl.scaled(w, config_id=10), 0)]
     q = binding.to_device(grps[0]["q_obs"])
@@ -192,7 +194,7 @@ def test_group_plan_replays_the_group_call():
         before = binding.wkv_launch_count()
         plan.launch()
         torch.cuda.synchronize()
-        assert binding.wkv_launch_count() - before >= 2
+        assert binding.wkv_launch_count() - before == 2            # scores with selection, and the gather
         assert binding.device_status(work) == 0
         ref = pu.run_gpu_group(w, grp)
         np.testing.assert_array_equal(out["window_idx"].cpu().numpy(), ref["window_idx"])
@@ -306,13 +308,25 @@ def test_more_work_items_than_blocks():
 
 
 def test_long_window_list_is_reread_by_the_selection():
-    # 10,000 windows per unit: more than 8 per thread of the selecting block, which then streams
-    # the scores from L2 in every radix pass instead of holding them in registers
-    w = small(batch=1, n_q_heads=4, n_kv_heads=2, head_dim=64, max_seqlen=40008, l_obs=8, window=4,
+    # 16,400 windows per unit: more than the 16 per thread that the selecting block holds in registers (9,216 in
+    # the tensor-core kernel, 16,384 in the selection kernel behind the CUDA-core ones); it then streams the scores from L2 in
+    # every pass
+    w = small(batch=1, n_q_heads=4, n_kv_heads=2, head_dim=64, max_seqlen=65608, l_obs=8, window=4,
               budget_frac=0.1, n_planted=20, n_layers=1, gamma=1)
     for impl in ("tc", "simt"):
         grp, ref, gpu, (max_rel, swaps) = pu.full_check(w, score_impl=IMPLS[impl])
-        assert gpu["prob"].kw_max == 10000 and max_rel < 1e-4
+        assert gpu["prob"].kw_max == 16400 and max_rel < 1e-4
+
+
+def test_long_window_list_of_the_one_launch_form_is_reread():
+    # the CUDA-core form of one launch holds 4,096 windows per unit in registers: 4,097 of two tokens, and 8,000 of one
+    for window, n_windows in ((2, 4097), (1, 8000)):
+        w = small(dtype="f32", batch=1, n_q_heads=2, n_kv_heads=1, head_dim=64, max_seqlen=8 + window * n_windows, l_obs=8, window=window,
+                  budget_frac=0.1, n_planted=0, n_layers=1, gamma=1)
+        before = binding.wkv_launch_count()
+        grp, ref, gpu, (max_rel, swaps) = pu.full_check(w, score_impl=IMPLS["simt"])
+        assert binding.wkv_launch_count() - before == 2            # and the gather
+        assert gpu["prob"].kw_max == n_windows and max_rel < 1e-4
 
 
 def test_one_workspace_serves_different_problems_in_turn():
@@ -350,9 +364,11 @@ def test_same_result_twice_and_across_entry_points():
 
 
 # ------------------------------------------------------------------ selection, exact
-@pytest.mark.parametrize("kw_n,budget", [(40, 100), (127, 128), (1020, 983), (5000, 2048), (9000, 40000), (1, 64)])
+@pytest.mark.parametrize("kw_n,budget", [(40, 100), (127, 128), (1020, 983), (4097, 9000), (5000, 2048), (9000, 40000), (1, 64),
+                                         (16384, 9000), (16385, 9000), (40000, 200000)])
 def test_selection_bit_exact_on_given_scores(kw_n, budget):
-    # feed the same fp32 scores to both sides: indices must agree exactly, including ties
+    # feed the same fp32 scores to both sides: indices must agree exactly, including ties; up to 4, 8 and 16 windows
+    # per thread in registers (4,096, 8,192, 16,384 in all) and longer lists, which are read again in every pass
     alpha, omega = 8, 8
     n = alpha + kw_n * omega - 3            # ragged last window
     B, H = 2, 3
@@ -651,23 +667,30 @@ def test_host_buffer_entry_point_keeps_the_staged_inputs(budget_frac):
     pu.check_gather(w, grp, got)
 
 
+@pytest.mark.parametrize("form", ["one launch", "given normalisers", "two kernels"])
 @pytest.mark.parametrize("n_windows", [1, 15, 17, 2048, 2049])
-def test_selection_inside_and_behind_the_cuda_core_score_kernel(n_windows):
-    """Up to 2,048 windows per unit are selected by the score kernel's last block of the unit, more by the kernel of its
+def test_selection_inside_and_behind_the_cuda_core_score_kernel(n_windows, form):
+    """Where statistics, scores and selection are not one launch (the caller gives the normalisers, or windows straddle
+    tiles), up to 2,048 windows per unit are selected by the score kernel's last block of the unit, more by the kernel of its
     own; twice on one workspace, whose ticket words clear themselves."""
-    w = small(dtype="f32", head_dim=64, n_q_heads=4, l_obs=8, window=4, n_planted=0, budget_frac=0.25, batch=1,
-              max_seqlen=8 + 4 * n_windows - (1 if n_windows > 1 else 0))
+    window = 12 if form == "two kernels" else 4
+    w = small(dtype="f32", head_dim=64, n_q_heads=4, l_obs=8, window=window, n_planted=0, budget_frac=0.25, batch=1,
+              max_seqlen=8 + window * n_windows - (1 if n_windows > 1 else 0))
     grp = wl.make_group(w, 0)
     ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], **pu.oracle_kwargs(w, grp))
+    lse = torch.from_numpy(pu.lse_obs_reference(w, grp)).cuda() if form == "given normalisers" else None
     prob = binding.Problem.from_workload(w)
     assert prob.kw_max == n_windows
     q, k = binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0])
     work, out = prob.alloc_workspace(), prob.alloc_outputs(0)
+    launches = 1 if form == "one launch" else (1 if lse is not None else 2) + (1 if n_windows > 2048 else 0)
     for _ in range(2):
         out["window_idx"].fill_(-7)
         out["kept_len"].fill_(-7)
-        binding.wkv_select_leader_windows(prob, q, k, out["window_scores"], out["window_idx"], out["kept_len"], work)
+        before = binding.wkv_launch_count()
+        binding.wkv_select_leader_windows(prob, q, k, out["window_scores"], out["window_idx"], out["kept_len"], work, lse_obs=lse)
         torch.cuda.synchronize()
+        assert binding.wkv_launch_count() - before == launches
         assert binding.device_status(work) == 0
         got = {"prob": prob, "window_scores": out["window_scores"].cpu().numpy(),
                "window_idx": out["window_idx"].cpu().numpy(), "kept_len": out["kept_len"].cpu().numpy()}
@@ -920,11 +943,13 @@ def test_a_sequence_with_more_chunks_than_blocks():
 @pytest.mark.parametrize("rows,window,n,batch", [
     (16, 8, 64, 1), (16, 4, 65, 2), (17, 16, 512, 1), (32, 64, 513, 2), (33, 32, 577, 1), (64, 2, 1024 + 8, 1), (64, 1, 200, 1),
     (65, 16, 1100, 3), (128, 8, 1031, 2), (129, 8, 700, 1), (16, 48, 700, 1), (16, 8, 9, 1), (16, 8, 72, 1),
-    (16, 16, 3000, 20), (16, 16, 3000, 40)])
+    (16, 16, 3000, 20), (16, 16, 3000, 40),
+    (16, 12, 9, 1), (16, 3, 65, 2), (17, 5, 129, 1), (32, 24, 513, 2), (33, 100, 577, 1), (64, 3, 200, 1), (64, 96, 64 + 8, 3),
+    (65, 7, 1100, 1), (128, 12, 1031, 2), (256, 8, 300, 1)])
 def test_cuda_core_path_in_one_launch_and_in_two(dtype, rows, window, n, batch):
     """Statistics, scores and selection in one launch where its blocks of 64 keys are resident together: both sides of its
     limits (128 rows, windows that do not straddle tiles, clusters that fit), every row tile, first and last tiles with only
-    observation keys or one review key.  Twice on one workspace, with other inputs: nothing of the first call passes for the second's."""
+    observation keys or one review key, in both forms.  Twice on one workspace, with other inputs: nothing of the first call passes for the second's."""
     alpha = rows if rows % 8 else 8
     w = small(dtype=dtype, head_dim=64, n_kv_heads=2, n_q_heads=2 * rows // alpha, l_obs=alpha, window=window, batch=batch,
               max_seqlen=max(n, alpha + 1), n_layers=1, gamma=1, n_planted=0, budget_frac=0.4, top_p=max(1, window // 2))
@@ -1041,3 +1066,46 @@ def test_selection_from_published_words_that_do_not_all_come(n_words, k, missing
         np.testing.assert_array_equal(got[64:64 + k], _expected_selection(scores, k))
     elif n_words > 4096:
         assert (got == -7).all()
+
+
+@pytest.mark.parametrize("recorded", [False, True])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_two_streams_at_once(dtype, recorded):
+    """Two threads of an engine, each with a stream, a workspace and outputs of its own: launches whose blocks wait for one
+    another, each of more than half of the GPU, overlap or take turns, and give what they give alone."""
+    w = small(dtype=dtype, n_q_heads=16, n_kv_heads=4, max_seqlen=3900, l_obs=16, head_dim=64, n_planted=0)
+    grps = [wl.make_group(wl.scaled(w, config_id=c), 0) for c in (20, 21)]
+    alone = [pu.run_gpu_group(w, g) for g in grps]
+    if dtype == "f32":                       # 64 clusters of eight blocks in one launch
+        before = binding.wkv_launch_count()
+        _select_leader(w, grps[0], alone[0]["prob"])
+        assert binding.wkv_launch_count() - before == 1
+    sides = []
+    for grp in grps:
+        prob = binding.Problem.from_workload(w)
+        side = {"prob": prob, "q": binding.to_device(grp["q_obs"]), "k": [binding.to_device(x) for x in grp["k_layers"]],
+                "v": [binding.to_device(x) for x in grp["v_layers"]], "out": prob.alloc_outputs(w.gamma, fill_byte=pu.FILL_BYTE),
+                "work": prob.alloc_workspace(), "stream": torch.cuda.Stream()}
+        args = (side["q"], side["k"], side["v"], side["out"]["k_out"], side["out"]["v_out"], side["out"]["window_scores"],
+                side["out"]["window_idx"], side["out"]["kept_len"], side["work"])
+        if recorded:
+            plan = binding.GroupPlan(prob, *args, keep_capacity=side["out"]["keep_capacity"])
+            side["call"] = lambda plan=plan, st=side["stream"]: plan.launch(stream=st)
+        else:
+            side["call"] = lambda prob=prob, args=args, side=side: binding.wkv_compress_group(
+                prob, *args, keep_capacity=side["out"]["keep_capacity"], stream=side["stream"])
+        sides.append(side)
+    torch.cuda.synchronize()
+    for _ in range(10):
+        for _ in range(10):
+            for side in sides:
+                side["call"]()
+        torch.cuda.synchronize()
+        assert [binding.device_status(side["work"]) for side in sides] == [0, 0]
+    for side, ref in zip(sides, alone):
+        out = side["out"]
+        for name in ("window_scores", "window_idx", "kept_len"):
+            np.testing.assert_array_equal(out[name].cpu().numpy(), ref[name])
+        for l in range(w.gamma):
+            np.testing.assert_array_equal(binding.to_host_bits(out["k_out"][l]), ref["k_out"][l])
+            np.testing.assert_array_equal(binding.to_host_bits(out["v_out"][l]), ref["v_out"][l])
