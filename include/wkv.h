@@ -194,8 +194,9 @@ int wkv_score_windows(const wkv_shape *s, const void *q_obs, const void *k_leade
  * the scratch is a fixed area of twice WKV_STATIC_SCRATCH_BYTES inside the library image, which every
  * GPU that loads the library holds until the process exits.  The function allocates and frees
  * nothing.
- *   - Shapes whose wkv_workspace_bytes() exceeds WKV_STATIC_SCRATCH_BYTES are refused with
- *     WKV_ERR_LIMIT before anything is enqueued.
+ *   - Shapes that need more than WKV_STATIC_SCRATCH_BYTES, counted without window scores and with eight
+ *     bytes per row statistic, are refused with WKV_ERR_LIMIT before anything is enqueued.  (The macro is
+ *     this limit, half of what is held: some kernels' statistics take sixteen bytes.)
  *   - The first call on each device looks up the area's device address (with that device current);
  *     make that first call outside any stream capture.
  *   - All calls on a device share the one area: two calls whose kernels may overlap on the GPU
