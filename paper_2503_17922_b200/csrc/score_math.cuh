@@ -1,6 +1,6 @@
-// Device-side pieces shared by the tensor-core score kernels: the per-element work of the two sweeps
-// (Eq. 1's online statistics, Eq. 2's normalised sum), Eq. 4's pooling of one window, and the
-// acquire / release accesses and bounded polls of the hand-over between thread blocks.
+// Device-side pieces shared by the score kernels: the per-element work of the tensor-core kernels' two sweeps
+// (Eq. 1's online statistics, Eq. 2's normalised sum), Eq. 4's pooling of one window, and the hand-over between thread
+// blocks: published words, acquire / release accesses, bounded waits.
 #pragma once
 
 #include "tc_common.cuh"

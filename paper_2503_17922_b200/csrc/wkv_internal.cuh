@@ -78,15 +78,15 @@ __device__ inline SeqInfo seq_info(const KShape &s, int b)
 // Workspace carve-up (all offsets 256-byte aligned).
 struct Workspace {
     size_t status_off;   // int: device status word, only ever OR-ed by the kernels (0 = no error)
-    size_t count_off;    // LaunchCount of the tensor-core kernel, inside the status word's 64 bytes
+    size_t count_off;    // LaunchCount of the kernels that publish words, inside the status word's 64 bytes
     size_t sync_off;     // int [kSyncTickets + kSyncWordsPerUnit * units], self-resetting
     size_t pstats_off;   // u64 [units][n_stat_chunks][128]: self-validating (max, sum) entries of the pipelined kernel;
                          // zero between launches (the kernel that writes them clears them again)
-    size_t stats_off;    // partial (max, sum) per row: float2 [units][n_stat_chunks][R_pad], or the tensor-core kernel's
-                         // published words [units][chunks_per_unit][R_pad] of 16 bytes
+    size_t stats_off;    // partial (max, sum) per row: float2 [units][n_stat_chunks][R_pad], or published words of 16 bytes
+                         // [units][chunks][R_pad] (tensor-core kernel, CUDA-core form of one launch)
     size_t lse_off;      // float  [units][R_pad]                 log2 of the row normaliser
     size_t scores_off;   // float  [units][kw_max]                window scores when the caller passes none
-    size_t entries_off;  // published window scores [units][kw_max] of 16 bytes (tensor-core kernel with selection)
+    size_t entries_off;  // published window scores [units][kw_max] of 16 bytes (the same two, with selection)
     size_t total;
     size_t counted_off;  // scores_off as it would be with float2 statistics: what the built-in area admits shapes by
     unsigned salt;       // goes into the tags of published words (0 but for the built-in area)
@@ -95,8 +95,8 @@ struct Workspace {
 };
 
 // words of the synchronisation area before the per-unit words; unit u owns four words from
-// sync[kSyncTickets + 4u]: ticket count, arrivals of the statistics sweep, "selection published" flag
-// and gather job counter (the last two only in the kernel that also gathers)
+// sync[kSyncTickets + 4u]: ticket count, and in the pipelined kernel arrivals of the statistics sweep, "selection
+// published" flag and gather job counter
 constexpr int kSyncTickets = 16;
 constexpr int kSyncWordsPerUnit = 4;
 // The area has room for at least this many units whatever the shape (32 KB), so that what lies behind it never lands on
