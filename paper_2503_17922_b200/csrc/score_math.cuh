@@ -149,32 +149,76 @@ struct PublishedScores {
     }
 };
 
+// Two fp32 numbers in one register pair: the packed instructions round each half as the plain ones do and take one issue slot
+// for the two.
+__device__ __forceinline__ unsigned long long pair_of(float lo, float hi)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 halves_of(unsigned long long p)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma_pair(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ unsigned long long add_pair(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long exp2_pair(unsigned long long x)
+{
+    const float2 h = halves_of(x);
+    return pair_of(fast_exp2(h.x), fast_exp2(h.y));
+}
+
 // acc + 2^x on the FMA pipe: 2^x = 2^t * 2^f with t the nearest integer, and 2^f by a polynomial of degree six
 // (a Remez fit of the relative error on [-1/2, 1/2]).  With its coefficients in fp32 it is off by 1.6e-8 at most, evaluated in
 // fp32 by 7.9e-8.  From t = -127 on the power of two is zero, so that below -126.5 nothing is added, and at t = 128 it is infinite, so that beyond
 // 127.5 the result is; a NaN stays one.  AT_MOST_ZERO: x is not above zero (but for its rounding).
 template <bool AT_MOST_ZERO>
-__device__ __forceinline__ void add_exp2_fma(float &acc, float x)
+__device__ __forceinline__ void add_exp2_fma(unsigned long long &acc, unsigned long long x2)
 {
-    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x));      // -127
-    if (!AT_MOST_ZERO) asm("min.NaN.f32 %0, %0, 0f43000000;" : "+f"(x));      // 128
-    const float shifted = x + 12582912.f;                  // 1.5 * 2^23: the integer is in the low bits
-    const float f = x - (shifted - 12582912.f);
-    float p = 1.5345812e-4f;
-    p = fmaf(p, f, 1.3399931e-3f);
-    p = fmaf(p, f, 9.618489e-3f);
-    p = fmaf(p, f, 5.5503286e-2f);
-    p = fmaf(p, f, 2.4022646e-1f);
-    p = fmaf(p, f, 6.931472e-1f);
-    p = fmaf(p, f, 1.f);
-    acc = fmaf(p, __int_as_float((__float_as_int(shifted) << 23) + 0x3f800000), acc);
+    float2 x = halves_of(x2);
+    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x.x));      // -127
+    asm("max.NaN.f32 %0, %0, 0fC2FE0000;" : "+f"(x.y));
+    if (!AT_MOST_ZERO) {
+        asm("min.NaN.f32 %0, %0, 0f43000000;" : "+f"(x.x));      // 128
+        asm("min.NaN.f32 %0, %0, 0f43000000;" : "+f"(x.y));
+    }
+    auto both = [](float v) { return pair_of(v, v); };
+    x2 = pair_of(x.x, x.y);
+    const unsigned long long shifted = add_pair(x2, both(12582912.f));                  // 1.5 * 2^23: the integer is in the low bits
+    const unsigned long long f = fma_pair(add_pair(shifted, both(-12582912.f)), both(-1.f), x2);
+    unsigned long long p = both(1.5345812e-4f);
+    p = fma_pair(p, f, both(1.3399931e-3f));
+    p = fma_pair(p, f, both(9.618489e-3f));
+    p = fma_pair(p, f, both(5.5503286e-2f));
+    p = fma_pair(p, f, both(2.4022646e-1f));
+    p = fma_pair(p, f, both(6.931472e-1f));
+    p = fma_pair(p, f, both(1.f));
+    const float2 t = halves_of(shifted);
+    acc = fma_pair(p, pair_of(__int_as_float((__float_as_int(t.x) << 23) + 0x3f800000), __int_as_float((__float_as_int(t.y) << 23) + 0x3f800000)), acc);
 }
-// FMA_SHARE: one exponential in eight of both sweeps goes that way.  The special-function pipe is what bounds them where
-// keys come fast enough, and the FMA pipe is half idle.  Select call, us, none / one in eight / 3 in 16 / one in four: 8
-// heads x 32,768 keys, 128 rows, 35.8 / 35.0 / 35.0 / 36.1; 16 heads x 24,576 keys 47.4 / 46.3 / 46.7 / 47.1; 8 heads x 65,536
-// keys, 256 rows, 99.2 / 93.3.  Launches of several waves run long enough to meet the power limit, where the added work
-// costs what it saves: a whole group of 8 sequences of 32-64 K keys with 256 rows 1,033 / 1,050, so they go without.
-// Scores against 64 bits: 3.4-6.5e-7 rms with and without.
+constexpr int kFmaEveryStats = 8, kFmaEveryScore = 16;      // two of so many neighbouring exponentials
+// FMA_SHARE: one exponential in four of the statistics sweep and one in eight of the scoring sweep go that way, two neighbours as a
+// pair.  The special-function pipe is what bounds the sweeps where keys come fast enough, and the FMA pipe is half idle.  Whole
+// pass, us, plain instructions with one in eight in launches of one wave only / packed, none / one in eight / one in four: 4
+// layers of 8 heads x 16,384 keys, 128 rows, 36.7 / 37.7 / 36.2 / 36.0; 4 ragged sequences of 16-32 K keys, 128 rows, 176 / 179 /
+// 175 / 176; of 20-40 K, 256 rows, 343 / 348 / 339 / 335; 8 of 32-64 K, 256 rows, 1,005 / 1,006 / 981 / 992.
+// The two shares differ for precision's sake: ex2.approx lies 5e-8 too low on average (1.6e-8 near zero), the polynomial has no bias,
+// and the accumulators' rounding makes scores 1-2e-7 too high; a normaliser with more of the polynomial's terms makes up for the
+// terms of the score.  Window scores against 64 bits, rms over 24 inputs, before and now: 128 rows 3.01 and 2.99e-7, 256 rows 2.59 and
+// 2.57e-7, in several waves 2.493 and 2.490e-7, 2.049 and 2.045e-7 (one in eight of both there: 2.510 and 2.062e-7).
 
 // ---------------------------------------------------------------------------------------------
 // per-element work of the two sweeps
@@ -198,33 +242,34 @@ __device__ __forceinline__ void stats_update(float (&v)[32], bool fast, int jb, 
     const float m_new = fmaxf(m, fmaxf(g0, g1));
     if (m_new > -INFINITY) {
         const float mc = m_new * c;
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+        const unsigned long long c2 = pair_of(c, c), mc2 = pair_of(-mc, -mc);
+        unsigned long long a01 = 0ull, a23 = 0ull;
 #pragma unroll
         for (int x = 0; x < 32; x += 4) {
-            a0 += fast_exp2(fmaf(v[x], c, -mc));
-            a1 += fast_exp2(fmaf(v[x + 1], c, -mc));
-            a2 += fast_exp2(fmaf(v[x + 2], c, -mc));
-            if (FMA_SHARE && x % 8 == 0) add_exp2_fma<true>(a3, fmaf(v[x + 3], c, -mc));
-            else a3 += fast_exp2(fmaf(v[x + 3], c, -mc));
+            a01 = add_pair(a01, exp2_pair(fma_pair(pair_of(v[x], v[x + 1]), c2, mc2)));
+            const unsigned long long y = fma_pair(pair_of(v[x + 2], v[x + 3]), c2, mc2);
+            if (FMA_SHARE && x % kFmaEveryStats == 0) add_exp2_fma<true>(a23, y);
+            else a23 = add_pair(a23, exp2_pair(y));
         }
-        const float add = (a0 + a1) + (a2 + a3);
+        const float2 s01 = halves_of(a01), s23 = halves_of(a23);
+        const float add = (s01.x + s01.y) + (s23.x + s23.y);
         l = m_new == m ? l + add : l * fast_exp2((m - m_new) * c) + add;
         m = m_new;
     }
 }
 // sweep 2: adds exp2(x*c - lse2) of 32 (or 16) rows to the four partial sums of a key
 template <int N, bool FMA_SHARE = false>
-__device__ __forceinline__ void score_accumulate(const float (&v)[N], const float *nl_base, float c, float &a0,
-                                                 float &a1, float &a2, float &a3)
+__device__ __forceinline__ void score_accumulate(const float (&v)[N], const float *nl_base, float c, unsigned long long &a01,
+                                                 unsigned long long &a23)
 {
+    const unsigned long long c2 = pair_of(c, c);
 #pragma unroll
     for (int x = 0; x < N; x += 4) {
-        const float4 nl = *reinterpret_cast<const float4 *>(nl_base + x);
-        a0 += fast_exp2(fmaf(v[x], c, nl.x));
-        a1 += fast_exp2(fmaf(v[x + 1], c, nl.y));
-        a2 += fast_exp2(fmaf(v[x + 2], c, nl.z));
-        if (FMA_SHARE && x % 8 == 0) add_exp2_fma<false>(a3, fmaf(v[x + 3], c, nl.w));   // (a caller's normaliser may be too low)
-        else a3 += fast_exp2(fmaf(v[x + 3], c, nl.w));
+        const ulonglong2 nl = *reinterpret_cast<const ulonglong2 *>(nl_base + x);
+        a01 = add_pair(a01, exp2_pair(fma_pair(pair_of(v[x], v[x + 1]), c2, nl.x)));
+        const unsigned long long y = fma_pair(pair_of(v[x + 2], v[x + 3]), c2, nl.y);
+        if (FMA_SHARE && x % kFmaEveryScore == 0) add_exp2_fma<false>(a23, y);   // (a caller's normaliser may be too low)
+        else a23 = add_pair(a23, exp2_pair(y));
     }
 }
 

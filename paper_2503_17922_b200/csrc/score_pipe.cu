@@ -743,20 +743,21 @@ group_pipeline_tc(const __grid_constant__ CUtensorMap kmap, const __grid_constan
                     const int t = (int)(g - it);
                     if (!warp_wait(&bar.tfull[grp], (g / kBufs) & 1, &abort_s, lane)) break;
                     tc_fence_after_sync();
-                    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+                    unsigned long long a01 = 0ull, a23 = 0ull;
                     for (int sl = 0; sl < n32; ++sl) {
                         float v[32];
                         tmem_ld32(taddr_grp + sl * 32, v);
                         if (sl + 1 == n32 && !tail) warp_release(&bar.tempty[grp], lane);
-                        score_accumulate<32>(v, neg_lse2 + sl * 32, c, a0, a1, a2, a3);
+                        score_accumulate<32>(v, neg_lse2 + sl * 32, c, a01, a23);
                     }
                     if (tail) {
                         float vt[16];
                         tmem_ld16(taddr_grp + n32 * 32, vt);
                         warp_release(&bar.tempty[grp], lane);
-                        score_accumulate<16>(vt, neg_lse2 + n32 * 32, c, a0, a1, a2, a3);
+                        score_accumulate<16>(vt, neg_lse2 + n32 * 32, c, a01, a23);
                     }
-                    const float tj = (a0 + a1) + (a2 + a3);
+                    const float2 s01 = halves_of(a01), s23 = halves_of(a23);
+                    const float tj = (s01.x + s01.y) + (s23.x + s23.y);
                     const int j = e.j_begin + t * kTile + L;
                     if (j < e.j_end) {
                         t_chunk[j - e.j_begin] = tj;

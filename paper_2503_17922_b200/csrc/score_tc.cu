@@ -170,7 +170,7 @@ struct StatsSweep {
     int limit;              // last key the thread's row may attend to
     int j_begin, j_plain;   // first key of the item; tiles that end before j_plain need no masking
 };
-template <int MB, bool FMA_SHARE>
+template <int MB>
 __device__ __forceinline__ float2 stats_sweep(GroupBarriers gb, StatsSweep w, uint32_t taddr, uint32_t it, int n_tiles, int grp, float c)
 {
     constexpr int NG = groups_for(MB);
@@ -188,7 +188,7 @@ __device__ __forceinline__ float2 stats_sweep(GroupBarriers gb, StatsSweep w, ui
             float x[32];
             tmem_ld32(taddr + sl * 32, x);
             if (sl + 1 == w.nslot) warp_release(tempty, lane);   // the buffer may be overwritten now
-            stats_update<FMA_SHARE>(x, fast, tile0 + w.col0 + sl * 32, w.limit, c, m, l);
+            stats_update<true>(x, fast, tile0 + w.col0 + sl * 32, w.limit, c, m, l);
         }
     }
     return make_float2(m, l);
@@ -200,7 +200,7 @@ struct ScoreSweep {
     bool reuse;
     float *token_out;       // or null
 };
-template <int MB, bool FMA_SHARE>
+template <int MB>
 __device__ __forceinline__ void score_sweep(GroupBarriers gb, ScoreSweep w, uint32_t taddr, uint32_t it, int n_tiles, int grp, int L, float c)
 {
     constexpr int NG = groups_for(MB);
@@ -215,20 +215,21 @@ __device__ __forceinline__ void score_sweep(GroupBarriers gb, ScoreSweep w, uint
         if ((int)(v % NG) != grp) continue;
         if (!warp_wait(tfull, (v / NG) & 1, abort_flag, lane)) break;
         tc_fence_after_sync();
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+        unsigned long long a01 = 0ull, a23 = 0ull;
         for (int sl = 0; sl < n32; ++sl) {
             float x[32];
             tmem_ld32(taddr + sl * 32, x);
             if (sl + 1 == n32 && !tail) warp_release(tempty, lane);   // the buffer may be overwritten now
-            score_accumulate<32, FMA_SHARE>(x, neg_lse2 + sl * 32, c, a0, a1, a2, a3);
+            score_accumulate<32, true>(x, neg_lse2 + sl * 32, c, a01, a23);
         }
         if (tail) {
             float x[16];
             tmem_ld16(taddr + n32 * 32, x);
             warp_release(tempty, lane);
-            score_accumulate<16, FMA_SHARE>(x, neg_lse2 + n32 * 32, c, a0, a1, a2, a3);
+            score_accumulate<16, true>(x, neg_lse2 + n32 * 32, c, a01, a23);
         }
-        const float tj = (a0 + a1) + (a2 + a3);
+        const float2 s01 = halves_of(a01), s23 = halves_of(a23);
+        const float tj = (s01.x + s01.y) + (s23.x + s23.y);
         const int j = tile_at<stages_for(MB)>(w.reuse, n_tiles, (int)(v / MB - it)) * kTile + L;
         if (j < w.n_keys) {
             t_out[j] = tj;
@@ -519,7 +520,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         w.j_begin = im.j_begin;
         w.j_plain = min(im.n_r + 1, im.j_end);
         const uint32_t taddr = taddr_grp + w.col0;
-        sh.part[grp][L] = stats_sweep<MB, ONE>(gb, w, taddr, it, im.n_tiles, grp, c);
+        sh.part[grp][L] = stats_sweep<MB>(gb, w, taddr, it, im.n_tiles, grp, c);
     };
 
     // kMergers neighbouring threads share an observation row when partial statistics are merged, within the block and
@@ -560,7 +561,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         w.n_keys = im.j_end - im.j_begin;
         w.reuse = im.reuse;
         w.token_out = MB == 1 && a.token_scores ? a.token_scores + (size_t)im.unit * s.nr_max + im.j_begin : nullptr;
-        score_sweep<MB, ONE>(gb, w, taddr_grp, it, im.n_tiles, grp, L, c);
+        score_sweep<MB>(gb, w, taddr_grp, it, im.n_tiles, grp, L, c);
     };
 
     auto block_barrier = [&]() {
