@@ -445,6 +445,17 @@ int wkv_probe_colsum_rate(float *scratch_dev, int32_t blocks, int32_t threads, i
 int wkv_probe_published_select(const void *words_dev, int32_t n_words, uint64_t tag, int32_t k, int32_t *window_idx_dev,
                                int32_t *status_dev, void *cuda_stream);
 
+/*
+ * Test aid (no counterpart in the paper): wkv_select_leader_windows (tensor-core path) whose blocks look `looks` >= 1 times for
+ * what another block of the launch publishes before they do without it, computing it themselves or leaving the selection to
+ * the unit's last block.  The library's own calls look often enough for that to happen only where another stream's
+ * kernel keeps blocks of the launch from starting.  Shapes whose blocks all start together only (one wave); the results are the same
+ * to within rounding.
+ */
+int wkv_probe_impatient_select(const wkv_shape *s, const void *q_obs_leader, const void *k_leader, const float *lse_obs,
+                               int32_t looks, float *window_scores, int32_t *window_idx, int32_t *kept_len, void *workspace,
+                               size_t workspace_bytes, void *cuda_stream);
+
 const char *wkv_status_string(int status);
 const char *wkv_last_error_detail(void);
 /* Number of kernels the library has launched from this process (all threads). */

@@ -26,7 +26,7 @@ EXPORTED_SYMBOLS = [
     "wkv_num_windows", "wkv_num_selected", "wkv_keep_len", "wkv_workspace_sync_words", "wkv_kw_max", "wkv_k_max", "wkv_keep_max", "wkv_group_budgets", "wkv_jaccard_windows",
     "wkv_workspace_bytes", "wkv_score_windows", "wkv_score_windows_static", "wkv_select_topk_windows", "wkv_gather_kv", "wkv_gather_kv_paged", "wkv_compact_kv_inplace",
     "wkv_compress_group", "wkv_compress_group_host", "wkv_compress_group_host_rows", "wkv_score_windows_lse", "wkv_compress_group_lse",
-    "wkv_select_leader_windows", "wkv_probe_ex2_rate", "wkv_probe_colsum_rate", "wkv_probe_published_select", "wkv_group_plan_create", "wkv_group_plan_launch", "wkv_group_plan_destroy", "wkv_status_string", "wkv_last_error_detail",
+    "wkv_select_leader_windows", "wkv_probe_ex2_rate", "wkv_probe_colsum_rate", "wkv_probe_published_select", "wkv_probe_impatient_select", "wkv_group_plan_create", "wkv_group_plan_launch", "wkv_group_plan_destroy", "wkv_status_string", "wkv_last_error_detail",
     "wkv_launch_count",
 ]
 
@@ -136,6 +136,8 @@ def lib() -> ctypes.CDLL:
     L.wkv_probe_colsum_rate.argtypes = [vp, i32, i32, i32, ctypes.POINTER(ctypes.c_int64), vp]
     L.wkv_probe_published_select.restype = ctypes.c_int
     L.wkv_probe_published_select.argtypes = [vp, i32, ctypes.c_uint64, i32, vp, vp, vp]
+    L.wkv_probe_impatient_select.restype = ctypes.c_int
+    L.wkv_probe_impatient_select.argtypes = [sp, vp, vp, vp, i32, vp, vp, vp, vp, sz, vp]
     L.wkv_status_string.restype = ctypes.c_char_p
     L.wkv_status_string.argtypes = [ctypes.c_int]
     L.wkv_last_error_detail.restype = ctypes.c_char_p
@@ -541,6 +543,14 @@ def wkv_probe_published_select(words, tag: int, window_idx, status, stream=None)
     """Selects the window_idx.numel() highest of the published scores `words` (int64 [n, 2]: score bits, tag)."""
     _check(lib().wkv_probe_published_select(_ptr(words), words.shape[0], tag, window_idx.numel(), _ptr(window_idx), _ptr(status),
                                             _stream(stream)), "wkv_probe_published_select")
+
+
+def wkv_probe_impatient_select(prob: Problem, q_obs_leader, k_leader, looks: int, window_scores, window_idx, kept_len, workspace,
+                               lse_obs=None, stream=None) -> None:
+    """wkv_select_leader_windows whose blocks look for one another's words `looks` times, then do without."""
+    _check(lib().wkv_probe_impatient_select(ctypes.byref(prob.shape), _ptr(q_obs_leader), _ptr(k_leader), _ptr(lse_obs), looks,
+                                            _ptr(window_scores), _ptr(window_idx), _ptr(kept_len), _ptr(workspace),
+                                            workspace.numel(), _stream(stream)), "wkv_probe_impatient_select")
 
 
 def device_status(workspace) -> int:

@@ -86,6 +86,26 @@ __device__ __forceinline__ void wait_entries(const StatEntry *p, size_t step, un
         }
     }
 }
+// The same for a caller that can do without the words: it looks `looks` times (each is a trip to L2, 0.6 us and more), then raises
+// the flag, which ends the search of all that share it.
+template <int N>
+__device__ __forceinline__ void look_for_entries(const StatEntry *p, size_t step, unsigned wanted, unsigned long long tag,
+                                                 StatEntry (&e)[N], volatile int *late_flag, int looks)
+{
+    for (;;) {
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+            if (wanted >> u & 1u) e[u] = read_entry(p + u * step);
+#pragma unroll
+        for (int u = 0; u < N; ++u)
+            if ((wanted >> u & 1u) && e[u].tag == tag) wanted &= ~(1u << u);
+        if (!wanted || *late_flag) return;
+        if (--looks <= 0) {
+            *late_flag = 1;
+            return;
+        }
+    }
+}
 
 // Launches on a workspace, counted so that each has a tag of its own.  Every block reads the count before it counts
 // itself, and the launch's last block to do so raises it: the blocks of one launch agree on it, the next one's
@@ -115,13 +135,15 @@ __device__ __forceinline__ void count_launch(LaunchCount *c, unsigned long long 
 }
 
 // The selection reads the published window scores, waiting for those that are still to come: LOOK words at a time.
-template <int LOOK>
+// PATIENT: until they come or the wait expires, else for `looks` looks.
+template <int LOOK, bool PATIENT = true>
 struct PublishedScores {
     static constexpr bool kWaits = true;
     const StatEntry *entries;
     unsigned long long tag;
     volatile int *abort_flag;
     int hint;
+    int looks = 0;
     template <int N>
     __device__ __forceinline__ void keys(unsigned (&key)[N], int lo, int hi) const
     {
@@ -130,8 +152,9 @@ struct PublishedScores {
         for (int e0 = 0; e0 < N; e0 += kLook) {
             StatEntry v[kLook];
             const int left = hi - lo - e0;
-            wait_entries<kLook>(entries + lo + e0, 1, left >= kLook ? (1u << kLook) - 1u : left > 0 ? (1u << left) - 1u : 0u, tag, v,
-                                abort_flag);
+            const unsigned wanted = left >= kLook ? (1u << kLook) - 1u : left > 0 ? (1u << left) - 1u : 0u;
+            if (PATIENT) wait_entries<kLook>(entries + lo + e0, 1, wanted, tag, v, abort_flag);
+            else look_for_entries<kLook>(entries + lo + e0, 1, wanted, tag, v, abort_flag, looks);
 #pragma unroll
             for (int e = 0; e < kLook; ++e) key[e0 + e] = e < left ? topk_order_key(__uint_as_float((unsigned)v[e].value)) : 0u;
         }

@@ -1,5 +1,5 @@
 // Tensor-core score kernel (tcgen05 + tensor memory + TMA) for bf16 inputs: Eq. 1-4 of the leader
-// and, when asked, the budgeted selection, in ONE cooperative launch.
+// and, when asked, the budgeted selection, in ONE launch.
 //
 // The token score of Eq. 2, t_j = sum_i exp(s_ij) / Z_i, needs every row's softmax normaliser
 // Z_i (a reduction over all keys) before any column sum can be finished, so the keys are swept
@@ -27,6 +27,10 @@
 //
 // Every wait is bounded (mbarriers and the wait for a unit's statistics): on expiry the block sets bit 0 of the
 // status word, drains its own TMA loads, frees its tensor memory and returns.
+//
+// Where the whole problem is one wave (ONE) the launch is a programmatic dependent and guarantees nothing about which
+// blocks run together: a block looks for what others publish for a while and then does without them
+// (stats_in_others_place, late_selection).  With several waves the launch is cooperative.
 #include "tc_common.cuh"
 #include "score_math.cuh"
 #include "topk_block.cuh"
@@ -75,6 +79,8 @@ struct TcArgs {
     int slot_tok, slot_h, slot_b;   // which tensor-map coordinate (1..3) carries token / head / batch
     unsigned alpha_inverse; // ceil(2^16 / alpha): r * alpha_inverse >> 16 is r / alpha for r, alpha <= 256
     int r16;                // observation rows rounded up to a multiple of 16
+    int looks;              // ONE: how often a block looks for another's words before it does without
+    const __nv_bfloat16 *k; // the keys behind the tensor map, for what a block computes in another's place
 };
 
 __device__ __forceinline__ uint8_t *align_1024(uint8_t *p)
@@ -118,14 +124,15 @@ __device__ __forceinline__ void warp_release(uint64_t *bar, int lane)
     if (lane == 0) mbar_arrive(bar);
 }
 
-// Hand-over between blocks (all are resident: cooperative launch): every partial statistic and, where the launch
+// Hand-over between blocks: every partial statistic and, where the launch
 // selects, every window score is published as one 16-byte word of value and tag, written and read as a whole, so that
 // it says itself whether it is there: no fence, no counter, and the data arrives with the answer.  The tag holds the
 // number of this launch on the workspace (LaunchCount), which what an earlier launch has left behind, of whatever
 // shape, cannot equal.  8 heads x 4,096 keys: 2.3 us from the end of sweep 1 to the normalisers and 3.3 us from the pooled
 // windows to the selection; with counters raised by a release and polled it was 3.7 and 4.6 us.
-// No block waits before it has finished all its sweep-1 work, so every wait ends.  Bounded: a thread that
-// looks for longer than two seconds gives up and sets the block's abort flag.
+// No block waits before it has finished all its sweep-1 work, so every wait among running blocks ends; ONE does without
+// blocks that do not run, and in a cooperative launch all do.  Bounded there: a thread that looks for longer than two
+// seconds gives up and sets the block's abort flag.
 
 // The value, but nothing that is computed from it before this point: what only the ends of an item need would otherwise
 // be computed ahead of the tile loops and take their registers.
@@ -143,6 +150,29 @@ struct Item {
     int j_begin, j_end, n_tiles;
     int reuse;   // sweep 2: the stage ring still holds the item's last tiles from sweep 1
 };
+__device__ __forceinline__ void set_item(const TcArgs &a, int unit, int chunk, int review_only, Item &im)
+{
+    const KShape &s = a.s;
+    im.unit = unit;
+    im.chunk = chunk;
+    im.b = unit / s.hkv;
+    im.h = unit - im.b * s.hkv;
+    if (s.cu) {
+        const int lo = min(max(s.cu[im.b], 0), s.total_rows);
+        im.n = min(min(max(s.cu[im.b + 1] - s.cu[im.b], 0), s.n_cap), s.total_rows - lo);
+        im.off = lo;
+    } else {
+        im.n = s.max_seqlen;
+        im.off = 0;
+    }
+    im.n_r = im.n - s.alpha;
+    const int n_keys = review_only ? im.n_r : im.n;
+    const int len = tc_chunk_len(n_keys > 0 ? n_keys : 1, a.chunks_per_unit, review_only ? s.omega : 1);
+    im.j_begin = chunk * len;
+    im.j_end = min(n_keys, im.j_begin + len);
+    im.n_tiles = im.j_end > im.j_begin ? (im.j_end - im.j_begin + kTile - 1) / kTile : 0;
+    im.reuse = 0;
+}
 // Tile taken at step u of an item.  Sweep 1 and a sweep 2 that has to load everything go through the
 // tiles in ascending order.  A block that scores the item it has just taken statistics of still holds
 // that item's last STAGES tiles in the ring, in ring order: it scores those first, without
@@ -239,10 +269,10 @@ __device__ __forceinline__ void score_sweep(GroupBarriers gb, ScoreSweep w, uint
 }
 // Eq. 1's normaliser of every row from the published statistics of a unit's `used` chunks (row r's of chunk c at
 // st[c * r_pad + r]) -> -log2 of it in neg_lse2.  `tl`: number of the compute thread; MERGERS neighbouring ones share a row.
-// LOOK of a thread's words are looked at together.
-template <int MERGERS, int LOOK>
+// LOOK of a thread's words are looked at together, `looks` times, or (PATIENT) until they come or the wait expires.
+template <int MERGERS, int LOOK, bool PATIENT>
 __device__ __forceinline__ void merge_stats(const StatEntry *st, int used, int rows, int r_pad, unsigned long long tag, int tl,
-                                            float *neg_lse2, volatile int *abort_flag)
+                                            float *neg_lse2, volatile int *flag, int looks)
 {
     const int r = tl / MERGERS, mp = tl % MERGERS;
     float M = -INFINITY, sum = 0.f;
@@ -252,7 +282,8 @@ __device__ __forceinline__ void merge_stats(const StatEntry *st, int used, int r
 #pragma unroll
             for (int u = 0; u < LOOK; ++u) wanted |= (c0 + u * MERGERS < used ? 1u : 0u) << u;
             StatEntry e[LOOK];
-            wait_entries<LOOK>(st + r + (size_t)c0 * r_pad, (size_t)MERGERS * r_pad, wanted, tag, e, abort_flag);
+            if (PATIENT) wait_entries<LOOK>(st + r + (size_t)c0 * r_pad, (size_t)MERGERS * r_pad, wanted, tag, e, flag);
+            else look_for_entries<LOOK>(st + r + (size_t)c0 * r_pad, (size_t)MERGERS * r_pad, wanted, tag, e, flag, looks);
             float2 p[LOOK];
             float Mn = M;
 #pragma unroll
@@ -296,6 +327,8 @@ struct Shared {
     __align__(8) Barriers bar;
     uint32_t tmem_base;
     int abort;
+    int late;                                  // ONE: a word has not come in time
+    unsigned last_chunk;                       // ONE: the unit's last chunk that holds review keys
     unsigned long long tag;                    // what this launch marks its published words with
     float2 part[groups_for(MB)][128 + 8];      // sweep 1: a group's (max, sum) of the rows on its lanes
     __align__(16) float neg_lse2[256];         // -log2 of the row normaliser; -inf for padding rows
@@ -316,6 +349,94 @@ template <int MB>
 __device__ __noinline__ void select_call(PublishedScores<1> src, int kw, int k, int k_max, int *out, int *kept_len, int n, int alpha, int omega)
 {
     select_topk_block<block_threads(MB)>((int)threadIdx.x, shared_state<MB>().topk, src, kw, k, k_max, out, kept_len, n, alpha, omega);
+}
+
+// What a block of ONE does when words have not come in time.  The blocks that should publish them may not have started,
+// and may be unable to before this one ends (another stream's kernel, of this library or not, holds their SMs).  Two
+// streams that issue groups in turn do not get there and gain with the rest (24,576-key paged and 2-head ragged groups:
+// 106 us a pair in cooperative launches, 98 now; with one stream of higher priority, whose blocks do come between the other's,
+// 106 and 105).
+//
+// Statistics: every compute thread takes what its row still lacks from the inputs, with plain arithmetic, publishes it
+// in the place of that block, and the normalisers are merged anew.  A few milliseconds at most where a block does not
+// come meanwhile.
+template <int MB>
+__device__ __noinline__ void stats_in_others_place(const TcArgs &a, const __nv_bfloat16 *q)
+{
+    constexpr int kMergers = groups_for(MB) * 128 / (MB * 128);
+    Shared<MB> &sh = shared_state<MB>();
+    const KShape &s = a.s;
+    const unsigned long long tag = sh.tag;
+    const int unit = blockIdx.x / a.chunks_per_unit, tl = (int)threadIdx.x - 64, r = tl / kMergers;
+    StatEntry *const words = a.stats + (size_t)unit * a.n_stat_chunks * a.r_pad;
+    Item im;
+    set_item(a, unit, 0, 0, im);
+    const int used = (im.n + im.j_end - 1) / im.j_end;
+    const int g = (int)((unsigned)r * a.alpha_inverse >> 16), i = r - g * s.alpha;
+    const __nv_bfloat16 *const row = q + im.b * s.qsb + ((long long)im.h * s.G + g) * s.qsh + i * s.qst;
+    for (int chunk = r < s.R ? tl % kMergers : used; chunk < used; chunk += kMergers) {
+        StatEntry *const word = words + (size_t)chunk * a.r_pad + r;
+        set_item(a, unit, chunk, 0, im);
+        const __nv_bfloat16 *key = a.k + (im.off + im.j_begin) * s.st + (s.cu ? 0 : im.b * s.sb) + im.h * s.sh;
+        const int j_end = min(im.j_end, im.n_r + i + 1);
+        float m = -INFINITY, l = 0.f;
+        bool there = read_entry(word).tag == tag;
+        for (int j = im.j_begin; j < j_end && !there; ++j, key += s.st) {
+            float dot = 0.f;
+            for (int v = 0; v < s.d; v += 8) {
+                const int4 x4 = __ldg(reinterpret_cast<const int4 *>(row + v)), y4 = __ldg(reinterpret_cast<const int4 *>(key + v));
+                const __nv_bfloat162 *x = reinterpret_cast<const __nv_bfloat162 *>(&x4), *y = reinterpret_cast<const __nv_bfloat162 *>(&y4);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 xf = __bfloat1622float2(x[e]), yf = __bfloat1622float2(y[e]);
+                    dot = fmaf(xf.x, yf.x, dot);
+                    dot = fmaf(xf.y, yf.y, dot);
+                }
+            }
+            dot *= s.scale_log2;
+            if (dot > m) {
+                l = l * fast_exp2(m - dot) + 1.f;
+                m = dot;
+            } else if (dot > -INFINITY) {
+                l += fast_exp2(dot - m);
+            }
+            if ((j & 31) == 31) there = read_entry(word).tag == tag;
+        }
+        if (!there) publish_entry(word, (unsigned long long)__float_as_uint(m) | (unsigned long long)__float_as_uint(l) << 32, tag);
+    }
+    __syncwarp();
+    merge_stats<kMergers, 1, true>(words, used, s.R, a.r_pad, tag, tl, sh.neg_lse2, &sh.abort, 0);
+}
+// Window scores: the selection is left to the block that counts itself last on the unit's ticket, by when all blocks are
+// publishing.  `ticket[1]` says so.  By the whole block, at its end: the one that has waited in vain (the last may have
+// counted itself meanwhile: then it selects after all), or the one that has found it gone.
+template <int MB>
+__device__ __noinline__ void late_selection(const TcArgs &a)
+{
+    Shared<MB> &sh = shared_state<MB>();
+    const KShape &s = a.s;
+    const int unit = blockIdx.x / a.chunks_per_unit, chunk = blockIdx.x - unit * a.chunks_per_unit;
+    if (chunk == (int)sh.last_chunk) {
+        if (threadIdx.x == 0) {
+            int *const ticket = a.sync + kSyncTickets + kSyncWordsPerUnit * unit;
+            __threadfence();                        // what this block has written of a selection comes before the other's
+            atomicExch(ticket + 1, 1);
+            __threadfence();
+            sh.topk.remaining = atomicAdd(ticket, 0) == 0 && atomicExch(ticket + 1, 0) != 0;
+            __threadfence();
+        }
+        __syncthreads();
+        if (!sh.topk.remaining) return;
+        __syncthreads();
+    }
+    Item im;
+    set_item(a, unit, 0, 1, im);
+    const int budget = s.budgets ? s.budgets[im.b] : s.budget;
+    const int kw = num_windows(im.n, s.alpha, s.omega), k = num_selected_capped(im.n, s.alpha, s.omega, budget, s.k_max);
+    const PublishedScores<1> src = {a.scores + (size_t)unit * s.kw_max, sh.tag, &sh.abort, topk_hint(s.R, im.n)};
+    select_topk_block<block_threads(MB)>((int)threadIdx.x, sh.topk, src, kw, k, s.k_max, a.window_idx + (size_t)unit * s.k_max,
+                                         a.kept_len + unit, im.n, s.alpha, s.omega);
+    __syncthreads();
 }
 
 // One wave of a block.  The sweeps have no registers to spare, and inside a loop over waves or items everything that
@@ -365,27 +486,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
 
     // the query head, within the unit's G, that observation row r < 256 belongs to: r / alpha
     auto head_of = [&](int r) { return (int)((unsigned)r * a.alpha_inverse >> 16); };
-    auto make_item = [&](int unit, int chunk, int review_only, Item &im) {
-        im.unit = unit;
-        im.chunk = chunk;
-        im.b = unit / s.hkv;
-        im.h = unit - im.b * s.hkv;
-        if (s.cu) {
-            const int lo = min(max(s.cu[im.b], 0), s.total_rows);
-            im.n = min(min(max(s.cu[im.b + 1] - s.cu[im.b], 0), s.n_cap), s.total_rows - lo);
-            im.off = lo;
-        } else {
-            im.n = s.max_seqlen;
-            im.off = 0;
-        }
-        im.n_r = im.n - s.alpha;
-        const int n_keys = review_only ? im.n_r : im.n;
-        const int len = tc_chunk_len(n_keys > 0 ? n_keys : 1, cpu, review_only ? s.omega : 1);
-        im.j_begin = chunk * len;
-        im.j_end = min(n_keys, im.j_begin + len);
-        im.n_tiles = im.j_end > im.j_begin ? (im.j_end - im.j_begin + kTile - 1) / kTile : 0;
-        im.reuse = 0;
-    };
+    auto make_item = [&](int unit, int chunk, int review_only, Item &im) { set_item(a, unit, chunk, review_only, im); };
 
     // Called by every warp except the producer; ends with a barrier among those warps.  Four loads
     // are in flight per thread.  The producer starts streaming key tiles once these small loads
@@ -646,6 +747,10 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                 if (lane == 0 && (ONE || !sh.counted)) {
                     count_launch(a.count, launch_of(sh.tag), gridDim.x);
                     sh.counted = 1;
+                    if (ONE) {
+                        const int len2 = tc_chunk_len(im.n_r, cpu, s.omega);
+                        sh.last_chunk = (unsigned)((im.n_r - 1) / len2);
+                    }
                 }
             } else {
             const int tl = late((int)threadIdx.x) - 64;
@@ -665,9 +770,13 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                 go_producer();
                 const StatEntry *st = a.stats + (size_t)im.unit * a.n_stat_chunks * a.r_pad;
                 const int used1 = (im.n + len1 - 1) / len1;    // chunks of the unit that hold keys in sweep 1
-                merge_stats<kMergers, ONE ? 5 : 2>(st, used1, s.R, a.r_pad, sh.tag, tl, sh.neg_lse2, &sh.abort);
+                merge_stats<kMergers, ONE ? 5 : 2, !ONE>(st, used1, s.R, a.r_pad, sh.tag, tl, sh.neg_lse2, ONE ? &sh.late : &sh.abort, a.looks);
             }
             compute_barrier();
+            if (ONE && *static_cast<volatile int *>(&sh.late)) {
+                stats_in_others_place<MB>(a, q);
+                compute_barrier();
+            }
             compute_scores(im);
             }
         }
@@ -689,7 +798,25 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         // the unit's ticket counts the blocks that are past all waiting for one another
         int *ticket = a.sync + kSyncTickets + kSyncWordsPerUnit * im.unit;
         const bool last_chunk = im.j_end == im.n_r;     // of those that hold keys in sweep 2
-        if (a.window_idx && !a.lse_obs && !last_chunk && threadIdx.x == 0) atomicAdd(ticket, 1);
+        if (ONE) {
+            // Every block of the unit counts itself and the last leaves the ticket at zero.  By a thread of the last warp, which is
+            // the last to get windows to pool.
+            if (threadIdx.x == kThreads - 32) {
+                int left = 0;
+                if (a.window_idx) {
+                    const unsigned last = sh.last_chunk, before = atomicInc(reinterpret_cast<unsigned *>(ticket), last);
+                    if (before > last) atomicOr(a.status, kStatusWaitExpired);   // the workspace was not cleared
+                    if (before == last && !last_chunk) {
+                        __threadfence();
+                        left = atomicExch(ticket + 1, 0);
+                        __threadfence();
+                    }
+                }
+                sh.late = left;
+            }
+        } else if (a.window_idx && !a.lse_obs && !last_chunk && threadIdx.x == 0) {
+            atomicAdd(ticket, 1);
+        }
         // Eq. 3-4: the item's windows (its first key is a multiple of omega)
         {
             const int n_tok = im.j_end - im.j_begin;
@@ -732,30 +859,39 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         // The block of the unit's last chunk selects for the unit, from the published scores: that
         // chunk is usually a short one, so its block is done early and the selection does not sit
         // on the path of a block that the next wave is waiting for.
-        // With given normalisers nothing else makes a block wait for another, and the selection does not
-        // either: the block that counts itself last selects, so the launch need not be cooperative.
-        bool selects = last_chunk;
-        if (a.lse_obs && a.window_idx) {
-            if (threadIdx.x == 0) {
-                const int before = atomicAdd(ticket, 1);
-                const int len2 = tc_chunk_len(im.n_r, cpu, late(s.omega)), used2 = (im.n_r + len2 - 1) / len2;
-                if (before == used2 - 1) atomicExch(ticket, 0);
-                if (before < 0 || before >= used2) atomicOr(a.status, kStatusWaitExpired);   // workspace not cleared
-                sh.topk.remaining = before == used2 - 1;
-            }
+        if (ONE && a.window_idx && last_chunk) {
             __syncthreads();
-            selects = sh.topk.remaining != 0;
-        }
-        if (a.window_idx && selects) {
-            __syncthreads();                 // a wait that expires from here on is seen by all at the same place
-            const PublishedScores<ONE ? 4 : 1> src = {a.scores + (size_t)im.unit * s.kw_max, sh.tag, &sh.abort, topk_hint(s.R, im.n)};
+            const PublishedScores<4, false> src = {a.scores + (size_t)im.unit * s.kw_max, sh.tag, &sh.late, topk_hint(s.R, im.n), a.looks};
             const int kw = num_windows(im.n, s.alpha, late(s.omega));
             const int k = num_selected_capped(im.n, s.alpha, late(s.omega), budget, s.k_max);
-            int *const out = a.window_idx + (size_t)im.unit * s.k_max;
-            if constexpr (ONE) select_topk_block<kThreads>((int)threadIdx.x, sh.topk, src, kw, k, s.k_max, out, a.kept_len + im.unit, im.n, s.alpha, s.omega);
-            else select_call<MB>(src, kw, k, s.k_max, out, a.kept_len + im.unit, im.n, s.alpha, s.omega);
-            // the others counted themselves before they published what has just been read: no wait in practice
-            if (!a.lse_obs && threadIdx.x == 0 && poll_until_at_least(ticket, im.chunk, &sh.abort)) atomicExch(ticket, 0);
+            select_topk_block<kThreads>((int)threadIdx.x, sh.topk, src, kw, k, s.k_max, a.window_idx + (size_t)im.unit * s.k_max,
+                                        a.kept_len + im.unit, im.n, s.alpha, s.omega);
+        }
+        if constexpr (!ONE) {
+            bool selects = last_chunk;
+            // With given normalisers nothing else makes a block wait for another, and the selection does not
+            // either: the block that counts itself last selects, so the launch need not be cooperative.
+            if (a.lse_obs && a.window_idx) {
+                if (threadIdx.x == 0) {
+                    const int before = atomicAdd(ticket, 1);
+                    const int len2 = tc_chunk_len(im.n_r, cpu, late(s.omega)), used2 = (im.n_r + len2 - 1) / len2;
+                    if (before == used2 - 1) atomicExch(ticket, 0);
+                    if (before < 0 || before >= used2) atomicOr(a.status, kStatusWaitExpired);   // workspace not cleared
+                    sh.topk.remaining = before == used2 - 1;
+                }
+                __syncthreads();
+                selects = sh.topk.remaining != 0;
+            }
+            if (a.window_idx && selects) {
+                __syncthreads();                 // a wait that expires from here on is seen by all at the same place
+                const PublishedScores<1> src = {a.scores + (size_t)im.unit * s.kw_max, sh.tag, &sh.abort, topk_hint(s.R, im.n)};
+                const int kw = num_windows(im.n, s.alpha, late(s.omega));
+                const int k = num_selected_capped(im.n, s.alpha, late(s.omega), budget, s.k_max);
+                int *const out = a.window_idx + (size_t)im.unit * s.k_max;
+                select_call<MB>(src, kw, k, s.k_max, out, a.kept_len + im.unit, im.n, s.alpha, s.omega);
+                // the others counted themselves before they published what has just been read: no wait in practice
+                if (!a.lse_obs && threadIdx.x == 0 && poll_until_at_least(ticket, im.chunk, &sh.abort)) atomicExch(ticket, 0);
+            }
         }
         if (!ONE) __syncthreads();   // t_chunk, neg_lse2 and the selection scratch are reused by the next item
     } while (!SINGLE && (item += gridDim.x) < n_items);
@@ -774,6 +910,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     if (threadIdx.x == 0) {
         init_barriers(bar);
         sh.abort = 0;
+        sh.late = 0;
         sh.counted = 0;
     }
     if (warp == 1) tmem_alloc(&sh.tmem_base, kTmemCols);
@@ -793,6 +930,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
 
     // ------------------------------------------------------------------ teardown
     __syncthreads();
+    if (ONE && *static_cast<volatile int *>(&sh.late) && !*static_cast<volatile int *>(&sh.abort)) late_selection<MB>(a);
     if (threadIdx.x == 32 && !sh.counted) count_launch(a.count, launches_so_far(a.count) + 1, gridDim.x);    // a block without an item
     if (warp == 0 && elect_one()) {
         // nothing of this block may be in flight when it ends: the last MMAs must have released
@@ -971,6 +1109,8 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
     a.slot_tok = slot[0];
     a.slot_h = slot[1];
     a.slot_b = slot[2];
+    a.k = static_cast<const __nv_bfloat16 *>(k);
+    a.looks = ws.looks;
     a.alpha_inverse = (65536u + ks.alpha - 1) / ks.alpha;
     a.r16 = (ks.R + 15) / 16 * 16;
 
@@ -1012,9 +1152,11 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
     const __nv_bfloat16 *qp = static_cast<const __nv_bfloat16 *>(q);
     if (err == cudaSuccess) {
         void *params[3] = {&tmap, &a, &qp};
-        // with given normalisers no block waits for another: a plain launch, which may start while the kernel in front
-        // drains (a cooperative one may not: 2 us)
-        if (lse_obs) err = launch_pdl(kernel, dim3(grid), threads, smem, stream, 1, tmap, a, qp);
+        // A plain launch may start while the kernel in front drains; a cooperative one may not, and begins on a tick of 2 us
+        // behind it.  With given normalisers no block waits for another, and in one wave none depends on it (above).  Group
+        // calls back to back, cooperative / plain, us: 8 heads x 4,096 keys 18.4 / 16.6, 8,192 26.7 / 24.8, 16,384 38.9 / 36.2; 3
+        // ragged sequences of 2 heads x 12,289 32.8 / 30.0.
+        if (lse_obs || form == 2) err = launch_pdl(kernel, dim3(grid), threads, smem, stream, 1, tmap, a, qp);
         else err = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), params, smem, stream);
     }
     if (err != cudaSuccess) {

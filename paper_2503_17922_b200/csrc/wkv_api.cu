@@ -57,6 +57,7 @@ Workspace plan_workspace(const KShape &ks, int sync_units)
     w.scores_off = off;
     w.counted_off = align_up(align_up(w.stats_off + units * w.r_pad * stats, 256) + units * w.r_pad * sizeof(float), 256);
     w.salt = 0;
+    w.looks = kPatientLooks;
     off = align_up(off + units * (size_t)ks.kw_max * sizeof(float), 256);
     w.entries_off = off;
     off = align_up(off + units * (size_t)ks.kw_max * 16, 256);
@@ -505,9 +506,10 @@ int wkv_score_windows_lse(const wkv_shape *s, const void *q_obs, const void *k_l
                                cuda_stream);
 }
 
-int wkv_select_leader_windows(const wkv_shape *s, const void *q_obs_leader, const void *k_leader,
-                              const float *lse_obs, float *window_scores, int32_t *window_idx, int32_t *kept_len,
-                              void *workspace, size_t workspace_bytes, void *cuda_stream)
+// wkv_select_leader_windows; `looks` > 0: as wkv_probe_impatient_select
+static int select_leader_entry(const wkv_shape *s, const void *q_obs_leader, const void *k_leader, const float *lse_obs, int looks,
+                               float *window_scores, int32_t *window_idx, int32_t *kept_len, void *workspace,
+                               size_t workspace_bytes, void *cuda_stream)
 {
     KShape ks;
     int st = resolve(s, ks);
@@ -516,13 +518,34 @@ int wkv_select_leader_windows(const wkv_shape *s, const void *q_obs_leader, cons
         set_error_detail("q_obs_leader / k_leader / window_idx / kept_len is NULL");
         return WKV_ERR_NULL;
     }
-    const Workspace ws = plan_workspace(ks);
+    Workspace ws = plan_workspace(ks);
+    if (looks > 0) ws.looks = looks;
     st = check_workspace(ws, workspace, workspace_bytes);
     if (st != WKV_OK) return st;
     float *scores = window_scores ? window_scores
                                   : reinterpret_cast<float *>(static_cast<char *>(workspace) + ws.scores_off);
     return do_score(s, ks, ws, q_obs_leader, k_leader, scores, nullptr, window_idx, kept_len, workspace,
                     static_cast<cudaStream_t>(cuda_stream), lse_obs);
+}
+
+int wkv_select_leader_windows(const wkv_shape *s, const void *q_obs_leader, const void *k_leader,
+                              const float *lse_obs, float *window_scores, int32_t *window_idx, int32_t *kept_len,
+                              void *workspace, size_t workspace_bytes, void *cuda_stream)
+{
+    return select_leader_entry(s, q_obs_leader, k_leader, lse_obs, 0, window_scores, window_idx, kept_len, workspace, workspace_bytes,
+                               cuda_stream);
+}
+
+int wkv_probe_impatient_select(const wkv_shape *s, const void *q_obs_leader, const void *k_leader, const float *lse_obs,
+                               int32_t looks, float *window_scores, int32_t *window_idx, int32_t *kept_len, void *workspace,
+                               size_t workspace_bytes, void *cuda_stream)
+{
+    if (looks < 1) {
+        set_error_detail("%d looks", looks);
+        return WKV_ERR_SHAPE;
+    }
+    return select_leader_entry(s, q_obs_leader, k_leader, lse_obs, looks, window_scores, window_idx, kept_len, workspace,
+                               workspace_bytes, cuda_stream);
 }
 
 int wkv_select_topk_windows(const wkv_shape *s, const float *window_scores, int32_t *window_idx,

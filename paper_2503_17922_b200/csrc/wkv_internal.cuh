@@ -90,6 +90,7 @@ struct Workspace {
     size_t total;
     size_t counted_off;  // scores_off as it would be with float2 statistics: what the built-in area admits shapes by
     unsigned salt;       // goes into the tags of published words (0 but for the built-in area)
+    int looks;           // how often a block that can do without another's words looks for them
     int n_stat_chunks;
     int r_pad;
 };
@@ -102,6 +103,12 @@ constexpr int kSyncWordsPerUnit = 4;
 // The area has room for at least this many units whatever the shape (32 KB), so that what lies behind it never lands on
 // the words of another shape: one workspace may serve shapes of up to so many units in turn.
 constexpr int kSyncUnits = 2048;
+
+// A look is a trip to L2 of 0.6 us or more.  The blocks of a launch that has the GPU to itself begin within a few us of one
+// another, those of one that shares it with short kernels of other streams within some tens: 600 us and more of looking
+// before a block takes it that another one cannot start.  (With 100 us two streams of different priority took 112 us for the
+// pair of groups that takes 105 so, and 106 in cooperative launches.)
+constexpr int kPatientLooks = 1000;
 
 // per-device host state (kernel attributes, device properties) is kept for this many device ordinals
 constexpr int kMaxDevices = 64;

@@ -1109,3 +1109,60 @@ def test_two_streams_at_once(dtype, recorded):
         for l in range(w.gamma):
             np.testing.assert_array_equal(binding.to_host_bits(out["k_out"][l]), ref["k_out"][l])
             np.testing.assert_array_equal(binding.to_host_bits(out["v_out"][l]), ref["v_out"][l])
+
+
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("case", [
+    dict(),                                                              # 64 rows, ragged last window
+    dict(n_q_heads=8, n_kv_heads=1, l_obs=32, max_seqlen=2100, batch=1),          # 256 rows
+    dict(l_obs=32, head_dim=64, max_seqlen=4096 + 32, window=16),        # 128 rows, head dimension 64
+    dict(ragged=True, batch=4, max_seqlen=3000, n_q_heads=6),            # packed, 48 rows, units of different lengths
+    dict(n_q_heads=32, n_kv_heads=8, max_seqlen=16384, window=16, batch=1, l_obs=32),  # 18 chunks per unit
+    dict(n_kv_heads=4, max_seqlen=130, batch=2, window=4),               # two tiles, the second for the causal edge alone
+], ids=lambda c: "-".join(f"{k}{v}" for k, v in c.items()) or "base")
+def test_blocks_that_do_without_one_another(case, given):
+    """A block that looks for another's words only once or twice computes the statistics itself and leaves the selection to the unit's last
+    block: the same selection, scores within the tolerance of the other tests, call after call on one workspace."""
+    w = small(**case)
+    grp = wl.make_group(w, 0)
+    ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], want_tokens=True, **pu.oracle_kwargs(w, grp))
+    prob = binding.Problem.from_workload(w)
+    q, k = binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0])
+    lse = torch.from_numpy(pu.lse_obs_reference(w, grp)).cuda() if given else None
+    work = prob.alloc_workspace()
+    for looks in (1, 2, 1, 4, 1):
+        out = prob.alloc_outputs(1, fill_byte=pu.FILL_BYTE)
+        binding.wkv_probe_impatient_select(prob, q, k, looks, out["window_scores"], out["window_idx"], out["kept_len"], work, lse_obs=lse)
+        torch.cuda.synchronize()
+        assert binding.device_status(work) == 0
+        gpu = {"prob": prob, **{n: out[n].cpu().numpy() for n in ("window_scores", "window_idx", "kept_len")}}
+        pu.check_selection(w, grp, gpu, ref)
+
+
+@pytest.mark.parametrize("case", [dict(n_q_heads=32, n_kv_heads=8, max_seqlen=16384, window=16, batch=1, l_obs=32),
+                                  dict(n_q_heads=8, n_kv_heads=1, l_obs=32, max_seqlen=8000, batch=4, ragged=True)],
+                         ids=["128rows", "256rows"])
+def test_selection_beside_a_kernel_that_holds_most_of_the_gpu(case):
+    """Another stream's kernel keeps two thirds of the SMs for some milliseconds, so that most blocks of the launch cannot start:
+    those that have started do without them."""
+    w = small(**case)
+    grp = wl.make_group(w, 0)
+    ref = oracle.select_leader(grp["q_obs"], grp["k_layers"][0], want_tokens=True, **pu.oracle_kwargs(w, grp))
+    prob = binding.Problem.from_workload(w)
+    q, k = binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0])
+    work, out = prob.alloc_workspace(), prob.alloc_outputs(1, fill_byte=pu.FILL_BYTE)
+    scratch, other, mine = torch.zeros(16, device="cuda"), torch.cuda.Stream(), torch.cuda.Stream()
+    binding.wkv_probe_ex2_rate(scratch, 1, 1024, 1)
+    torch.cuda.synchronize()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    # 1,024 threads of 8 exponentials: 512 clocks a round, beside which no block of the score kernel finds its registers
+    binding.wkv_probe_ex2_rate(scratch, sms * 2 // 3, 1024, 20000, stream=other)
+    with torch.cuda.stream(mine):
+        start.record()
+        binding.wkv_select_leader_windows(prob, q, k, out["window_scores"], out["window_idx"], out["kept_len"], work, stream=mine)
+        end.record()
+    torch.cuda.synchronize()
+    assert binding.device_status(work) == 0
+    gpu = {"prob": prob, **{n: out[n].cpu().numpy() for n in ("window_scores", "window_idx", "kept_len")}}
+    pu.check_selection(w, grp, gpu, ref)
