@@ -250,7 +250,17 @@ __device__ __forceinline__ void fetch_window(const KShape &s, const char *tensor
         asm volatile("prefetch.global.L2 [%0];" ::"l"(at + r * row_bytes + (long long)(x - r * row_lines) * 128));
     }
 }
-// `cluster`: blocks per cluster along x (1: none)
+// `cluster`: blocks per cluster along x (1: none); the attributes of such a launch, and their number
+inline int pdl_attributes(cudaLaunchAttribute (&attr)[2], int cluster)
+{
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    return cluster > 1 ? 2 : 1;
+}
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t stream,
                               int cluster, const Args &...args)
@@ -261,17 +271,8 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, 
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 1;
-    if (cluster > 1) {
-        attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = cluster;
-        attr[1].val.clusterDim.y = 1;
-        attr[1].val.clusterDim.z = 1;
-        cfg.numAttrs = 2;
-    }
     cfg.attrs = attr;
+    cfg.numAttrs = pdl_attributes(attr, cluster);
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 

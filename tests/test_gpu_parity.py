@@ -1111,6 +1111,35 @@ def test_two_streams_at_once(dtype, recorded):
             np.testing.assert_array_equal(binding.to_host_bits(out["v_out"][l]), ref["v_out"][l])
 
 
+def test_plan_that_moves_between_streams():
+    """Replays of one plan follow one another whatever streams they are on: each of many leaves
+    what the direct call leaves."""
+    w = small(n_q_heads=32, n_kv_heads=8, max_seqlen=6000, l_obs=16)
+    grp = wl.make_group(w, 0)
+    ref = pu.run_gpu_group(w, grp)
+    prob = binding.Problem.from_workload(w)
+    q = binding.to_device(grp["q_obs"])
+    ks, vs = ([binding.to_device(x) for x in grp[n]] for n in ("k_layers", "v_layers"))
+    work = prob.alloc_workspace()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for pattern in ((0, 0, 0, 1, 0, 1, 1), (0, 1), (1,) * 5):
+        out = prob.alloc_outputs(w.gamma, fill_byte=pu.FILL_BYTE)
+        torch.cuda.synchronize()
+        plan = binding.GroupPlan(prob, q, ks, vs, out["k_out"], out["v_out"], out["window_scores"], out["window_idx"],
+                                 out["kept_len"], work, keep_capacity=out["keep_capacity"])
+        before = binding.wkv_launch_count()
+        for i in pattern * 4:
+            plan.launch(stream=streams[i])
+        torch.cuda.synchronize()
+        assert binding.wkv_launch_count() - before == 2 * 4 * len(pattern)
+        assert binding.device_status(work) == 0
+        for name in ("window_scores", "window_idx", "kept_len"):
+            np.testing.assert_array_equal(out[name].cpu().numpy(), ref[name])
+        for l in range(w.gamma):
+            np.testing.assert_array_equal(binding.to_host_bits(out["k_out"][l]), ref["k_out"][l])
+        plan.close()
+
+
 @pytest.mark.parametrize("given", [False, True])
 @pytest.mark.parametrize("case", [
     dict(),                                                              # 64 rows, ragged last window
