@@ -897,6 +897,36 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
     } while (!SINGLE && (item += gridDim.x) < n_items);
 }
 
+// The unit's Q and the block's first key tile on their way to L2 while the kernel in front drains.  Nothing is read here that
+// the kernel goes on with (L2 is where the GPU's memory is coherent), and a place that is not the final one is no more than a
+// wasted fetch inside the tensors.  Passes back to back, us, without / with one tile / two / four / sixteen: 8 heads x 8,192 keys 24.8 /
+// 23.8 / 23.9 / 24.2 / 24.2, 16,384 36.3 / 34.6 / 34.6 / 35.0 / 36.0, 32,768 53.5 / 52.0 / 52.2 / 52.5 / 54.8, 3 ragged
+// sequences of 2 heads x 12,289 30.1 / 28.5 / 28.7 / 29.1 / 29.2: more only takes bandwidth from the kernel in front.
+template <int MB>
+__device__ __forceinline__ void fetch_ahead(const CUtensorMap *tmap, const TcArgs &a, const __nv_bfloat16 *q)
+{
+    const KShape &s = a.s;
+    const int unit = blockIdx.x / a.chunks_per_unit;
+    Item im;
+    set_item(a, unit, blockIdx.x - unit * a.chunks_per_unit, a.lse_obs != nullptr, im);
+    if (threadIdx.x < 32) {
+        if (im.n_tiles > 0 && elect_one()) {
+            const int tok = (int)im.off + im.j_begin, bcoord = s.cu ? 0 : im.b;
+            const int c1 = a.slot_tok == 1 ? tok : (a.slot_h == 1 ? im.h : bcoord);
+            const int c2 = a.slot_tok == 2 ? tok : (a.slot_h == 2 ? im.h : bcoord);
+            const int c3 = a.slot_tok == 3 ? tok : (a.slot_h == 3 ? im.h : bcoord);
+            for (int kb = 0; kb < a.kblocks; ++kb) tma_prefetch_4d(tmap, kb * 64, c1, c2, c3);
+        }
+    } else {
+        const int shift = a.kblocks - 1;            // a row is one or two lines of 128 bytes
+        const __nv_bfloat16 *const q_unit = q + im.b * s.qsb + (long long)im.h * s.G * s.qsh;
+        for (int x = (int)threadIdx.x - 32; x < s.R << shift; x += block_threads(MB) - 32) {
+            const int r = x >> shift, g = (int)((unsigned)r * a.alpha_inverse >> 16), i = r - g * s.alpha;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(q_unit + g * s.qsh + i * s.qst + (x & shift) * 64));
+        }
+    }
+}
+
 template <int MB, bool ONE, bool SINGLE>
 // 18 warps put five on one SM sub-partition (16K registers): 96 registers per thread at most
 __global__ void __launch_bounds__(block_threads(MB), 1)
@@ -917,8 +947,9 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    pdl_wait();                 // nothing above touches memory of anybody else
     if (threadIdx.x == 0) tma_prefetch_desc(&tmap);
+    if (ONE) fetch_ahead<MB>(&tmap, a, q);
+    pdl_wait();                 // nothing above reads or writes what another kernel may have written or may still read
 
     Carry carry = {0, 0, -1};
     if (ONE) {
