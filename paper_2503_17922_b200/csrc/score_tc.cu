@@ -358,7 +358,7 @@ __device__ __noinline__ void select_call(PublishedScores<1> src, int kw, int k, 
 // 106 and 105).
 //
 // Statistics: every compute thread takes what its row still lacks from the inputs, with plain arithmetic, publishes it
-// in the place of that block, and the normalisers are merged anew.  A few milliseconds at most where a block does not
+// in the place of that block, and the normalisers are merged anew.  Some milliseconds where a block does not
 // come meanwhile.
 template <int MB>
 __device__ __noinline__ void stats_in_others_place(const TcArgs &a, const __nv_bfloat16 *q)
