@@ -446,11 +446,14 @@ int wkv_probe_published_select(const void *words_dev, int32_t n_words, uint64_t 
                                int32_t *status_dev, void *cuda_stream);
 
 /*
- * Test aid (no counterpart in the paper): wkv_select_leader_windows (tensor-core path) whose blocks look `looks` >= 1 times for
- * what another block of the launch publishes before they do without it, computing it themselves or leaving the selection to
- * the unit's last block.  The library's own calls look often enough for that to happen only where another stream's
- * kernel keeps blocks of the launch from starting.  Shapes whose blocks all start together only (one wave); the results are the same
- * to within rounding.
+ * Test aid (no counterpart in the paper): wkv_select_leader_windows (tensor-core path) whose blocks do without one another: each
+ * computes the row statistics of all keys of its unit itself, and one that looks for the unit's window scores and does not find
+ * them `looks` >= 1 times leaves the selection to the unit's last block.  In the library's own calls that happens only to words
+ * that a block has looked for about a thousand times, that is where another stream's
+ * kernel keeps blocks of the launch from starting.  The results are the same, bit for bit.  Shapes whose blocks all start together
+ * (one wave); with others, and on the CUDA-core path, no block does without another and `looks` has no effect.
+ * How often it has happened since the workspace was zeroed, in any call on it: the int32 at byte 20 counts chunks of keys whose
+ * row statistics a block has computed in another's place, the one at byte 24 selections left to the unit's last block.
  */
 int wkv_probe_impatient_select(const wkv_shape *s, const void *q_obs_leader, const void *k_leader, const float *lse_obs,
                                int32_t looks, float *window_scores, int32_t *window_idx, int32_t *kept_len, void *workspace,

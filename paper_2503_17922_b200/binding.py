@@ -547,10 +547,17 @@ def wkv_probe_published_select(words, tag: int, window_idx, status, stream=None)
 
 def wkv_probe_impatient_select(prob: Problem, q_obs_leader, k_leader, looks: int, window_scores, window_idx, kept_len, workspace,
                                lse_obs=None, stream=None) -> None:
-    """wkv_select_leader_windows whose blocks look for one another's words `looks` times, then do without."""
+    """wkv_select_leader_windows whose blocks compute all row statistics themselves and look `looks` times for window scores."""
     _check(lib().wkv_probe_impatient_select(ctypes.byref(prob.shape), _ptr(q_obs_leader), _ptr(k_leader), _ptr(lse_obs), looks,
                                             _ptr(window_scores), _ptr(window_idx), _ptr(kept_len), _ptr(workspace),
                                             workspace.numel(), _stream(stream)), "wkv_probe_impatient_select")
+
+
+def device_stand_ins(workspace):
+    """How often blocks of score launches on the workspace have done without one another's words since it was zeroed
+    (synchronises): (chunks of statistics computed in another block's place, selections left to a unit's last block)."""
+    words = workspace[20:28].view(__import__("torch").int32).tolist()
+    return words[0], words[1]
 
 
 def device_status(workspace) -> int:

@@ -111,7 +111,10 @@ __device__ __forceinline__ void look_for_entries(const StatEntry *p, size_t step
 // itself, and the launch's last block to do so raises it: the blocks of one launch agree on it, the next one's
 // find it changed.
 struct LaunchCount {
-    unsigned blocks, unused[3];
+    unsigned blocks;
+    unsigned stood_in;      // for diagnosis: chunks whose statistics a block has taken because their block's had not come,
+    unsigned left_over;     // and selections left to the block that counts itself last (score_tc.cu)
+    unsigned unused;
     unsigned long long launches;
 };
 // The tag's upper bits make its upper word a NaN with a payload that no arithmetic produces, so that neither numbers

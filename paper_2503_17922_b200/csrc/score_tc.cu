@@ -30,7 +30,7 @@
 //
 // Where the whole problem is one wave (ONE) the launch is a programmatic dependent and guarantees nothing about which
 // blocks run together: a block looks for what others publish for a while and then does without them
-// (stats_in_others_place, late_selection).  With several waves the launch is cooperative.
+// (stand_in, late_selection), with the same results.  With several waves the launch is cooperative.
 #include "tc_common.cuh"
 #include "score_math.cuh"
 #include "topk_block.cuh"
@@ -80,7 +80,7 @@ struct TcArgs {
     unsigned alpha_inverse; // ceil(2^16 / alpha): r * alpha_inverse >> 16 is r / alpha for r, alpha <= 256
     int r16;                // observation rows rounded up to a multiple of 16
     int looks;              // ONE: how often a block looks for another's words before it does without
-    const __nv_bfloat16 *k; // the keys behind the tensor map, for what a block computes in another's place
+    int alone;              // ONE: it does without all statistics but its own, whether they have come or not
 };
 
 __device__ __forceinline__ uint8_t *align_1024(uint8_t *p)
@@ -327,7 +327,8 @@ struct Shared {
     __align__(8) Barriers bar;
     uint32_t tmem_base;
     int abort;
-    int late;                                  // ONE: a word has not come in time
+    int late;                                  // ONE: a statistic has not come in time
+    int left_over;                             // ONE: a window score has not, or another block's selection is left to this one
     unsigned last_chunk;                       // ONE: the unit's last chunk that holds review keys
     unsigned long long tag;                    // what this launch marks its published words with
     float2 part[groups_for(MB)][128 + 8];      // sweep 1: a group's (max, sum) of the rows on its lanes
@@ -352,61 +353,8 @@ __device__ __noinline__ void select_call(PublishedScores<1> src, int kw, int k, 
 }
 
 // What a block of ONE does when words have not come in time.  The blocks that should publish them may not have started,
-// and may be unable to before this one ends (another stream's kernel, of this library or not, holds their SMs).  Two
-// streams that issue groups in turn do not get there and gain with the rest (24,576-key paged and 2-head ragged groups:
-// 106 us a pair in cooperative launches, 98 now; with one stream of higher priority, whose blocks do come between the other's,
-// 106 and 105).
+// and may be unable to before this one ends (another stream's kernel, of this library or not, holds their SMs).
 //
-// Statistics: every compute thread takes what its row still lacks from the inputs, with plain arithmetic, publishes it
-// in the place of that block, and the normalisers are merged anew.  Some milliseconds where a block does not
-// come meanwhile.
-template <int MB>
-__device__ __noinline__ void stats_in_others_place(const TcArgs &a, const __nv_bfloat16 *q)
-{
-    constexpr int kMergers = groups_for(MB) * 128 / (MB * 128);
-    Shared<MB> &sh = shared_state<MB>();
-    const KShape &s = a.s;
-    const unsigned long long tag = sh.tag;
-    const int unit = blockIdx.x / a.chunks_per_unit, tl = (int)threadIdx.x - 64, r = tl / kMergers;
-    StatEntry *const words = a.stats + (size_t)unit * a.n_stat_chunks * a.r_pad;
-    Item im;
-    set_item(a, unit, 0, 0, im);
-    const int used = (im.n + im.j_end - 1) / im.j_end;
-    const int g = (int)((unsigned)r * a.alpha_inverse >> 16), i = r - g * s.alpha;
-    const __nv_bfloat16 *const row = q + im.b * s.qsb + ((long long)im.h * s.G + g) * s.qsh + i * s.qst;
-    for (int chunk = r < s.R ? tl % kMergers : used; chunk < used; chunk += kMergers) {
-        StatEntry *const word = words + (size_t)chunk * a.r_pad + r;
-        set_item(a, unit, chunk, 0, im);
-        const __nv_bfloat16 *key = a.k + (im.off + im.j_begin) * s.st + (s.cu ? 0 : im.b * s.sb) + im.h * s.sh;
-        const int j_end = min(im.j_end, im.n_r + i + 1);
-        float m = -INFINITY, l = 0.f;
-        bool there = read_entry(word).tag == tag;
-        for (int j = im.j_begin; j < j_end && !there; ++j, key += s.st) {
-            float dot = 0.f;
-            for (int v = 0; v < s.d; v += 8) {
-                const int4 x4 = __ldg(reinterpret_cast<const int4 *>(row + v)), y4 = __ldg(reinterpret_cast<const int4 *>(key + v));
-                const __nv_bfloat162 *x = reinterpret_cast<const __nv_bfloat162 *>(&x4), *y = reinterpret_cast<const __nv_bfloat162 *>(&y4);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 xf = __bfloat1622float2(x[e]), yf = __bfloat1622float2(y[e]);
-                    dot = fmaf(xf.x, yf.x, dot);
-                    dot = fmaf(xf.y, yf.y, dot);
-                }
-            }
-            dot *= s.scale_log2;
-            if (dot > m) {
-                l = l * fast_exp2(m - dot) + 1.f;
-                m = dot;
-            } else if (dot > -INFINITY) {
-                l += fast_exp2(dot - m);
-            }
-            if ((j & 31) == 31) there = read_entry(word).tag == tag;
-        }
-        if (!there) publish_entry(word, (unsigned long long)__float_as_uint(m) | (unsigned long long)__float_as_uint(l) << 32, tag);
-    }
-    __syncwarp();
-    merge_stats<kMergers, 1, true>(words, used, s.R, a.r_pad, tag, tl, sh.neg_lse2, &sh.abort, 0);
-}
 // Window scores: the selection is left to the block that counts itself last on the unit's ticket, by when all blocks are
 // publishing.  `ticket[1]` says so.  By the whole block, at its end: the one that has waited in vain (the last may have
 // counted itself meanwhile: then it selects after all), or the one that has found it gone.
@@ -424,6 +372,7 @@ __device__ __noinline__ void late_selection(const TcArgs &a)
             __threadfence();
             sh.topk.remaining = atomicAdd(ticket, 0) == 0 && atomicExch(ticket + 1, 0) != 0;
             __threadfence();
+            atomicAdd(&a.count->left_over, 1u);
         }
         __syncthreads();
         if (!sh.topk.remaining) return;
@@ -442,8 +391,9 @@ __device__ __noinline__ void late_selection(const TcArgs &a)
 // One wave of a block.  The sweeps have no registers to spare, and inside a loop over waves or items everything that
 // lives on counts: 8 heads x 65,536 keys, 128 rows, one wave, take 58.1 us as ONE and 61.0 us as the form with a
 // loop (65.2 us where that looks at five published words at a time and has the selection inlined, as ONE does).  MB: 128-row blocks of observation rows, 1 (R <= 128) or 2 (R <= 256).  SINGLE: no block has more
-// than one item of a wave.  ONE: and there is one wave, so that nothing is kept from item to item.
-template <int MB, bool ONE, bool SINGLE>
+// than one item of a wave.  ONE: and there is one wave, so that nothing is kept from item to item.  STAND_IN: with the
+// statistics that others have not published (stand_in).
+template <int MB, bool ONE, bool SINGLE, bool STAND_IN>
 __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs &a, const __nv_bfloat16 *__restrict__ q, int u0,
                                           Carry &carry)
 {
@@ -621,13 +571,15 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         w.j_begin = im.j_begin;
         w.j_plain = min(im.n_r + 1, im.j_end);
         const uint32_t taddr = taddr_grp + w.col0;
-        sh.part[grp][L] = stats_sweep<MB>(gb, w, taddr, it, im.n_tiles, grp, c);
+        // (STAND_IN: to the place of the group that has these tiles where they are the block's first)
+        sh.part[STAND_IN ? (grp - (int)(it * MB)) & (NG - 1) : grp][L] = stats_sweep<MB>(gb, w, taddr, it, im.n_tiles, grp, c);
     };
 
     // kMergers neighbouring threads share an observation row when partial statistics are merged, within the block and
     // between the chunks; both in a fixed order
     constexpr int kComputeThreads = kThreads - 64;
     constexpr int kMergers = kComputeThreads / q_rows;
+    constexpr int kLook = ONE ? 5 : 2;         // (the rounding of a normaliser depends on it)
     auto compute_barrier = [&]() { asm volatile("bar.sync 3, %0;" ::"n"(kComputeThreads) : "memory"); };
 
     // combines the compute groups and the column slices of each row and publishes the item's statistics
@@ -673,10 +625,40 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
     const int n_items = ONE ? (int)gridDim.x : min(a.units_per_wave, units - u0) * cpu;
     int item;
 
+    if constexpr (STAND_IN) {
+        static_assert((NG & (NG - 1)) == 0, "groups are numbered modulo a power of two");
+        Item im;
+        const int unit = (int)blockIdx.x / cpu, own = (int)blockIdx.x - unit * cpu;
+        make_item(unit, 0, 0, im);
+        const int used1 = (im.n + im.j_end - 1) / im.j_end;     // chunks of the unit that hold keys in sweep 1
+        const StatEntry *const words = a.stats + (size_t)unit * a.n_stat_chunks * a.r_pad;
+        unsigned taken = 0;
+        for (int x = 1; x <= used1; ++x) {
+            const int chunk = (own + x) % used1;
+            const int lacks = tid < s.R && (a.alone ? chunk != own : read_entry(words + (size_t)chunk * a.r_pad + tid).tag != sh.tag);
+            if (!__syncthreads_or(lacks)) continue;
+            make_item(unit, chunk, 0, im);
+            if (warp == 0) {
+                produce(im, 0, im.n_tiles);
+            } else if (warp == 1) {
+                issue_mma(im, std::false_type{});
+            } else {
+                compute_stats(im);
+                compute_barrier();
+                publish_stats(im);
+            }
+            it += im.n_tiles;
+            ++taken;
+            block_barrier();
+            if (*static_cast<volatile int *>(&sh.abort)) return;
+        }
+        if (threadIdx.x == 0 && taken) atomicAdd(&a.count->stood_in, taken);
+    }
+
     // ------------------------------------------------------------------ sweep 1
     // (not needed when the caller supplies the normalisers: sweep 2 then reads the keys from HBM)
     item = blockIdx.x;
-    if (!a.lse_obs && (ONE || item < n_items)) do {
+    if (!STAND_IN && !a.lse_obs && (ONE || item < n_items)) do {
         Item im;
         const int nth = item / cpu;
         make_item(u0 + nth, item - nth * cpu, 0, im);
@@ -727,7 +709,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         const int len1 = tc_chunk_len(im.n, cpu, 1);
         // the ring holds the last tiles of the block's one item of the wave, if they are this sweep's tiles too
         const int keys1 = min(im.n - im.chunk * len1, len1);
-        im.reuse = !a.lse_obs && (SINGLE || (item == (int)blockIdx.x && item + (int)gridDim.x >= n_items)) &&
+        im.reuse = !STAND_IN && !a.lse_obs && (SINGLE || (item == (int)blockIdx.x && item + (int)gridDim.x >= n_items)) &&
                    im.n_tiles >= kStages && im.chunk * len1 == im.j_begin && (keys1 + kTile - 1) / kTile == im.n_tiles;
         if (warp == 0) {
             // ahead of the small loads of this item: the tiles the ring still holds (no traffic), or
@@ -744,7 +726,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                 go_producer();
                 issue_mma(im, std::true_type{});
                 // the block counts itself, once, now that it has read the number of launches
-                if (lane == 0 && (ONE || !sh.counted)) {
+                if (lane == 0 && !STAND_IN && (ONE || !sh.counted)) {
                     count_launch(a.count, launch_of(sh.tag), gridDim.x);
                     sh.counted = 1;
                     if (ONE) {
@@ -770,20 +752,18 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                 go_producer();
                 const StatEntry *st = a.stats + (size_t)im.unit * a.n_stat_chunks * a.r_pad;
                 const int used1 = (im.n + len1 - 1) / len1;    // chunks of the unit that hold keys in sweep 1
-                merge_stats<kMergers, ONE ? 5 : 2, !ONE>(st, used1, s.R, a.r_pad, sh.tag, tl, sh.neg_lse2, ONE ? &sh.late : &sh.abort, a.looks);
+                constexpr bool patient = !ONE || STAND_IN;
+                merge_stats<kMergers, kLook, patient>(st, used1, s.R, a.r_pad, sh.tag, tl, sh.neg_lse2, patient ? &sh.abort : &sh.late, a.looks);
             }
             compute_barrier();
-            if (ONE && *static_cast<volatile int *>(&sh.late)) {
-                stats_in_others_place<MB>(a, q);
-                compute_barrier();
-            }
-            compute_scores(im);
+            compute_scores(im);     // (for nothing if a statistic is late: the accumulators on their way have to be taken)
             }
         }
         q_unit_loaded = im.unit;
         it += im.n_tiles;
         block_barrier();
         if (sh.abort) break;
+        if (ONE && !STAND_IN && *static_cast<volatile int *>(&sh.late)) break;     // (stand_in, at the block's end)
         float *t_item = &sh.t_chunk[0][0];
         if (MB == 2) {
             // Eq. 2 sums over all rows: add the two halves' sums of every key
@@ -812,7 +792,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                         __threadfence();
                     }
                 }
-                sh.late = left;
+                sh.left_over = left;
             }
         } else if (a.window_idx && !a.lse_obs && !last_chunk && threadIdx.x == 0) {
             atomicAdd(ticket, 1);
@@ -861,7 +841,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         // on the path of a block that the next wave is waiting for.
         if (ONE && a.window_idx && last_chunk) {
             __syncthreads();
-            const PublishedScores<4, false> src = {a.scores + (size_t)im.unit * s.kw_max, sh.tag, &sh.late, topk_hint(s.R, im.n), a.looks};
+            const PublishedScores<4, false> src = {a.scores + (size_t)im.unit * s.kw_max, sh.tag, &sh.left_over, topk_hint(s.R, im.n), a.looks};
             const int kw = num_windows(im.n, s.alpha, late(s.omega));
             const int k = num_selected_capped(im.n, s.alpha, late(s.omega), budget, s.k_max);
             select_topk_block<kThreads>((int)threadIdx.x, sh.topk, src, kw, k, s.k_max, a.window_idx + (size_t)im.unit * s.k_max,
@@ -895,6 +875,25 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         }
         if (!ONE) __syncthreads();   // t_chunk, neg_lse2 and the selection scratch are reused by the next item
     } while (!SINGLE && (item += gridDim.x) < n_items);
+}
+
+// Statistics that have not come in time: the block takes those of every chunk that still lacks some, tile by tile as that
+// chunk's block does, in the same order and by the same instructions, so that no bit of the result depends on which of the two
+// a normaliser comes from.  By the whole block, at its end; sweep 2, which has taken the accumulators on their way, is repeated.
+// Blocks that stand in together begin with different chunks and take what another of them has published.  A chunk of 37 tiles
+// takes some 30 us, and a unit has at most 148 of them.  Returns the number of tiles whose loads the block has issued.
+// Inlined, and not called ahead of the pooling: what a call keeps on the stack cost every launch 0.1 to 0.5 us of 16 to 53.
+template <int MB>
+__device__ __forceinline__ uint32_t stand_in(const CUtensorMap *tmap, const TcArgs &a, const __nv_bfloat16 *q)
+{
+    const int unit = blockIdx.x / a.chunks_per_unit, chunk = blockIdx.x - unit * a.chunks_per_unit;
+    Item first, second;
+    set_item(a, unit, chunk, 0, first);
+    set_item(a, unit, chunk, 1, second);
+    const uint32_t tiles = first.n_tiles + second.n_tiles;      // all that the block has had so far
+    Carry carry = {tiles, tiles, unit};
+    take_wave<MB, true, true, true>(tmap, a, q, 0, carry);
+    return carry.issued;
 }
 
 // The unit's Q and the block's first key tile on their way to L2 while the kernel in front drains.  Nothing is read here that
@@ -940,7 +939,8 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     if (threadIdx.x == 0) {
         init_barriers(bar);
         sh.abort = 0;
-        sh.late = 0;
+        sh.late = a.alone;
+        sh.left_over = 0;
         sh.counted = 0;
     }
     if (warp == 1) tmem_alloc(&sh.tmem_base, kTmemCols);
@@ -953,15 +953,20 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
 
     Carry carry = {0, 0, -1};
     if (ONE) {
-        take_wave<MB, true, true>(&tmap, a, q, 0, carry);
+        take_wave<MB, true, true, false>(&tmap, a, q, 0, carry);
     } else {
         for (int u0 = 0; u0 < a.s.batch * a.s.hkv && !*static_cast<volatile int *>(&sh.abort); u0 += a.units_per_wave)
-            take_wave<MB, false, SINGLE>(&tmap, a, q, u0, carry);
+            take_wave<MB, false, SINGLE, false>(&tmap, a, q, u0, carry);
     }
 
     // ------------------------------------------------------------------ teardown
     __syncthreads();
-    if (ONE && *static_cast<volatile int *>(&sh.late) && !*static_cast<volatile int *>(&sh.abort)) late_selection<MB>(a);
+    // (of the blocks that have counted themselves: those with keys to score)
+    if (ONE && *static_cast<volatile int *>(&sh.late) && sh.counted && !*static_cast<volatile int *>(&sh.abort)) {
+        carry.issued = stand_in<MB>(&tmap, a, q);
+        __syncthreads();
+    }
+    if (ONE && *static_cast<volatile int *>(&sh.left_over) && !*static_cast<volatile int *>(&sh.abort)) late_selection<MB>(a);
     if (threadIdx.x == 32 && !sh.counted) count_launch(a.count, launches_so_far(a.count) + 1, gridDim.x);    // a block without an item
     if (warp == 0 && elect_one()) {
         // nothing of this block may be in flight when it ends: the last MMAs must have released
@@ -1140,8 +1145,8 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
     a.slot_tok = slot[0];
     a.slot_h = slot[1];
     a.slot_b = slot[2];
-    a.k = static_cast<const __nv_bfloat16 *>(k);
     a.looks = ws.looks;
+    a.alone = ws.alone && !lse_obs;
     a.alpha_inverse = (65536u + ks.alpha - 1) / ks.alpha;
     a.r16 = (ks.R + 15) / 16 * 16;
 

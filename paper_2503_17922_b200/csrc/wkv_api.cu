@@ -58,6 +58,7 @@ Workspace plan_workspace(const KShape &ks, int sync_units)
     w.counted_off = align_up(align_up(w.stats_off + units * w.r_pad * stats, 256) + units * w.r_pad * sizeof(float), 256);
     w.salt = 0;
     w.looks = kPatientLooks;
+    w.alone = false;
     off = align_up(off + units * (size_t)ks.kw_max * sizeof(float), 256);
     w.entries_off = off;
     off = align_up(off + units * (size_t)ks.kw_max * 16, 256);
@@ -519,7 +520,10 @@ static int select_leader_entry(const wkv_shape *s, const void *q_obs_leader, con
         return WKV_ERR_NULL;
     }
     Workspace ws = plan_workspace(ks);
-    if (looks > 0) ws.looks = looks;
+    if (looks > 0) {
+        ws.looks = looks;
+        ws.alone = true;
+    }
     st = check_workspace(ws, workspace, workspace_bytes);
     if (st != WKV_OK) return st;
     float *scores = window_scores ? window_scores

@@ -91,6 +91,7 @@ struct Workspace {
     size_t counted_off;  // scores_off as it would be with float2 statistics: what the built-in area admits shapes by
     unsigned salt;       // goes into the tags of published words (0 but for the built-in area)
     int looks;           // how often a block that can do without another's words looks for them
+    bool alone;          // it does without all statistics but its own (test aid)
     int n_stat_chunks;
     int r_pad;
 };

@@ -1195,3 +1195,82 @@ def test_selection_beside_a_kernel_that_holds_most_of_the_gpu(case):
     assert binding.device_status(work) == 0
     gpu = {"prob": prob, **{n: out[n].cpu().numpy() for n in ("window_scores", "window_idx", "kept_len")}}
     pu.check_selection(w, grp, gpu, ref)
+
+
+def _impatient_equals_ordinary(w, grp, looks, scale=1.0, given=False, seen=(0, 0)):
+    """One call whose blocks look `looks` times and one that waits: the same bytes.  Returns how often blocks did without one
+    another."""
+    prob = binding.Problem.from_workload(w)
+    q, k = binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0])
+    q *= scale
+    lse = torch.from_numpy(pu.lse_obs_reference(w, grp)).cuda() if given else None
+    work, hasty = prob.alloc_workspace(), prob.alloc_workspace()
+    ref = prob.alloc_outputs(1, fill_byte=pu.FILL_BYTE)
+    binding.wkv_select_leader_windows(prob, q, k, ref["window_scores"], ref["window_idx"], ref["kept_len"], work, lse_obs=lse)
+    for _ in range(6):
+        out = prob.alloc_outputs(1, fill_byte=pu.FILL_BYTE)
+        binding.wkv_probe_impatient_select(prob, q, k, looks, out["window_scores"], out["window_idx"], out["kept_len"], hasty, lse_obs=lse)
+        torch.cuda.synchronize()
+        assert binding.device_status(hasty) == 0
+        for name in ("window_scores", "window_idx", "kept_len"):
+            assert torch.equal(out[name].view(torch.int32), ref[name].view(torch.int32)), name
+    assert binding.device_status(work) == 0
+    return binding.device_stand_ins(hasty)
+
+
+@pytest.mark.parametrize("scale", [1.0, 12.0])                    # logits of a few and of several tens
+@pytest.mark.parametrize("case", [
+    dict(n_q_heads=32, n_kv_heads=8, max_seqlen=16384, window=16, batch=1, l_obs=32),        # 128 rows, 18 chunks of 8 tiles
+    dict(n_q_heads=8, n_kv_heads=2, max_seqlen=9001, window=16, batch=1, l_obs=16),          # 64 rows, in two copies
+    dict(n_q_heads=4, n_kv_heads=4, max_seqlen=5000, window=8, batch=2, l_obs=16),           # 16 rows, in four copies
+    dict(n_q_heads=8, n_kv_heads=1, l_obs=32, max_seqlen=40000, batch=1),                    # 256 rows
+    dict(n_q_heads=6, n_kv_heads=1, l_obs=32, max_seqlen=7000, batch=3, ragged=True),        # 192 rows, packed
+    dict(n_q_heads=8, n_kv_heads=2, l_obs=32, head_dim=64, max_seqlen=30000, window=12, batch=1),
+], ids=lambda c: "-".join(f"{k}{v}" for k, v in c.items()))
+def test_doing_without_one_another_changes_no_bit(case, scale):
+    """The statistics that a block computes in another's place have that block's bits, whatever the logits."""
+    w = small(**case)
+    counts = [_impatient_equals_ordinary(w, wl.make_group(w, 0), looks, scale) for looks in (1, 2)]
+    assert counts[0][0] > 0                                        # it did happen
+
+
+def test_one_long_unit_whose_blocks_do_without_one_another():
+    """148 chunks of 37 tiles, 256 rows: each block may take every other's chunk, within all limits of waiting."""
+    w = small(n_q_heads=8, n_kv_heads=1, l_obs=32, max_seqlen=148 * 37 * 128 - 100, batch=1, window=16, gamma=1)
+    assert _impatient_equals_ordinary(w, wl.make_group(w, 0), 1)[0] > 0
+
+
+@pytest.mark.parametrize("case", [dict(n_q_heads=4, n_kv_heads=1, max_seqlen=16384, window=16, batch=1, l_obs=32),
+                                  dict(n_q_heads=8, n_kv_heads=1, l_obs=32, max_seqlen=18000, batch=1),
+                                  dict(n_q_heads=12, n_kv_heads=2, l_obs=16, max_seqlen=9000, batch=1)],
+                         ids=["one-unit-128rows", "one-unit-256rows", "two-units"])
+def test_blocks_that_cannot_start_change_no_bit(case):
+    """Another stream's kernel holds two thirds of the SMs for milliseconds, and a unit has more blocks than the other SMs take:
+    those that have started do without the rest, and the result is that of a call that has the GPU to itself."""
+    w = small(**case)
+    grp = wl.make_group(w, 0)
+    prob = binding.Problem.from_workload(w)
+    q, k = binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0])
+    runs = [(prob.alloc_workspace(), prob.alloc_outputs(1, fill_byte=pu.FILL_BYTE)) for _ in range(2)]
+    scratch, other, mine = torch.zeros(16, device="cuda"), torch.cuda.Stream(), torch.cuda.Stream()
+    binding.wkv_probe_ex2_rate(scratch, 1, 1024, 1)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+
+    def select(work, out):
+        binding.wkv_select_leader_windows(prob, q, k, out["window_scores"], out["window_idx"], out["kept_len"], work, stream=mine)
+    select(*runs[0])
+    torch.cuda.synchronize()
+    assert binding.device_stand_ins(runs[0][0]) == (0, 0)
+    ended, let_go = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    # 1,024 threads of 8 exponentials: 512 clocks a round, beside which no block of the score kernel finds its registers
+    binding.wkv_probe_ex2_rate(scratch, sms * 2 // 3, 1024, 40000, stream=other)
+    let_go.record(other)
+    select(*runs[1])
+    ended.record(mine)
+    torch.cuda.synchronize()
+    work, out = runs[1]
+    assert binding.device_status(work) == 0
+    assert binding.device_stand_ins(work)[0] > 0                   # blocks were held back, and others stood in
+    assert ended.elapsed_time(let_go) > 0                          # (and made room for them: all while the other kernel ran)
+    for name in ("window_scores", "window_idx", "kept_len"):
+        assert torch.equal(out[name].view(torch.int32), runs[0][1][name].view(torch.int32)), name
