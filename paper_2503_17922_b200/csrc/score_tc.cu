@@ -150,6 +150,7 @@ struct Item {
     int j_begin, j_end, n_tiles;
     int reuse;   // sweep 2: the stage ring still holds the item's last tiles from sweep 1
 };
+template <bool EARLY = false>
 __device__ __forceinline__ void set_item(const TcArgs &a, int unit, int chunk, int review_only, Item &im)
 {
     const KShape &s = a.s;
@@ -158,8 +159,8 @@ __device__ __forceinline__ void set_item(const TcArgs &a, int unit, int chunk, i
     im.b = unit / s.hkv;
     im.h = unit - im.b * s.hkv;
     if (s.cu) {
-        const int lo = min(max(s.cu[im.b], 0), s.total_rows);
-        im.n = min(min(max(s.cu[im.b + 1] - s.cu[im.b], 0), s.n_cap), s.total_rows - lo);
+        const int from = length_word<EARLY>(s.cu + im.b), to = length_word<EARLY>(s.cu + im.b + 1), lo = min(max(from, 0), s.total_rows);
+        im.n = min(min(max(to - from, 0), s.n_cap), s.total_rows - lo);
         im.off = lo;
     } else {
         im.n = s.max_seqlen;
@@ -896,9 +897,8 @@ __device__ __forceinline__ uint32_t stand_in(const CUtensorMap *tmap, const TcAr
     return carry.issued;
 }
 
-// The unit's Q and the block's first key tile on their way to L2 while the kernel in front drains.  Nothing is read here that
-// the kernel goes on with (L2 is where the GPU's memory is coherent), and a place that is not the final one is no more than a
-// wasted fetch inside the tensors.  Passes back to back, us, without / with one tile / two / four / sixteen: 8 heads x 8,192 keys 24.8 /
+// The unit's Q and the block's first key tile on their way to L2 while the kernel in front drains.  Only a sequence's lengths are
+// read here, from L2 and anew behind the wait; lengths that are not the final ones make no more than a wasted fetch inside the tensors.  Passes back to back, us, without / with one tile / two / four / sixteen: 8 heads x 8,192 keys 24.8 /
 // 23.8 / 23.9 / 24.2 / 24.2, 16,384 36.3 / 34.6 / 34.6 / 35.0 / 36.0, 32,768 53.5 / 52.0 / 52.2 / 52.5 / 54.8, 3 ragged
 // sequences of 2 heads x 12,289 30.1 / 28.5 / 28.7 / 29.1 / 29.2: more only takes bandwidth from the kernel in front.
 template <int MB>
@@ -907,7 +907,7 @@ __device__ __forceinline__ void fetch_ahead(const CUtensorMap *tmap, const TcArg
     const KShape &s = a.s;
     const int unit = blockIdx.x / a.chunks_per_unit;
     Item im;
-    set_item(a, unit, blockIdx.x - unit * a.chunks_per_unit, a.lse_obs != nullptr, im);
+    set_item<true>(a, unit, blockIdx.x - unit * a.chunks_per_unit, a.lse_obs != nullptr, im);
     if (threadIdx.x < 32) {
         if (im.n_tiles > 0 && elect_one()) {
             const int tok = (int)im.off + im.j_begin, bcoord = s.cu ? 0 : im.b;
@@ -949,7 +949,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     tc_fence_after_sync();
     if (threadIdx.x == 0) tma_prefetch_desc(&tmap);
     if (ONE) fetch_ahead<MB>(&tmap, a, q);
-    pdl_wait();                 // nothing above reads or writes what another kernel may have written or may still read
+    pdl_wait();                 // but for what fetch_ahead says, nothing above touches memory of anybody else
 
     Carry carry = {0, 0, -1};
     if (ONE) {
