@@ -57,7 +57,9 @@ __host__ __device__ constexpr int groups_for(int) { return 4; }
 __host__ __device__ constexpr int block_threads(int mb) { return 64 + groups_for(mb) * 128; }
 constexpr int kTile = kTcTileKeys;                       // keys per tile
 constexpr int kRegion = kTile * 128;                     // bytes of one 64-column block of a key tile
-constexpr uint32_t kTmemCols = 512;                      // all of tensor memory: four accumulator buffers
+constexpr uint32_t kTmemCols = 512;                      // all of tensor memory: four accumulator buffers,
+constexpr uint32_t kTmemBase = 0;                        // which therefore begin with its first column
+constexpr uint32_t kNoTmem = ~0u;
 constexpr int kChunkCap = kTcChunkCap;                   // token scores a block may hold
 
 struct TcArgs {
@@ -326,7 +328,7 @@ template <int MB>
 struct Shared {
     int counted;                               // the block is among the launch's counted blocks
     __align__(8) Barriers bar;
-    uint32_t tmem_base;
+    uint32_t tmem_base;                        // kNoTmem until tensor memory has been taken
     int abort;
     int late;                                  // ONE: a statistic has not come in time
     int left_over;                             // ONE: a window score has not, or another block's selection is left to this one
@@ -426,7 +428,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
     const int ksteps = s.d / 16;
     const uint32_t leader = elect_one();     // lane that acts for its warp where a whole warp issues
 
-    const uint32_t tmem_base = sh.tmem_base;
+    constexpr uint32_t tmem_base = kTmemBase;
     uint32_t &it = carry.it, &p_issued = carry.issued;
     int &q_unit_loaded = carry.q_unit_loaded;
 
@@ -482,6 +484,14 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
             fence_proxy_async_smem();
             if (first && threadIdx.x == 32) sh.tag = launch_tag(launches, a.salt);
             asm volatile("bar.sync 1, %0;" ::"n"(kLoaders) : "memory");
+            // The warp that issues the MMAs takes tensor memory, and does so behind the wait for the kernel in front: a block
+            // of that kernel which shares the SM and has yet to take its own would wait for this one, which waits for that
+            // kernel.  Here the first key tile is still on its way (ahead of the wait or here 15.70 us for 8 heads x 4,096 keys,
+            // between the wait and the loads 16.05).
+            if (first && warp == 1) {
+                __syncwarp();
+                tmem_alloc(&sh.tmem_base, kTmemCols);
+            }
         } else if (signal) {
             go_producer();
         }
@@ -939,14 +949,12 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     if (threadIdx.x == 0) {
         init_barriers(bar);
         sh.abort = 0;
+        sh.tmem_base = kNoTmem;
         sh.late = a.alone;
         sh.left_over = 0;
         sh.counted = 0;
     }
-    if (warp == 1) tmem_alloc(&sh.tmem_base, kTmemCols);
-    tc_fence_before_sync();
     __syncthreads();
-    tc_fence_after_sync();
     if (threadIdx.x == 0) tma_prefetch_desc(&tmap);
     if (ONE) fetch_ahead<MB>(&tmap, a, q);
     pdl_wait();                 // but for what fetch_ahead says, nothing above touches memory of anybody else
@@ -984,7 +992,7 @@ score_windows_tc(const __grid_constant__ CUtensorMap tmap, const __grid_constant
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    if (warp == 1) tmem_dealloc(sh.tmem_base, kTmemCols);
+    if (warp == 1 && sh.tmem_base != kNoTmem) tmem_dealloc(sh.tmem_base, kTmemCols);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -76,3 +76,17 @@ def test_a_size_that_does_not_fit_is_remembered(fake):
     for _ in range(2):
         assert fake(rows=128, head_dim=288, device=device) == (0, TWO, 0)
         assert fake(rows=128, head_dim=64, device=device) == (0, ONE, 0)
+
+
+def test_nothing_that_a_block_may_wait_for_is_taken_ahead_of_the_kernel_in_front():
+    """A block that starts while the kernel in front still runs holds its SM's tensor memory from no other block: one of that
+    kernel's that waited for it would never end, and this block waits for that kernel.  (Read in the source: the way it fails is a GPU
+    that hangs.)"""
+    with open(os.path.join(build.CSRC, "score_tc.cu")) as f:
+        source = f.read()
+    body = source[source.index("score_windows_tc(const __grid_constant__ CUtensorMap tmap"):]
+    ahead, behind = body[:body.index("pdl_wait();")], body[body.index("pdl_wait();"):]
+    assert "take_wave<" in behind and "tmem_alloc" not in ahead and "take_wave<" not in ahead
+    helper = source[source.index("void fetch_ahead("):]
+    assert "fetch_ahead<" in ahead and "tmem_alloc" not in helper[:helper.index("score_windows_tc(")]
+    assert source.count("tmem_alloc(") == 1
