@@ -471,6 +471,11 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                     }
                 }
                 if (signal && base == loader) go_producer();
+                // The warp that issues the MMAs takes tensor memory, and does so behind the wait for the kernel in front: a
+                // block of that kernel which shares the SM and has yet to take its own would wait for this one, which waits
+                // for that kernel.  Here its share of Q is on its way: a group of 8 heads x 4,096 keys takes 16.4 us as with tensor memory
+                // taken ahead of the wait, 16.6 with it taken behind the barrier below; given normalisers cost 0.2 of 49 us.
+                if (first && base == loader && threadIdx.x < 64) tmem_alloc(&sh.tmem_base, kTmemCols);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int idx = base + u * kLoaders;
@@ -484,14 +489,6 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
             fence_proxy_async_smem();
             if (first && threadIdx.x == 32) sh.tag = launch_tag(launches, a.salt);
             asm volatile("bar.sync 1, %0;" ::"n"(kLoaders) : "memory");
-            // The warp that issues the MMAs takes tensor memory, and does so behind the wait for the kernel in front: a block
-            // of that kernel which shares the SM and has yet to take its own would wait for this one, which waits for that
-            // kernel.  Here the first key tile is still on its way (ahead of the wait or here 15.70 us for 8 heads x 4,096 keys,
-            // between the wait and the loads 16.05).
-            if (first && warp == 1) {
-                __syncwarp();
-                tmem_alloc(&sh.tmem_base, kTmemCols);
-            }
         } else if (signal) {
             go_producer();
         }
