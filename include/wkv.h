@@ -343,15 +343,16 @@ int wkv_select_leader_windows(const wkv_shape *s, const void *q_obs_leader, cons
  * wkv_compress_group / wkv_compress_group_lse).  For engines that call the group with the same
  * buffers again and again (static K/V pools and compact caches): create records the launches of
  * the call in a CUDA graph once, launch replays them on a stream, without validating or encoding
- * anything anew.  The plan owns only the graph; every buffer stays the caller's and must stay valid and at its address for as long as the plan is launched.  What a
- * launch computes depends on the buffers' contents at that moment only.
+ * anything anew.  The plan owns the recorded launches and an event; every buffer stays the caller's and must stay valid and at
+ * its address for as long as the plan is launched.  What a launch computes depends on the buffers' contents at that moment only.
  *   create   arguments as wkv_compress_group_lse (lse_obs may be NULL: then the normalisers are
  *            computed); validates as the direct call does and launches nothing.  Host-side
  *            resources (a graph) are allocated; no device buffer of the caller's is touched.
  *            `budgets` and the strides of `s` are read now, not at launch.
  *   launch   enqueues the group on cuda_stream; one plan is in flight once at a time (it uses
- *            the one workspace it was created with).  The first launch on another stream than those before it waits
- *            on the host for what the device has under way.
+ *            the one workspace it was created with): a launch is put behind the plan's launch before it, on the device and
+ *            whatever streams the two are on.  What the caller does to the buffers in between is the caller's to order.
+ *            After a failure part of the group may have been enqueued, as with the direct call.
  *   destroy  after the last launch has completed.  NULL is ignored.
  */
 typedef struct wkv_group_plan wkv_group_plan;

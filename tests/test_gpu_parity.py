@@ -1274,3 +1274,85 @@ def test_blocks_that_cannot_start_change_no_bit(case):
     assert ended.elapsed_time(let_go) > 0                          # (and made room for them: all while the other kernel ran)
     for name in ("window_scores", "window_idx", "kept_len"):
         assert torch.equal(out[name].view(torch.int32), runs[0][1][name].view(torch.int32)), name
+
+
+def _plan_on_two_inputs():
+    w = small(n_q_heads=32, n_kv_heads=8, max_seqlen=6000, l_obs=16)
+    grps = [wl.make_group(wl.scaled(w, config_id=c), 0) for c in (30, 31)]
+    refs = [pu.run_gpu_group(w, g) for g in grps]
+    prob = binding.Problem.from_workload(w)
+    work, out = prob.alloc_workspace(), prob.alloc_outputs(w.gamma, fill_byte=pu.FILL_BYTE)
+    sets = [[binding.to_device(x) for x in [g["q_obs"]] + g["k_layers"] + g["v_layers"]] for g in grps]
+    ins = [torch.empty_like(x) for x in sets[0]]
+    plan = binding.GroupPlan(prob, ins[0], ins[1:1 + w.gamma], ins[1 + w.gamma:], out["k_out"], out["v_out"], out["window_scores"],
+                             out["window_idx"], out["kept_len"], work, keep_capacity=out["keep_capacity"])
+    return w, refs, work, out, sets, ins, plan
+
+
+def test_every_replay_of_a_plan_that_moves_computes():
+    """Replays on two streams in turn, with other inputs and cleared outputs each time: each leaves what the direct call leaves
+    for the inputs it found."""
+    w, refs, work, out, sets, ins, plan = _plan_on_two_inputs()
+    names = ("window_scores", "window_idx", "kept_len")
+    results = [out[n] for n in names] + out["k_out"] + out["v_out"]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    left, turn = [], None
+    for i, at in enumerate((0, 0, 1, 0, 1, 1, 0)):
+        with torch.cuda.stream(streams[at]):
+            if turn:
+                turn.wait()                                  # what the test does to the buffers is the test's to order
+            for dst, src in zip(ins, sets[i % 2]):
+                dst.copy_(src)
+            for t in results:
+                t.view(torch.uint8).fill_(pu.FILL_BYTE)
+            plan.launch(stream=streams[at])
+            left.append([t.clone() for t in results])
+            turn = streams[at].record_event()
+    torch.cuda.synchronize()
+    assert binding.device_status(work) == 0
+    for i, got in enumerate(left):
+        ref = refs[i % 2]
+        for name, t in zip(names, got):
+            np.testing.assert_array_equal(t.cpu().numpy(), ref[name])
+        for t, r in zip(got[3:], ref["k_out"] + ref["v_out"]):
+            np.testing.assert_array_equal(binding.to_host_bits(t), r)
+    plan.close()
+
+
+def test_a_plan_that_moves_blocks_nobody():
+    """A replay on another stream than the one before is enqueued behind it and no more: the host goes on while the first has not
+    even begun, and a third stream may be under recording meanwhile."""
+    import time
+    w, refs, work, out, sets, ins, plan = _plan_on_two_inputs()
+    for dst, src in zip(ins, sets[0]):
+        dst.copy_(src)
+    first, second, third = (torch.cuda.Stream() for _ in range(3))
+    scratch, x = torch.zeros(16, device="cuda"), torch.zeros(64, device="cuda")
+    binding.wkv_probe_ex2_rate(scratch, 1, 1024, 1)
+    plan.launch(stream=first)
+    torch.cuda.synchronize()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    binding.wkv_probe_ex2_rate(scratch, sms, 1024, 400000, stream=first)            # 0.1 s ahead of the first replay
+    held, done = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    held.record(first)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(third):
+        graph.capture_begin(capture_error_mode="thread_local")
+        x.add_(1.0)
+        plan.launch(stream=first)
+        t0 = time.perf_counter()
+        plan.launch(stream=second)
+        seconds = time.perf_counter() - t0
+        x.add_(1.0)
+        graph.capture_end()
+    done.record(second)
+    torch.cuda.synchronize()
+    assert seconds < 0.03
+    assert held.elapsed_time(done) > 0
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(x.sum()) == 128.0
+    assert binding.device_status(work) == 0
+    np.testing.assert_array_equal(out["window_scores"].cpu().numpy(), refs[0]["window_scores"])
+    plan.close()

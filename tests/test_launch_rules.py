@@ -90,3 +90,40 @@ def test_nothing_that_a_block_may_wait_for_is_taken_ahead_of_the_kernel_in_front
     helper = source[source.index("void fetch_ahead("):]
     assert "fetch_ahead<" in ahead and "tmem_alloc" not in helper[:helper.index("score_windows_tc(")]
     assert source.count("tmem_alloc(") == 1
+
+
+@pytest.fixture(scope="module")
+def replays(tmp_path_factory):
+    nvcc = build._nvcc()
+    try:
+        subprocess.check_output([nvcc, "--version"])
+    except OSError:
+        pytest.skip("no nvcc")
+    so = str(tmp_path_factory.mktemp("fake-plan") / "libfakeplan.so")
+    subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=compute_100a", "-O0", "-std=c++17", "-Xcompiler", "-fPIC", "-shared",
+                           "-cudart", "none", "-Xlinker", "-Bsymbolic", "-I", os.path.join(build.ROOT, "include"), "-I", build.CSRC, "-o", so,
+                           os.path.join(build.CSRC, "group_plan.cu"), os.path.join(HERE, "fake_plan_runtime.cu")])
+    lib = ctypes.CDLL(so)
+
+    def run(script, failing=""):
+        log = ctypes.create_string_buffer(1024)
+        lib.fake_replays(script.encode(), failing.encode(), log, ctypes.c_size_t(1024))
+        return [step.strip() for step in log.value.decode().split("|")[:-1]]
+    return run
+
+
+A, B = "score:A gather:A record:A", "score:B gather:B record:B"
+
+
+@pytest.mark.parametrize("script,failing,steps", [
+    ("AA", "", [A, A]),
+    ("ABBA", "", [A, "wait:B " + B, B, "wait:A " + A]),      # ordered on the device, never on the host
+    ("ABB", "wait:B ", [A, "wait:B -", "wait:B " + B]),                    # a move that fails is made again
+    ("ABA", "gather:B ", [A, "wait:B score:B gather:B record:B -", "wait:A " + A]),     # what has been launched stays in the order
+    ("ABA", "score:B ", [A, "wait:B score:B -", A]),
+    ("A!BAB", "", [A, "graph:B -", A, "wait:B " + B]),                     # refused in a recording, and nothing lost
+    ("A1BB0A", "", [A, "wait:B graph:B", "wait:B graph:B", "wait:A graph:A"]),      # another device's stream: as a graph from then on
+])
+def test_replays_of_a_plan_follow_one_another(replays, script, failing, steps):
+    """A replay is put behind the one before it by an event, whatever streams the two are on; the host waits for nothing."""
+    assert replays(script, failing) == steps
