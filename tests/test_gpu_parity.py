@@ -1356,3 +1356,59 @@ def test_a_plan_that_moves_blocks_nobody():
     assert binding.device_status(work) == 0
     np.testing.assert_array_equal(out["window_scores"].cpu().numpy(), refs[0]["window_scores"])
     plan.close()
+
+
+# (In one wave, the shape of test_expired_wait_sets_the_status_word_and_the_context_survives[tc], a ticket that is none of the launch's
+# own is noticed at once and nothing waits for it.  In several waves the block that selects still does.)
+def test_expired_wait_of_the_score_kernel_in_several_waves():
+    """The ticket of unit 0 can never reach its target: the block that waits for it gives up after two seconds, those of the
+    next wave that wait for that block's statistics with it.  Each drains its loads, frees its tensor memory and ends; the status
+    bit is set, and on a zeroed workspace the same call is correct."""
+    w = small(batch=25, n_kv_heads=8, n_q_heads=16, max_seqlen=300, n_planted=0)          # 200 units: more than one wave holds
+    prob = binding.Problem.from_workload(w, score_impl=IMPLS["tc"])
+    grp = wl.make_group(w, 0)
+    ref = pu.run_gpu_group(w, grp, score_impl=IMPLS["tc"])
+    q, k = binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0])
+    work, out = prob.alloc_workspace(), prob.alloc_outputs(1, fill_byte=pu.FILL_BYTE)
+    ticket_off, _ = binding.workspace_sync_words(prob, 0)
+    work[ticket_off: ticket_off + 4].view(torch.int32)[0] = -1000000
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    start.record()
+    binding.wkv_select_leader_windows(prob, q, k, out["window_scores"], out["window_idx"], out["kept_len"], work)
+    end.record()
+    torch.cuda.synchronize()
+    assert binding.device_status(work) & 1
+    assert start.elapsed_time(end) > 1900                          # ms: it did wait
+    work.zero_()
+    binding.wkv_select_leader_windows(prob, q, k, out["window_scores"], out["window_idx"], out["kept_len"], work)
+    torch.cuda.synchronize()
+    assert binding.device_status(work) == 0
+    for name in ("window_scores", "window_idx", "kept_len"):
+        np.testing.assert_array_equal(out[name].cpu().numpy(), ref[name])
+
+
+@pytest.mark.parametrize("n_q_heads", [4, 8], ids=["128rows", "256rows"])
+def test_token_scores_of_blocks_that_stand_in(n_q_heads):
+    """Beside a kernel that holds two thirds of the SMs, the token scores of a unit of more blocks than are left have the bits that
+    they have alone."""
+    w = small(n_q_heads=n_q_heads, n_kv_heads=1, max_seqlen=17000, window=16, batch=1, l_obs=32)
+    grp = wl.make_group(w, 0)
+    prob = binding.Problem.from_workload(w)
+    q, k = binding.to_device(grp["q_obs"]), binding.to_device(grp["k_layers"][0])
+    scratch, other, mine = torch.zeros(16, device="cuda"), torch.cuda.Stream(), torch.cuda.Stream()
+    binding.wkv_probe_ex2_rate(scratch, 1, 1024, 1)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    got = []
+    for held in (False, True):
+        work, out = prob.alloc_workspace(), prob.alloc_outputs(1, fill_byte=pu.FILL_BYTE)
+        tokens = torch.full((1, 1, prob.nr_max), float("nan"), dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        if held:
+            binding.wkv_probe_ex2_rate(scratch, sms * 2 // 3, 1024, 40000, stream=other)
+        binding.wkv_score_windows(prob, q, k, out["window_scores"], tokens, work, stream=mine)
+        torch.cuda.synchronize()
+        assert binding.device_status(work) == 0
+        assert (binding.device_stand_ins(work)[0] > 0) == held
+        got.append((tokens, out["window_scores"]))
+    for a, b in zip(*got):
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32)) and not torch.isnan(a[..., : w.max_seqlen - w.l_obs]).any()
