@@ -157,7 +157,7 @@ size_t wkv_workspace_bytes(const wkv_shape *s);
 
 /* Byte offsets, inside the workspace of this shape, of the two words through which the blocks of a
  * launch synchronise on `unit` (a ticket count and, in the pipelined kernel, a count of arrived
- * statistics chunks; both are zero between launches).  Diagnostic helper (no counterpart in the paper): lets a test or a
+ * statistics chunks, in the tensor-core kernel a flag that its selection is left over; both are zero between launches).  Diagnostic helper (no counterpart in the paper): lets a test or a
  * debugger inspect or disturb the hand-over without knowing the workspace layout.  Either output
  * may be NULL.  The status word is always at byte 0. */
 int wkv_workspace_sync_words(const wkv_shape *s, int32_t unit, size_t *ticket_byte_offset,

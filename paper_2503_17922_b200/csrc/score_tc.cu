@@ -1158,8 +1158,8 @@ int launch_score_tc(const KShape &ks, const void *q, const void *k, float *windo
     const int mb = ks.R > 128 ? 2 : 1;
     const int threads = block_threads(mb);
     const size_t smem = tc_smem_bytes(a.kblocks, mb);
-    // persistent blocks, one per SM at most; every block of a cooperative launch is resident, which
-    // the hand-over of the statistics between the sweeps relies on
+    // persistent blocks, one per SM at most.  With several waves the hand-over of the statistics between the sweeps relies on
+    // all being resident, which a cooperative launch sees to; in one wave nothing does.
     int grid = plan.units_per_wave * plan.chunks_per_unit;
     if (grid > di.sm_count) grid = di.sm_count;
     const int form = grid < plan.units_per_wave * plan.chunks_per_unit ? 0 : (plan.units_per_wave < units ? 1 : 2);

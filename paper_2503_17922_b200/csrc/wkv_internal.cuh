@@ -106,7 +106,7 @@ struct Workspace {
 
 // words of the synchronisation area before the per-unit words; unit u owns four words from
 // sync[kSyncTickets + 4u]: ticket count, and in the pipelined kernel arrivals of the statistics sweep, "selection
-// published" flag and gather job counter
+// published" flag and gather job counter; the second is the "selection left over" flag of the tensor-core kernel of one wave
 constexpr int kSyncTickets = 16;
 constexpr int kSyncWordsPerUnit = 4;
 // The area has room for at least this many units whatever the shape (32 KB), so that what lies behind it never lands on
