@@ -441,11 +441,11 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
     auto head_of = [&](int r) { return (int)((unsigned)r * a.alpha_inverse >> 16); };
     auto make_item = [&](int unit, int chunk, int review_only, Item &im) { set_item(a, unit, chunk, review_only, im); };
 
-    // Called by every warp except the producer; ends with a barrier among those warps.  Four loads
-    // are in flight per thread.  The producer starts streaming key tiles once these small loads
+    // Called by every warp except the producer; ends with a barrier among those warps.  The compute warps load, four loads
+    // in flight per thread.  The producer starts streaming key tiles once these small loads
     // have been ISSUED (go_producer): a tile burst issued first would sit in front of them in the
     // SM's memory pipeline for microseconds.
-    constexpr int kLoaders = kThreads - 32;
+    constexpr int kLoaders = kThreads - 64;               // the compute warps
     auto go_producer = [&]() { asm volatile("bar.arrive 2, %0;" ::"n"(kThreads) : "memory"); };
     auto load_q_image = [&](const Item &im, bool signal) {
         if (ONE ? q_unit_loaded < 0 : q_unit_loaded != im.unit) {
@@ -453,9 +453,21 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
             const bool first = q_unit_loaded < 0;      // the number is raised while the launch runs: it is read once
             if (first && threadIdx.x == 32) launches = launches_so_far(a.count);
             const __nv_bfloat16 *q_unit = q + im.b * s.qsb + (long long)im.h * s.G * s.qsh;
-            const int loader = late((int)threadIdx.x) - 32;
             const int vshift = s.d == 128 ? 4 : 3;            // log2(16-byte vectors per row)
             const int total = q_rows << vshift;
+            const int loader = warp == 1 ? total : late((int)threadIdx.x) - 64;
+            if (warp == 1) {
+                if (signal) go_producer();
+                // The warp that issues the MMAs takes tensor memory meanwhile, at the block's first item and so behind the wait for
+                // the kernel in front: a block of that kernel which shares the SM and has yet to take its own would wait for
+                // this one, which waits for that kernel.  That takes as long as the loads, so it comes first: groups of 8 heads, us,
+                // ahead of the wait / so / behind a share of the loads / behind the barrier below: 4,096 keys 16.35 / 16.29 / 16.40 /
+                // 16.50, 8,192 23.98 / 23.80 / 23.99 / -, selection and four gathers of 32,768 keys, given normalisers 49.3 / 49.4 / 49.5 / -.
+                if (first) {
+                    __syncwarp();
+                    tmem_alloc(&sh.tmem_base, kTmemCols);
+                }
+            }
             for (int base = loader; base < total; base += kLoaders * 4) {
                 int4 v[4];
 #pragma unroll
@@ -471,11 +483,6 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                     }
                 }
                 if (signal && base == loader) go_producer();
-                // The warp that issues the MMAs takes tensor memory, and does so behind the wait for the kernel in front: a
-                // block of that kernel which shares the SM and has yet to take its own would wait for this one, which waits
-                // for that kernel.  Here its share of Q is on its way: a group of 8 heads x 4,096 keys takes 16.4 us as with tensor memory
-                // taken ahead of the wait, 16.6 with it taken behind the barrier below; given normalisers cost 0.2 of 49 us.
-                if (first && base == loader && threadIdx.x < 64) tmem_alloc(&sh.tmem_base, kTmemCols);
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int idx = base + u * kLoaders;
@@ -485,10 +492,10 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                     }
                 }
             }
-            if (signal && loader >= total) go_producer();   // a thread without a share of the image
+            if (signal && warp != 1 && loader >= total) go_producer();   // a thread without a share of the image
             fence_proxy_async_smem();
             if (first && threadIdx.x == 32) sh.tag = launch_tag(launches, a.salt);
-            asm volatile("bar.sync 1, %0;" ::"n"(kLoaders) : "memory");
+            asm volatile("bar.sync 1, %0;" ::"n"(kLoaders + 32) : "memory");
         } else if (signal) {
             go_producer();
         }
