@@ -466,6 +466,7 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
                 if (first) {
                     __syncwarp();
                     tmem_alloc(&sh.tmem_base, kTmemCols);
+                    asm volatile("bar.arrive 4, 64;" ::: "memory");
                 }
             }
             for (int base = loader; base < total; base += kLoaders * 4) {
@@ -508,6 +509,8 @@ __device__ __forceinline__ void take_wave(const CUtensorMap *tmap, const TcArgs 
         for (int t = t_begin; t < t_end; ++t) {
             const uint32_t g = it + t;
             const int st = g % kStages;
+            // (the limit of the waits counts from when tensor memory has been had: another kernel on the SM may hold it)
+            if (g == kStages) asm volatile("bar.sync 4, 64;" ::: "memory");
             if (g >= kStages && !mbar_wait(&bar.empty[st], ((g / kStages) - 1) & 1, &sh.abort)) return;
             if (im.reuse && t < kStages) {
                 // the stage holds this tile already: complete the phase without a load
